@@ -759,7 +759,7 @@ struct BatchLayout {
 spgemm_status batch_layout(int n, const spgemm_csr* As, const spgemm_csr* Bs, const spgemm_opts& o,
                            BatchLayout* L, std::vector<sg::BatchDesc>* desc) {
   if (n < 0 || (n > 0 && (!As || !Bs))) return SPGEMM_ERR_INVALID_ARG;
-  long long rows = 0, ks = 0, ncols = 0, an = 0, bn = 0;
+  long long rows = 0, ks = 0, ncols = 0, ncols_max = 0, an = 0, bn = 0;
   if (desc) desc->resize((size_t)n);
   for (int i = 0; i < n; ++i) {
     spgemm_status s;
@@ -772,9 +772,10 @@ spgemm_status batch_layout(int n, const spgemm_csr* As, const spgemm_csr* Bs, co
       D.b_rp = Bs[i].row_ptr; D.b_ci = Bs[i].col_idx; D.b_v = Bs[i].vals;
       D.m = As[i].nrows; D.k = As[i].ncols; D.n = Bs[i].ncols;
       D.a_nnz = As[i].nnz; D.b_nnz = Bs[i].nnz;
-      D.roff = rows; D.koff = ks; D.noff = ncols; D.aoff = an; D.boff = bn;
+      D.roff = rows; D.koff = ks; D.aoff = an; D.boff = bn;
     }
     rows += As[i].nrows; ks += As[i].ncols; ncols += Bs[i].ncols; an += As[i].nnz; bn += Bs[i].nnz;
+    if (Bs[i].ncols > ncols_max) ncols_max = Bs[i].ncols;
   }
   const long long lim = (1ll << 31) - 1;
   if (rows >= lim || ks >= lim || ncols >= lim || an >= lim || bn >= lim) return SPGEMM_ERR_INDEX_OVERFLOW;
@@ -790,7 +791,7 @@ spgemm_status batch_layout(int n, const spgemm_csr* As, const spgemm_csr* Bs, co
   L->bounds = off; off = align_up(off + sizeof(int32_t) * (size_t)(n + 1));
   L->plan = off;
   L->A = spgemm_csr{rows, ks, an, nullptr, nullptr, nullptr};
-  L->B = spgemm_csr{ks, ncols, bn, nullptr, nullptr, nullptr};
+  L->B = spgemm_csr{ks, ncols_max, bn, nullptr, nullptr, nullptr};  // every instance's own columns
   // the inner plan's size depends only on the stacked shapes
   L->A.row_ptr = (const int32_t*)16;
   L->B.row_ptr = (const int32_t*)16;
@@ -904,11 +905,9 @@ spgemm_status spgemm_batch_numeric(spgemm_batch* b, const int32_t* c_row_ptr, in
   if (b->plan->nnz_c == 0) return SPGEMM_OK;
   if (!c_col_idx || !c_vals) return SPGEMM_ERR_INVALID_ARG;
   sg::LaunchCtx c = ctx_of(b->plan, stream);
-  if (sg::launch_stack_values(c, b->n, b->dtype, b->d_desc, b->a_v, b->b_v) != cudaSuccess) return SPGEMM_ERR_CUDA;
-  spgemm_status s = spgemm_numeric(b->plan, b->a_v, b->b_v, c_row_ptr, c_col_idx, c_vals, stream);
-  if (s != SPGEMM_OK) return s;
-  if (sg::launch_unstack_columns(c, b->n, b->d_desc, c_row_ptr, c_col_idx) != cudaSuccess) return SPGEMM_ERR_CUDA;
-  return SPGEMM_OK;
+  if (sg::launch_stack_values(c, b->n, b->dtype, b->d_desc, b->a_v, b->b_v, b->a_nnz, b->b_nnz) != cudaSuccess)
+    return SPGEMM_ERR_CUDA;
+  return spgemm_numeric(b->plan, b->a_v, b->b_v, c_row_ptr, c_col_idx, c_vals, stream);
 }
 
 spgemm_status spgemm_batch_capture(spgemm_batch* b, const int32_t* c_row_ptr, int32_t* c_col_idx, void* c_vals,
@@ -967,6 +966,7 @@ spgemm_status spgemm_batch_products(int32_t n, const spgemm_csr* As, const spgem
   spgemm_batch_products_workspace_size(n, &need);
   if (!workspace || workspace_bytes < need || ((uintptr_t)workspace) % 16) return SPGEMM_ERR_WORKSPACE;
   std::vector<sg::BatchDesc> desc((size_t)n);
+  long long total_a_nnz = 0;
   for (int i = 0; i < n; ++i) {
     spgemm_status s;
     if ((s = check_csr(&As[i])) != SPGEMM_OK) return s;
@@ -976,6 +976,8 @@ spgemm_status spgemm_batch_products(int32_t n, const spgemm_csr* As, const spgem
     D = sg::BatchDesc{};
     D.a_rp = As[i].row_ptr; D.a_ci = As[i].col_idx; D.b_rp = Bs[i].row_ptr; D.b_ci = Bs[i].col_idx;
     D.m = As[i].nrows; D.k = As[i].ncols; D.n = Bs[i].ncols; D.a_nnz = As[i].nnz; D.b_nnz = Bs[i].nnz;
+    D.aoff = total_a_nnz;
+    total_a_nnz += As[i].nnz;
   }
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return SPGEMM_ERR_CUDA;
@@ -986,7 +988,7 @@ spgemm_status spgemm_batch_products(int32_t n, const spgemm_csr* As, const spgem
   if (cudaMemcpyAsync(workspace, desc.data(), sizeof(sg::BatchDesc) * (size_t)n, cudaMemcpyHostToDevice,
                       c.stream) != cudaSuccess)
     return SPGEMM_ERR_CUDA;
-  if (sg::launch_batch_products(c, n, (const sg::BatchDesc*)workspace, (long long*)products) != cudaSuccess)
+  if (sg::launch_batch_products(c, n, (const sg::BatchDesc*)workspace, total_a_nnz, (long long*)products) != cudaSuccess)
     return SPGEMM_ERR_CUDA;
   return SPGEMM_OK;
 }

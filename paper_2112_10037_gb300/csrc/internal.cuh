@@ -325,16 +325,17 @@ struct BatchDesc {
   const void* b_v;
   long long m, k, n;     // A_i is m x k, B_i is k x n
   long long a_nnz, b_nnz;
-  long long roff, koff, noff, aoff, boff;  // offsets in the stacked arrays
+  long long roff, koff, aoff, boff;  // offsets in the stacked arrays
 };
 cudaError_t launch_stack_structure(const LaunchCtx& c, int n, const BatchDesc* d, long long total_rows,
                                    long long total_k, int32_t* a_rp, int32_t* a_ci, int32_t* b_rp, int32_t* b_ci,
                                    long long total_a_nnz, long long total_b_nnz);
-cudaError_t launch_stack_values(const LaunchCtx& c, int n, int dtype, const BatchDesc* d, void* a_v, void* b_v);
-cudaError_t launch_unstack_columns(const LaunchCtx& c, int n, const BatchDesc* d, const int32_t* c_rp, int32_t* c_ci);
+cudaError_t launch_stack_values(const LaunchCtx& c, int n, int dtype, const BatchDesc* d, void* a_v, void* b_v,
+                                long long total_a_nnz, long long total_b_nnz);
 cudaError_t launch_batch_bounds(const LaunchCtx& c, int n, const BatchDesc* d, const int32_t* c_rp, long long total_rows,
                                 int32_t* out);
-cudaError_t launch_batch_products(const LaunchCtx& c, int n, const BatchDesc* d, long long* products);
+cudaError_t launch_batch_products(const LaunchCtx& c, int n, const BatchDesc* d, long long total_a_nnz,
+                                  long long* products);
 
 // Split (heavy) rows: list positions [*hs, *hs + return value) -- the rows of
 // bins [heavy_bin, hi_bin], at most hcap of them; split row h of both passes
