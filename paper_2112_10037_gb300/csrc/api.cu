@@ -73,7 +73,7 @@ size_t transpose_layout(size_t off, long long n, long long nnz, int vbytes, size
   return off;
 }
 
-int numeric_block_bin(const spgemm_opts& o);
+int numeric_block_bin(const spgemm_opts& o, long long ncols_b);
 
 // Last bin of the register-sort path: rows of at most 128, 256 or 512
 // products (opts.sort_max; bin b holds products in (2^(b-2), 2^(b-1)]).
@@ -109,7 +109,7 @@ int small_hi_bin(const spgemm_opts& o) {
 void split_geometry(const spgemm_opts& o, int window, long long mloc, long long ncols_b, sg::SplitInfo* sp,
                     size_t* hcnt_entries) {
   sp->heavy_bin = sg::NBINS;
-  sp->hi_bin = numeric_block_bin(o) - 1;  // the warp kernel's last bin
+  sp->hi_bin = numeric_block_bin(o, ncols_b) - 1;  // the warp kernel's last bin
   if (sp->hi_bin > sg::NBINS - 1) sp->hi_bin = sg::NBINS - 1;
   sp->hcap = 0;
   sp->wf_shift = 0;
@@ -118,7 +118,7 @@ void split_geometry(const spgemm_opts& o, int window, long long mloc, long long 
   *hcnt_entries = 0;
   if (o.split_min < 0 || o.force_path >= 0 || mloc <= 0 || sp->ntf < 2) return;
   const long long smin = o.split_min > 0 ? o.split_min : 131072;
-  if (sg::bin_of(smin) + 1 >= numeric_block_bin(o)) return;  // those rows use the block window
+  if (sg::bin_of(smin) + 1 >= numeric_block_bin(o, ncols_b)) return;  // those rows use the block window
   long long cap = mloc < 16384 ? mloc : 16384;
   const long long lim = ((long long)1 << 24) / sp->ntf;
   if (cap > lim) cap = lim;
@@ -132,13 +132,22 @@ void split_geometry(const spgemm_opts& o, int window, long long mloc, long long 
   *hcnt_entries = (size_t)cap * (size_t)sp->ntf;
 }
 
-// First bin of rows whose numeric pass uses the block-wide window.
-int numeric_block_bin(const spgemm_opts& o) {
+// First bin of rows whose numeric pass uses the block-wide window: by default
+// rows of more than 2048 products per window of B's columns, within 8192 to
+// 65,536.  (A window costs the block a few thousand cycles whatever it holds;
+// a warp that owns a whole row of 65,536 products over two windows runs alone
+// long after the other rows are done: on a graph of 12,345 vertices the warp
+// window took 1.15 ms for the rows of 8,193 to 65,536 products.)
+int numeric_block_bin(const spgemm_opts& o, long long ncols_b) {
   if (o.force_path == 1 || o.force_path == 3) return sg::NBINS;  // warp window only
   if (o.force_path == 2) return tiny_hi_bin(o) + 1;                 // every row above the register sort
   if (o.force_path == 4) return 1;                                 // every non-empty row
   if (o.num_block_min < 0) return sg::NBINS;
-  const long long m = o.num_block_min > 0 ? o.num_block_min : 65536;
+  long long m = o.num_block_min;
+  if (m == 0) {
+    m = 2048 * ((ncols_b + 8191) / 8192);
+    m = m < 8192 ? 8192 : (m > 65536 ? 65536 : m);
+  }
   const int b = sg::bin_of(m) + 1;
   return b < small_hi_bin(o) + 1 ? small_hi_bin(o) + 1 : b;
 }
@@ -151,6 +160,14 @@ int numeric_rank_bin(const spgemm_opts& o) {
   const long long m = o.rank_min;
   const int b = sg::bin_of(m) + 1;
   return b < small_hi_bin(o) + 1 ? small_hi_bin(o) + 1 : b;
+}
+
+// Last bin of the rows whose numeric pass keeps every product in registers
+// (numonce.cuh: at most 8192 products); 0 when off: a forced path, or the
+// warp window asked for by its width.
+int numeric_once_bin(const spgemm_opts& o) {
+  if (o.force_path >= 0 || o.window_warp > 0) return 0;
+  return sg::bin_of(8192);
 }
 
 int numeric_window(const spgemm_opts& o) {
@@ -182,7 +199,7 @@ Layout layout_for(const spgemm_opts& o, long long mloc, long long nnz_a, long lo
   }
   L.hcnt = off; off = align_up(off + sizeof(int32_t) * nh);
   L.rrb = L.runsb = 0;
-  if (own_b && numeric_block_bin(o) < sg::NBINS) {  // run list at the block window's width
+  if (own_b && numeric_block_bin(o, ncols_b) < sg::NBINS) {  // run list at the block window's width
     L.rrb = off; off = align_up(off + sizeof(int32_t) * (size_t)(nrows_b + 1));
     L.runsb = off; off = align_up(off + sizeof(int2) * (size_t)(nnz_b + nrows_b + sg::RUNS_PAD));
   }
@@ -237,14 +254,15 @@ static void block_geometry(const spgemm_opts& o, int* w, int* nw) {
 }
 
 // Bin ranges of the paths from the options (see sg::bin_of for the bins).
-void choose_paths(const spgemm_opts& o, sg::PathBins* pb, sg::Tuning* tu) {
+void choose_paths(const spgemm_opts& o, long long ncols_b, sg::PathBins* pb, sg::Tuning* tu) {
   const int last = sg::NBINS - 1;
   tu->warp_max = o.warp_max > 0 ? o.warp_max : 8192;
   tu->window_warp = numeric_window(o);
   block_geometry(o, &tu->window_block, &tu->block_warps);
   const int HASH_HI = hash_hi_bin(o);
   tu->hash_max = HASH_HI > 0 ? 1 << (HASH_HI - 1) : 0;
-  tu->num_lo_block = numeric_block_bin(o);
+  tu->num_hi_once = numeric_once_bin(o);
+  tu->num_lo_block = numeric_block_bin(o, ncols_b);
   tu->num_lo_rank = numeric_rank_bin(o);
   tu->rank_accum = o.rank_accum == 1 ? 1 : 0;
   const int TINY_HI = tiny_hi_bin(o);  // register sort up to opts.sort_max products
@@ -368,10 +386,11 @@ static spgemm_status analyse_impl(const spgemm_csr* A, const spgemm_csr* B, cons
   p->cursor = (int32_t*)(p->ws + L.cursor);
   p->nxt = (int32_t*)(p->ws + L.nxt);
   p->scan_part = (long long*)(p->ws + L.scan);
-  choose_paths(o, &p->pb, &p->tu);
+  choose_paths(o, B->ncols, &p->pb, &p->tu);
   {
     size_t nh = 0;
     split_geometry(o, p->tu.window_warp, p->mloc, B->ncols, &p->sp, &nh);
+    if (nh && p->tu.num_hi_once >= p->sp.heavy_bin) p->tu.num_hi_once = p->sp.heavy_bin - 1;  // split rows: warp window
     p->sp.hcnt = nh ? (int32_t*)(p->ws + L.hcnt) : nullptr;
     p->sp.wb_shift = 0;
     while ((1 << p->sp.wb_shift) < p->tu.window_block) ++p->sp.wb_shift;
@@ -405,6 +424,7 @@ static spgemm_status analyse_impl(const spgemm_csr* A, const spgemm_csr* B, cons
     int win_lo = sg::NBINS;
     for (int q : {sg::PATH_WARP, sg::PATH_BLOCK})
       if (p->pb.hi[q] >= p->pb.lo[q] && p->pb.lo[q] < win_lo) win_lo = p->pb.lo[q];
+    if (p->tu.num_hi_once >= win_lo) win_lo = p->tu.num_hi_once + 1;
     if (rb != 0 || re != A->nrows) win_lo = 0;
     e = sg::launch_runs(c, p->B, p->sp, p->runs_part, win_lo);
   }

@@ -85,6 +85,7 @@ struct Tuning {
   int window_block;    // numeric window width (columns) of the block accumulator
   int hash_max;        // largest P of the hash path (0: path disabled)
   int warp_max;        // largest P of the symbolic warp path
+  int num_hi_once;     // numeric bins <= this (above the small-row bins) keep a row in registers (0: none)
   int num_lo_block;    // numeric bins >= this use the block kernel (NBINS: never)
   int num_lo_rank;     // numeric bins >= this (below num_lo_block) use the rank kernel (NBINS: never)
   int rank_accum;      // 0: rank kernel values reduced in global memory; 1: in shared-memory chunks

@@ -29,13 +29,19 @@ int kernel_blocks_per_sm(Kern kernel, int threads, size_t smem) {
     auto it = cache.find(key);
     if (it != cache.end()) return it->second;
   }
+  std::lock_guard<std::mutex> g(mu);
   if (smem > 48 * 1024) {
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-      return 0;
+    // a kernel launched with several sizes keeps the largest opt-in
+    static std::unordered_map<unsigned long long, size_t> opted;
+    size_t& most = opted[((unsigned long long)(uintptr_t)(const void*)kernel) ^ ((unsigned long long)dev << 58)];
+    if (smem > most) {
+      if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        return 0;
+      most = smem;
+    }
   }
   int n = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, smem) != cudaSuccess) n = 0;
-  std::lock_guard<std::mutex> g(mu);
   cache[key] = n;
   return n;
 }

@@ -8,6 +8,7 @@
 
 #include "launch_util.cuh"
 #include "numblock.cuh"
+#include "numonce.cuh"
 #include "numrank.cuh"
 #include "numwarp.cuh"
 #include "rowhash.cuh"
@@ -72,6 +73,43 @@ static cudaError_t hash_dispatch(const int* hist, int lo, int hi, F1 f1, F2 f2, 
   if ((e = clip(7, 7, f2))) return e;
   if ((e = clip(8, 8, f4))) return e;
   return cudaSuccess;
+}
+
+template <typename T, int NT, int SR>
+static cudaError_t once_num(const LaunchCtx& c, const Csr& A, const Csr& B, const T* av, const T* bv,
+                            const RowInfo& ri, int lo, int hi, const int32_t* c_rp, int32_t* c_ci, T* c_v,
+                            const int* hist) {
+  auto k = k_num_once<NT, T, SR>;
+  int wlog = 10;  // the narrowest bitmap that holds a row of B, up to the widest
+  while (wlog < once_wlog_max<NT>() && (1ll << wlog) < B.ncols) ++wlog;
+  const size_t smem = once_smem_bytes<NT, T>(wlog);
+  const int occ = kernel_blocks_per_sm(k, NT, smem);
+  if (occ <= 0) return cudaErrorInvalidConfiguration;
+  long long rows = hist ? 0 : -1;
+  for (int b = lo; hist && b <= hi; ++b) rows += hist[b];
+  const int grid = persistent_grid(rows, 1, c.nsm, occ);
+  k<<<grid, NT, smem, c.stream>>>(A, B, av, bv, ri, c.st, lo, hi, wlog, c_rp, c_ci, c_v, c.err);
+  count_launch(c);
+  return cudaGetLastError();
+}
+
+// Bins lo..hi (at most 8192 products) by the threads whose registers hold a
+// row: 64 threads up to 512 products, then twice the threads per bin.
+template <typename T, int SR>
+static cudaError_t once_dispatch(const LaunchCtx& c, const Csr& A, const Csr& B, const T* av, const T* bv,
+                                 const RowInfo& ri, int lo, int hi, const int32_t* c_rp, int32_t* c_ci, T* c_v,
+                                 const int* hist) {
+  cudaError_t e = cudaSuccess;
+  auto clip = [&](int a, int b, auto f) {
+    const int l = lo > a ? lo : a, h = hi < b ? hi : b;
+    if (e == cudaSuccess && l <= h && !empty_bins(hist, l, h)) e = f(c, A, B, av, bv, ri, l, h, c_rp, c_ci, c_v, hist);
+  };
+  clip(14, 14, once_num<T, 1024, SR>);  // longest rows first
+  clip(13, 13, once_num<T, 512, SR>);
+  clip(12, 12, once_num<T, 256, SR>);
+  clip(11, 11, once_num<T, 128, SR>);
+  clip(1, 10, once_num<T, 64, SR>);
+  return e;
 }
 
 template <typename T, int W, int SR>
@@ -281,11 +319,17 @@ static cudaError_t numeric_t(const LaunchCtx& c, const Csr& A, const Csr& B, con
   }
   if (hi >= lo && !empty_bins(hist, lo, hi)) {
     timer_mark(c, T_NUM_WARP, 0);
-    switch (SR == SPGEMM_PLUS_TIMES ? tu.window_warp : 1024) {
-      case 2048: e = warp_num<T, 2048, SR>(c, A, B, av, bv, ri, lo, hi, sp, cur, nxt, c_rp, c_ci, c_v, rows_wide); break;
-      case 4096: e = warp_num<T, 4096, SR>(c, A, B, av, bv, ri, lo, hi, sp, cur, nxt, c_rp, c_ci, c_v, rows_wide); break;
-      default: e = warp_num<T, 1024, SR>(c, A, B, av, bv, ri, lo, hi, sp, cur, nxt, c_rp, c_ci, c_v, rows_wide); break;
+    if (tu.num_hi_once >= lo) {  // rows whose products fit a block's registers
+      const int ohi = hi < tu.num_hi_once ? hi : tu.num_hi_once;
+      e = once_dispatch<T, SR>(c, A, B, av, bv, ri, lo, ohi, c_rp, c_ci, c_v, hist);
+      lo = ohi + 1;
     }
+    if (!e && hi >= lo && !empty_bins(hist, lo, hi))
+      switch (SR == SPGEMM_PLUS_TIMES ? tu.window_warp : 1024) {
+        case 2048: e = warp_num<T, 2048, SR>(c, A, B, av, bv, ri, lo, hi, sp, cur, nxt, c_rp, c_ci, c_v, rows_wide); break;
+        case 4096: e = warp_num<T, 4096, SR>(c, A, B, av, bv, ri, lo, hi, sp, cur, nxt, c_rp, c_ci, c_v, rows_wide); break;
+        default: e = warp_num<T, 1024, SR>(c, A, B, av, bv, ri, lo, hi, sp, cur, nxt, c_rp, c_ci, c_v, rows_wide); break;
+      }
     timer_mark(c, T_NUM_WARP, 1);
     if (e) return e;
   }
