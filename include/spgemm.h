@@ -89,7 +89,9 @@ typedef struct spgemm_opts {
                           force_path >= 0 or sort_max is 256 or 512.  Rows of at most
                           16 products always use the register sort */
   int32_t window_warp; /* columns of the numeric dense window (one per warp):
-                          1024, 2048 or 4096 (0: default 1024) */
+                          1024, 2048 or 4096 (0: default 1024).  With 1024, rows of up
+                          to 8192 products that no other option routes elsewhere keep
+                          their products in a block's registers instead */
   int32_t window_block;/* columns of the numeric block window, with block_warps one of
                           the pairs (2048, 4), (2048, 8), (4096, 4), (4096, 8),
                           (4096, 16), (8192, 8), (8192, 16), (16384, 16); 0 or any
@@ -101,8 +103,9 @@ typedef struct spgemm_opts {
   int32_t backward;    /* nonzero: the plan also keeps the transpose of A's structure,
                           which spgemm_backward needs (more workspace) */
   int32_t num_block_min;/* rows with more products than this run the numeric pass
-                          with a block-wide window (0: default 65536; -1: never, then
-                          heavy rows are split as split_min says) */
+                          with a block-wide window (0: 2048 products per 8192 columns
+                          of B, at least 8192 and at most 65536; -1: never, then heavy
+                          rows are split as split_min says) */
   int32_t block_warps; /* warps sharing a numeric block window (see window_block) */
   int32_t sort_max;    /* rows of at most this many products are merged by a sort in
                           registers: 128, 256 or 512 (0: 128); rows of 17 or more

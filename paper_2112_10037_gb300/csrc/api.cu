@@ -163,10 +163,10 @@ int numeric_rank_bin(const spgemm_opts& o) {
 }
 
 // Last bin of the rows whose numeric pass keeps every product in registers
-// (numonce.cuh: at most 8192 products); 0 when off: a forced path, or the
-// warp window asked for by its width.
+// (numonce.cuh: at most 8192 products); 0 when off: a forced path, or a warp
+// window of another width than the default asked for.
 int numeric_once_bin(const spgemm_opts& o) {
-  if (o.force_path >= 0 || o.window_warp > 0) return 0;
+  if (o.force_path >= 0 || o.window_warp == 2048 || o.window_warp == 4096) return 0;
   return sg::bin_of(8192);
 }
 
