@@ -247,9 +247,11 @@ spgemm_status spgemm_plan_check(spgemm_plan* plan, spgemm_stream_t stream);
  * of A's nonzeros; entries of rows outside the plan's row range are left
  * untouched) and db_vals (aligned with B's col_idx; sums over the plan's
  * rows only) are overwritten; either may be NULL to skip it.  Each output is
- * summed in a fixed order -- one fused multiply-add chain when it has at most
- * 128 terms, otherwise 32 lane chains added by a fixed shuffle tree -- so the
- * result is deterministic (the same bits on every call).
+ * summed in a fixed order (chains of fused multiply-adds and fixed trees of
+ * additions), so the result is deterministic (the same bits on every call).
+ * db_vals uses a buffer of at most 128 MB in the plan's workspace: calls on
+ * one plan follow one another on the GPU whatever streams they are given; a
+ * graph captured from this call must not run beside another of the plan's.
  * Does not block, allocates nothing. */
 spgemm_status spgemm_backward(spgemm_plan* plan, const void* a_vals, const void* b_vals,
                               const int32_t* c_row_ptr, const int32_t* c_col_idx,

@@ -31,6 +31,13 @@ struct spgemm_plan {
   int32_t* at_src = nullptr;
   int32_t* a_row = nullptr;  // row of every nonzero of A (backward)
   int32_t* b_row = nullptr;  // row of every entry of B (backward)
+  // product offsets and the product buffer (backward)
+  long long *row_off = nullptr, *p_off = nullptr, *t_off = nullptr;
+  void* grad_buf = nullptr;
+  long long grad_buf_entries = 0;
+  std::mutex grad_mu;                // calls that use the buffer follow one another
+  cudaEvent_t grad_done = nullptr;   // end of the last one outside a capture
+  cudaStream_t grad_stream = nullptr;
   // host state
   sg::PathBins pb{};
   sg::Tuning tu{};
@@ -48,6 +55,7 @@ struct spgemm_plan {
   ~spgemm_plan() {
     for (auto& ev : timers)
       if (ev) cudaEventDestroy(ev);
+    if (grad_done) cudaEventDestroy(grad_done);
   }
 };
 
@@ -59,6 +67,8 @@ inline size_t align_up(size_t x) { return (x + ALIGN - 1) & ~(ALIGN - 1); }
 struct Layout {
   size_t st, prod, cmin, cmax, rows, cursor, nxt, scan, rr, runs, runs_part, hcnt, rrb, runsb;
   size_t at_rp, at_ci, at_src, at_tmp, at_table, at_part, a_row, b_row;  // opts.backward only
+  size_t row_off, off_part, p_off, t_off, gbuf;  // opts.backward, and rows of B that fit the product buffer
+  long long gbuf_entries;
   size_t total;
 };
 
@@ -210,6 +220,15 @@ Layout layout_for(const spgemm_opts& o, long long mloc, long long nnz_a, long lo
     L.a_row = off; off = align_up(off + sizeof(int32_t) * (size_t)nnz_a);
     L.b_row = off; off = align_up(off + sizeof(int32_t) * (size_t)nnz_b);
     off = transpose_layout(off, nrows_b, nnz_a, 0, &L.at_tmp, &L.at_table, &L.at_part);
+    const int vb = o.dtype == SPGEMM_F32 ? 4 : 8;
+    L.gbuf_entries = sg::grad_buffer_entries(nnz_a, nnz_b, ncols_b, vb);
+    if (L.gbuf_entries > 0) {
+      L.row_off = off; off = align_up(off + sizeof(long long) * (size_t)(mloc + 1));
+      L.off_part = off; off = align_up(off + sizeof(long long) * sg::scan_partials_count(mloc));
+      L.p_off = off; off = align_up(off + sizeof(long long) * (size_t)nnz_a);
+      L.t_off = off; off = align_up(off + sizeof(long long) * (size_t)nnz_a);
+      L.gbuf = off; off = align_up(off + (size_t)vb * (size_t)L.gbuf_entries);
+    }
   }
   L.total = off;
   return L;
@@ -439,6 +458,15 @@ static spgemm_status analyse_impl(const spgemm_csr* A, const spgemm_csr* B, cons
     p->b_row = (int32_t*)(p->ws + L.b_row);
     if (e == cudaSuccess) e = sg::launch_row_index(c, A->row_ptr, A->nrows, p->a_row);
     if (e == cudaSuccess) e = sg::launch_row_index(c, B->row_ptr, B->nrows, p->b_row);
+    if (e == cudaSuccess && L.gbuf_entries > 0) {
+      p->row_off = (long long*)(p->ws + L.row_off);
+      p->p_off = (long long*)(p->ws + L.p_off);
+      p->t_off = (long long*)(p->ws + L.t_off);
+      p->grad_buf = p->ws + L.gbuf;
+      p->grad_buf_entries = L.gbuf_entries;
+      e = sg::launch_grad_offsets(c, p->A, p->B, p->row_begin, p->mloc, p->prod, p->at_ci, p->at_src, p->row_off,
+                                  (long long*)(p->ws + L.off_part), p->p_off, p->t_off);
+    }
   }
   if (e != cudaSuccess) { delete p; return SPGEMM_ERR_CUDA; }
   *plan = p;
@@ -651,13 +679,41 @@ spgemm_status spgemm_backward(spgemm_plan* p, const void* a_vals, const void* b_
   if (!c_row_ptr || (p->nnz_c > 0 && (!c_col_idx || !dc_vals))) return SPGEMM_ERR_INVALID_ARG;
   if ((da_vals && p->B.nnz > 0 && !b_vals) || (db_vals && p->A.nnz > 0 && !a_vals)) return SPGEMM_ERR_INVALID_ARG;
   sg::LaunchCtx c = ctx_of(p, stream);
+  // rows outside the plan's range keep their dA; a plan without rows zeroes dB
   cudaError_t e = cudaSuccess;
-  // rows outside the plan's range keep their dA; zero nothing else
-  if (db_vals && p->B.nnz > 0)
+  if (db_vals && p->B.nnz > 0 && p->mloc <= 0)
     e = cudaMemsetAsync(db_vals, 0, (size_t)p->B.nnz * (p->opts.dtype == SPGEMM_F32 ? 4 : 8), c.stream);
-  if (e == cudaSuccess)
-    e = sg::launch_backward(c, p->opts.dtype, p->A, p->B, p->row_begin, p->mloc, a_vals, b_vals, p->a_row, p->b_row,
-                            p->at_rp, p->at_ci, p->at_src, c_row_ptr, c_col_idx, dc_vals, da_vals, db_vals);
+  sg::GradArgs g;
+  g.A = p->A;
+  g.B = p->B;
+  g.ri = rowinfo_of(p);
+  g.a_row = p->a_row; g.b_row = p->b_row;
+  g.t_rp = p->at_rp; g.t_ci = p->at_ci; g.t_src = p->at_src;
+  g.c_rp = c_row_ptr; g.c_ci = c_col_idx;
+  g.row_off = p->row_off; g.p_off = p->p_off; g.t_off = p->t_off;
+  g.total = (long long)p->host_st.total_products;
+  g.hist = p->host_st.hist;
+  g.buf = p->grad_buf;
+  g.buf_entries = p->grad_buf_entries;
+  if (e == cudaSuccess && p->mloc > 0) {
+    // the product buffer serves one call at a time: the launches of a call are
+    // not mixed with another thread's, and a call on another stream waits for
+    // the last one (not inside a capture, which takes no outside event)
+    std::lock_guard<std::mutex> lock(p->grad_mu);
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    const bool order = p->grad_buf_entries > 0 && db_vals;
+    if (order) e = cudaStreamIsCapturing(c.stream, &cs);
+    const bool eager = order && cs == cudaStreamCaptureStatusNone;
+    if (e == cudaSuccess && eager && !p->grad_done)
+      e = cudaEventCreateWithFlags(&p->grad_done, cudaEventDisableTiming);
+    else if (e == cudaSuccess && eager && p->grad_stream != c.stream)
+      e = cudaStreamWaitEvent(c.stream, p->grad_done, 0);
+    if (e == cudaSuccess) e = sg::launch_backward(c, p->opts.dtype, g, a_vals, b_vals, dc_vals, da_vals, db_vals);
+    if (e == cudaSuccess && eager) {
+      e = cudaEventRecord(p->grad_done, c.stream);
+      p->grad_stream = c.stream;
+    }
+  }
   return e == cudaSuccess ? SPGEMM_OK : SPGEMM_ERR_CUDA;
 }
 

@@ -3,17 +3,31 @@
 //   dA(i,k) = sum_j dC(i,j) * B(k,j)   on the pattern of A   (dC * B^T sampled)
 //   dB(k,j) = sum_i A(i,k) * dC(i,j)   on the pattern of B   (A^T * dC sampled)
 // Every (i,k,j) with A(i,k), B(k,j) nonzero has C(i,j) in C's pattern, so
-// each lookup of dC(i,j) succeeds; it is a binary search in the sorted row i
-// of C.
+// each lookup of dC(i,j) succeeds.  Both gradients need the same lookup, one
+// per scalar product of the forward pass; everything else is streaming.
 //
-// Work is cut into slabs of 32 consecutive outputs (nonzeros of A for dA,
-// of B for dB), one warp per slab, so a power-law input spreads its long
-// rows over many warps.  An output whose sum has few terms (at most 128) is
-// summed by its own lane as a chain of fused multiply-adds; an output with
-// more terms is summed by the whole warp -- lane l takes terms l, l+32, ...,
-// each lane chains its own terms, and a fixed shuffle tree adds the 32
-// partial sums.  Both orders are fixed, so the result is deterministic (the
-// same bits on every run), and nothing is accumulated atomically.
+// The lookups run once, in the order of A's rows, where row i of C is at
+// hand: k_grad_rows stages its values with a presence bitmap of its columns
+// in shared memory, finds dC(i,j) as a rank (one bitmap word and its prefix),
+// sums dA(i,k) on the spot and writes the values dC(i,j) to a buffer in
+// product order -- B(k,:) long and contiguous for every nonzero (i,k).
+// k_grad_cols then sums dB(k,:) over the nonzeros of A^T(k,:), each a
+// contiguous read of the buffer.  The buffer holds a chunk of the products at
+// a time (64 MB, so that it stays in the L2 cache between the two kernels);
+// the chunks follow each other in product order and add to dB in that order.
+// Rows of C that are too short to be worth a block or too long or too wide
+// for its shared memory are searched in global memory by k_grad_slabs.
+//
+// Orders are fixed (a lane's own chain, fixed shuffle trees, chunks in
+// order), nothing is accumulated atomically: the same bits on every run.
+//
+// 65,536 rows of 32 x 32 products, FP32: a binary search in C's row per
+// product and gradient (the kernels that still serve products whose rows of
+// B exceed the buffer) took 0.82 ms for dA and 1.88 ms for dB, bound by the
+// memory latency and the 32-byte sectors of scattered searches in C (533 MB).
+// Here k_grad_rows takes 0.62 ms for four chunks (bound by the latency of a
+// row's loads, 8 of 16 warps per scheduler resident at 64 registers),
+// k_grad_cols 0.20 ms (2.6 TB/s of DRAM and L1 59 % busy).
 #include "launch_util.cuh"
 
 namespace sg {
@@ -22,6 +36,9 @@ namespace sg {
 // summing up to this many terms each, their chains run side by side; a sum
 // far longer than its neighbours' (a hub row) would hold the warp alone.
 constexpr int GRAD_LANE_MAX = 128;
+
+constexpr long long GRAD_BUFFER_BYTES = 64ll << 20;  // a chunk of the products' dC values: half the L2 cache
+constexpr int GRAD_ROW_CAP = 4096;                   // entries of a row of C staged in shared memory
 
 __device__ __forceinline__ int find_col(const int32_t* __restrict__ ci, int lo, int hi, int c) {
   while (lo < hi) {
@@ -173,6 +190,435 @@ __global__ void __launch_bounds__(256) k_grad_b(Csr B, const T* __restrict__ av,
   }
 }
 
+// ------------------------------------------------- product offsets (plan)
+// off[r] = exclusive prefix sum of cnt (64 bits), off[n] the total: tile sums,
+// one block over the tile sums, tiles again.
+constexpr int OFF_THREADS = 256;
+constexpr int OFF_TILE = OFF_THREADS * 16;
+
+__device__ __forceinline__ long long off_block_scan(long long v, long long* total) {
+  __shared__ long long s_w[OFF_THREADS / 32];
+  const int lane = lane_id(), warp = threadIdx.x >> 5;
+  const long long incl = warp_incl_scan(v);
+  __syncthreads();
+  if (lane == 31) s_w[warp] = incl;
+  __syncthreads();
+  long long before = 0, all = 0;
+  for (int w = 0; w < OFF_THREADS / 32; ++w) {
+    if (w < warp) before += s_w[w];
+    all += s_w[w];
+  }
+  *total = all;
+  return before + incl - v;
+}
+
+__global__ void __launch_bounds__(OFF_THREADS) k_off_tiles(const long long* __restrict__ cnt, long long n,
+                                                          long long* __restrict__ part) {
+  const long long base = (long long)blockIdx.x * OFF_TILE;
+  long long v = 0, total;
+  for (int u = 0; u < 16; ++u) {
+    const long long r = base + u * OFF_THREADS + threadIdx.x;
+    if (r < n) v += cnt[r];
+  }
+  off_block_scan(v, &total);
+  if (threadIdx.x == 0) part[blockIdx.x] = total;
+}
+
+__global__ void __launch_bounds__(OFF_THREADS) k_off_partials(long long* __restrict__ part, long long tiles) {
+  long long carry = 0;
+  for (long long b = 0; b < tiles; b += OFF_THREADS) {
+    const long long i = b + threadIdx.x;
+    long long total;
+    const long long ex = off_block_scan(i < tiles ? part[i] : 0, &total);
+    if (i < tiles) part[i] = carry + ex;
+    carry += total;
+  }
+}
+
+__global__ void __launch_bounds__(OFF_THREADS) k_off_down(const long long* __restrict__ cnt, long long n,
+                                                         const long long* __restrict__ part,
+                                                         long long* __restrict__ off) {
+  const long long base = (long long)blockIdx.x * OFF_TILE;
+  long long carry = part[blockIdx.x];
+  for (int u = 0; u < 16; ++u) {
+    const long long r = base + u * OFF_THREADS + threadIdx.x;
+    const long long v = r < n ? cnt[r] : 0;
+    long long total;
+    const long long ex = off_block_scan(v, &total);
+    if (r < n) off[r] = carry + ex;
+    if (r == n - 1) off[n] = carry + ex + v;
+    carry += total;
+  }
+}
+
+// p_off[e] = products before nonzero e of A (rows of the plan's range): the
+// row's offset plus the lengths of the row's earlier rows of B.  A warp per row.
+__global__ void __launch_bounds__(256) k_product_offsets(Csr A, Csr B, long long row_begin, long long mloc,
+                                                         const long long* __restrict__ row_off,
+                                                         long long* __restrict__ p_off, const DevStats* st) {
+  if (block_skip(st)) return;
+  const int lane = lane_id();
+  const long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+  const long long nw = (gridDim.x * (long long)blockDim.x) >> 5;
+  for (long long r = w; r < mloc; r += nw) {
+    const int a0 = A.rp[row_begin + r], a1 = A.rp[row_begin + r + 1];
+    long long before = row_off[r];
+    for (int e0 = a0; e0 < a1; e0 += 32) {
+      const int e = e0 + lane;
+      int len = 0;
+      if (e < a1) {
+        const int k = A.ci[e];
+        if (k >= 0 && (long long)k < B.nrows) len = B.rp[k + 1] - B.rp[k];
+      }
+      const long long incl = warp_incl_scan((long long)len);
+      if (e < a1) p_off[e] = before + incl - len;
+      before += __shfl_sync(FULL, incl, 31);
+    }
+  }
+}
+
+// The same offsets in the order of A^T; rows before and after the plan's
+// range lie below and above every product.
+__global__ void __launch_bounds__(256) k_transposed_offsets(long long nnz, const int32_t* __restrict__ t_ci,
+                                                            const int32_t* __restrict__ t_src, long long row_begin,
+                                                            long long row_end, const long long* __restrict__ p_off,
+                                                            long long* __restrict__ t_off, const DevStats* st) {
+  if (block_skip(st)) return;
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < nnz; t += (long long)gridDim.x * blockDim.x) {
+    const long long i = t_ci[t];
+    t_off[t] = i < row_begin ? -1ll : (i >= row_end ? LLONG_MAX : p_off[t_src[t]]);
+  }
+}
+
+// First index of the non-decreasing v[lo, hi) with v[index] >= x (hi if none).
+template <typename I>
+__device__ __forceinline__ I first_at_least(const long long* __restrict__ v, I lo, I hi, long long x) {
+  while (lo < hi) {
+    const I mid = lo + (hi - lo) / 2;
+    if (v[mid] < x) lo = mid + 1; else hi = mid;
+  }
+  return lo;
+}
+
+// The same for a whole warp with one x: 32 probes a step (a block's single
+// search over millions of offsets would otherwise be 20 dependent loads).
+__device__ __forceinline__ long long warp_first_at_least(const long long* __restrict__ v, long long lo, long long hi,
+                                                         long long x) {
+  while (lo < hi) {
+    const long long step = (hi - lo + 31) / 32;
+    const long long q = lo + (long long)lane_id() * step;
+    const unsigned below = __ballot_sync(FULL, q < hi && v[q < hi ? q : lo] < x);
+    if (!below) return lo;
+    const int last = 31 - __clz(below);  // v is non-decreasing: lanes 0..last are below x
+    lo += last * step + 1;
+    hi = min(hi, lo + step - 1);
+  }
+  return lo;
+}
+
+// ---------------------------------------------------- both gradients' lookups
+// Which rows of C k_grad_rows takes: more than GRAD_ROW_MIN entries, at most
+// `cap`, and a column span inside one bitmap of 2^wlog columns.
+constexpr int GRAD_ROW_MIN = 128;
+
+__device__ __forceinline__ bool grad_row_staged(int n, int cmin, int cmax, int cap, int wlog) {
+  return n > GRAD_ROW_MIN && n <= cap && (long long)cmax - (cmin & ~31) < (1ll << wlog);
+}
+
+// One chunk [c0, c1) of the products, rows of C staged in shared memory, one
+// block per row.  G lanes take a nonzero (i,k) and walk B(k,:) together; a
+// warp keeps 8 nonzeros per lane group in flight and folds their 8 partial
+// sums with one exchange tree (FP64 additions cost a warp the same with any
+// number of lanes: 8 separate trees would take 8 * log2(G) of them, the folded
+// one 7 + log2(G) - 3).  buf may be null (dB not wanted), da as well.
+template <int NT, int G, typename T>
+__global__ void __launch_bounds__(NT)
+k_grad_rows(Csr A, Csr B, const T* __restrict__ bv, RowInfo ri, const long long* __restrict__ row_off,
+            const long long* __restrict__ p_off, const int32_t* __restrict__ c_rp, const int32_t* __restrict__ c_ci,
+            const T* __restrict__ dc, T* __restrict__ da, T* __restrict__ buf, long long c0, long long c1, int cap,
+            int wlog, uint32_t* err) {
+  constexpr int NW = NT / 32, GPW = 32 / G, S = 8;
+  constexpr int LG = G == 32 ? 5 : (G == 16 ? 4 : 3);
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* const sdc = reinterpret_cast<T*>(smem_raw);
+  uint32_t* const bits = reinterpret_cast<uint32_t*>(sdc + cap);
+  uint16_t* const pre = reinterpret_cast<uint16_t*>(bits + ((1 << wlog) >> 5));
+  __shared__ long long s_first;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = lane_id(), gl = lane & (G - 1), g = lane / G;
+  for (int t = tid; t < (1 << wlog) / 32; t += NT) bits[t] = 0u;
+  // first row with a product or an empty nonzero at or past c0
+  if (warp == 0) {
+    const long long f = c0 <= 0 ? 0 : warp_first_at_least(row_off, 1, ri.mloc + 1, c0) - 1;
+    if (lane == 0) s_first = f;
+  }
+  __syncthreads();
+  for (long long r = s_first + blockIdx.x; r < ri.mloc; r += gridDim.x) {
+    if (row_off[r] >= c1) break;
+    const int p0 = c_rp[r], n = c_rp[r + 1] - p0;
+    const int cmn = ri.cmin[r], cmx = ri.cmax[r];
+    if (!grad_row_staged(n, cmn, cmx, cap, wlog)) continue;
+    const int base = cmn & ~31;
+    const int a0 = A.rp[ri.row_begin + r], a1 = A.rp[ri.row_begin + r + 1];
+    // this lane group's nonzeros of a round: e0 + s * (NW * GPW).  The first
+    // round's are read before C's row is staged, both in flight together
+    int b0[S], len[S], at[S];  // at: position in the buffer, -1 outside the chunk
+    auto fetch = [&](int e0) {
+      int k[S];
+#pragma unroll
+      for (int s = 0; s < S; ++s) {
+        const int e = e0 + s * (NW * GPW);
+        b0[s] = len[s] = 0;
+        at[s] = -1;
+        k[s] = -1;
+        if (e < a1) {
+          const long long po = p_off[e];
+          k[s] = A.ci[e];
+          if (po >= c0 && po < c1) at[s] = buf ? (int)(po - c0) : 0;  // without dB the chunk is every product
+        }
+      }
+#pragma unroll
+      for (int s = 0; s < S; ++s)
+        if (at[s] >= 0) {
+          b0[s] = B.rp[k[s]];
+          len[s] = B.rp[k[s] + 1] - b0[s];
+        }
+    };
+    fetch(a0 + warp * GPW + g);
+    for (int p = tid; p < n; p += NT) {
+      const int c = c_ci[p0 + p] - base;
+      sdc[p] = dc[p0 + p];
+      if ((unsigned)c < (1u << wlog)) {
+        atomicOr(&bits[c >> 5], 1u << (c & 31));
+        if (p == 0 || ((c_ci[p0 + p - 1] - base) >> 5) != (c >> 5)) pre[c >> 5] = (uint16_t)p;
+      }
+    }
+    __syncthreads();
+    for (int e0 = a0 + warp * GPW + g; e0 - g < a1; e0 += S * NW * GPW) {  // warp-uniform
+      if (e0 - g - warp * GPW != a0) fetch(e0);
+      T part[S];
+#pragma unroll
+      for (int s = 0; s < S; ++s) part[s] = T(0);
+      int most = 0;
+#pragma unroll
+      for (int s = 0; s < S; ++s) most = max(most, len[s]);
+      for (int l = gl; l < most; l += G) {
+        int col[S];
+        T b[S];
+#pragma unroll
+        for (int s = 0; s < S; ++s) {
+          col[s] = 0;
+          b[s] = T(0);
+          if (l < len[s]) {
+            col[s] = B.ci[b0[s] + l];
+            b[s] = bv[b0[s] + l];
+          }
+        }
+#pragma unroll
+        for (int s = 0; s < S; ++s) {
+          if (l < len[s]) {
+            const int j = col[s] - base;
+            const unsigned m = 1u << (j & 31);
+            T d = T(0);
+            const uint32_t word = (unsigned)j < (1u << wlog) ? bits[j >> 5] : 0u;
+            if (word & m) d = sdc[pre[j >> 5] + __popc(word & (m - 1u))];
+            else atomicOr(err, EB_INTERNAL);  // C's pattern holds every product
+            part[s] = fma(d, b[s], part[s]);
+            if (buf) buf[at[s] + l] = d;
+          }
+        }
+      }
+      if (da) {
+        // fold 8 sums per lane into one: lane bits LG-1, LG-2, LG-3 choose the
+        // nonzero, then the remaining lanes add up
+#pragma unroll
+        for (int h = S / 2, d = G / 2; h >= 1; h >>= 1, d >>= 1) {
+          const bool up = (gl & d) != 0;
+#pragma unroll
+          for (int x = 0; x < h; ++x) {
+            const T send = up ? part[x] : part[x + h];
+            const T keep = up ? part[x + h] : part[x];
+            part[x] = keep + __shfl_xor_sync(FULL, send, d);
+          }
+        }
+#pragma unroll
+        for (int d = G / 16; d >= 1; d >>= 1) part[0] += __shfl_xor_sync(FULL, part[0], d);
+        const int s = gl >> (LG - 3);
+        int mine = -1;
+#pragma unroll
+        for (int x = 0; x < S; ++x)
+          if (x == s) mine = at[x];
+        if (mine >= 0 && (gl & ((1 << (LG - 3)) - 1)) == 0) da[e0 + s * (NW * GPW)] = part[0];
+      }
+    }
+    __syncthreads();
+    const int nwords = ((cmx - base) >> 5) + 1;
+    for (int t = tid * 4; t < nwords; t += NT * 4) *reinterpret_cast<uint4*>(bits + t) = make_uint4(0, 0, 0, 0);
+    __syncthreads();
+  }
+}
+
+// The other rows: slabs of 32 nonzeros of A, dC(i,j) by a binary search in
+// C's row in global memory.
+template <typename T>
+__global__ void __launch_bounds__(256)
+k_grad_slabs(Csr A, Csr B, const T* __restrict__ bv, RowInfo ri, const int32_t* __restrict__ a_row,
+             const long long* __restrict__ p_off, const int32_t* __restrict__ c_rp, const int32_t* __restrict__ c_ci,
+             const T* __restrict__ dc, T* __restrict__ da, T* __restrict__ buf, long long c0, long long c1, int cap,
+             int wlog, uint32_t* err) {
+  __shared__ long long s_lo, s_hi;
+  if (threadIdx.x < 32) {
+    const long long lo = A.rp[ri.row_begin], hi = A.rp[ri.row_begin + ri.mloc];
+    const long long f = c0 <= 0 ? lo : warp_first_at_least(p_off, lo, hi, c0);
+    const long long l = c1 >= LLONG_MAX - 1 ? hi : warp_first_at_least(p_off, lo, hi, c1);
+    if (threadIdx.x == 0) {
+      s_lo = f;
+      s_hi = l;
+    }
+  }
+  __syncthreads();
+  const int lane = lane_id();
+  const long long e_lo = s_lo, e_hi = s_hi;
+  const long long nslab = (e_hi - e_lo + 31) >> 5;
+  const long long w0 = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+  const long long nw = (gridDim.x * (long long)blockDim.x) >> 5;
+  for (long long s = w0; s < nslab; s += nw) {
+    const long long e = e_lo + (s << 5) + lane;
+    bool have = e < e_hi;
+    int b0 = 0, b1 = 0, p0 = 0, p1 = 0;
+    long long at = 0;
+    if (have) {
+      const long long r = (long long)a_row[e] - ri.row_begin;
+      p0 = c_rp[r];
+      p1 = c_rp[r + 1];
+      have = !grad_row_staged(p1 - p0, ri.cmin[r], ri.cmax[r], cap, wlog);
+      if (have) {
+        const int k = A.ci[e];
+        b0 = B.rp[k];
+        b1 = B.rp[k + 1];
+        at = p_off[e] - c0;
+      }
+    }
+    if (!__any_sync(FULL, have)) continue;
+    const bool wide = have && b1 - b0 > GRAD_LANE_MAX;
+    T acc = T(0);
+    if (have && !wide) {
+      int lo = p0;
+      for (int q = b0; q < b1; ++q) {
+        const int j = B.ci[q];
+        const int pos = find_col(c_ci, lo, p1, j);
+        T d = T(0);
+        if (pos < p1 && c_ci[pos] == j) {
+          d = dc[pos];
+          lo = pos + 1;
+        } else {
+          atomicOr(err, EB_INTERNAL);
+        }
+        acc = fma(d, bv[q], acc);
+        if (buf) buf[at + (q - b0)] = d;
+      }
+    }
+    unsigned wm = __ballot_sync(FULL, wide);
+    while (wm) {
+      const int L = __ffs(wm) - 1;
+      wm &= wm - 1;
+      const int lb0 = __shfl_sync(FULL, b0, L), lb1 = __shfl_sync(FULL, b1, L);
+      const int lp0 = __shfl_sync(FULL, p0, L), lp1 = __shfl_sync(FULL, p1, L);
+      const long long lat = __shfl_sync(FULL, at, L);
+      T part = T(0);
+      for (int q = lb0 + lane; q < lb1; q += 32) {
+        const int j = B.ci[q];
+        const int pos = find_col(c_ci, lp0, lp1, j);
+        T d = T(0);
+        if (pos < lp1 && c_ci[pos] == j) d = dc[pos];
+        else atomicOr(err, EB_INTERNAL);
+        part = fma(d, bv[q], part);
+        if (buf) buf[lat + (q - lb0)] = d;
+      }
+      const T tot = warp_sum_fixed(part);
+      if (lane == L) acc = tot;
+    }
+    if (have && da) da[e] = acc;
+  }
+}
+
+// dB from one chunk of the buffer: slabs of 32 outputs of B per warp, each
+// output its lane's chain over the chunk's nonzeros of A^T(k,:) (lanes of one
+// row of B read consecutive buffer entries).  A slab with an output of more
+// than GRAD_COL_MAX terms is summed by the whole block, each warp an eighth of
+// every output's terms, the eighths added in order.
+constexpr int GRAD_COL_MAX = 512;
+
+template <typename T>
+__device__ __forceinline__ T grad_col_sum(const T* __restrict__ av, const int32_t* __restrict__ t_src,
+                                          const long long* __restrict__ t_off, const T* __restrict__ buf,
+                                          long long c0, int l, int t0, int t1, T acc) {
+  int t = t0;
+  for (; t + 4 <= t1; t += 4) {
+    T a[4], d[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      a[u] = av[t_src[t + u]];
+      d[u] = buf[t_off[t + u] - c0 + l];
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) acc = fma(a[u], d[u], acc);
+  }
+  for (; t < t1; ++t) acc = fma(av[t_src[t]], buf[t_off[t] - c0 + l], acc);
+  return acc;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256)
+k_grad_cols(Csr B, const T* __restrict__ av, const int32_t* __restrict__ b_row, const int32_t* __restrict__ t_rp,
+            const int32_t* __restrict__ t_src, const long long* __restrict__ t_off, const T* __restrict__ buf,
+            T* __restrict__ db, long long c0, long long c1, int first, int whole) {
+  __shared__ int s_big[8];
+  __shared__ int s_l[32], s_t0[32], s_t1[32];
+  __shared__ T s_part[8][32];
+  const int warp = threadIdx.x >> 5, lane = lane_id();
+  const long long nslab = (B.nnz + 31) >> 5;
+  for (long long s0 = blockIdx.x * 8ll; s0 < nslab; s0 += gridDim.x * 8ll) {
+    const long long q = ((s0 + warp) << 5) + lane;
+    const bool have = q < B.nnz;
+    int l = 0, t0 = 0, t1 = 0;
+    if (have) {
+      const int k = b_row[q];
+      l = (int)(q - B.rp[k]);
+      t0 = t_rp[k];
+      t1 = t_rp[k + 1];
+      if (!whole) {  // one chunk of every row of A needs no search
+        t0 = first_at_least(t_off, t0, t1, c0);
+        t1 = first_at_least(t_off, t0, t1, c1);
+      }
+    }
+    const bool big = __any_sync(FULL, t1 - t0 > GRAD_COL_MAX);
+    if (!big && have && (first || t1 > t0))
+      db[q] = grad_col_sum(av, t_src, t_off, buf, c0, l, t0, t1, first ? T(0) : db[q]);
+    if (lane == 0) s_big[warp] = big;
+    if (!__syncthreads_or(big)) continue;
+    for (int w = 0; w < 8; ++w) {
+      if (!s_big[w]) continue;  // block-uniform
+      if (warp == w) {
+        s_l[lane] = l;
+        s_t0[lane] = t0;
+        s_t1[lane] = t1;
+      }
+      __syncthreads();
+      const int u0 = s_t0[lane], n = s_t1[lane] - u0;
+      s_part[warp][lane] = grad_col_sum(av, t_src, t_off, buf, c0, s_l[lane], u0 + (int)((long long)n * warp / 8),
+                                        u0 + (int)((long long)n * (warp + 1) / 8), T(0));
+      __syncthreads();
+      if (warp == w && have) {
+        T acc = first ? T(0) : db[q];
+        for (int v = 0; v < 8; ++v) acc += s_part[v][lane];
+        db[q] = acc;
+      }
+      __syncthreads();
+    }
+    __syncthreads();
+  }
+}
+
 static int grid_for(long long slabs, int nsm) {
   long long g = (slabs + 7) / 8;  // 8 warps (slabs in flight) per block
   const long long cap = (long long)nsm * 8;
@@ -187,32 +633,129 @@ cudaError_t launch_row_index(const LaunchCtx& c, const int32_t* rp, long long nr
   return cudaGetLastError();
 }
 
-cudaError_t launch_backward(const LaunchCtx& c, int dtype, const Csr& A, const Csr& B, long long row_begin,
-                            long long mloc, const void* av, const void* bv, const int32_t* a_row,
-                            const int32_t* b_row, const int32_t* t_rp, const int32_t* t_ci, const int32_t* t_src,
-                            const int32_t* c_rp, const int32_t* c_ci, const void* dc, void* da, void* db) {
+long long grad_buffer_entries(long long nnz_a, long long nnz_b, long long ncols_b, int vbytes) {
+  const long long chunk = GRAD_BUFFER_BYTES / vbytes;
+  const long long longest = ncols_b < nnz_b ? ncols_b : nnz_b;  // no row of B is longer
+  if (longest > chunk || nnz_a <= 0 || longest <= 0) return 0;
+  // a chunk's last nonzero may start just inside it
+  const long long all = nnz_a < chunk / longest ? nnz_a * longest : chunk;
+  return (all < chunk ? all : chunk) + longest;
+}
+
+cudaError_t launch_grad_offsets(const LaunchCtx& c, const Csr& A, const Csr& B, long long row_begin, long long mloc,
+                                const long long* prod, const int32_t* t_ci, const int32_t* t_src, long long* row_off,
+                                long long* part, long long* p_off, long long* t_off) {
+  if (mloc <= 0) return cudaSuccess;
+  const long long tiles = (mloc + OFF_TILE - 1) / OFF_TILE;
+  k_off_tiles<<<(unsigned)tiles, OFF_THREADS, 0, c.stream>>>(prod, mloc, part);
+  k_off_partials<<<1, OFF_THREADS, 0, c.stream>>>(part, tiles);
+  k_off_down<<<(unsigned)tiles, OFF_THREADS, 0, c.stream>>>(prod, mloc, part, row_off);
+  k_product_offsets<<<grid_for(mloc, c.nsm), 256, 0, c.stream>>>(A, B, row_begin, mloc, row_off, p_off, c.st);
+  k_transposed_offsets<<<grid_for((A.nnz + 31) / 32, c.nsm), 256, 0, c.stream>>>(
+      A.nnz, t_ci, t_src, row_begin, row_begin + mloc, p_off, t_off, c.st);
+  for (int i = 0; i < 5; ++i) count_launch(c);
+  return cudaGetLastError();
+}
+
+template <int NT, int G, typename T>
+static cudaError_t grad_rows(const LaunchCtx& c, const GradArgs& g, const T* bv, const T* dc, T* da, T* buf,
+                             long long c0, long long c1, int cap, int wlog, long long rows) {
+  auto k = k_grad_rows<NT, G, T>;
+  const size_t smem = (size_t)cap * sizeof(T) + ((size_t)1 << wlog) / 32 * 6;
+  const int occ = kernel_blocks_per_sm(k, NT, smem);
+  if (occ <= 0) return cudaErrorInvalidConfiguration;
+  k<<<persistent_grid(rows, 1, c.nsm, occ), NT, smem, c.stream>>>(g.A, g.B, bv, g.ri, g.row_off, g.p_off, g.c_rp,
+                                                                 g.c_ci, dc, da, buf, c0, c1, cap, wlog, c.err);
+  count_launch(c);
+  return cudaGetLastError();
+}
+
+// Both gradients through the product buffer (g.buf_entries > 0).
+template <typename T>
+static cudaError_t backward_buffered(const LaunchCtx& c, const GradArgs& g, const T* av, const T* bv, const T* dc,
+                                     T* da, T* db) {
+  const long long longest = g.B.ncols < g.B.nnz ? g.B.ncols : g.B.nnz;
+  const long long chunk = db ? g.buf_entries - longest : LLONG_MAX;
+  T* const buf = db ? (T*)g.buf : nullptr;
+  // rows of C staged in shared memory: a row has at most its products'
+  // entries, so the rows' bins bound them
+  int hi = 0;
+  long long rows = 0;
+  for (int b = bin_of(GRAD_ROW_MIN + 1); b < NBINS; ++b)
+    if (g.hist[b]) {
+      hi = b;
+      rows += g.hist[b];
+    }
+  int cap = 256;
+  while (cap < GRAD_ROW_CAP && cap < (hi > 0 ? (hi < 14 ? 1 << (hi - 1) : GRAD_ROW_CAP) : 0)) cap *= 2;
+  int wlog = 10;
+  while (wlog < (cap > 2048 ? 18 : 17) && (1ll << wlog) < g.B.ncols) ++wlog;
+  const double avg = g.B.nrows > 0 ? (double)g.B.nnz / (double)g.B.nrows : 0.0;
+  for (long long c0 = 0; c0 < g.total || c0 == 0; c0 += chunk) {
+    const bool last = c0 + chunk >= g.total || chunk == LLONG_MAX;
+    const long long c1 = last ? LLONG_MAX - 1 : c0 + chunk;
+    cudaError_t e = cudaSuccess;
+    if (hi > 0) {
+#define SG_GRAD_ROWS(GG)                                                                               \
+  e = cap > 2048 ? grad_rows<256, GG, T>(c, g, bv, dc, da, buf, c0, c1, cap, wlog, rows)                \
+                 : grad_rows<128, GG, T>(c, g, bv, dc, da, buf, c0, c1, cap, wlog, rows)
+      if (avg >= 20) SG_GRAD_ROWS(32);
+      else if (avg >= 10) SG_GRAD_ROWS(16);
+      else SG_GRAD_ROWS(8);
+#undef SG_GRAD_ROWS
+      if (e != cudaSuccess) return e;
+    }
+    k_grad_slabs<T><<<grid_for(g.A.nnz / 32 + 1, c.nsm), 256, 0, c.stream>>>(
+        g.A, g.B, bv, g.ri, g.a_row, g.p_off, g.c_rp, g.c_ci, dc, da, buf, c0, c1, hi > 0 ? cap : 0, wlog, c.err);
+    count_launch(c);
+    if (db) {
+      k_grad_cols<T><<<grid_for((g.B.nnz + 31) / 32, c.nsm), 256, 0, c.stream>>>(
+          g.B, av, g.b_row, g.t_rp, g.t_src, g.t_off, buf, db, c0, c1, c0 == 0 ? 1 : 0,
+          c0 == 0 && last && g.ri.row_begin == 0 && g.ri.mloc == g.A.nrows ? 1 : 0);
+      count_launch(c);
+    }
+    if ((e = cudaGetLastError()) != cudaSuccess || last) return e;
+  }
+  return cudaSuccess;
+}
+
+cudaError_t launch_backward(const LaunchCtx& c, int dtype, const GradArgs& g, const void* av, const void* bv,
+                            const void* dc, void* da, void* db) {
+  const Csr &A = g.A, &B = g.B;
+  const long long row_begin = g.ri.row_begin, mloc = g.ri.mloc;
+  if (g.buf_entries > 0 && mloc > 0 && B.nnz > 0) {
+    if (dtype == SPGEMM_F32)
+      return backward_buffered<float>(c, g, (const float*)av, (const float*)bv, (const float*)dc, (float*)da,
+                                      (float*)db);
+    return backward_buffered<double>(c, g, (const double*)av, (const double*)bv, (const double*)dc, (double*)da,
+                                     (double*)db);
+  }
+  // rows of B longer than the buffer: a search per product and gradient
+  if (db && B.nnz > 0) {
+    const cudaError_t e = cudaMemsetAsync(db, 0, (size_t)B.nnz * (dtype == SPGEMM_F32 ? 4 : 8), c.stream);
+    if (e != cudaSuccess) return e;
+  }
   if (da && mloc > 0) {
     const long long slabs = A.nnz / 32 + 1;  // an upper bound; the kernel reads the range's own extent
     if (dtype == SPGEMM_F32)
-      k_grad_a<float><<<grid_for(slabs, c.nsm), 256, 0, c.stream>>>(A, B, (const float*)bv, row_begin, mloc, a_row, c_rp,
-                                                                    c_ci, (const float*)dc, (float*)da, c.err);
+      k_grad_a<float><<<grid_for(slabs, c.nsm), 256, 0, c.stream>>>(A, B, (const float*)bv, row_begin, mloc, g.a_row,
+                                                                    g.c_rp, g.c_ci, (const float*)dc, (float*)da, c.err);
     else
-      k_grad_a<double><<<grid_for(slabs, c.nsm), 256, 0, c.stream>>>(A, B, (const double*)bv, row_begin, mloc, a_row,
-                                                                     c_rp,
-                                                                     c_ci, (const double*)dc, (double*)da, c.err);
+      k_grad_a<double><<<grid_for(slabs, c.nsm), 256, 0, c.stream>>>(A, B, (const double*)bv, row_begin, mloc, g.a_row,
+                                                                     g.c_rp, g.c_ci, (const double*)dc, (double*)da, c.err);
     count_launch(c);
   }
   if (db && B.nnz > 0) {
     const long long slabs = (B.nnz + 31) / 32;
     if (dtype == SPGEMM_F32)
-      k_grad_b<float><<<grid_for(slabs, c.nsm), 256, 0, c.stream>>>(B, (const float*)av, b_row, t_rp, t_ci, t_src,
-                                                                     row_begin,
-                                                                     row_begin + mloc, c_rp, c_ci, (const float*)dc,
+      k_grad_b<float><<<grid_for(slabs, c.nsm), 256, 0, c.stream>>>(B, (const float*)av, g.b_row, g.t_rp, g.t_ci,
+                                                                     g.t_src, row_begin, row_begin + mloc, g.c_rp,
+                                                                     g.c_ci, (const float*)dc,
                                                                      (float*)db, c.err);
     else
-      k_grad_b<double><<<grid_for(slabs, c.nsm), 256, 0, c.stream>>>(B, (const double*)av, b_row, t_rp, t_ci,
-                                                                      t_src,
-                                                                      row_begin, row_begin + mloc, c_rp, c_ci,
+      k_grad_b<double><<<grid_for(slabs, c.nsm), 256, 0, c.stream>>>(B, (const double*)av, g.b_row, g.t_rp, g.t_ci,
+                                                                      g.t_src,
+                                                                      row_begin, row_begin + mloc, g.c_rp, g.c_ci,
                                                                       (const double*)dc, (double*)db, c.err);
     count_launch(c);
   }

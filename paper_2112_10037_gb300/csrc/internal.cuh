@@ -311,10 +311,27 @@ cudaError_t launch_masked(const LaunchCtx& c, int dtype, int semiring, const Csr
                           const void* av, const void* bv, const void* mv, void* out);
 // out[q] = row of entry q of a CSR with row pointer rp (nrows rows).
 cudaError_t launch_row_index(const LaunchCtx& c, const int32_t* rp, long long nrows, int32_t* out);
-cudaError_t launch_backward(const LaunchCtx& c, int dtype, const Csr& A, const Csr& B, long long row_begin,
-                            long long mloc, const void* av, const void* bv, const int32_t* a_row,
-                            const int32_t* b_row, const int32_t* t_rp, const int32_t* t_ci, const int32_t* t_src,
-                            const int32_t* c_rp, const int32_t* c_ci, const void* dc, void* da, void* db);
+// What the adjoint reads besides values: structure, A^T (t_rp, t_ci, t_src),
+// the row of every nonzero (a_row, b_row), C's structure, and the offsets of
+// the products (row_off per row and their total, p_off per nonzero of A, t_off
+// the same in A^T's order).  buf: a product buffer of buf_entries values (0:
+// none, rows of B too long for it).
+struct GradArgs {
+  Csr A, B;
+  RowInfo ri;
+  const int32_t *a_row, *b_row, *t_rp, *t_ci, *t_src, *c_rp, *c_ci;
+  const long long *row_off, *p_off, *t_off;
+  long long total;   // products of the plan's rows
+  const int* hist;   // host: rows per bin
+  void* buf;
+  long long buf_entries;
+};
+long long grad_buffer_entries(long long nnz_a, long long nnz_b, long long ncols_b, int vbytes);
+cudaError_t launch_grad_offsets(const LaunchCtx& c, const Csr& A, const Csr& B, long long row_begin, long long mloc,
+                                const long long* prod, const int32_t* t_ci, const int32_t* t_src, long long* row_off,
+                                long long* part, long long* p_off, long long* t_off);
+cudaError_t launch_backward(const LaunchCtx& c, int dtype, const GradArgs& g, const void* av, const void* bv,
+                            const void* dc, void* da, void* db);
 
 // One instance of a batched product (see batch.cu).
 struct BatchDesc {

@@ -1,0 +1,107 @@
+"""GPU parity of the adjoint where its kernels hand over to each other: rows of
+C at the edges of what a block stages in shared memory (128 and 4096 entries,
+one bitmap of columns), rows of B of average length below and above the lane
+groups' sizes, columns of A with more terms than a lane's chain takes, one
+gradient at a time, and calls on two streams."""
+import numpy as np
+import pytest
+
+from paper_2112_10037_gb300 import gen
+from parity import abs_csr, max_rel_err
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def api():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2112_10037_gb300 import build
+    build.build()
+    from paper_2112_10037_gb300 import api as a
+    return a
+
+
+def _edge_operands(ncols, blen, seed):
+    """A's rows reach 0, 1, 127..130, 1000 and 4094..4098 distinct columns:
+    B's rows are disjoint runs of `blen` columns, and single columns after
+    them; every row of A also holds column 0 of B's rows (a hub: one long
+    column sum)."""
+    rng = np.random.default_rng(seed)
+    runs = 4200 // blen
+    step = ncols // (runs * blen + 64)
+    place = np.arange(runs * blen + 64, dtype=np.int64) * step + step // 2
+    lens = np.concatenate([np.full(runs, blen), np.ones(64, np.int64), [0]])
+    rp = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    order = rng.permutation(runs * blen)  # runs interleave over the whole width
+    ci = np.concatenate([np.sort(place[order[k * blen:(k + 1) * blen]]) for k in range(runs)] + [place[runs * blen:]])
+    B = gen.CSR(len(lens), ncols, rp, ci.astype(np.int32), rng.standard_normal(len(ci))).check()
+    rows = []
+    for want in [0, 1, 127, 128, 129, 130, 1000, 4094, 4095, 4096, 4097, 4098] + [blen] * 700:
+        n = min(want // blen, runs)
+        ones = min(want - n * blen, 64)
+        ks = np.concatenate([np.arange(n), runs + np.arange(ones), [len(lens) - 1] if want % 2 else []])
+        rows.append(np.sort(ks).astype(np.int64))
+    arp = np.concatenate([[0], np.cumsum([len(r) for r in rows])]).astype(np.int32)
+    aci = np.concatenate(rows).astype(np.int32)
+    return gen.CSR(len(rows), B.nrows, arp, aci, rng.standard_normal(len(aci))).check(), B
+
+
+def _reference(oracle_mod, A, B, W):
+    C = oracle_mod.spgemm(A, B)
+    da, db = oracle_mod.backward(A, B, C.row_ptr, C.col_idx, W)
+    sa, sb = oracle_mod.backward(abs_csr(A), abs_csr(B), C.row_ptr, C.col_idx, np.abs(W))
+    return da, db, sa, sb
+
+
+@pytest.mark.parametrize("dtype,tol", [(torch.float64, 1e-12), (torch.float32, 2e-4)])
+@pytest.mark.parametrize("ncols", [5000, 600_000])
+@pytest.mark.parametrize("blen", [7, 15, 60])
+def test_row_edges(api, oracle_mod, blen, ncols, dtype, tol):
+    A, B = _edge_operands(ncols, blen, blen)
+    dA, dB = api.DeviceCSR.from_host(A, dtype=dtype), api.DeviceCSR.from_host(B, dtype=dtype)
+    plan = api.Plan(dA, dB, dtype=dtype, backward=True)
+    _, nnz = plan.symbolic()
+    plan.numeric(dA.vals, dB.vals)
+    W = np.random.default_rng(1).standard_normal(nnz).astype(np.float32).astype(np.float64)
+    dW = torch.from_numpy(W).to(device="cuda", dtype=dtype)
+    da, db = plan.backward(dA.vals, dB.vals, dW)
+    only_a, none_b = plan.backward(dA.vals, dB.vals, dW, need_b=False)
+    none_a, only_b = plan.backward(dA.vals, dB.vals, dW, need_a=False)
+    torch.cuda.synchronize()
+    plan.check()
+    assert none_a is None and none_b is None
+    assert torch.equal(da, only_a) and torch.equal(db, only_b)
+    if dtype == torch.float32:
+        A, B = (M.astype(np.float32).astype(np.float64) for M in (A, B))
+    ra, rb, sa, sb = _reference(oracle_mod, A, B, W)
+    assert max_rel_err(da.double().cpu().numpy(), ra, sa) <= tol
+    assert max_rel_err(db.double().cpu().numpy(), rb, sb) <= tol
+    plan.close()
+
+
+def test_two_streams(api):
+    """Calls on one plan from two streams give what each gives alone."""
+    A = gen.random_rows(3000, 3000, np.full(3000, 40), np.random.default_rng(3))
+    dA = api.DeviceCSR.from_host(A)
+    plan = api.Plan(dA, dA, backward=True)
+    _, nnz = plan.symbolic()
+    plan.numeric(dA.vals, dA.vals)
+    gen_ = torch.Generator(device="cuda").manual_seed(1)
+    ws = [torch.randn(nnz, generator=gen_, device="cuda", dtype=torch.float64) for _ in range(2)]
+    alone = [plan.backward(dA.vals, dA.vals, w) for w in ws]
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in ws]
+    home = plan.stream
+    got = []
+    for _ in range(5):
+        for s, w in zip(streams, ws):
+            plan.stream = int(s.cuda_stream)
+            with torch.cuda.stream(s):
+                got.append(plan.backward(dA.vals, dA.vals, w))
+    torch.cuda.synchronize()
+    plan.stream = home
+    for i, (da, db) in enumerate(got):
+        assert torch.equal(da, alone[i % 2][0]) and torch.equal(db, alone[i % 2][1])
+    plan.close()
