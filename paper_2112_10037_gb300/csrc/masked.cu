@@ -8,19 +8,36 @@
 //
 // Work is cut into units of 32 consecutive nonzeros of A (so rows of any
 // length spread over many warps and the dense core of a power-law graph
-// does not hold one warp for long); each lane finds its entry's row by a
-// binary search over A's row pointer.  The unit's products are formed in
-// full 32-lane batches (a prefix sum over the lanes' B row lengths, then a
-// search for each lane's owner).  A product whose column lies in its row of
-// M adds its rounded value A(i,k)*B(k,j) to that entry:
-//  * when the whole unit lies in one row and that row of M has at most
-//    MASK_CAP columns, the row's mask columns and one accumulator each are
-//    staged in shared memory, each product's column is found there by binary
-//    search, hits add with a shared-memory reduction, and the unit ends by
-//    adding its nonzero accumulators to the output with global FP64
-//    reductions (other units of the row add to the same entries);
-//  * otherwise each product searches its row of M in global memory and a hit
-//    adds straight to the output with a global FP64 reduction.
+// does not hold one warp for long).  A warp finds the row of its unit's first
+// nonzero by a 32-way search over A's row pointer, the others follow from it.
+// A product whose column lies in its row of M adds its rounded value
+// A(i,k)*B(k,j) to that entry.
+//
+// Few products do (6 % in triangle counting on R-MAT graphs), so turning the
+// others away decides the speed.  The part of a row of A inside the unit that
+// forms at least MASK_MIN_PRODUCTS products, and MASK_RATIO for each mask
+// column, is handled by itself, with the row's mask columns and one
+// accumulator each in shared memory (up to MASK_CAP columns; longer mask rows
+// stay in global memory):
+//  * a row of B much longer than the mask row is not read at all: each mask
+//    column is searched in it, four rows of B at a time,
+//  * otherwise the mask columns set bits of a hashed bitmap in shared memory
+//    (the column's low 12 bits) and a product costs one load of its column
+//    and one test; rows of B of at least 32 entries are walked directly by
+//    the warp, shorter ones are flattened so that every lane has a product,
+//  * products that pass wait in a queue and are looked up 32 at a time, all
+//    lanes busy, by a binary search over the mask row; hits add with a
+//    shared-memory reduction, and the row ends by adding its nonzero
+//    accumulators to the output with global reductions (other units of the
+//    row add to the same entries).
+// The remaining products are flattened over all their rows and search the
+// mask row in global memory one by one: parts of few products, where staging
+// does not pay, and masks that most products hit (the full pattern of A*B has
+// no more columns than products).
+//
+// A block is one warp and takes one unit, so that the hardware's block
+// scheduler balances units of very different work.
+//
 // The output is zeroed before and, with M's values, scaled by them after
 // (the sum is finished before the factor, as in the definition).
 #include <type_traits>
@@ -29,15 +46,41 @@
 
 namespace sg {
 
-constexpr int MASK_WARPS = 8;
-constexpr int MASK_CAP = 512;   // mask columns staged per warp
+constexpr int MASK_CAP = 384;             // mask columns staged per warp (32 warps share an SM)
+constexpr int MASK_BITS = 4096;           // bits of the hashed bitmap
+constexpr int MASK_FILTER_MAX = 2048;     // longest mask row worth the bitmap (two bits per column)
+constexpr int MASK_MIN_PRODUCTS = 128;    // fewest products worth staging a row,
+constexpr int MASK_RATIO = 4;             // and per mask column,
+constexpr int MASK_UNIT_PRODUCTS = 512;   // in a unit of this many in all (a stencil's units have 224)
+constexpr int MASK_QUEUE = 64;            // products that passed the bitmap (fewer than 32 wait)
 
-// Largest r with rp[r] <= e (the row holding position e), over rows [0, m).
-__device__ __forceinline__ int row_of(const int32_t* __restrict__ rp, int m, int e) {
-  int lo = 0, hi = m - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (rp[mid] <= e) lo = mid; else hi = mid - 1;
+// Largest r with rp[r] <= e (the row holding position e) over rows [0, m),
+// the same e on every lane: 32 probes a step.
+__device__ __forceinline__ int warp_row_of(const int32_t* __restrict__ rp, int m, int e) {
+  int lo = 0, hi = m;  // rp[lo] <= e, rp[hi] > e or hi == m
+  while (hi - lo > 1) {
+    const int step = (hi - lo + 31) >> 5;
+    const long long q = (long long)lo + (long long)lane_id() * step;
+    const unsigned b = __ballot_sync(FULL, q < hi && rp[q < hi ? q : lo] <= e);
+    const int last = b ? 31 - __clz(b) : 0;
+    lo += last * step;
+    hi = min(hi, lo + step);
+  }
+  return lo;
+}
+
+// Row holding position e, searched upward from `row` (rp[row] <= e).
+__device__ __forceinline__ int row_from(const int32_t* __restrict__ rp, int m, int row, int e) {
+  if (row + 1 >= m || rp[row + 1] > e) return row;
+  int lo = row + 1, step = 1;  // rp[lo] <= e
+  while (lo + step < m && rp[lo + step] <= e) {
+    lo += step;
+    step <<= 1;
+  }
+  int hi = min(lo + step, m);
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (rp[mid] <= e) lo = mid; else hi = mid;
   }
   return lo;
 }
@@ -112,24 +155,45 @@ __device__ __forceinline__ void sr_reduce_global(T* p, T v) {
   else *p = T(1);
 }
 
+// Shared memory of one warp.
+template <typename T>
+struct MaskWarp {
+  T acc[MASK_CAP];
+  int2 queue[MASK_QUEUE];  // (entry of B, lane whose nonzero of A owns it)
+  int col[MASK_CAP];
+  uint32_t bits[MASK_BITS / 32];
+};
+
+// acc (+)= v for an accumulator that only this lane updates meanwhile.
+template <int SR, typename T>
+__device__ __forceinline__ void sr_add_own(T* p, T v) {
+  if (SR == 0) *p += v;
+  else if (SR == 1) { if (v < *p) *p = v; }
+  else if (SR == 2) { if (v > *p) *p = v; }
+  else if (v != T(0)) *p = T(1);
+}
+
+// Searching the mask's n columns in a row of B of len entries costs about
+// 10 * log2(len) instructions per 32 columns, reading the row 50 per 32
+// entries.
+__device__ __forceinline__ bool mask_search_pays(int n, int len) {
+  return len >= 32 && ((n + 31) >> 5) * (32 - __clz(len)) * 6 < len;
+}
+
 template <typename T, int SR>
-__global__ void __launch_bounds__(MASK_WARPS * 32)
+__global__ void __launch_bounds__(32, 32)
 k_masked(Csr A, Csr B, Csr M, const T* __restrict__ av, const T* __restrict__ bv, T* __restrict__ out) {
-  __shared__ __align__(16) int s_col[MASK_WARPS][MASK_CAP];
-  __shared__ __align__(16) T s_acc[MASK_WARPS][MASK_CAP];
-  const int warp = threadIdx.x >> 5, lane = lane_id();
-  int* mc = s_col[warp];
-  T* acc = s_acc[warp];
-  const long long units = (A.nnz + 31) / 32;
-  const long long w = (long long)blockIdx.x * MASK_WARPS + warp;
-  const long long nw = (long long)gridDim.x * MASK_WARPS;
-  for (long long u = w; u < units; u += nw) {
+  __shared__ MaskWarp<T> sm;
+  const int lane = lane_id();
+  const unsigned lt = lanemask_lt();
+  {
+    const long long u = blockIdx.x;
     const int e = (int)(32 * u) + lane;
     const bool ve = e < A.nnz;
-    int i = 0, sb = 0, len = 0;
+    int i = warp_row_of(A.rp, (int)A.nrows, (int)(32 * u)), sb = 0, len = 0;
     T a = T(0);
     if (ve) {
-      i = row_of(A.rp, (int)A.nrows, e);
+      i = row_from(A.rp, (int)A.nrows, i, e);
       const int k = A.ci[e];
       if (k >= 0 && (long long)k < B.nrows) {  // a column of A out of range names no row of B
         sb = B.rp[k];
@@ -137,23 +201,134 @@ k_masked(Csr A, Csr B, Csr M, const T* __restrict__ av, const T* __restrict__ bv
         a = av[e];
       }
     }
-    const int last = min(31, (int)(A.nnz - 32 * u) - 1);  // last valid lane
-    const int i0 = __shfl_sync(FULL, i, 0), i1 = __shfl_sync(FULL, i, last);
-    const int m0 = M.rp[i0], m1 = M.rp[i0 + 1];
-    const bool staged = i0 == i1 && m1 - m0 <= MASK_CAP;  // warp-uniform
-    if (staged) {
-      for (int t = lane; t < m1 - m0; t += 32) {
-        mc[t] = M.ci[m0 + t];
-        acc[t] = sr_zero<SR, T>();
+    const int mr0 = M.rp[i], mr1 = M.rp[i + 1];  // the row's mask range (lanes past the end: unused)
+    unsigned todo = __ballot_sync(FULL, ve && len > 0 && mr1 > mr0);
+    if (!(todo >> lane & 1u)) len = 0;
+    // ---- rows of many products, one at a time
+    unsigned left = warp_sum(min(len, 1 << 20)) >= MASK_UNIT_PRODUCTS ? todo : 0u;
+    while (left) {
+      const int L = __ffs(left) - 1;
+      const int i0 = __shfl_sync(FULL, i, L);
+      const int m0 = __shfl_sync(FULL, mr0, L), n = __shfl_sync(FULL, mr1, L) - m0;
+      const unsigned mine = __ballot_sync(FULL, i == i0) & left;
+      left &= ~mine;
+      const bool in = mine >> lane & 1u;
+      // (lengths capped: the sum only decides whether staging pays)
+      const int products = warp_sum(in ? min(len, 1 << 20) : 0);
+      if (products < MASK_MIN_PRODUCTS || products < MASK_RATIO * n || n > MASK_FILTER_MAX) continue;
+      const bool staged = n <= MASK_CAP;
+      const bool search = in && mask_search_pays(n, len);
+      const bool filter = __any_sync(FULL, in && !search);  // some row of B is read
+      if (filter)
+        for (int t = lane; t < MASK_BITS / 32; t += 32) sm.bits[t] = 0u;
+      __syncwarp();
+      for (int t = lane; t < n; t += 32) {
+        const int c = M.ci[m0 + t];
+        if (filter) atomicOr(&sm.bits[(c >> 5) & (MASK_BITS / 32 - 1)], 1u << (c & 31));
+        if (staged) {
+          sm.col[t] = c;
+          sm.acc[t] = sr_zero<SR, T>();
+        }
       }
       __syncwarp();
+      // ---- mask columns searched in long rows of B, four rows at a time
+      unsigned sm4 = __ballot_sync(FULL, search);
+      while (sm4) {
+        int s4[4], n4[4];
+        T a4[4];
+        int most = 0;
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+          const int o = sm4 ? __ffs(sm4) - 1 : -1;
+          sm4 &= sm4 - 1;  // 0 stays 0
+          s4[v] = __shfl_sync(FULL, sb, o & 31);
+          n4[v] = __shfl_sync(FULL, len, o & 31);
+          a4[v] = __shfl_sync(FULL, a, o & 31);
+          if (o < 0) n4[v] = 0;
+          most = max(most, n4[v]);
+        }
+        const int top = 1 << (31 - __clz(most));
+        for (int t = lane; t < n; t += 32) {
+          const int c = staged ? sm.col[t] : M.ci[m0 + t];
+          int at[4] = {0, 0, 0, 0};  // entries of the row below c
+          for (int step = top; step > 0; step >>= 1) {
+#pragma unroll
+            for (int v = 0; v < 4; ++v)
+              if (at[v] + step <= n4[v] && B.ci[s4[v] + at[v] + step - 1] < c) at[v] += step;
+          }
+#pragma unroll
+          for (int v = 0; v < 4; ++v)
+            if (at[v] < n4[v] && B.ci[s4[v] + at[v]] == c) {
+              const T x = sr_product<SR>(a4[v], bv[s4[v] + at[v]]);
+              if (staged) sr_add_own<SR>(&sm.acc[t], x);
+              else sr_reduce_global<SR>(&out[m0 + t], x);
+            }
+        }
+      }
+      __syncwarp();
+      const bool rd = in && !search;
+      int qn = 0;  // waiting products
+      auto look_up = [&](int cnt) {  // the last cnt (at most 32) of the queue
+        int2 x = make_int2(0, 0);
+        if (lane < cnt) x = sm.queue[qn - cnt + lane];
+        const T oa = __shfl_sync(FULL, a, x.y);
+        if (lane < cnt) {
+          const int j = B.ci[x.x];
+          if (staged) {
+            const int p = find_in(sm.col, 0, n, j);
+            if (p >= 0) sr_reduce_shared<SR>(&sm.acc[p], sr_product<SR>(oa, bv[x.x]));
+          } else {
+            const int p = find_in(M.ci, m0, m0 + n, j);
+            if (p >= 0) sr_reduce_global<SR>(&out[p], sr_product<SR>(oa, bv[x.x]));
+          }
+        }
+        qn -= cnt;
+        __syncwarp();  // the entries are read before later ones overwrite them
+      };
+      auto offer = [&](int j, int bi, int owner, bool act) {
+        const bool pass = act && (sm.bits[(j >> 5) & (MASK_BITS / 32 - 1)] >> (j & 31) & 1u);
+        const unsigned b = __ballot_sync(FULL, pass);
+        if (!b) return;
+        if (pass) sm.queue[qn + __popc(b & lt)] = make_int2(bi, owner);
+        qn += __popc(b);
+        __syncwarp();
+        if (qn >= 32) look_up(32);
+      };
+      // rows of B of at least 32 entries, four loads in flight
+      unsigned lm = __ballot_sync(FULL, rd && len >= 32);
+      const int sl = rd && len < 32 ? len : 0;
+      while (lm) {
+        const int o = __ffs(lm) - 1;
+        lm &= lm - 1;
+        const int s = __shfl_sync(FULL, sb, o), ln = __shfl_sync(FULL, len, o);
+        for (int t = lane; t - lane < ln; t += 128) {
+          int j[4];
+#pragma unroll
+          for (int v = 0; v < 4; ++v) j[v] = t + 32 * v < ln ? B.ci[s + t + 32 * v] : 0;
+#pragma unroll
+          for (int v = 0; v < 4; ++v)
+            if (t - lane + 32 * v < ln) offer(j[v], s + t + 32 * v, o, t + 32 * v < ln);  // warp-uniform
+        }
+      }
+      // shorter ones, flattened
+      const int incl = warp_incl_scan(sl);
+      const int tot = __shfl_sync(FULL, incl, 31);
+      const int delta = sb - (incl - sl);  // entry of B minus stream position
+      for (int q0 = 0; q0 < tot; q0 += 32) {
+        const int q = q0 + lane;
+        const int o = warp_owner(incl, q);
+        const int bi = __shfl_sync(FULL, delta, o & 31) + q;
+        offer(q < tot ? B.ci[bi] : 0, bi, o & 31, q < tot);
+      }
+      if (qn > 0) look_up(qn);
+      if (staged) {
+        __syncwarp();
+        for (int t = lane; t < n; t += 32) sr_reduce_global<SR>(&out[m0 + t], sm.acc[t]);
+      }
+      __syncwarp();  // the row's columns and bits are read before the next row's
+      if (in) len = 0;
     }
-    // per lane: its row's mask range (the owner's is read by shuffle)
-    int mr0 = 0, mr1 = 0;
-    if (ve && !staged) {
-      mr0 = M.rp[i];
-      mr1 = M.rp[i + 1];
-    }
+    // ---- the others: every lane a product, searched in global memory
     const int incl = warp_incl_scan(len);
     const int tot = __shfl_sync(FULL, incl, 31);
     const int excl = incl - len;
@@ -167,19 +342,9 @@ k_masked(Csr A, Csr B, Csr M, const T* __restrict__ av, const T* __restrict__ bv
       if (q < tot) {
         const int bi = os + q - oex;
         const int j = B.ci[bi];
-        if (staged) {
-          const int p = (m1 > m0) ? find_in(mc, 0, m1 - m0, j) : -1;
-          if (p >= 0) sr_reduce_shared<SR>(&acc[p], sr_product<SR>(oa, bv[bi]));
-        } else if (ohi > olo) {
-          const int p = find_in(M.ci, olo, ohi, j);
-          if (p >= 0) sr_reduce_global<SR>(&out[p], sr_product<SR>(oa, bv[bi]));
-        }
+        const int p = find_in(M.ci, olo, ohi, j);
+        if (p >= 0) sr_reduce_global<SR>(&out[p], sr_product<SR>(oa, bv[bi]));
       }
-    }
-    if (staged) {
-      __syncwarp();
-      for (int t = lane; t < m1 - m0; t += 32) sr_reduce_global<SR>(&out[m0 + t], acc[t]);
-      __syncwarp();
     }
   }
 }
@@ -213,9 +378,7 @@ static cudaError_t masked_t(const LaunchCtx& c, const Csr& A, const Csr& B, cons
   }
   if (e != cudaSuccess || A.nnz <= 0) return e;
   auto k = k_masked<T, SR>;
-  const int occ = kernel_blocks_per_sm(k, MASK_WARPS * 32, 0);
-  const int grid = persistent_grid((A.nnz + 31) / 32, MASK_WARPS, c.nsm, occ);
-  k<<<grid, MASK_WARPS * 32, 0, c.stream>>>(A, B, M, av, bv, out);
+  k<<<(unsigned)((A.nnz + 31) / 32), 32, 0, c.stream>>>(A, B, M, av, bv, out);
   count_launch(c);
   if ((e = cudaGetLastError()) != cudaSuccess || SR != 0 || !mv) return e;
   k_scale<T><<<eg, 256, 0, c.stream>>>(out, mv, M.nnz);
