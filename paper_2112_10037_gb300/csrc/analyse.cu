@@ -78,16 +78,16 @@ __global__ void __launch_bounds__(256) k_analyse(Csr A, Csr B, long long row_beg
   constexpr int RPW = 32 / G;  // rows per warp step
   __shared__ int s_hist[NBINS];
   __shared__ unsigned long long s_total, s_max;
-  __shared__ unsigned s_wide;
+  __shared__ unsigned s_wide, s_wide8;
   if (threadIdx.x < NBINS) s_hist[threadIdx.x] = 0;
-  if (threadIdx.x == 0) { s_total = 0; s_max = 0; s_wide = 0; }
+  if (threadIdx.x == 0) { s_total = 0; s_max = 0; s_wide = 0; s_wide8 = 0; }
   if (block_skip(st)) return;  // validated input was rejected
   const int lane = lane_id();
   const int gl = lane & (G - 1), g = lane / G;
   const long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const long long nw = (gridDim.x * (long long)blockDim.x) >> 5;
   unsigned long long my_total = 0, my_max = 0;
-  unsigned my_wide = 0;
+  unsigned my_wide = 0, my_wide8 = 0;
   bool bad = false;
   for (long long r0 = w * RPW; r0 < mloc; r0 += nw * RPW) {
     const long long r = r0 + g;
@@ -136,6 +136,7 @@ __global__ void __launch_bounds__(256) k_analyse(Csr A, Csr B, long long row_beg
     mx = group_max<G>(mx);
     if (vr && gl == 0) {
       my_wide += a1 - a0 > 32 ? 1u : 0u;
+      my_wide8 += a1 - a0 > 8 ? 1u : 0u;
       prod[r] = p;
       cmin[r] = mn;
       cmax[r] = mx;
@@ -149,6 +150,7 @@ __global__ void __launch_bounds__(256) k_analyse(Csr A, Csr B, long long row_beg
     atomicMax(&s_max, my_max);
   }
   if (gl == 0 && my_wide) atomicAdd(&s_wide, my_wide);
+  if (gl == 0 && my_wide8) atomicAdd(&s_wide8, my_wide8);
   if (__any_sync(FULL, bad) && lane == 0) atomicOr(&st->err, EB_UNSORTED);
   __syncthreads();
   if (threadIdx.x < NBINS && s_hist[threadIdx.x]) atomicAdd(&st->hist[threadIdx.x], s_hist[threadIdx.x]);
@@ -157,6 +159,7 @@ __global__ void __launch_bounds__(256) k_analyse(Csr A, Csr B, long long row_beg
     atomicMax(&st->max_products, s_max);
   }
   if (threadIdx.x == 0 && s_wide) atomicAdd(&st->rows_wide, s_wide);
+  if (threadIdx.x == 0 && s_wide8) atomicAdd(&st->rows_wide8, s_wide8);
 }
 
 // Counting sort of the non-empty rows by bin, largest bin first.  Each block

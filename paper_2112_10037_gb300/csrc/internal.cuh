@@ -47,6 +47,7 @@ struct DevStats {
   long long scratch_total;  // total of the transpose's prefix sum
   uint32_t err;
   uint32_t rows_wide;  // rows of the plan with more than 32 nonzeros of A
+  uint32_t rows_wide8;  // rows with more than 8 (LANE_MERGE_K)
   int hist[NBINS];   // rows per bin
   int fill[NBINS];   // scatter cursors
   unsigned int work[8];  // dynamic work counters (reset before each use)
@@ -280,6 +281,7 @@ cudaError_t launch_numeric(const LaunchCtx& c, const Csr& A, const Csr& B, const
                            const int32_t* c_rp, int32_t* c_ci, void* c_v,
                            const int* path_rows /* host, may be null */,
                            long long rows_wide /* rows with more than 32 nonzeros, -1: unknown */,
+                           long long rows_wide8 /* rows with more than 8, -1: unknown */,
                            const int* hist /* host rows per bin, may be null: bins without rows
                                               are not launched */,
                            int semiring /* spgemm_semiring_kind */);
@@ -288,7 +290,7 @@ cudaError_t launch_numeric(const LaunchCtx& c, const Csr& A, const Csr& B, const
   cudaError_t NAME(const LaunchCtx& c, const Csr& A, const Csr& B, const RowInfo& ri, const PathBins& pb,     \
                    const Tuning& tu, const SplitInfo& sp, int dtype, const void* av, const void* bv,          \
                    int32_t* cur, int32_t* nxt, const int32_t* c_rp, int32_t* c_ci, void* c_v,                 \
-                   const int* path_rows, long long rows_wide, const int* hist)
+                   const int* path_rows, long long rows_wide, long long rows_wide8, const int* hist)
 SG_NUMERIC_SR_DECL(launch_numeric_min_plus);
 SG_NUMERIC_SR_DECL(launch_numeric_max_plus);
 SG_NUMERIC_SR_DECL(launch_numeric_or_and);

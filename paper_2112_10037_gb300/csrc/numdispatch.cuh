@@ -234,9 +234,16 @@ template <typename T, int SR>
 static cudaError_t numeric_t(const LaunchCtx& c, const Csr& A, const Csr& B, const RowInfo& ri,
                              const PathBins& pb, const Tuning& tu, const SplitInfo& sp, const T* av,
                              const T* bv, int32_t* cur, int32_t* nxt, const int32_t* c_rp, int32_t* c_ci,
-                             T* c_v, const int* path_rows, long long rows_wide, const int* hist) {
+                             T* c_v, const int* path_rows, long long rows_wide, long long rows_wide8, const int* hist) {
   cudaError_t e = cudaSuccess;
-  if (pb.hi[PATH_TINY] >= pb.lo[PATH_TINY]) {
+  // When no row has more than LANE_MERGE_K nonzeros (stencil products, and
+  // stencils times an aggregation), rows of at most 64 products are merged by
+  // one lane each, the smallest ones too: the register sort exchanges every
+  // product of a row with its neighbours log2(P)^2 / 2 times (96^3 Galerkin,
+  // A*P with 7 products a row: 107 us).
+  const bool merge = rows_wide8 == 0 && path_rows && pb.hi[PATH_HASH] >= pb.lo[PATH_HASH] &&
+                     pb.hi[PATH_TINY] + 1 == pb.lo[PATH_HASH];
+  if (pb.hi[PATH_TINY] >= pb.lo[PATH_TINY] && !merge) {
     const long long rows = rows_in(path_rows, PATH_TINY);
     timer_mark(c, T_NUM_TINY, 0);
     e = tiny_dispatch(hist, pb.lo[PATH_TINY], pb.hi[PATH_TINY],
@@ -261,10 +268,11 @@ static cudaError_t numeric_t(const LaunchCtx& c, const Csr& A, const Csr& B, con
     long long all_rows = 0;
     if (path_rows)
       for (int q = 0; q < NPATHS; ++q) all_rows += path_rows[q];
-    const bool lanes = path_rows && 2 * (long long)path_rows[PATH_HASH] >= all_rows;
-    const int llo = pb.lo[PATH_HASH], lhi = lanes ? (pb.hi[PATH_HASH] < 7 ? pb.hi[PATH_HASH] : 7) : 0;
+    const bool lanes = merge || (path_rows && 2 * (long long)path_rows[PATH_HASH] >= all_rows);
+    const int llo = merge ? pb.lo[PATH_TINY] : pb.lo[PATH_HASH], lhi = lanes ? (pb.hi[PATH_HASH] < 7 ? pb.hi[PATH_HASH] : 7) : 0;
     if (llo <= lhi && !empty_bins(hist, llo, lhi))
-      e = lane_rows<true, T, SR>(c, A, B, av, bv, ri, llo, lhi, nullptr, c_rp, c_ci, c_v, rows);
+      e = lane_rows<true, T, SR>(c, A, B, av, bv, ri, llo, lhi, nullptr, c_rp, c_ci, c_v,
+                                 merge ? rows + path_rows[PATH_TINY] : rows, rows_wide8);
     const int wlo = lhi >= llo ? lhi + 1 : llo;
     if (!e && pb.hi[PATH_HASH] >= wlo)
       e = hash_dispatch(hist, wlo, pb.hi[PATH_HASH],
@@ -343,12 +351,12 @@ static cudaError_t launch_numeric_sr(const LaunchCtx& c, const Csr& A, const Csr
                                      const PathBins& pb, const Tuning& tu, const SplitInfo& sp, int dtype,
                                      const void* av, const void* bv, int32_t* cur, int32_t* nxt,
                                      const int32_t* c_rp, int32_t* c_ci, void* c_v, const int* path_rows,
-                                     long long rows_wide, const int* hist) {
+                                     long long rows_wide, long long rows_wide8, const int* hist) {
   if (dtype == SPGEMM_F32)
     return numeric_t<float, SR>(c, A, B, ri, pb, tu, sp, (const float*)av, (const float*)bv, cur, nxt, c_rp, c_ci,
-                                (float*)c_v, path_rows, rows_wide, hist);
+                                (float*)c_v, path_rows, rows_wide, rows_wide8, hist);
   return numeric_t<double, SR>(c, A, B, ri, pb, tu, sp, (const double*)av, (const double*)bv, cur, nxt, c_rp, c_ci,
-                               (double*)c_v, path_rows, rows_wide, hist);
+                               (double*)c_v, path_rows, rows_wide, rows_wide8, hist);
 }
 
 }  // namespace sg

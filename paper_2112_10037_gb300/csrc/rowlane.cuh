@@ -23,9 +23,8 @@
 // A row of P <= 64 products has at most 64 distinct columns, so its table
 // never overflows (the probe loop is bounded by the table size).
 //
-// In the numeric pass, rows with at most 8 nonzeros of A (the 7-point
-// stencil's) skip the table: k_lane_merge stages the row's B rows in the
-// same shared memory and merges them in column order.
+// Rows with at most 8 nonzeros of A (the 7-point stencil's) skip the table:
+// their B rows are merged in column order from registers (lane_merge_rows).
 #pragma once
 
 #include "launch_util.cuh"
@@ -169,32 +168,125 @@ k_lane_rows(Csr A, Csr B, const T* __restrict__ av, const T* __restrict__ bv, Ro
 }
 
 // Rows with at most LANE_MERGE_K nonzeros of A (every row of a 7-point
-// stencil product): one lane per row stages its B rows (each sorted, at most
-// 64 products in all: columns and values) in its slot-major shared-memory
-// column, then merges them -- the next output column is the smallest head column, its
-// value the products of the heads that hold it, each head advanced past it
-// -- so the row comes out in column order with no table and no ranking.  The
-// sums run in A's order, every product fused into the running sum from the
-// semiring's identity (for plus-times the first product is a*b rounded,
+// stencil product and of a stencil times an aggregation): one lane per row
+// merges its B rows -- the next output column is the smallest head column,
+// its value the products of the heads that hold it, each head advanced past
+// it -- so the row comes out in column order with no table and no ranking.
+// The sums run in A's order, every product fused into the running sum from
+// the semiring's identity (for plus-times the first product is a*b rounded,
 // +0 where that product is exactly -0).
-// (Measured on the 96^3 stencil: staging only the columns, for more warps
-// per SM, and reading B's values from global memory was 13 % slower; one
-// product per inner round, to issue fewer FP64 warp instructions, 14 %.)
+//
+// A head's column, the column after it and its value are in registers, read
+// one step before they are needed, so no shared memory holds B rows and an SM
+// keeps as many warps as the registers allow.  Outputs are collected 8 per
+// row and written by 8 lanes per row: lanes that wrote their own rows would
+// touch 32 sectors with every store.  96^3 stencil squared in FP64: 0.37 ms
+// with the B rows staged in shared memory (8 warps per SM, lanes storing their
+// own rows), 0.20 ms here (20 warps at 96 registers); the floor of one FP64
+// operation per product and full warps is 0.07 ms, that of the bytes 0.04 ms.
+// A heads' test issues its FP64 instruction when any lane of the warp matches.
 constexpr int LANE_MERGE_K = 8;
+constexpr int LANE_OUT = 8;          // outputs collected per row
+constexpr int LANE_OUT_CI = 36;      // strides of the collecting arrays that keep both
+constexpr int LANE_OUT_V = 34;       // sides of the exchange free of bank conflicts
+
+template <typename T>
+struct LaneOut {
+  T val[LANE_OUT * LANE_OUT_V];
+  int col[LANE_OUT * LANE_OUT_CI];
+};
+
+// The 8 outputs from `first` on of every lane's row (n: the row's outputs so
+// far, its entries go to [ob, oe)).  Every lane must call it.
+template <typename T>
+__device__ __forceinline__ void lane_flush(const LaneOut<T>& so, int first, int n, int ob, int oe,
+                                           int32_t* __restrict__ c_ci, T* __restrict__ c_v) {
+  const int lane = lane_id(), t = lane & 7;
+  __syncwarp();
+#pragma unroll
+  for (int g = 0; g < 8; ++g) {
+    const int j = g * 4 + (lane >> 3);
+    const int nj = __shfl_sync(FULL, n, j), oj = __shfl_sync(FULL, ob, j), ej = __shfl_sync(FULL, oe, j);
+    const int o = oj + first + t;
+    if (first + t < nj && o < ej) {
+      c_ci[o] = so.col[t * LANE_OUT_CI + j];
+      c_v[o] = so.val[t * LANE_OUT_V + j];
+    }
+  }
+  __syncwarp();
+}
+
+// One warp's 32 rows (a0 == a1: none).  NUM: columns and values to [ob, oe);
+// returns the lane's distinct columns.
+template <bool NUM, typename T, int SR>
+__device__ __forceinline__ int lane_merge_rows(const Csr& A, const Csr& B, const T* __restrict__ av,
+                                               const T* __restrict__ bv, int a0, int a1, LaneOut<T>* so, int ob,
+                                               int oe, int32_t* __restrict__ c_ci, T* __restrict__ c_v) {
+  using Ops = SrOps<T, SR>;
+  constexpr int K = LANE_MERGE_K;
+  const int lane = lane_id();
+  int hs[K], he[K], hc[K], hn[K];  // head position, end, head column, the column after it
+  T a[K], v[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    hs[k] = he[k] = 0;
+    a[k] = v[k] = T(0);
+    if (a0 + k < a1) {
+      const int kk = A.ci[a0 + k];
+      hs[k] = B.rp[kk];
+      he[k] = B.rp[kk + 1];
+      if (NUM) a[k] = av[a0 + k];
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    hc[k] = hs[k] < he[k] ? B.ci[hs[k]] : INT_MAX;
+    hn[k] = hs[k] + 1 < he[k] ? B.ci[hs[k] + 1] : INT_MAX;
+    if (NUM && hs[k] < he[k]) v[k] = bv[hs[k]];
+  }
+  int n = 0;
+  for (int step = 0;; ++step) {
+    int m = hc[0];
+#pragma unroll
+    for (int k = 1; k < K; ++k) m = min(m, hc[k]);
+    const bool act = m != INT_MAX;
+    if (NUM && step > 0 && (step & (LANE_OUT - 1)) == 0) lane_flush(*so, step - LANE_OUT, n, ob, oe, c_ci, c_v);
+    if (!__any_sync(FULL, act)) {
+      if (NUM && (step & (LANE_OUT - 1)) != 0) lane_flush(*so, step & ~(LANE_OUT - 1), n, ob, oe, c_ci, c_v);
+      break;
+    }
+    if (act) {
+      T acc = Ops::zero();
+      bool any = false;
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        if (hc[k] == m) {
+          if (NUM) acc = Ops::madd(a[k], v[k], any ? acc : Ops::zero());  // one FP64 instruction per head test
+          any = true;
+          ++hs[k];
+          hc[k] = hn[k];
+          hn[k] = hs[k] + 1 < he[k] ? B.ci[hs[k] + 1] : INT_MAX;
+          if (NUM && hs[k] < he[k]) v[k] = bv[hs[k]];
+        }
+      }
+      if (NUM) {
+        so->col[(step & (LANE_OUT - 1)) * LANE_OUT_CI + lane] = m;
+        so->val[(step & (LANE_OUT - 1)) * LANE_OUT_V + lane] = acc;
+      }
+      ++n;
+    }
+  }
+  return n;
+}
 
 template <typename T, int SR>
 __global__ void __launch_bounds__(LANE_WARPS * 32)
 k_lane_merge(Csr A, Csr B, const T* __restrict__ av, const T* __restrict__ bv, RowInfo ri, const DevStats* st,
              int bin_lo, int bin_hi, const int32_t* __restrict__ c_rp, int32_t* __restrict__ c_ci,
              T* __restrict__ c_v, uint32_t* err) {
-  using Ops = SrOps<T, SR>;
-  constexpr int K = LANE_MERGE_K;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ LaneOut<T> s_out[LANE_WARPS];
   __shared__ int s_lb, s_le;
   const int warp = threadIdx.x >> 5, lane = lane_id();
-  const size_t per_warp = (size_t)LANE_SLOTS * 32 * (sizeof(int) + sizeof(T));
-  int* scol = reinterpret_cast<int*>(smem_raw + warp * per_warp);  // [slot][lane]
-  T* sval = reinterpret_cast<T*>(smem_raw + warp * per_warp + (size_t)LANE_SLOTS * 32 * sizeof(int));
   if (threadIdx.x == 0) bin_range(st, bin_lo, bin_hi, &s_lb, &s_le);
   if (block_skip(st)) return;
   const long long lb = s_lb, le = s_le;
@@ -202,78 +294,19 @@ k_lane_merge(Csr A, Csr B, const T* __restrict__ av, const T* __restrict__ bv, R
   const long long nw = (long long)gridDim.x * LANE_WARPS;
   for (long long base = lb + gw * 32; base < le; base += nw * 32) {
     const long long idx = base + lane;
-    if (idx >= le) continue;
-    const int r = ri.rows[idx];
-    const long long i = ri.row_begin + r;
-    const int a0 = A.rp[i], a1 = A.rp[i + 1];
-    if (a1 - a0 > K) continue;  // k_lane_rows takes the row
-    // stage B(k,:), the row's k-th nonzero, into slots [hs[k], he[k])
-    int hs[K], he[K];
-    T a[K];
-    int q = 0;
-    bool over = false;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      hs[k] = q;
-      he[k] = q;
-      a[k] = T(0);
-      if (a0 + k < a1) {
-        const int kk = A.ci[a0 + k];
-        a[k] = av[a0 + k];
-        const int s0 = B.rp[kk];
-        int len = B.rp[kk + 1] - s0;
-        if (q + len > LANE_SLOTS) {
-          over = true;
-          len = LANE_SLOTS - q;
-        }
-        for (int g = 0; g < len; g += 4) {
-          int cc[4];
-          T vv[4];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            cc[u] = g + u < len ? B.ci[s0 + g + u] : 0;
-            vv[u] = g + u < len ? bv[s0 + g + u] : T(0);
-          }
-#pragma unroll
-          for (int u = 0; u < 4; ++u)
-            if (g + u < len) {
-              scol[(q + g + u) * 32 + lane] = cc[u];
-              sval[(q + g + u) * 32 + lane] = vv[u];
-            }
-        }
-        q += len;
-        he[k] = q;
+    int a0 = 0, a1 = 0, ob = 0, oe = 0;
+    if (idx < le) {
+      const int r = ri.rows[idx];
+      a0 = A.rp[ri.row_begin + r];
+      a1 = A.rp[ri.row_begin + r + 1];
+      if (a1 - a0 > LANE_MERGE_K) a0 = a1;  // k_lane_rows takes the row
+      if (a1 > a0) {
+        ob = c_rp[r];
+        oe = c_rp[r + 1];
       }
     }
-    int hc[K];  // head column of each staged row (INT_MAX when exhausted)
-#pragma unroll
-    for (int k = 0; k < K; ++k) hc[k] = hs[k] < he[k] ? scol[hs[k] * 32 + lane] : INT_MAX;
-    const int ob = c_rp[r], oe = c_rp[r + 1];
-    int o = ob;
-    while (true) {
-      int m = hc[0];
-#pragma unroll
-      for (int k = 1; k < K; ++k) m = min(m, hc[k]);
-      if (m == INT_MAX) break;
-      T acc = Ops::zero();
-      bool any = false;
-#pragma unroll
-      for (int k = 0; k < K; ++k) {
-        if (hc[k] == m) {
-          const T b = sval[hs[k] * 32 + lane];
-          acc = Ops::madd(a[k], b, any ? acc : Ops::zero());  // one FP64 instruction per head test
-          any = true;
-          ++hs[k];
-          hc[k] = hs[k] < he[k] ? scol[hs[k] * 32 + lane] : INT_MAX;
-        }
-      }
-      if (o < oe) {
-        c_ci[o] = m;
-        c_v[o] = acc;
-      }
-      ++o;
-    }
-    if (over || o != oe) atomicOr(err, EB_INTERNAL);  // the row's bin and the symbolic count rule both out
+    const int n = lane_merge_rows<true, T, SR>(A, B, av, bv, a0, a1, &s_out[warp], ob, oe, c_ci, c_v);
+    if (a1 > a0 && ob + n != oe) atomicOr(err, EB_INTERNAL);  // the symbolic count rules this out
   }
 }
 
@@ -284,24 +317,24 @@ constexpr size_t lane_rows_smem() {
 
 // Launch over the rows of bins [lo, hi] (rows: their number, -1 unknown).
 // The numeric pass merges rows of at most LANE_MERGE_K nonzeros of A
-// (k_lane_merge) and hashes the others; the symbolic pass hashes all.
+// (k_lane_merge) and hashes the others (wide8: rows of the plan with more, -1
+// unknown); the symbolic pass hashes all.
 template <bool NUM, typename T, int SR = SPGEMM_PLUS_TIMES>
 static cudaError_t lane_rows(const LaunchCtx& c, const Csr& A, const Csr& B, const T* av, const T* bv,
                              const RowInfo& ri, int lo, int hi, int32_t* c_cnt, const int32_t* c_rp,
-                             int32_t* c_ci, T* c_v, long long rows) {
-  const size_t smem = lane_rows_smem<NUM, T>();
+                             int32_t* c_ci, T* c_v, long long rows, long long wide8) {
   if constexpr (NUM) {
     auto km = k_lane_merge<T, SR>;
-    const size_t smem_m = smem;  // columns and values of 64 staged products per lane
-    const int occm = kernel_blocks_per_sm(km, LANE_WARPS * 32, smem_m);
+    const int occm = kernel_blocks_per_sm(km, LANE_WARPS * 32, 0);
     if (occm <= 0) return cudaErrorInvalidConfiguration;
     const int gridm = persistent_grid(rows, LANE_WARPS * 32, c.nsm, occm);
-    km<<<gridm, LANE_WARPS * 32, smem_m, c.stream>>>(A, B, av, bv, ri, c.st, lo, hi, c_rp, c_ci, c_v, c.err);
+    km<<<gridm, LANE_WARPS * 32, 0, c.stream>>>(A, B, av, bv, ri, c.st, lo, hi, c_rp, c_ci, c_v, c.err);
     count_launch(c);
     const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess || wide8 == 0) return e;
   }
   auto k = k_lane_rows<NUM, T, SR>;
+  const size_t smem = lane_rows_smem<NUM, T>();
   const int occ = kernel_blocks_per_sm(k, LANE_WARPS * 32, smem);
   if (occ <= 0) return cudaErrorInvalidConfiguration;
   const int grid = persistent_grid(rows, LANE_WARPS * 32, c.nsm, occ);

@@ -126,7 +126,7 @@ cudaError_t launch_symbolic(const LaunchCtx& c, const Csr& A, const Csr& B, cons
     // rows of at most 64 products: one lane per row; 65..128: a warp per row
     const int llo = pb.lo[PATH_HASH], lhi = pb.hi[PATH_HASH] < 7 ? pb.hi[PATH_HASH] : 7;
     if (llo <= lhi)
-      e = lane_rows<false, double>(c, A, B, nullptr, nullptr, ri, llo, lhi, c_cnt, nullptr, nullptr, nullptr, rows);
+      e = lane_rows<false, double>(c, A, B, nullptr, nullptr, ri, llo, lhi, c_cnt, nullptr, nullptr, nullptr, rows, -1);
     if (!e && pb.hi[PATH_HASH] >= 8)
       e = hash_dispatch(8, pb.hi[PATH_HASH],
           [&](int l, int h) { return hash_sym<1>(c, A, B, ri, l, h, c_cnt, rows); },
