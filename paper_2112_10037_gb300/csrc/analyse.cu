@@ -64,77 +64,66 @@ __device__ __forceinline__ int group_max(int v) {
   }
 }
 
-// G lanes per row of A (32: one warp; 8: four rows per warp, for matrices
-// of short rows, where a warp per row leaves most lanes idle and each
-// warp's rows form one long chain of dependent loads): P_i, the smallest and
-// largest column any product of the row reaches (first and last column of
-// each touched B row, since B's rows are sorted), histogram of bins, total
-// and maximum P.
-template <int G>
+// This lane's share of the row of A at [a0, a1), a warp walking it: products,
+// smallest and largest column reached.  Four entries per lane per step, their
+// dependent loads in flight together (long rows of power-law matrices
+// otherwise form the tail).
+__device__ __forceinline__ void analyse_walk(const Csr& A, const Csr& B, int a0, int a1, long long* p, int* mn,
+                                             int* mx, bool* bad) {
+  for (int e0 = a0 + lane_id(); e0 < a1; e0 += 128) {
+    int kk[4], ss[4], tt[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) kk[u] = e0 + 32 * u < a1 ? A.ci[e0 + 32 * u] : -1;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      ss[u] = tt[u] = 0;
+      if (e0 + 32 * u < a1) {
+        if (kk[u] < 0 || (long long)kk[u] >= B.nrows) {
+          *bad = true;
+        } else {
+          ss[u] = B.rp[kk[u]];
+          tt[u] = B.rp[kk[u] + 1];
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      if (tt[u] > ss[u]) {
+        *p += tt[u] - ss[u];
+        *mn = min(*mn, B.ci[ss[u]]);
+        *mx = max(*mx, B.ci[tt[u] - 1]);
+      }
+    }
+  }
+}
+
+// One warp per row of A: P_i, the smallest and largest column any product of
+// the row reaches (first and last column of each touched B row, since B's rows
+// are sorted), histogram of bins, total and maximum P.
 __global__ void __launch_bounds__(256) k_analyse(Csr A, Csr B, long long row_begin, long long mloc,
                                                  long long* __restrict__ prod, int* __restrict__ cmin,
                                                  int* __restrict__ cmax, DevStats* st) {
-  static_assert(G == 8 || G == 16 || G == 32, "lanes per row");
-  constexpr int RPW = 32 / G;  // rows per warp step
   __shared__ int s_hist[NBINS];
   __shared__ unsigned long long s_total, s_max;
   __shared__ unsigned s_wide, s_wide8;
   if (threadIdx.x < NBINS) s_hist[threadIdx.x] = 0;
   if (threadIdx.x == 0) { s_total = 0; s_max = 0; s_wide = 0; s_wide8 = 0; }
   if (block_skip(st)) return;  // validated input was rejected
-  const int lane = lane_id();
-  const int gl = lane & (G - 1), g = lane / G;
+  const int lane = lane_id(), gl = lane;
   const long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const long long nw = (gridDim.x * (long long)blockDim.x) >> 5;
   unsigned long long my_total = 0, my_max = 0;
   unsigned my_wide = 0, my_wide8 = 0;
   bool bad = false;
-  for (long long r0 = w * RPW; r0 < mloc; r0 += nw * RPW) {
-    const long long r = r0 + g;
-    const bool vr = r < mloc;
-    const long long i = row_begin + r;
-    int a0 = 0, a1 = 0;
-    if (vr) {
-      a0 = A.rp[i];
-      a1 = A.rp[i + 1];
-    }
+  for (long long r = w; r < mloc; r += nw) {
+    const int a0 = A.rp[row_begin + r], a1 = A.rp[row_begin + r + 1];
     long long p = 0;
     int mn = INT_MAX, mx = -1;
-    // four entries per lane per step, their dependent loads in flight
-    // together (long rows of power-law matrices otherwise form the tail)
-    for (int e0 = a0 + gl; e0 < a1; e0 += 4 * G) {
-      int kk[4], ss[4], tt[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int e = e0 + G * u;
-        kk[u] = e < a1 ? A.ci[e] : -1;
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int e = e0 + G * u;
-        ss[u] = tt[u] = 0;
-        if (e < a1) {
-          if (kk[u] < 0 || (long long)kk[u] >= B.nrows) {
-            bad = true;
-          } else {
-            ss[u] = B.rp[kk[u]];
-            tt[u] = B.rp[kk[u] + 1];
-          }
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        if (tt[u] > ss[u]) {
-          p += tt[u] - ss[u];
-          mn = min(mn, B.ci[ss[u]]);
-          mx = max(mx, B.ci[tt[u] - 1]);
-        }
-      }
-    }
-    p = group_sum<G>(p);
-    mn = group_min<G>(mn);
-    mx = group_max<G>(mx);
-    if (vr && gl == 0) {
+    analyse_walk(A, B, a0, a1, &p, &mn, &mx, &bad);
+    p = warp_sum(p);
+    mn = warp_min(mn);
+    mx = warp_max(mx);
+    if (lane == 0) {
       my_wide += a1 - a0 > 32 ? 1u : 0u;
       my_wide8 += a1 - a0 > 8 ? 1u : 0u;
       prod[r] = p;
@@ -162,10 +151,145 @@ __global__ void __launch_bounds__(256) k_analyse(Csr A, Csr B, long long row_beg
   if (threadIdx.x == 0 && s_wide8) atomicAdd(&st->rows_wide8, s_wide8);
 }
 
+// The same for matrices of short rows (stencils, aggregation operators): 8
+// lanes per row, four rows per group in flight, so that the chain of dependent
+// loads (row pointer, column, row pointer of B) is paid once per 16 rows of a
+// warp; rows of more than 32 nonzeros are walked by the warp.  Column spans are read in a second walk and only for rows of more than
+// span_min products (the paths of smaller rows never use them).  96^3 stencil
+// squared: 76 us with one row per group and every row's span, 40 us here.
+__global__ void __launch_bounds__(256) k_analyse_short(Csr A, Csr B, long long row_begin, long long mloc,
+                                                       long long* __restrict__ prod, int* __restrict__ cmin,
+                                                       int* __restrict__ cmax, DevStats* st, long long span_min) {
+  constexpr int G = 8, RPW = 32 / G, U = 4;
+  __shared__ int s_hist[NBINS];
+  __shared__ unsigned long long s_total, s_max;
+  __shared__ unsigned s_wide, s_wide8;
+  if (threadIdx.x < NBINS) s_hist[threadIdx.x] = 0;
+  if (threadIdx.x == 0) { s_total = 0; s_max = 0; s_wide = 0; s_wide8 = 0; }
+  if (block_skip(st)) return;  // validated input was rejected
+  const int lane = lane_id();
+  const int gl = lane & (G - 1), g = lane / G;
+  const long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+  const long long nw = (gridDim.x * (long long)blockDim.x) >> 5;
+  unsigned long long my_total = 0, my_max = 0;
+  unsigned my_wide = 0, my_wide8 = 0;
+  bool bad = false;
+  for (long long r0 = w * RPW * U; r0 < mloc; r0 += nw * RPW * U) {
+    int a0[U], a1[U], k[U];
+    long long p[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const long long r = r0 + u * RPW + g;
+      a0[u] = a1[u] = 0;
+      if (r < mloc) {
+        a0[u] = A.rp[row_begin + r];
+        a1[u] = A.rp[row_begin + r + 1];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) k[u] = (a0[u] + gl < a1[u] && a1[u] - a0[u] <= 32) ? A.ci[a0[u] + gl] : -1;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      p[u] = 0;
+      if (a0[u] + gl < a1[u] && a1[u] - a0[u] <= 32) {
+        if (k[u] < 0 || (long long)k[u] >= B.nrows) bad = true;
+        else p[u] = B.rp[k[u] + 1] - B.rp[k[u]];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const bool wide = a1[u] - a0[u] > 32;
+      if (!wide)
+        for (int e = a0[u] + G + gl; e < a1[u]; e += G) {  // rows of more than 8 nonzeros
+          const int kk = A.ci[e];
+          if (kk < 0 || (long long)kk >= B.nrows) bad = true;
+          else p[u] += B.rp[kk + 1] - B.rp[kk];
+        }
+      p[u] = group_sum<G>(p[u]);
+      const long long r = r0 + u * RPW + g;
+      unsigned wm = __ballot_sync(FULL, wide && gl == 0);
+      while (wm) {
+        const int L = __ffs(wm) - 1;
+        wm &= wm - 1;
+        long long wp = 0;
+        int mn = INT_MAX, mx = -1;
+        analyse_walk(A, B, __shfl_sync(FULL, a0[u], L), __shfl_sync(FULL, a1[u], L), &wp, &mn, &mx, &bad);
+        wp = warp_sum(wp);
+        mn = warp_min(mn);
+        mx = warp_max(mx);
+        if (g == L / G) p[u] = wp;
+        if (lane == L) {
+          cmin[r] = mn;
+          cmax[r] = mx;
+        }
+      }
+      if (__any_sync(FULL, p[u] > span_min && !wide)) {
+        int mn = INT_MAX, mx = -1;
+        if (p[u] > span_min && !wide)
+          for (int e = a0[u] + gl; e < a1[u]; e += G) {
+            const int kk = A.ci[e];
+            if (kk >= 0 && (long long)kk < B.nrows) {
+              const int s = B.rp[kk], t = B.rp[kk + 1];
+              if (t > s) {
+                mn = min(mn, B.ci[s]);
+                mx = max(mx, B.ci[t - 1]);
+              }
+            }
+          }
+        mn = group_min<G>(mn);
+        mx = group_max<G>(mx);
+        if (gl == 0 && r < mloc && p[u] > span_min && !wide) {
+          cmin[r] = mn;
+          cmax[r] = mx;
+        }
+      }
+      if (gl == 0 && r < mloc) {
+        my_wide += a1[u] - a0[u] > 32 ? 1u : 0u;
+        my_wide8 += a1[u] - a0[u] > 8 ? 1u : 0u;
+        prod[r] = p[u];
+        atomicAdd(&s_hist[bin_of(p[u])], 1);
+        my_total += (unsigned long long)p[u];
+        my_max = my_max > (unsigned long long)p[u] ? my_max : (unsigned long long)p[u];
+      }
+    }
+  }
+  if (gl == 0 && my_total) {
+    atomicAdd(&s_total, my_total);
+    atomicMax(&s_max, my_max);
+  }
+  if (gl == 0 && my_wide) atomicAdd(&s_wide, my_wide);
+  if (gl == 0 && my_wide8) atomicAdd(&s_wide8, my_wide8);
+  if (__any_sync(FULL, bad) && lane == 0) atomicOr(&st->err, EB_UNSORTED);
+  __syncthreads();
+  if (threadIdx.x < NBINS && s_hist[threadIdx.x]) atomicAdd(&st->hist[threadIdx.x], s_hist[threadIdx.x]);
+  if (threadIdx.x == 0 && s_total) {
+    atomicAdd(&st->total_products, s_total);
+    atomicMax(&st->max_products, s_max);
+  }
+  if (threadIdx.x == 0 && s_wide) atomicAdd(&st->rows_wide, s_wide);
+  if (threadIdx.x == 0 && s_wide8) atomicAdd(&st->rows_wide8, s_wide8);
+}
+
 // Counting sort of the non-empty rows by bin, largest bin first.  Each block
 // takes a contiguous chunk of rows: counts per bin in shared memory, reserves
 // one range per bin with a single global atomic, then places its rows.
-constexpr int SCATTER_ROWS = 4096;
+// (1024 rows: a matrix of a few thousand rows otherwise fits one block.)  Lanes
+// of one bin -- in a stencil's product all of them -- count with one atomic.
+constexpr int SCATTER_ROWS = 1024;
+
+// Adds one per lane to cnt[b] (active lanes: b > 0); returns the lane's place.
+__device__ __forceinline__ int bin_add(int* cnt, int b) {
+  const int lane = lane_id();
+  const unsigned act = __ballot_sync(FULL, b > 0);
+  if (!act) return 0;
+  const int b0 = __shfl_sync(FULL, b, __ffs(act) - 1);
+  if (__all_sync(FULL, b == 0 || b == b0)) {
+    int at = 0;
+    if (lane == __ffs(act) - 1) at = atomicAdd(&cnt[b0], __popc(act));
+    return __shfl_sync(FULL, at, __ffs(act) - 1) + __popc(act & lanemask_lt());
+  }
+  return b > 0 ? atomicAdd(&cnt[b], 1) : 0;
+}
 
 __global__ void __launch_bounds__(256) k_bin_scatter(const long long* __restrict__ prod, long long mloc,
                                                      DevStats* st, int* __restrict__ rows) {
@@ -182,10 +306,14 @@ __global__ void __launch_bounds__(256) k_bin_scatter(const long long* __restrict
   __syncthreads();
   const long long r0 = (long long)blockIdx.x * SCATTER_ROWS;
   const long long r1 = min(mloc, r0 + SCATTER_ROWS);
-  for (long long r = r0 + threadIdx.x; r < r1; r += blockDim.x) {
-    const int b = bin_of(prod[r]);
-    if (b) atomicAdd(&s_cnt[b], 1);
+  int bins[SCATTER_ROWS / 256];
+#pragma unroll
+  for (int u = 0; u < SCATTER_ROWS / 256; ++u) {
+    const long long r = r0 + u * 256 + threadIdx.x;
+    bins[u] = r < r1 ? bin_of(prod[r]) : 0;
   }
+#pragma unroll
+  for (int u = 0; u < SCATTER_ROWS / 256; ++u) bin_add(s_cnt, bins[u]);
   __syncthreads();
   if (threadIdx.x < NBINS) {
     const int b = threadIdx.x;
@@ -193,27 +321,14 @@ __global__ void __launch_bounds__(256) k_bin_scatter(const long long* __restrict
     s_cnt[b] = 0;
   }
   __syncthreads();
-  for (long long r = r0 + threadIdx.x; r < r1; r += blockDim.x) {
-    const int b = bin_of(prod[r]);
-    if (b) rows[s_base[b] + atomicAdd(&s_cnt[b], 1)] = (int)r;
+#pragma unroll
+  for (int u = 0; u < SCATTER_ROWS / 256; ++u) {
+    const int at = bin_add(s_cnt, bins[u]);
+    if (bins[u]) rows[s_base[bins[u]] + at] = (int)(r0 + u * 256 + threadIdx.x);
   }
 }
 
 static int grid_for_warps(long long nwarps, int warps_per_block, int nsm);
-
-// True (for the whole block) when win_lo > 0 and the analysis put no row in
-// bins win_lo and above, i.e. no row takes a numeric window path and the
-// window-run lists will never be read.
-__device__ __forceinline__ bool no_window_rows(const DevStats* st, int win_lo) {
-  __shared__ int s_none;
-  if (threadIdx.x == 0) {
-    int n = 0;
-    for (int b = win_lo > 0 ? win_lo : NBINS; b < NBINS; ++b) n += st->hist[b];
-    s_none = win_lo > 0 && n == 0;
-  }
-  __syncthreads();
-  return s_none != 0;
-}
 
 // Window-run lists of B (see SplitInfo), at two window widths (shifts s1
 // and s2) from one read of B: pass 1 counts the runs of each row (plus its
@@ -221,18 +336,11 @@ __device__ __forceinline__ bool no_window_rows(const DevStats* st, int win_lo) {
 // (window id, first position) of every run.  One warp per row; a run starts
 // where the window id differs from the previous entry's.  A null second list
 // is skipped.  With no row in a window bin (win_lo, see no_window_rows) the
-// counts are written as zeros and the lists stay unbuilt.
+// lists stay unbuilt.
 __global__ void __launch_bounds__(256) k_runs_count(Csr B, int s1, int32_t* __restrict__ rr1, int s2,
                                                     int32_t* __restrict__ rr2, const DevStats* st, int win_lo) {
   if (block_skip(st)) return;
-  if (no_window_rows(st, win_lo)) {
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < B.nrows;
-         k += (long long)gridDim.x * blockDim.x) {
-      rr1[k] = 0;
-      if (rr2) rr2[k] = 0;
-    }
-    return;
-  }
+  if (no_window_rows(st, win_lo)) return;
   const int lane = lane_id();
   const long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const long long nw = (gridDim.x * (long long)blockDim.x) >> 5;
@@ -317,8 +425,7 @@ cudaError_t launch_runs(const LaunchCtx& c, const Csr& B, const SplitInfo& sp, l
   count_launch(c);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  e = launch_scan(c, sp.rr, B.nrows, partials, &c.st->nruns);
-  if (e == cudaSuccess && two) e = launch_scan(c, sp.rrb, B.nrows, partials, &c.st->nruns_b);
+  e = launch_scan_runs(c, sp.rr, two ? sp.rrb : nullptr, B.nrows, partials, win_lo);
   if (e != cudaSuccess) return e;
   k_runs_fill<<<grid, 256, 0, c.stream>>>(B, sp.wf_shift, sp.rr, sp.runs, sp.wb_shift, two ? sp.rrb : nullptr,
                                           two ? sp.runsb : nullptr, c.st, win_lo);
@@ -340,16 +447,16 @@ cudaError_t launch_validate(const LaunchCtx& c, const Csr& M) {
 }
 
 cudaError_t launch_analyse(const LaunchCtx& c, const Csr& A, const Csr& B, long long row_begin,
-                           long long mloc, long long* prod, int* cmin, int* cmax, int* rows) {
+                           long long mloc, long long* prod, int* cmin, int* cmax, int* rows,
+                           long long span_min) {
   if (mloc <= 0) return cudaSuccess;
   timer_mark(c, T_ANALYSE, 0);
   // short rows on average (stencils, aggregation operators): 8 lanes per row
   if (A.nrows > 0 && A.nnz <= 12 * A.nrows)
-    k_analyse<8><<<grid_for_warps((mloc + 3) / 4, 8, c.nsm), 256, 0, c.stream>>>(A, B, row_begin, mloc, prod,
-                                                                                 cmin, cmax, c.st);
+    k_analyse_short<<<grid_for_warps((mloc + 15) / 16, 8, c.nsm), 256, 0, c.stream>>>(A, B, row_begin, mloc, prod,
+                                                                                     cmin, cmax, c.st, span_min);
   else
-    k_analyse<32><<<grid_for_warps(mloc, 8, c.nsm), 256, 0, c.stream>>>(A, B, row_begin, mloc, prod, cmin,
-                                                                       cmax, c.st);
+    k_analyse<<<grid_for_warps(mloc, 8, c.nsm), 256, 0, c.stream>>>(A, B, row_begin, mloc, prod, cmin, cmax, c.st);
   count_launch(c);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;

@@ -205,7 +205,7 @@ Layout layout_for(const spgemm_opts& o, long long mloc, long long nnz_a, long lo
   if (own_b) {
     L.rr = off; off = align_up(off + sizeof(int32_t) * (size_t)(nrows_b + 1));
     L.runs = off; off = align_up(off + sizeof(int2) * (size_t)(nnz_b + nrows_b + sg::RUNS_PAD));
-    L.runs_part = off; off = align_up(off + sizeof(long long) * sg::scan_partials_count(nrows_b));
+    L.runs_part = off; off = align_up(off + 2 * sizeof(long long) * sg::scan_partials_count(nrows_b));
   }
   L.hcnt = off; off = align_up(off + sizeof(int32_t) * nh);
   L.rrb = L.runsb = 0;
@@ -430,12 +430,20 @@ static spgemm_status analyse_impl(const spgemm_csr* A, const spgemm_csr* B, cons
 
   cudaStream_t st = (cudaStream_t)stream;
   sg::LaunchCtx c = ctx_of(p, stream);
+  // small rows (at most 128 products, the adjoint's limit for short rows of C)
+  // never look at their column span
+  long long span_min = 0;
+  if (o.force_path < 0) {
+    const int b = small_hi_bin(o) < sg::bin_of(128) ? small_hi_bin(o) : sg::bin_of(128);
+    span_min = 1ll << (b - 1);
+  }
   cudaError_t e = cudaMemsetAsync(p->st, 0, sizeof(sg::DevStats), st);
   if (e == cudaSuccess && o.validate) {
     e = sg::launch_validate(c, p->A);
     if (e == cudaSuccess) e = sg::launch_validate(c, p->B);
   }
-  if (e == cudaSuccess) e = sg::launch_analyse(c, p->A, p->B, p->row_begin, p->mloc, p->prod, p->cmin, p->cmax, p->rows);
+  if (e == cudaSuccess) e = sg::launch_analyse(c, p->A, p->B, p->row_begin, p->mloc, p->prod, p->cmin, p->cmax, p->rows,
+                                               span_min);
   if (e == cudaSuccess && !base) {
     // Only the numeric window paths read the run lists.  A plan of every row
     // of A may leave them unbuilt when none of its rows takes such a path:
@@ -577,10 +585,10 @@ spgemm_status spgemm_symbolic(spgemm_plan* p, int32_t* c_row_ptr, int64_t* c_nnz
   cudaStream_t st = (cudaStream_t)stream;
   sg::LaunchCtx c = ctx_of(p, stream);
   const sg::RowInfo ri = rowinfo_of(p);
-  cudaError_t e = cudaMemsetAsync(c_row_ptr, 0, sizeof(int32_t) * (size_t)(p->mloc + 1), st);
-  if (e == cudaSuccess && p->mloc > 0)
-    e = sg::launch_symbolic(c, p->A, p->B, ri, p->pb, p->tu, p->sp, p->cursor, c_row_ptr, nullptr);
-  if (e == cudaSuccess) e = sg::launch_scan(c, c_row_ptr, p->mloc, p->scan_part);
+  cudaError_t e = cudaSuccess;
+  if (p->mloc > 0) e = sg::launch_symbolic(c, p->A, p->B, ri, p->pb, p->sp, p->cursor, c_row_ptr);
+  // rows without products were not visited: the scan takes them as empty
+  if (e == cudaSuccess) e = sg::launch_scan(c, c_row_ptr, p->mloc, p->scan_part, nullptr, p->prod, &p->st->work[4]);
   if (e != cudaSuccess) return SPGEMM_ERR_CUDA;
   spgemm_status s = read_stats(p, st);
   if (s != SPGEMM_OK) return s;

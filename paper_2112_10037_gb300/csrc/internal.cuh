@@ -50,7 +50,8 @@ struct DevStats {
   uint32_t rows_wide8;  // rows with more than 8 (LANE_MERGE_K)
   int hist[NBINS];   // rows per bin
   int fill[NBINS];   // scatter cursors
-  unsigned int work[8];  // dynamic work counters (reset before each use)
+  unsigned int work[8];  // dynamic work counters (0, 1, 3: reset before each use; 4, 5: the symbolic
+                         // pass's, zero between passes)
 };
 
 // Paths a non-empty row can take.
@@ -234,6 +235,31 @@ __device__ __forceinline__ void bin_range(const DevStats* st, int lo, int hi, in
   *end = b + e;
 }
 
+// The same for a whole block, into shared memory: warp 0 reads the histogram
+// at once (the caller's next barrier publishes it).
+__device__ __forceinline__ void block_bin_range(const DevStats* st, int lo, int hi, int* begin, int* end) {
+  if (threadIdx.x < 32) {
+    const int k0 = threadIdx.x, k1 = threadIdx.x + 32;
+    const int h0 = k0 >= 1 ? st->hist[k0] : 0, h1 = k1 < NBINS ? st->hist[k1] : 0;
+    const int b = warp_sum((k0 > hi ? h0 : 0) + (k1 > hi ? h1 : 0));
+    const int n = warp_sum((k0 >= lo && k0 <= hi ? h0 : 0) + (k1 >= lo && k1 <= hi ? h1 : 0));
+    if (threadIdx.x == 0) {
+      *begin = b;
+      *end = b + n;
+    }
+  }
+}
+
+// True (for the whole block) when win_lo > 0 and the analysis put no row in
+// bins win_lo and above, i.e. no row takes a numeric window path and the
+// window-run lists will never be read.
+__device__ __forceinline__ bool no_window_rows(const DevStats* st, int win_lo) {
+  if (win_lo <= 0) return false;
+  int mine = 0;
+  if (threadIdx.x < NBINS && (int)threadIdx.x >= win_lo) mine = st->hist[threadIdx.x];
+  return !__syncthreads_or(mine);
+}
+
 // ------------------------------------------------------------ host launchers
 struct LaunchCtx {
   cudaStream_t stream;
@@ -264,16 +290,22 @@ inline void count_launch(const LaunchCtx& c) {
 
 cudaError_t launch_validate(const LaunchCtx& c, const Csr& M);
 cudaError_t launch_analyse(const LaunchCtx& c, const Csr& A, const Csr& B, long long row_begin,
-                           long long mloc, long long* prod, int* cmin, int* cmax, int* rows);
+                           long long mloc, long long* prod, int* cmin, int* cmax, int* rows,
+                           long long span_min /* rows of at most this many products need no column span */);
 // win_lo > 0: skip building the lists when the analysis put no row in bins
 // win_lo and above (only valid when no other plan reads this plan's lists
 // for rows outside it).
 cudaError_t launch_runs(const LaunchCtx& c, const Csr& B, const SplitInfo& sp, long long* partials, int win_lo);
 cudaError_t launch_symbolic(const LaunchCtx& c, const Csr& A, const Csr& B, const RowInfo& ri,
-                            const PathBins& pb, const Tuning& tu, const SplitInfo& sp, int32_t* cursor,
-                            int32_t* c_rp, const int* path_rows /* host, may be null */);
+                            const PathBins& pb, const SplitInfo& sp, int32_t* cursor, int32_t* c_rp);
+// prod: rows of no product count as size 0 whatever c_rp holds (null: no
+// such rows); reset: two words set to zero (null: none).
 cudaError_t launch_scan(const LaunchCtx& c, int32_t* c_rp, long long mloc, long long* partials,
-                        long long* total_out = nullptr);
+                        long long* total_out = nullptr, const long long* prod = nullptr, unsigned* reset = nullptr);
+// The run pointers of B's window-run lists (rrb may be null), both sums in the
+// same launches; win_lo as for launch_runs.
+cudaError_t launch_scan_runs(const LaunchCtx& c, int32_t* rr, int32_t* rrb, long long m, long long* partials,
+                             int win_lo);
 size_t scan_partials_count(long long mloc);
 cudaError_t launch_numeric(const LaunchCtx& c, const Csr& A, const Csr& B, const RowInfo& ri,
                            const PathBins& pb, const Tuning& tu, const SplitInfo& sp, int dtype,

@@ -238,8 +238,8 @@ k_num_block(Csr A, Csr B, const T* __restrict__ av, const T* __restrict__ bv, Ro
   const int warp = threadIdx.x >> 5, lane = lane_id();
   for (int t = threadIdx.x; t < W; t += NW * 32) acc[t] = SrOps<T, SR>::zero();
   for (int t = threadIdx.x; t < 2 * NWORDS; t += NW * 32) bits0[t] = 0u;
+  block_bin_range(st, bin_lo, bin_hi, &s_lb, &s_le);
   if (threadIdx.x == 0) {
-    bin_range(st, bin_lo, bin_hi, &s_lb, &s_le);
     s_pack[0] = 0ull;
     s_pack[1] = 0ull;
   }

@@ -271,8 +271,8 @@ static cudaError_t numeric_t(const LaunchCtx& c, const Csr& A, const Csr& B, con
     const bool lanes = merge || (path_rows && 2 * (long long)path_rows[PATH_HASH] >= all_rows);
     const int llo = merge ? pb.lo[PATH_TINY] : pb.lo[PATH_HASH], lhi = lanes ? (pb.hi[PATH_HASH] < 7 ? pb.hi[PATH_HASH] : 7) : 0;
     if (llo <= lhi && !empty_bins(hist, llo, lhi))
-      e = lane_rows<true, T, SR>(c, A, B, av, bv, ri, llo, lhi, nullptr, c_rp, c_ci, c_v,
-                                 merge ? rows + path_rows[PATH_TINY] : rows, rows_wide8);
+      e = lane_rows<T, SR>(c, A, B, av, bv, ri, llo, lhi, c_rp, c_ci, c_v,
+                           merge ? rows + path_rows[PATH_TINY] : rows, rows_wide8);
     const int wlo = lhi >= llo ? lhi + 1 : llo;
     if (!e && pb.hi[PATH_HASH] >= wlo)
       e = hash_dispatch(hist, wlo, pb.hi[PATH_HASH],

@@ -88,7 +88,7 @@ k_num_once(Csr A, Csr B, const T* __restrict__ av, const T* __restrict__ bv, Row
   const int tid = threadIdx.x, warp = tid >> 5, lane = lane_id();
   for (int t = tid; t < W / 32; t += NT) bits[t] = 0u;
   for (int t = tid; t < HW; t += NT) marks[t] = 0u;
-  if (tid == 0) bin_range(st, bin_lo, bin_hi, &s_lb, &s_le);
+  block_bin_range(st, bin_lo, bin_hi, &s_lb, &s_le);
   if (block_skip(st)) return;
   const int lb = s_lb, le = s_le;
   const unsigned le_mask = lane == 31 ? FULL : (2u << lane) - 1u;

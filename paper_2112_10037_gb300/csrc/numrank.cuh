@@ -209,7 +209,7 @@ k_num_rank(Csr A, Csr B, const T* __restrict__ av, const T* __restrict__ bv, Row
   __shared__ int s_wsum[NW];
   __shared__ unsigned long long s_pack;
   const int tid = threadIdx.x, warp = tid >> 5, lane = lane_id();
-  if (tid == 0) bin_range(st, bin_lo, bin_hi, &s_lb, &s_le);
+  block_bin_range(st, bin_lo, bin_hi, &s_lb, &s_le);
   if (block_skip(st)) return;
   const int lb = s_lb, le = s_le;
 

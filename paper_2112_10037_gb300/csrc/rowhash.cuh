@@ -191,23 +191,16 @@ __device__ __forceinline__ void hash_row_loop(const Csr& A, const Csr& B, const 
 }
 
 // Symbolic pass: the number of distinct columns of each row (the count of
-// slots its products claimed).
+// slots its products claimed).  Rows at list positions [lb, le), warp w of nw
+// takes its share; key (64 * E slots, all HASH_EMPTY): this warp's.
 template <int E>
-__global__ void __launch_bounds__(HASH_WARPS * 32)
-k_hash_sym(Csr A, Csr B, RowInfo ri, const DevStats* st, int bin_lo, int bin_hi, int32_t* __restrict__ c_cnt,
-           uint32_t* err) {
+__device__ __forceinline__ void hash_sym_rows(const Csr& A, const Csr& B, const RowInfo& ri, long long lb,
+                                              long long le, long long w, long long nw, int* key,
+                                              int32_t* __restrict__ c_cnt, uint32_t* err) {
   constexpr int LG = 6 + (E >= 4 ? 2 : (E >= 2 ? 1 : 0));
-  constexpr int H = 1 << LG;
-  static_assert(H == 64 * E, "table of twice the slots");
-  __shared__ int s_lb, s_le;
-  __shared__ __align__(16) int s_key[HASH_WARPS][H];
-  const int warp = threadIdx.x >> 5, lane = lane_id();
-  int* key = s_key[warp];
-  for (int t = lane; t < H; t += 32) key[t] = HASH_EMPTY;
-  if (threadIdx.x == 0) bin_range(st, bin_lo, bin_hi, &s_lb, &s_le);
-  if (block_skip(st)) return;
-  const long long nw = (long long)gridDim.x * HASH_WARPS;
-  hash_row_loop<false, float>(A, B, nullptr, ri, s_lb, s_le, (long long)blockIdx.x * HASH_WARPS + warp, nw,
+  static_assert((1 << LG) == 64 * E, "table of twice the slots");
+  const int lane = lane_id();
+  hash_row_loop<false, float>(A, B, nullptr, ri, lb, le, w, nw,
                               [&](int r, int a0, int a1, const Chunk0<float>& c0, auto& between) {
     int col[E];
     float pv[E];
@@ -256,7 +249,7 @@ k_hash_num(Csr A, Csr B, const T* __restrict__ av, const T* __restrict__ bv, Row
   int* dk = s_dk[warp];
   T* dv = s_dv[warp];
   for (int t = lane; t < H; t += 32) key[t] = HASH_EMPTY;
-  if (threadIdx.x == 0) bin_range(st, bin_lo, bin_hi, &s_lb, &s_le);
+  block_bin_range(st, bin_lo, bin_hi, &s_lb, &s_le);
   if (block_skip(st)) return;
   const long long nw = (long long)gridDim.x * HASH_WARPS;
   hash_row_loop<true, T>(A, B, av, ri, s_lb, s_le, (long long)blockIdx.x * HASH_WARPS + warp, nw,

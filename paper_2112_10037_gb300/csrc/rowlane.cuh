@@ -36,15 +36,20 @@ constexpr int LANE_SLOTS = 64;     // table slots per lane (rows of at most 64 p
 constexpr int LANE_WARPS = 4;      // warps per block
 constexpr int LANE_EMPTY = -1;
 
-__device__ __forceinline__ unsigned lane_hash(int c) { return ((unsigned)c * 0x9E3779B1u) >> 26; }
+template <int SLOTS>
+__device__ __forceinline__ unsigned lane_hash(int c) {
+  return ((unsigned)c * 0x9E3779B1u) >> (SLOTS == 64 ? 26 : 27);
+}
 
 // Slot of column j in the lane's table (claimed if absent; *fresh tells).
 // keys: this warp's table base, slot-major.  -1 if the table is full of
 // other columns (ruled out by the row's product count).
+template <int SLOTS>
 __device__ __forceinline__ int lane_probe(int* keys, int lane, int j, bool* fresh) {
-  unsigned h = lane_hash(j);
+  static_assert(SLOTS == 64 || SLOTS == 32, "slots per lane");
+  unsigned h = lane_hash<SLOTS>(j);
   *fresh = false;
-  for (int it = 0; it < LANE_SLOTS; ++it) {
+  for (int it = 0; it < SLOTS; ++it) {
     int* kp = &keys[h * 32 + lane];
     const int k = *kp;
     if (k == j) return (int)h;
@@ -53,31 +58,24 @@ __device__ __forceinline__ int lane_probe(int* keys, int lane, int j, bool* fres
       *fresh = true;
       return (int)h;
     }
-    h = (h + 1u) & (LANE_SLOTS - 1);
+    h = (h + 1u) & (SLOTS - 1);
   }
   return -1;
 }
 
 // NUM = false: c_cnt[r] = distinct columns of row r.  NUM = true: C's
-// columns and values at [c_rp[r], c_rp[r+1]).
-template <bool NUM, typename T, int SR = SPGEMM_PLUS_TIMES>
-__global__ void __launch_bounds__(LANE_WARPS * 32)
-k_lane_rows(Csr A, Csr B, const T* __restrict__ av, const T* __restrict__ bv, RowInfo ri, const DevStats* st,
-            int bin_lo, int bin_hi, int32_t* __restrict__ c_cnt, const int32_t* __restrict__ c_rp,
-            int32_t* __restrict__ c_ci, T* __restrict__ c_v, uint32_t* err, int skip_upto) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int s_lb, s_le;
-  const int warp = threadIdx.x >> 5, lane = lane_id();
-  // per warp: keys [64][32] int32, then (numeric) values [64][32] T
-  const size_t per_warp = (size_t)LANE_SLOTS * 32 * (sizeof(int) + (NUM ? sizeof(T) : 0));
-  int* keys = reinterpret_cast<int*>(smem_raw + warp * per_warp);
-  T* vals = reinterpret_cast<T*>(smem_raw + warp * per_warp + (size_t)LANE_SLOTS * 32 * sizeof(int));
-  for (int h = 0; h < LANE_SLOTS; ++h) keys[h * 32 + lane] = LANE_EMPTY;
-  if (threadIdx.x == 0) bin_range(st, bin_lo, bin_hi, &s_lb, &s_le);
-  if (block_skip(st)) return;
-  const long long lb = s_lb, le = s_le;
-  const long long gw = (long long)blockIdx.x * LANE_WARPS + warp;
-  const long long nw = (long long)gridDim.x * LANE_WARPS;
+// columns and values at [c_rp[r], c_rp[r+1]).  Rows at list positions
+// [lb, le), warp gw of nw takes its share; rows of at most skip_upto nonzeros
+// are left out.  keys (all LANE_EMPTY) and vals: this warp's.  SLOTS: 64, or
+// 32 for rows of at most 16 products.
+template <bool NUM, typename T, int SR = SPGEMM_PLUS_TIMES, int SLOTS = LANE_SLOTS>
+__device__ __forceinline__ void lane_hash_rows(const Csr& A, const Csr& B, const T* __restrict__ av,
+                                               const T* __restrict__ bv, const RowInfo& ri, long long lb,
+                                               long long le, long long gw, long long nw, int* keys, T* vals,
+                                               int32_t* __restrict__ c_cnt, const int32_t* __restrict__ c_rp,
+                                               int32_t* __restrict__ c_ci, T* __restrict__ c_v, uint32_t* err,
+                                               int skip_upto) {
+  const int lane = lane_id();
   for (long long base = lb + gw * 32; base < le; base += nw * 32) {
     const long long idx = base + lane;
     if (idx < le) {
@@ -107,7 +105,7 @@ k_lane_rows(Csr A, Csr B, const T* __restrict__ av, const T* __restrict__ bv, Ro
           for (int u = 0; u < 8; ++u) {
             if (jj[u] < 0) continue;
             bool fresh;
-            const int h = lane_probe(keys, lane, jj[u], &fresh);
+            const int h = lane_probe<SLOTS>(keys, lane, jj[u], &fresh);
             ++np;
             if (h < 0) {
               over = true;
@@ -121,16 +119,16 @@ k_lane_rows(Csr A, Csr B, const T* __restrict__ av, const T* __restrict__ bv, Ro
           }
         }
       }
-      if (over || np > LANE_SLOTS) atomicOr(err, EB_INTERNAL);  // the row's bin rules this out
+      if (over || np > SLOTS) atomicOr(err, EB_INTERNAL);  // the row's bin rules this out
       if (!NUM) {
         c_cnt[r] = nd;
-        for (int h = 0; h < LANE_SLOTS; ++h) keys[h * 32 + lane] = LANE_EMPTY;
+        for (int h = 0; h < SLOTS; ++h) keys[h * 32 + lane] = LANE_EMPTY;
       } else {
         // compact the occupied slots into slots [0, nd) of a list kept in
         // the same columns (read slot h before writing entry d <= h), and
         // clear the rest of the table
         int d = 0;
-        for (int h = 0; h < LANE_SLOTS; ++h) {
+        for (int h = 0; h < SLOTS; ++h) {
           const int k = keys[h * 32 + lane];
           if (k != LANE_EMPTY) {
             const T v = vals[h * 32 + lane];
@@ -165,6 +163,25 @@ k_lane_rows(Csr A, Csr B, const T* __restrict__ av, const T* __restrict__ bv, Ro
       }
     }
   }
+}
+
+template <typename T, int SR = SPGEMM_PLUS_TIMES>
+__global__ void __launch_bounds__(LANE_WARPS * 32)
+k_lane_rows(Csr A, Csr B, const T* __restrict__ av, const T* __restrict__ bv, RowInfo ri, const DevStats* st,
+            int bin_lo, int bin_hi, const int32_t* __restrict__ c_rp, int32_t* __restrict__ c_ci,
+            T* __restrict__ c_v, uint32_t* err, int skip_upto) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int s_lb, s_le;
+  const int warp = threadIdx.x >> 5, lane = lane_id();
+  // per warp: keys [64][32] int32, then values [64][32] T
+  const size_t per_warp = (size_t)LANE_SLOTS * 32 * (sizeof(int) + sizeof(T));
+  int* keys = reinterpret_cast<int*>(smem_raw + warp * per_warp);
+  T* vals = reinterpret_cast<T*>(smem_raw + warp * per_warp + (size_t)LANE_SLOTS * 32 * sizeof(int));
+  for (int h = 0; h < LANE_SLOTS; ++h) keys[h * 32 + lane] = LANE_EMPTY;
+  block_bin_range(st, bin_lo, bin_hi, &s_lb, &s_le);
+  if (block_skip(st)) return;
+  lane_hash_rows<true, T, SR>(A, B, av, bv, ri, s_lb, s_le, (long long)blockIdx.x * LANE_WARPS + warp,
+                              (long long)gridDim.x * LANE_WARPS, keys, vals, nullptr, c_rp, c_ci, c_v, err, skip_upto);
 }
 
 // Rows with at most LANE_MERGE_K nonzeros of A (every row of a 7-point
@@ -216,9 +233,9 @@ __device__ __forceinline__ void lane_flush(const LaneOut<T>& so, int first, int 
   __syncwarp();
 }
 
-// One warp's 32 rows (a0 == a1: none).  NUM: columns and values to [ob, oe);
+// One warp's 32 rows (a0 == a1: none): columns and values to [ob, oe);
 // returns the lane's distinct columns.
-template <bool NUM, typename T, int SR>
+template <typename T, int SR>
 __device__ __forceinline__ int lane_merge_rows(const Csr& A, const Csr& B, const T* __restrict__ av,
                                                const T* __restrict__ bv, int a0, int a1, LaneOut<T>* so, int ob,
                                                int oe, int32_t* __restrict__ c_ci, T* __restrict__ c_v) {
@@ -235,14 +252,14 @@ __device__ __forceinline__ int lane_merge_rows(const Csr& A, const Csr& B, const
       const int kk = A.ci[a0 + k];
       hs[k] = B.rp[kk];
       he[k] = B.rp[kk + 1];
-      if (NUM) a[k] = av[a0 + k];
+      a[k] = av[a0 + k];
     }
   }
 #pragma unroll
   for (int k = 0; k < K; ++k) {
     hc[k] = hs[k] < he[k] ? B.ci[hs[k]] : INT_MAX;
     hn[k] = hs[k] + 1 < he[k] ? B.ci[hs[k] + 1] : INT_MAX;
-    if (NUM && hs[k] < he[k]) v[k] = bv[hs[k]];
+    if (hs[k] < he[k]) v[k] = bv[hs[k]];
   }
   int n = 0;
   for (int step = 0;; ++step) {
@@ -250,9 +267,9 @@ __device__ __forceinline__ int lane_merge_rows(const Csr& A, const Csr& B, const
 #pragma unroll
     for (int k = 1; k < K; ++k) m = min(m, hc[k]);
     const bool act = m != INT_MAX;
-    if (NUM && step > 0 && (step & (LANE_OUT - 1)) == 0) lane_flush(*so, step - LANE_OUT, n, ob, oe, c_ci, c_v);
+    if (step > 0 && (step & (LANE_OUT - 1)) == 0) lane_flush(*so, step - LANE_OUT, n, ob, oe, c_ci, c_v);
     if (!__any_sync(FULL, act)) {
-      if (NUM && (step & (LANE_OUT - 1)) != 0) lane_flush(*so, step & ~(LANE_OUT - 1), n, ob, oe, c_ci, c_v);
+      if ((step & (LANE_OUT - 1)) != 0) lane_flush(*so, step & ~(LANE_OUT - 1), n, ob, oe, c_ci, c_v);
       break;
     }
     if (act) {
@@ -261,18 +278,16 @@ __device__ __forceinline__ int lane_merge_rows(const Csr& A, const Csr& B, const
 #pragma unroll
       for (int k = 0; k < K; ++k) {
         if (hc[k] == m) {
-          if (NUM) acc = Ops::madd(a[k], v[k], any ? acc : Ops::zero());  // one FP64 instruction per head test
+          acc = Ops::madd(a[k], v[k], any ? acc : Ops::zero());  // one FP64 instruction per head test
           any = true;
           ++hs[k];
           hc[k] = hn[k];
           hn[k] = hs[k] + 1 < he[k] ? B.ci[hs[k] + 1] : INT_MAX;
-          if (NUM && hs[k] < he[k]) v[k] = bv[hs[k]];
+          if (hs[k] < he[k]) v[k] = bv[hs[k]];
         }
       }
-      if (NUM) {
-        so->col[(step & (LANE_OUT - 1)) * LANE_OUT_CI + lane] = m;
-        so->val[(step & (LANE_OUT - 1)) * LANE_OUT_V + lane] = acc;
-      }
+      so->col[(step & (LANE_OUT - 1)) * LANE_OUT_CI + lane] = m;
+      so->val[(step & (LANE_OUT - 1)) * LANE_OUT_V + lane] = acc;
       ++n;
     }
   }
@@ -287,7 +302,7 @@ k_lane_merge(Csr A, Csr B, const T* __restrict__ av, const T* __restrict__ bv, R
   __shared__ LaneOut<T> s_out[LANE_WARPS];
   __shared__ int s_lb, s_le;
   const int warp = threadIdx.x >> 5, lane = lane_id();
-  if (threadIdx.x == 0) bin_range(st, bin_lo, bin_hi, &s_lb, &s_le);
+  block_bin_range(st, bin_lo, bin_hi, &s_lb, &s_le);
   if (block_skip(st)) return;
   const long long lb = s_lb, le = s_le;
   const long long gw = (long long)blockIdx.x * LANE_WARPS + warp;
@@ -305,41 +320,37 @@ k_lane_merge(Csr A, Csr B, const T* __restrict__ av, const T* __restrict__ bv, R
         oe = c_rp[r + 1];
       }
     }
-    const int n = lane_merge_rows<true, T, SR>(A, B, av, bv, a0, a1, &s_out[warp], ob, oe, c_ci, c_v);
+    const int n = lane_merge_rows<T, SR>(A, B, av, bv, a0, a1, &s_out[warp], ob, oe, c_ci, c_v);
     if (a1 > a0 && ob + n != oe) atomicOr(err, EB_INTERNAL);  // the symbolic count rules this out
   }
 }
 
-template <bool NUM, typename T>
+template <typename T>
 constexpr size_t lane_rows_smem() {
-  return (size_t)LANE_WARPS * LANE_SLOTS * 32 * (sizeof(int) + (NUM ? sizeof(T) : 0));
+  return (size_t)LANE_WARPS * LANE_SLOTS * 32 * (sizeof(int) + sizeof(T));
 }
 
-// Launch over the rows of bins [lo, hi] (rows: their number, -1 unknown).
-// The numeric pass merges rows of at most LANE_MERGE_K nonzeros of A
-// (k_lane_merge) and hashes the others (wide8: rows of the plan with more, -1
-// unknown); the symbolic pass hashes all.
-template <bool NUM, typename T, int SR = SPGEMM_PLUS_TIMES>
+// Numeric launch over the rows of bins [lo, hi] (rows: their number, -1
+// unknown): rows of at most LANE_MERGE_K nonzeros of A are merged, the others
+// (wide8: rows of the plan with more, -1 unknown) go through the tables.
+template <typename T, int SR = SPGEMM_PLUS_TIMES>
 static cudaError_t lane_rows(const LaunchCtx& c, const Csr& A, const Csr& B, const T* av, const T* bv,
-                             const RowInfo& ri, int lo, int hi, int32_t* c_cnt, const int32_t* c_rp,
-                             int32_t* c_ci, T* c_v, long long rows, long long wide8) {
-  if constexpr (NUM) {
-    auto km = k_lane_merge<T, SR>;
-    const int occm = kernel_blocks_per_sm(km, LANE_WARPS * 32, 0);
-    if (occm <= 0) return cudaErrorInvalidConfiguration;
-    const int gridm = persistent_grid(rows, LANE_WARPS * 32, c.nsm, occm);
-    km<<<gridm, LANE_WARPS * 32, 0, c.stream>>>(A, B, av, bv, ri, c.st, lo, hi, c_rp, c_ci, c_v, c.err);
-    count_launch(c);
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess || wide8 == 0) return e;
-  }
-  auto k = k_lane_rows<NUM, T, SR>;
-  const size_t smem = lane_rows_smem<NUM, T>();
+                             const RowInfo& ri, int lo, int hi, const int32_t* c_rp, int32_t* c_ci, T* c_v,
+                             long long rows, long long wide8) {
+  auto km = k_lane_merge<T, SR>;
+  const int occm = kernel_blocks_per_sm(km, LANE_WARPS * 32, 0);
+  if (occm <= 0) return cudaErrorInvalidConfiguration;
+  km<<<persistent_grid(rows, LANE_WARPS * 32, c.nsm, occm), LANE_WARPS * 32, 0, c.stream>>>(
+      A, B, av, bv, ri, c.st, lo, hi, c_rp, c_ci, c_v, c.err);
+  count_launch(c);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess || wide8 == 0) return e;
+  auto k = k_lane_rows<T, SR>;
+  const size_t smem = lane_rows_smem<T>();
   const int occ = kernel_blocks_per_sm(k, LANE_WARPS * 32, smem);
   if (occ <= 0) return cudaErrorInvalidConfiguration;
-  const int grid = persistent_grid(rows, LANE_WARPS * 32, c.nsm, occ);
-  k<<<grid, LANE_WARPS * 32, smem, c.stream>>>(A, B, av, bv, ri, c.st, lo, hi, c_cnt, c_rp, c_ci, c_v, c.err,
-                                               NUM ? LANE_MERGE_K : -1);
+  k<<<persistent_grid(rows, LANE_WARPS * 32, c.nsm, occ), LANE_WARPS * 32, smem, c.stream>>>(
+      A, B, av, bv, ri, c.st, lo, hi, c_rp, c_ci, c_v, c.err, LANE_MERGE_K);
   count_launch(c);
   return cudaGetLastError();
 }

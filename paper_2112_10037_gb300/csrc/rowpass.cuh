@@ -33,25 +33,20 @@ namespace sg {
 // so every slot is a run of G consecutive elements after the sort; the
 // bitonic network exchanges through shuffles (partner distance < G) or
 // between a lane's own slots (distance >= G).
+// [lb, le): the rows' positions in the list; warp_g of nwarps takes its share.
 template <int G, int E, bool NUM, typename T, int SR = SPGEMM_PLUS_TIMES>
-__global__ void __launch_bounds__(256)
-k_tiny(Csr A, Csr B, const T* __restrict__ av, const T* __restrict__ bv, RowInfo ri,
-       const DevStats* st, int bin_lo, int bin_hi, int32_t* __restrict__ c_cnt,
-       const int32_t* __restrict__ c_rp, int32_t* __restrict__ c_ci, T* __restrict__ c_v,
-       uint32_t* err) {
+__device__ __forceinline__ void tiny_rows(const Csr& A, const Csr& B, const T* __restrict__ av,
+                                          const T* __restrict__ bv, const RowInfo& ri, int lb, int le,
+                                          long long warp_g, long long nwarps, int32_t* __restrict__ c_cnt,
+                                          const int32_t* __restrict__ c_rp, int32_t* __restrict__ c_ci,
+                                          T* __restrict__ c_v, uint32_t* err) {
   static_assert(E == 1 || G == 32, "multi-slot rows use whole warps");
   constexpr int N = G * E;
-  __shared__ int s_lb, s_le;
-  if (threadIdx.x == 0) bin_range(st, bin_lo, bin_hi, &s_lb, &s_le);
-  if (block_skip(st)) return;
-  const int lb = s_lb, le = s_le;
   const int lane = lane_id();
   const int gl = lane & (G - 1);
   const int gi = lane / G;
   constexpr int GPW = 32 / G;
   const unsigned gmask = (G == 32) ? FULL : (((1u << G) - 1u) << (gi * G));
-  const long long warp_g = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
-  const long long nwarps = (gridDim.x * (long long)blockDim.x) >> 5;
   for (long long wb = lb + warp_g * GPW; wb < le; wb += nwarps * GPW) {
     const long long idx = wb + gi;
     const bool vrow = idx < le;
@@ -205,22 +200,27 @@ k_tiny(Csr A, Csr B, const T* __restrict__ av, const T* __restrict__ bv, RowInfo
   }
 }
 
-// ------------------------------------------------------- bitmap-window path
-// Symbolic pass for rows above the register-sort limit: a group of GW warps
-// owns a presence bitmap of W columns; each product sets its column's bit
-// (shared-memory atomicOr after a plain test), and the row size is the
-// popcount of the window.  Windows start at a multiple of 32 at or below the
-// smallest unread column.  For split rows the popcounts are also added up
-// per fine tile into hcnt, which fixes where each tile's entries go.
-template <int GW>
-__device__ __forceinline__ void group_sync(int g) {
-  if (GW == 1) {
-    __syncwarp();
-  } else {
-    asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "r"(GW * 32) : "memory");
-  }
+template <int G, int E, bool NUM, typename T, int SR = SPGEMM_PLUS_TIMES>
+__global__ void __launch_bounds__(256)
+k_tiny(Csr A, Csr B, const T* __restrict__ av, const T* __restrict__ bv, RowInfo ri,
+       const DevStats* st, int bin_lo, int bin_hi, int32_t* __restrict__ c_cnt,
+       const int32_t* __restrict__ c_rp, int32_t* __restrict__ c_ci, T* __restrict__ c_v,
+       uint32_t* err) {
+  __shared__ int s_lb, s_le;
+  block_bin_range(st, bin_lo, bin_hi, &s_lb, &s_le);
+  if (block_skip(st)) return;
+  tiny_rows<G, E, NUM, T, SR>(A, B, av, bv, ri, s_lb, s_le,
+                              (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5,
+                              (gridDim.x * (long long)blockDim.x) >> 5, c_cnt, c_rp, c_ci, c_v, err);
 }
 
+// ------------------------------------------------------- bitmap-window path
+// Symbolic pass for rows above the register-sort limit: a warp owns a presence
+// bitmap of W columns; each product sets its column's bit (shared-memory
+// atomicOr after a plain test), and the row size is the popcount of the
+// window.  Windows start at a multiple of 32 at or below the smallest unread
+// column.  For split rows the popcounts are also added up per fine tile into
+// hcnt, which fixes where each tile's entries go.
 __device__ __forceinline__ void bit_insert(uint32_t* bits, int j, int W, uint32_t* err) {
   if ((unsigned)j >= (unsigned)W) {  // only reachable with unsorted input
     atomicOr(err, EB_UNSORTED);
@@ -233,42 +233,39 @@ __device__ __forceinline__ void bit_insert(uint32_t* bits, int j, int W, uint32_
 // Smallest fine-tile width the symbolic kernel sizes its tile counters for.
 constexpr int SYM_MIN_FINE = 1024;
 
-template <int W, int GW, int WF = SYM_MIN_FINE>
-__host__ __device__ constexpr size_t sym_group_bytes() {
-  return (((size_t)(W / 32) * 4 + (size_t)GW * 8 + (size_t)(W / WF + 2) * 4) + 15) & ~(size_t)15;
+// Shared memory of one warp: the bitmap, marks and positions of 32 flattened
+// segments, and the fine tiles' counts.
+template <int W>
+__host__ __device__ constexpr size_t sym_window_bytes() {
+  return (((size_t)(W / 32) * 4 + 64 * 4 + (size_t)(W / SYM_MIN_FINE + 2) * 4) + 15) & ~(size_t)15;
 }
 
-// GW warps per row (group), CW warps per block, W columns per window; the
-// fine tile width is 2^sp.wf_shift >= SYM_MIN_FINE columns.
-template <int GW, int CW, int W>
-__global__ void __launch_bounds__(CW * 32)
-k_sym_window(Csr A, Csr B, RowInfo ri, const DevStats* st, int bin_lo, int bin_hi, SplitInfo sp,
-             int32_t* __restrict__ cursor, int32_t* __restrict__ c_cnt, uint32_t* err) {
-  static_assert(CW % GW == 0 && W % 32 == 0, "bad shape");
+// The rows at list positions [lb, le), handed out to warps by a counter;
+// split rows are positions [hs, hs + nh); the fine tile width is
+// 2^sp.wf_shift >= SYM_MIN_FINE columns.  mem: this warp's.
+template <int W>
+__device__ __forceinline__ void sym_window_rows(const Csr& A, const Csr& B, const RowInfo& ri, int lb, int le, int hs,
+                                                int nh, const SplitInfo& sp, int32_t* __restrict__ cursor,
+                                                int32_t* __restrict__ c_cnt, unsigned* counter, unsigned char* mem,
+                                                uint32_t* err) {
   constexpr int NWORDS = W / 32;
-  constexpr int NG = CW / GW;
   constexpr int NTW = W / SYM_MIN_FINE + 2;  // fine tiles a window can touch
-  constexpr size_t GB = sym_group_bytes<W, GW>();
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int s_lb, s_le, s_nh, s_hs;
-  const int warp = threadIdx.x >> 5, lane = lane_id();
-  const int g = warp / GW, wig = warp % GW;
-  unsigned char* gbase = smem_raw + (size_t)g * GB;
-  uint32_t* bits = reinterpret_cast<uint32_t*>(gbase);
-  int* wcnt = reinterpret_cast<int*>(bits + NWORDS);
-  int* wnext = wcnt + GW;
-  int* tcnt = wnext + GW;
-  for (int t = wig * 32 + lane; t < NWORDS; t += GW * 32) bits[t] = 0u;
-  for (int t = wig * 32 + lane; t < NTW; t += GW * 32) tcnt[t] = 0;
-  if (threadIdx.x == 0) {
-    bin_range(st, bin_lo, bin_hi, &s_lb, &s_le);
-    s_nh = split_rows(st, sp, &s_hs);
-  }
-  if (block_skip(st)) return;
-  const int lb = s_lb, le = s_le, nh = s_nh, hs = s_hs;
+  const int lane = lane_id();
+  uint32_t* bits = reinterpret_cast<uint32_t*>(mem);
+  uint32_t* marks = bits + NWORDS;                    // where flattened segments start, a bit per product
+  int* at = reinterpret_cast<int*>(marks + 32);       // entry of B minus product, per flattened segment
+  int* tcnt = at + 32;
+  const unsigned le_mask = lane == 31 ? FULL : (2u << lane) - 1u;
+  for (int t = lane; t < NWORDS; t += 32) bits[t] = 0u;
+  for (int t = lane; t < NTW; t += 32) tcnt[t] = 0;
+  __syncwarp();
   const int wf_shift = sp.wf_shift;
-
-  for (long long idx = lb + (long long)blockIdx.x * NG + g; idx < le; idx += (long long)gridDim.x * NG) {
+  while (true) {
+    unsigned item = 0;
+    if (lane == 0) item = atomicAdd(counter, 1u);
+    item = __shfl_sync(FULL, item, 0);
+    if (item >= (unsigned)(le - lb)) break;
+    const int idx = lb + (int)item;
     const int r = ri.rows[idx];
     const bool split = idx >= hs && idx < hs + nh;
     const long long hrow = idx - hs;  // row of the per-window count table
@@ -276,24 +273,21 @@ k_sym_window(Csr A, Csr B, RowInfo ri, const DevStats* st, int bin_lo, int bin_h
     const int a0 = A.rp[i], a1 = A.rp[i + 1], nA = a1 - a0;
     int base = ri.cmin[r] & ~31;
     const int last = ri.cmax[r];
-    const int CS = min(32, max(1, (nA + GW - 1) / GW));  // nonzeros per chunk
-    const int nch = (nA + CS - 1) / CS;
-    const bool regcur = nch <= GW;  // one chunk per warp: cursor stays in a register
+    const bool regcur = nA <= 32;  // the cursors stay in registers
     int rcur = 0;
     long long rowcount = 0;
     bool first = true;
     if (split) {
-      for (int t = wig * 32 + lane; t < sp.ntf; t += GW * 32) sp.hcnt[(size_t)hrow * sp.ntf + t] = 0;
-      group_sync<GW>(g);
+      for (int t = lane; t < sp.ntf; t += 32) sp.hcnt[(size_t)hrow * sp.ntf + t] = 0;
+      __syncwarp();
     }
     while (true) {
       const int wend = (int)min((long long)base + W, (long long)INT_MAX);
       int mynext = INT_MAX;
-      for (int c = wig; c < nch; c += GW) {
-        const int e = a0 + c * CS + lane;
-        const bool ve = lane < CS && e < a1;
+      for (int e0 = a0; e0 < a1; e0 += 32) {
+        const int e = e0 + lane;
         int s = 0, len = 0;
-        if (ve) {
+        if (e < a1) {
           const int k = A.ci[e];
           const int rs = B.rp[k], re = B.rp[k + 1];
           const int cur = first ? rs : (regcur ? rcur : cursor[e]);
@@ -332,64 +326,78 @@ k_sym_window(Csr A, Csr B, RowInfo ri, const DevStats* st, int bin_lo, int bin_h
           }
           for (; t < ln; t += 32) bit_insert(bits, B.ci[ls + t] - base, W, err);
         }
-        // Short segments: flattened so every lane takes one product.
+        // Short segments (fewer than 32 * 32 products): flattened so that every
+        // lane takes one product, its segment the number of segment starts up
+        // to it.
         const int sl = len < 32 ? len : 0;
         const int incl = warp_incl_scan(sl);
         const int tot = __shfl_sync(FULL, incl, 31);
-        const int excl = incl - sl;
-        for (int p0 = 0; p0 < tot; p0 += 64) {
-          const int p = p0 + lane, p2 = p + 32;
-          const int o = warp_owner(incl, p), o2 = warp_owner(incl, p2);
-          const int os = __shfl_sync(FULL, s, o), oex = __shfl_sync(FULL, excl, o);
-          const int os2 = __shfl_sync(FULL, s, o2), oex2 = __shfl_sync(FULL, excl, o2);
-          const int c0 = p < tot ? B.ci[os + p - oex] : 0;
-          const int c1 = p2 < tot ? B.ci[os2 + p2 - oex2] : 0;
-          if (p < tot) bit_insert(bits, c0 - base, W, err);
-          if (p2 < tot) bit_insert(bits, c1 - base, W, err);
+        if (tot) {
+          const int excl = incl - sl;
+          const int k = __popc(__ballot_sync(FULL, sl > 0) & lanemask_lt());
+          marks[lane] = 0u;
+          __syncwarp();
+          if (sl > 0) {
+            atomicOr(&marks[excl >> 5], 1u << (excl & 31));
+            at[k] = s - excl;
+          }
+          __syncwarp();
+          int k0 = -1;
+          for (int p0 = 0; p0 < tot; p0 += 128) {
+            int c[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              const int p = p0 + 32 * u + lane;
+              const unsigned m = p0 + 32 * u < tot ? marks[(p0 >> 5) + u] : 0u;
+              const int q = k0 + __popc(m & le_mask);
+              k0 += __popc(m);
+              c[u] = p < tot ? B.ci[at[q] + p] : 0;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+              if (p0 + 32 * u + lane < tot) bit_insert(bits, c[u] - base, W, err);
+          }
+          __syncwarp();
         }
       }
-      mynext = warp_min(mynext);
+      const int nb = warp_min(mynext);
       const int hic = min(wend - 1, last);
       const int nw = hic >= base ? ((hic - base) >> 5) + 1 : 0;
-      group_sync<GW>(g);
-      const int wpw = (nw + GW - 1) / GW;
-      const int w0 = min(nw, wig * wpw), w1 = min(nw, w0 + wpw);
       const int tile0 = base >> wf_shift;
+      __syncwarp();
       int cnt = 0;
-      for (int j = w0 + lane; j < w1; j += 32) {
-        const int pc = __popc(bits[j]);
-        bits[j] = 0u;
-        cnt += pc;
-        if (split && pc) atomicAdd(&tcnt[((base + 32 * j) >> wf_shift) - tile0], pc);
+      if (!split) {  // four words at a time (words past the last one are clear)
+        for (int j = lane * 4; j < nw; j += 128) {
+          const uint4 x = *reinterpret_cast<const uint4*>(bits + j);
+          cnt += __popc(x.x) + __popc(x.y) + __popc(x.z) + __popc(x.w);
+          *reinterpret_cast<uint4*>(bits + j) = make_uint4(0, 0, 0, 0);
+        }
+      } else {
+        for (int j = lane; j < nw; j += 32) {
+          const int pc = __popc(bits[j]);
+          bits[j] = 0u;
+          cnt += pc;
+          if (pc) atomicAdd(&tcnt[((base + 32 * j) >> wf_shift) - tile0], pc);
+        }
       }
-      cnt = warp_sum(cnt);
-      if (lane == 0) {
-        wcnt[wig] = cnt;
-        wnext[wig] = mynext;
-      }
-      group_sync<GW>(g);
-      int total = 0, nb = INT_MAX;
-      for (int w = 0; w < GW; ++w) {
-        total += wcnt[w];
-        nb = min(nb, wnext[w]);
-      }
+      rowcount += warp_sum(cnt);
+      __syncwarp();
       if (split) {
         const int ntw = min(NTW, sp.ntf - tile0);
-        for (int t = wig * 32 + lane; t < ntw; t += GW * 32) {
+        for (int t = lane; t < ntw; t += 32) {
           const int v = tcnt[t];
           if (v) {
             atomicAdd(&sp.hcnt[(size_t)hrow * sp.ntf + tile0 + t], v);
             tcnt[t] = 0;
           }
         }
+        __syncwarp();
       }
-      rowcount += total;
-      group_sync<GW>(g);
       first = false;
       if (nb == INT_MAX) break;
       base = nb & ~31;
     }
-    if (wig == 0 && lane == 0) c_cnt[r] = (int)rowcount;
+    if (lane == 0) c_cnt[r] = (int)rowcount;
   }
 }
 

@@ -80,35 +80,33 @@ __device__ __forceinline__ void sb_range(const Csr& B, const int* off, const int
   }
 }
 
-// cursor: per nonzero of A, the first entry of its B row not yet counted.
+// The rows at list positions [lb, le), handed out to blocks by a counter; split
+// rows are positions [hs, hs + nh).  cursor: per nonzero of A, the first entry
+// of its B row not yet counted.
 template <int W, int NW>
-__global__ void __launch_bounds__(NW * 32)
-k_sym_block(Csr A, Csr B, RowInfo ri, const DevStats* st, int bin_lo, int bin_hi, SplitInfo sp,
-            int32_t* __restrict__ cursor, int32_t* __restrict__ c_cnt, unsigned* counter, uint32_t* err) {
+__device__ __forceinline__ void sym_block_rows(const Csr& A, const Csr& B, const RowInfo& ri, int lb, int le, int hs,
+                                               int nh, const SplitInfo& sp, int32_t* __restrict__ cursor,
+                                               int32_t* __restrict__ c_cnt, unsigned* counter,
+                                               unsigned char* smem_raw, uint32_t* err) {
   static_assert(W % 32 == 0 && W >= SYM_MIN_FINE, "bad window");
   constexpr int NWORDS = W / 32;
   constexpr int SEGCAP = sb_segcap<NW>();
   constexpr int NTW = W / SYM_MIN_FINE + 2;  // fine tiles a window can touch
-  extern __shared__ __align__(16) unsigned char smem_raw[];
   uint32_t* bits = reinterpret_cast<uint32_t*>(smem_raw);
   int* seg_off = reinterpret_cast<int*>(bits + NWORDS);
   int* seg_s = seg_off + SEGCAP;
   int* wcnt = seg_s + SEGCAP;
   int* wnext = wcnt + NW;
   int* tcnt = wnext + NW;
-  __shared__ int s_lb, s_le, s_nh, s_hs, s_item;
+  __shared__ int s_item;
   __shared__ unsigned long long s_pack[2];
   const int warp = threadIdx.x >> 5, lane = lane_id();
   for (int t = threadIdx.x; t < NWORDS; t += NW * 32) bits[t] = 0u;
   for (int t = threadIdx.x; t < NTW; t += NW * 32) tcnt[t] = 0;
   if (threadIdx.x == 0) {
-    bin_range(st, bin_lo, bin_hi, &s_lb, &s_le);
-    s_nh = split_rows(st, sp, &s_hs);
     s_pack[0] = 0ull;
     s_pack[1] = 0ull;
   }
-  if (block_skip(st)) return;
-  const int lb = s_lb, le = s_le, nh = s_nh, hs = s_hs;
   const int wf_shift = sp.wf_shift;
   int parity = 0;
 
