@@ -461,7 +461,7 @@ static spgemm_status analyse_impl(const spgemm_csr* A, const spgemm_csr* B, cons
     p->at_src = (int32_t*)(p->ws + L.at_src);
     e = sg::launch_transpose(c, A->nrows, A->ncols, A->nnz, A->row_ptr, A->col_idx, p->at_rp, p->at_ci, p->at_src,
                              0, nullptr, nullptr, (int32_t*)(p->ws + L.at_tmp), (int32_t*)(p->ws + L.at_table),
-                             (long long*)(p->ws + L.at_part));
+                             (long long*)(p->ws + L.at_part), (int32_t*)(p->ws + L.a_row) /* filled below */);
     p->a_row = (int32_t*)(p->ws + L.a_row);
     p->b_row = (int32_t*)(p->ws + L.b_row);
     if (e == cudaSuccess) e = sg::launch_row_index(c, A->row_ptr, A->nrows, p->a_row);
@@ -731,7 +731,7 @@ spgemm_status spgemm_transpose_workspace_size(int64_t nrows, int64_t ncols, int6
   if (nnz >= (1ll << 31) || ncols >= (1ll << 31) - 1) return SPGEMM_ERR_INDEX_OVERFLOW;
   size_t tmp, table, part;
   size_t off = align_up(sizeof(sg::DevStats));
-  off = align_up(off + sizeof(int32_t) * (size_t)nnz);  // source positions if the caller wants none
+  off = align_up(off + sizeof(int32_t) * (size_t)nnz);  // the sorted columns
   *bytes = transpose_layout(off, ncols, nnz, 8, &tmp, &table, &part);  // room for FP64 values
   return SPGEMM_OK;
 }
@@ -756,17 +756,16 @@ spgemm_status spgemm_transpose(const spgemm_csr* M, int32_t dtype, int32_t* t_ro
   c.st = (sg::DevStats*)ws;
   c.err = &c.st->err;
   size_t off = align_up(sizeof(sg::DevStats));
-  int32_t* own_src = (int32_t*)(ws + off);
+  int32_t* sorted = (int32_t*)(ws + off);
   off = align_up(off + sizeof(int32_t) * (size_t)M->nnz);
   size_t tmp, table, part;
   transpose_layout(off, M->ncols, M->nnz, 8, &tmp, &table, &part);
-  int32_t* src = t_src ? t_src : own_src;
   const int vbytes = t_vals ? (dtype == SPGEMM_F32 ? 4 : 8) : 0;
   cudaError_t e = cudaMemsetAsync(c.st, 0, sizeof(sg::DevStats), c.stream);
   if (e == cudaSuccess)
-    e = sg::launch_transpose(c, M->nrows, M->ncols, M->nnz, M->row_ptr, M->col_idx, t_row_ptr, t_col_idx, src,
+    e = sg::launch_transpose(c, M->nrows, M->ncols, M->nnz, M->row_ptr, M->col_idx, t_row_ptr, t_col_idx, t_src,
                              vbytes, M->vals, t_vals, (int32_t*)(ws + tmp), (int32_t*)(ws + table),
-                             (long long*)(ws + part));
+                             (long long*)(ws + part), sorted);
   return e == cudaSuccess ? SPGEMM_OK : SPGEMM_ERR_CUDA;
 }
 

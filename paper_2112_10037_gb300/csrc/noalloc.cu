@@ -35,7 +35,8 @@ struct NaLayout {
   size_t st, src, tmp, table, part, total;
 };
 
-// The source positions get scratch only when the caller passes no t_src;
+// The sorted columns get scratch only when the caller passes no t_src (what
+// fits the fixed array does not depend on how the row pointer is found);
 // values (vbytes each, 0 without t_vals) travel through the scratch.
 NaLayout na_layout(long long ncols, long long nnz, bool need_src, int vbytes) {
   const TransposeScratch s = transpose_scratch(ncols, nnz, vbytes);
@@ -103,12 +104,12 @@ extern "C" spgemm_status spgemm_transpose_noalloc(const spgemm_csr* M, int32_t d
   c.nsm = nsm;
   c.st = (DevStats*)(ws + L.st);
   c.err = &c.st->err;
-  int32_t* src = t_src ? t_src : (int32_t*)(ws + L.src);
+  int32_t* sorted = t_src ? nullptr : (int32_t*)(ws + L.src);
   // the stats word (error bits, scan total) must start at zero every call
   cudaError_t e = cudaMemsetAsync(c.st, 0, sizeof(DevStats), c.stream);
   if (e == cudaSuccess)
-    e = launch_transpose(c, M->nrows, M->ncols, M->nnz, M->row_ptr, M->col_idx, t_row_ptr, t_col_idx, src,
+    e = launch_transpose(c, M->nrows, M->ncols, M->nnz, M->row_ptr, M->col_idx, t_row_ptr, t_col_idx, t_src,
                          vbytes, M->vals, t_vals, (int32_t*)(ws + L.tmp), (int32_t*)(ws + L.table),
-                         (long long*)(ws + L.part));
+                         (long long*)(ws + L.part), sorted);
   return e == cudaSuccess ? SPGEMM_OK : SPGEMM_ERR_CUDA;
 }
