@@ -446,12 +446,14 @@ static spgemm_status analyse_impl(const spgemm_csr* A, const spgemm_csr* B, cons
                                                span_min);
   if (e == cudaSuccess && !base) {
     // Only the numeric window paths read the run lists.  A plan of every row
-    // of A may leave them unbuilt when none of its rows takes such a path:
+    // of A may leave them unbuilt when none of its rows can take such a path:
     // plans derived from it cover subsets of those rows.
-    int win_lo = sg::NBINS;
+    int lo = sg::NBINS;  // first bin above the small rows
     for (int q : {sg::PATH_WARP, sg::PATH_BLOCK})
-      if (p->pb.hi[q] >= p->pb.lo[q] && p->pb.lo[q] < win_lo) win_lo = p->pb.lo[q];
-    if (p->tu.num_hi_once >= win_lo) win_lo = p->tu.num_hi_once + 1;
+      if (p->pb.hi[q] >= p->pb.lo[q] && p->pb.lo[q] < lo) lo = p->pb.lo[q];
+    int win_lo = lo > p->tu.num_hi_once ? lo : p->tu.num_hi_once + 1;  // bins the register path leaves over,
+    const int block_lo = lo > p->tu.num_lo_block ? lo : p->tu.num_lo_block;  // or the block window takes first
+    if (block_lo < win_lo) win_lo = block_lo;
     if (rb != 0 || re != A->nrows) win_lo = 0;
     e = sg::launch_runs(c, p->B, p->sp, p->runs_part, win_lo);
   }

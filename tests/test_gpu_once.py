@@ -96,3 +96,17 @@ def test_infinities_and_nan(api, oracle_mod):
     assert np.array_equal(np.isnan(got.vals), np.isnan(R.vals))
     inf = np.isinf(R.vals)
     assert np.array_equal(got.vals[inf], R.vals[inf]) and np.array_equal(np.isinf(got.vals), inf)
+
+
+@pytest.mark.parametrize("ncols", [9000, 200_000])
+@pytest.mark.parametrize("num_block_min", [256, 4096])
+def test_block_window_before_the_registers(api, oracle_mod, ncols, num_block_min):
+    """Rows of at most 8192 products that the block window takes by an option:
+    its run lists of B are built although no row is longer."""
+    A, B = _operands(ncols, "spread", 8)
+    keep = np.flatnonzero(np.array(EDGES) <= 8192)
+    A = oracle_mod.select_rows(A, keep)
+    got = api.spgemm(api.DeviceCSR.from_host(A), api.DeviceCSR.from_host(B), num_block_min=num_block_min).to_host()
+    R, S = oracle_with_scale(oracle_mod, A, B)
+    assert_structure_equal(got, R)
+    assert_values_close(got.vals, R.vals, S)
