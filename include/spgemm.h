@@ -103,9 +103,9 @@ typedef struct spgemm_opts {
   int32_t backward;    /* nonzero: the plan also keeps the transpose of A's structure,
                           which spgemm_backward needs (more workspace) */
   int32_t num_block_min;/* rows with more products than this run the numeric pass
-                          with a block-wide window (0: 2048 products per 8192 columns
-                          of B, at least 8192 and at most 65536; -1: never, then heavy
-                          rows are split as split_min says) */
+                          with a block-wide window (0: 65536, or down to 4096 where
+                          few rows are that long and rank_min is off; -1: never, then heavy rows are split
+                          as split_min says) */
   int32_t block_warps; /* warps sharing a numeric block window (see window_block) */
   int32_t sort_max;    /* rows of at most this many products are merged by a sort in
                           registers: 128, 256 or 512 (0: 128); rows of 17 or more
@@ -291,8 +291,8 @@ spgemm_status spgemm_transpose_check(void* workspace, spgemm_stream_t stream);
  * scratch would exceed it are rejected with SPGEMM_ERR_WORKSPACE: the need
  * is, for 513 to 262,144 columns, 12*nnz bytes plus 8*nnz (FP64) or 4*nnz
  * (FP32) when t_vals is given (none of this for at most 512 columns; 4*nnz
- * more above 262,144 columns), plus 4*nnz when t_src is NULL (the source
- * positions then need scratch too), plus the digit counts (4 bytes per
+ * more above 262,144 columns), plus 4*nnz when t_src is NULL (scratch for
+ * the sorted columns), plus the digit counts (4 bytes per
  * digit value and 4096 entries: at most nnz/2 bytes) and their scan partials
  * (8 bytes per 4096 counts or columns), plus about 2 KB of bookkeeping and
  * alignment; so about 400 K entries fit with t_src and FP64 t_vals given.

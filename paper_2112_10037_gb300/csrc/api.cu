@@ -142,22 +142,17 @@ void split_geometry(const spgemm_opts& o, int window, long long mloc, long long 
   *hcnt_entries = (size_t)cap * (size_t)sp->ntf;
 }
 
-// First bin of rows whose numeric pass uses the block-wide window: by default
-// rows of more than 2048 products per window of B's columns, within 8192 to
-// 65,536.  (A window costs the block a few thousand cycles whatever it holds;
-// a warp that owns a whole row of 65,536 products over two windows runs alone
-// long after the other rows are done: on a graph of 12,345 vertices the warp
-// window took 1.15 ms for the rows of 8,193 to 65,536 products.)
+// First bin of rows whose numeric pass may use the block-wide window; by
+// default rows of more than 8192 products, of more than 4096 where B has at
+// most 65,536 columns.  (Which of the bins up to 65,536 products do is decided
+// by their rows, see block_lo in numdispatch.cuh.)
 int numeric_block_bin(const spgemm_opts& o, long long ncols_b) {
   if (o.force_path == 1 || o.force_path == 3) return sg::NBINS;  // warp window only
   if (o.force_path == 2) return tiny_hi_bin(o) + 1;                 // every row above the register sort
   if (o.force_path == 4) return 1;                                 // every non-empty row
   if (o.num_block_min < 0) return sg::NBINS;
   long long m = o.num_block_min;
-  if (m == 0) {
-    m = 2048 * ((ncols_b + 8191) / 8192);
-    m = m < 8192 ? 8192 : (m > 65536 ? 65536 : m);
-  }
+  if (m == 0) m = o.rank_min > 0 ? 65536 : (ncols_b <= 65536 ? 4096 : 8192);
   const int b = sg::bin_of(m) + 1;
   return b < small_hi_bin(o) + 1 ? small_hi_bin(o) + 1 : b;
 }
@@ -257,11 +252,15 @@ spgemm_status check_csr(const spgemm_csr* M) {
 }
 
 // Window columns and warps of the numeric block kernel: one of the compiled
-// pairs, the default where the options name none or an unsupported one.
-static void block_geometry(const spgemm_opts& o, int* w, int* nw) {
+// pairs, the default where the options name none or an unsupported one: 8192
+// columns and 8 warps (three blocks on an SM), or 16,384 and 16 where B has at
+// most two such windows: there the longest rows set the time, and a row is
+// done in half of it (12,345 columns FP32: 0.36 ms for the rows above 4096
+// products, 0.22 so; 65,536 columns FP64: 3.4 and 3.9 ms).
+static void block_geometry(const spgemm_opts& o, long long ncols_b, int* w, int* nw) {
   static const int pairs[][2] = {{2048, 4}, {2048, 8}, {4096, 4}, {4096, 8}, {4096, 16}, {8192, 8}, {8192, 16},
                                  {16384, 16}};
-  const int dw = 8192, dn = 8;  // default geometry
+  const int dw = ncols_b <= 32768 ? 16384 : 8192, dn = ncols_b <= 32768 ? 16 : 8;
   const int ww = o.window_block > 0 ? o.window_block : dw, nn = o.block_warps > 0 ? o.block_warps : dn;
   *w = dw;
   *nw = dn;
@@ -277,11 +276,12 @@ void choose_paths(const spgemm_opts& o, long long ncols_b, sg::PathBins* pb, sg:
   const int last = sg::NBINS - 1;
   tu->warp_max = o.warp_max > 0 ? o.warp_max : 8192;
   tu->window_warp = numeric_window(o);
-  block_geometry(o, &tu->window_block, &tu->block_warps);
+  block_geometry(o, ncols_b, &tu->window_block, &tu->block_warps);
   const int HASH_HI = hash_hi_bin(o);
   tu->hash_max = HASH_HI > 0 ? 1 << (HASH_HI - 1) : 0;
   tu->num_hi_once = numeric_once_bin(o);
   tu->num_lo_block = numeric_block_bin(o, ncols_b);
+  tu->block_auto = o.force_path < 0 && o.num_block_min == 0 && o.rank_min <= 0;
   tu->num_lo_rank = numeric_rank_bin(o);
   tu->rank_accum = o.rank_accum == 1 ? 1 : 0;
   const int TINY_HI = tiny_hi_bin(o);  // register sort up to opts.sort_max products

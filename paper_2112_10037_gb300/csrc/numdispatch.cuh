@@ -230,6 +230,19 @@ static cudaError_t tiny_dispatch(const int* hist, int lo, int hi, F8 f8, F16 f16
   return cudaSuccess;
 }
 
+// First bin of the block window.  Rows of more than 65,536 products always take
+// it; a bin below does when it has fewer than 40 rows per SM: the warp window
+// runs one warp per row, 27 at a time on an SM, and with fewer rows the longest
+// of them run alone at the end (40,000 columns, 316 K nonzeros, rows above 4096
+// products in FP64: 2.4 ms with warps up to 65,536 products, 0.57 with blocks;
+// R-MAT scale 18, 7 K to 16 K rows a bin: 13.1 ms with warps, 15.6 with blocks).
+static int block_lo(const Tuning& tu, const int* hist, int nsm) {
+  if (!tu.block_auto || !hist) return tu.num_lo_block;
+  int b = bin_of(65536) + 1;
+  while (b > tu.num_lo_block && hist[b - 1] < 40 * nsm) --b;
+  return b;
+}
+
 template <typename T, int SR>
 static cudaError_t numeric_t(const LaunchCtx& c, const Csr& A, const Csr& B, const RowInfo& ri,
                              const PathBins& pb, const Tuning& tu, const SplitInfo& sp, const T* av,
@@ -282,7 +295,7 @@ static cudaError_t numeric_t(const LaunchCtx& c, const Csr& A, const Csr& B, con
     timer_mark(c, T_NUM_HASH, 1);
     if (e) return e;
   }
-  // every other row: the warp-owned dense window up to tu.num_lo_block,
+  // every other row: the warp-owned dense window up to block_lo,
   // the block-wide window from there on (rows of the symbolic warp and block
   // paths both land here)
   int lo = NBINS, hi = 0;
@@ -291,19 +304,20 @@ static cudaError_t numeric_t(const LaunchCtx& c, const Csr& A, const Csr& B, con
       lo = pb.lo[p] < lo ? pb.lo[p] : lo;
       hi = pb.hi[p] > hi ? pb.hi[p] : hi;
     }
-  const int blo = tu.num_lo_block > lo ? tu.num_lo_block : lo;
+  const int nlo = block_lo(tu, hist, c.nsm);
+  const int blo = nlo > lo ? nlo : lo;
   if (hi >= blo && !empty_bins(hist, blo, hi)) {
     timer_mark(c, T_NUM_BLOCK, 0);
 #define SG_BLOCK_NUM(WW, NWW) e = block_num<T, WW, NWW, SR>(c, A, B, av, bv, ri, blo, hi, sp, cur, nxt, c_rp, c_ci, c_v)
     // supported geometries (window columns, warps); others fall back to 8192 x 8
     const int wbk = tu.window_block, nwk = tu.block_warps;
-    if (SR != SPGEMM_PLUS_TIMES) SG_BLOCK_NUM(8192, 8);
+    if (wbk == 16384 && nwk == 16) SG_BLOCK_NUM(16384, 16);
+    else if (SR != SPGEMM_PLUS_TIMES) SG_BLOCK_NUM(8192, 8);
     else if (wbk == 2048 && nwk == 4) SG_BLOCK_NUM(2048, 4);
     else if (wbk == 2048 && nwk == 8) SG_BLOCK_NUM(2048, 8);
     else if (wbk == 4096 && nwk == 4) SG_BLOCK_NUM(4096, 4);
     else if (wbk == 4096 && nwk == 8) SG_BLOCK_NUM(4096, 8);
     else if (wbk == 4096 && nwk == 16) SG_BLOCK_NUM(4096, 16);
-    else if (wbk == 16384 && nwk == 16) SG_BLOCK_NUM(16384, 16);
     else if (wbk == 8192 && nwk == 16) SG_BLOCK_NUM(8192, 16);
     else SG_BLOCK_NUM(8192, 8);
 #undef SG_BLOCK_NUM

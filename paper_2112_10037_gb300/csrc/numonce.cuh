@@ -29,9 +29,9 @@
 // instruction issue (2.4 of 4 per clock, 152 warp instructions per 32 products
 // at 16,384 rows of 32 x 32) and the shared-memory traffic of random bits and
 // ranks (L1 74 % busy).  65,536 rows of 32 x 32 products over 65,536 columns
-// in FP32: 1.58 ms with the warp window, 0.41 ms here; 64 products of 1,024 to
+// in FP32: 1.58 ms with the warp window, 0.40 ms here; 64 products of 1,024 to
 // 50,000 rows (rows of up to 4,096 products, FP64): 10.9 ms and 4.1 ms; R-MAT
-// scale 18, rows of 129 to 8,192 products: 6.0 ms and 2.8 ms.
+// scale 18, rows of 129 to 8,192 products: 6.0 ms and 2.6 ms.
 //
 // The threads follow the row's products, 8 per thread.  Rows above 8192
 // products stay with the windows: their products no longer fit 64 registers
@@ -66,6 +66,17 @@ __host__ __device__ constexpr int once_blocks_per_sm() {
 template <int NT>
 __host__ __device__ constexpr int once_wlog_max() {
   return NT >= 512 ? 18 : (NT >= 128 ? 17 : 16);
+}
+
+// Exclusive sum of the NW warps' entries of v before this warp, and the total
+// of all (lane w reads entry w: a loop over the entries in every thread of a
+// 1024-thread block was a quarter of the kernel's instructions).
+template <int NW>
+__device__ __forceinline__ int once_before(const int* v, int warp, int* total) {
+  const int lane = lane_id();
+  const int x = lane < NW ? v[lane] : 0;
+  *total = __reduce_add_sync(FULL, x);
+  return __reduce_add_sync(FULL, lane < warp ? x : 0);
 }
 
 template <int NT, typename T, int SR = SPGEMM_PLUS_TIMES>
@@ -143,14 +154,8 @@ k_num_once(Csr A, Csr B, const T* __restrict__ av, const T* __restrict__ bv, Row
       const unsigned incl = warp_incl_scan(v);
       if (lane == 31) wsum[warp] = (int)incl;
       __syncthreads();
-      unsigned before = carry, total = 0;
-#pragma unroll 4
-      for (int w = 0; w < NW; ++w) {
-        const unsigned x = (unsigned)wsum[w];
-        total += x;
-        if (w < warp) before += x;
-      }
-      before += incl - v;
+      int total;
+      const unsigned before = carry + (unsigned)once_before<NW>(wsum, warp, &total) + incl - v;
       const int off = (int)(before & 0xffffu), k = (int)(before >> 16);
       if (len > 0) {
         if (off + len <= CAP && k < CAP) {
@@ -161,7 +166,7 @@ k_num_once(Csr A, Csr B, const T* __restrict__ av, const T* __restrict__ bv, Row
           atomicOr(err, EB_INTERNAL);
         }
       }
-      carry += total;
+      carry += (unsigned)total;
       __syncthreads();
     }
     const int P = min((int)(carry & 0xffffu), CAP);
@@ -246,15 +251,9 @@ k_num_once(Csr A, Csr B, const T* __restrict__ av, const T* __restrict__ bv, Row
       sum = warp_sum(sum);
       if (lane == 0) wsum[warp] = sum;
       __syncthreads();
-      int run = 0, total = 0;
-      next = INT_MAX;
-#pragma unroll 4
-      for (int w = 0; w < NW; ++w) {
-        const int x = wsum[w];
-        if (w < warp) run += x;
-        total += x;
-        next = min(next, wnext[w]);
-      }
+      int total;
+      int run = once_before<NW>(wsum, warp, &total);
+      next = warp_min(lane < NW ? wnext[lane] : INT_MAX);
       for (int t = t0; t < t1; ++t) {
         const int w0 = (t << 8) + lane * 8;
         uint4 x = make_uint4(0, 0, 0, 0), y = x;
