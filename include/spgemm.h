@@ -103,9 +103,12 @@ typedef struct spgemm_opts {
   int32_t backward;    /* nonzero: the plan also keeps the transpose of A's structure,
                           which spgemm_backward needs (more workspace) */
   int32_t num_block_min;/* rows with more products than this run the numeric pass
-                          with a block-wide window (0: 65536, or down to 4096 where
-                          few rows are that long and rank_min is off; -1: never, then heavy rows are split
-                          as split_min says) */
+                          with a block-wide window (-1: never, then heavy rows are split
+                          as split_min says).  0 or 65536 with the other options that
+                          choose a kernel for such rows (rank_min, split_min, window_warp,
+                          window_block, block_warps) at 0 or their defaults: rows of more
+                          than 4096 products (2048 on at most 65,536 columns) accumulate
+                          in bands of ranks, see csrc/numband.cuh */
   int32_t block_warps; /* warps sharing a numeric block window (see window_block) */
   int32_t sort_max;    /* rows of at most this many products are merged by a sort in
                           registers: 128, 256 or 512 (0: 128); rows of 17 or more

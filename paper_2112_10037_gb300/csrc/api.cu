@@ -84,6 +84,7 @@ size_t transpose_layout(size_t off, long long n, long long nnz, int vbytes, size
 }
 
 int numeric_block_bin(const spgemm_opts& o, long long ncols_b);
+bool default_long_rows(const spgemm_opts& o);
 
 // Last bin of the register-sort path: rows of at most 128, 256 or 512
 // products (opts.sort_max; bin b holds products in (2^(b-2), 2^(b-1)]).
@@ -126,7 +127,7 @@ void split_geometry(const spgemm_opts& o, int window, long long mloc, long long 
   while ((1 << sp->wf_shift) < window) ++sp->wf_shift;
   sp->ntf = (int)((ncols_b + window - 1) / window);
   *hcnt_entries = 0;
-  if (o.split_min < 0 || o.force_path >= 0 || mloc <= 0 || sp->ntf < 2) return;
+  if (o.split_min < 0 || o.force_path >= 0 || mloc <= 0 || sp->ntf < 2 || default_long_rows(o)) return;
   const long long smin = o.split_min > 0 ? o.split_min : 131072;
   if (sg::bin_of(smin) + 1 >= numeric_block_bin(o, ncols_b)) return;  // those rows use the block window
   long long cap = mloc < 16384 ? mloc : 16384;
@@ -142,18 +143,43 @@ void split_geometry(const spgemm_opts& o, int window, long long mloc, long long 
   *hcnt_entries = (size_t)cap * (size_t)sp->ntf;
 }
 
-// First bin of rows whose numeric pass may use the block-wide window; by
-// default rows of more than 8192 products, of more than 4096 where B has at
-// most 65,536 columns.  (Which of the bins up to 65,536 products do is decided
-// by their rows, see block_lo in numdispatch.cuh.)
+// Whether rows too long for the register path take the default routes (the
+// banded accumulator, see numeric_band_bin): no option that asks for another
+// kernel or another shape of one.  Options at their old defaults ask for none.
+bool default_long_rows(const spgemm_opts& o) {
+  return o.force_path < 0 && (o.num_block_min == 0 || o.num_block_min == 65536) && o.rank_min <= 0 &&
+         o.split_min <= 0 && (o.window_warp == 0 || o.window_warp == 1024) &&
+         (o.window_block == 0 || o.window_block == 8192) && (o.block_warps == 0 || o.block_warps == 8);
+}
+
+// First bin of rows whose numeric pass may use the block-wide window.  By
+// default only FP32 rows of more than 4096 products on at most 32,768 columns
+// (and of those only few rows, see numdispatch.cuh).
 int numeric_block_bin(const spgemm_opts& o, long long ncols_b) {
   if (o.force_path == 1 || o.force_path == 3) return sg::NBINS;  // warp window only
   if (o.force_path == 2) return tiny_hi_bin(o) + 1;                 // every row above the register sort
   if (o.force_path == 4) return 1;                                 // every non-empty row
   if (o.num_block_min < 0) return sg::NBINS;
-  long long m = o.num_block_min;
-  if (m == 0) m = o.rank_min > 0 ? 65536 : (ncols_b <= 65536 ? 4096 : 8192);
+  long long m = o.num_block_min > 0 ? o.num_block_min : 65536;
+  if (default_long_rows(o)) {
+    if (o.dtype != SPGEMM_F32 || ncols_b > 32768) return sg::NBINS;
+    m = 4096;
+  }
   const int b = sg::bin_of(m) + 1;
+  return b < small_hi_bin(o) + 1 ? small_hi_bin(o) + 1 : b;
+}
+
+// First bin of rows whose numeric pass uses the banded accumulator
+// (numband.cuh), NBINS when an option asks for another kernel.  Rows of more
+// than 4096 products, of more than 2048 where B has at most 65,536 columns:
+// there the bitmap of a row is small and the register path's block of 512 or
+// 1024 threads is alone on its SM (32,768 columns, 262 K nonzeros, FP64, rows
+// above 128 products: 0.56 ms with the line at 4096 products, 0.50 at 2048;
+// 150,000 columns: rows of 2,049 to 4,096 take 0.13 ms in registers, 0.16 in
+// bands).
+int numeric_band_bin(const spgemm_opts& o, long long ncols_b) {
+  if (!default_long_rows(o)) return sg::NBINS;
+  const int b = sg::bin_of(ncols_b <= 65536 ? 2048 : 4096) + 1;
   return b < small_hi_bin(o) + 1 ? small_hi_bin(o) + 1 : b;
 }
 
@@ -256,7 +282,7 @@ spgemm_status check_csr(const spgemm_csr* M) {
 // columns and 8 warps (three blocks on an SM), or 16,384 and 16 where B has at
 // most two such windows: there the longest rows set the time, and a row is
 // done in half of it (12,345 columns FP32: 0.36 ms for the rows above 4096
-// products, 0.22 so; 65,536 columns FP64: 3.4 and 3.9 ms).
+// products with 8192 and 8, 0.22 so).
 static void block_geometry(const spgemm_opts& o, long long ncols_b, int* w, int* nw) {
   static const int pairs[][2] = {{2048, 4}, {2048, 8}, {4096, 4}, {4096, 8}, {4096, 16}, {8192, 8}, {8192, 16},
                                  {16384, 16}};
@@ -281,7 +307,7 @@ void choose_paths(const spgemm_opts& o, long long ncols_b, sg::PathBins* pb, sg:
   tu->hash_max = HASH_HI > 0 ? 1 << (HASH_HI - 1) : 0;
   tu->num_hi_once = numeric_once_bin(o);
   tu->num_lo_block = numeric_block_bin(o, ncols_b);
-  tu->block_auto = o.force_path < 0 && o.num_block_min == 0 && o.rank_min <= 0;
+  tu->num_lo_band = numeric_band_bin(o, ncols_b);
   tu->num_lo_rank = numeric_rank_bin(o);
   tu->rank_accum = o.rank_accum == 1 ? 1 : 0;
   const int TINY_HI = tiny_hi_bin(o);  // register sort up to opts.sort_max products
@@ -453,9 +479,10 @@ static spgemm_status analyse_impl(const spgemm_csr* A, const spgemm_csr* B, cons
       if (p->pb.hi[q] >= p->pb.lo[q] && p->pb.lo[q] < lo) lo = p->pb.lo[q];
     int win_lo = lo > p->tu.num_hi_once ? lo : p->tu.num_hi_once + 1;  // bins the register path leaves over,
     const int block_lo = lo > p->tu.num_lo_block ? lo : p->tu.num_lo_block;  // or the block window takes first
-    if (block_lo < win_lo) win_lo = block_lo;
+    if (block_lo < win_lo || p->tu.num_lo_band < sg::NBINS) win_lo = block_lo;  // (bands need no lists)
+    const bool never = win_lo >= sg::NBINS && p->tu.num_lo_band < sg::NBINS;
     if (rb != 0 || re != A->nrows) win_lo = 0;
-    e = sg::launch_runs(c, p->B, p->sp, p->runs_part, win_lo);
+    if (!never) e = sg::launch_runs(c, p->B, p->sp, p->runs_part, win_lo);
   }
   if (e == cudaSuccess && o.backward) {
     p->at_rp = (int32_t*)(p->ws + L.at_rp);

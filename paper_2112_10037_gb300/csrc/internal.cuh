@@ -89,7 +89,8 @@ struct Tuning {
   int warp_max;        // largest P of the symbolic warp path
   int num_hi_once;     // numeric bins <= this (above the small-row bins) keep a row in registers (0: none)
   int num_lo_block;    // numeric bins >= this use the block kernel (NBINS: never)
-  bool block_auto;     // ... of those up to 65,536 products, the bins of few rows only
+  int num_lo_band;     // numeric bins >= this use the banded accumulator (NBINS: never); then the block
+                       // kernel serves few rows only
   int num_lo_rank;     // numeric bins >= this (below num_lo_block) use the rank kernel (NBINS: never)
   int rank_accum;      // 0: rank kernel values reduced in global memory; 1: in shared-memory chunks
   int block_warps;     // warps per numeric block window

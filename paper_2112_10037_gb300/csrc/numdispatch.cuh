@@ -7,6 +7,7 @@
 #include <cstddef>
 
 #include "launch_util.cuh"
+#include "numband.cuh"
 #include "numblock.cuh"
 #include "numonce.cuh"
 #include "numrank.cuh"
@@ -172,6 +173,25 @@ static cudaError_t block_num(const LaunchCtx& c, const Csr& A, const Csr& B, con
   return cudaGetLastError();
 }
 
+template <typename T, int SR>
+static cudaError_t band_num(const LaunchCtx& c, const Csr& A, const Csr& B, const T* av, const T* bv,
+                            const RowInfo& ri, int lo, int hi, int32_t* cur, int32_t* nxt, const int32_t* c_rp,
+                            int32_t* c_ci, T* c_v) {
+  auto k = k_num_band<T, SR>;
+  int wlog = 10;  // the narrowest bitmap that holds a row of B, up to the widest
+  while (wlog < BAND_WLOG && (1ll << wlog) < B.ncols) ++wlog;
+  const size_t smem = band_smem_bytes<T>(wlog);
+  const int occ = kernel_blocks_per_sm(k, BAND_THREADS, smem);
+  if (occ <= 0) return cudaErrorInvalidConfiguration;
+  unsigned* counter = &c.st->work[1];
+  cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned), c.stream);
+  if (e != cudaSuccess) return e;
+  k<<<c.nsm * occ, BAND_THREADS, smem, c.stream>>>(A, B, av, bv, ri, c.st, lo, hi, wlog, cur, nxt, c_rp, c_ci, c_v,
+                                                   counter, c.err);
+  count_launch(c);
+  return cudaGetLastError();
+}
+
 // Rank-compacted accumulator: 8 warps per block; values either reduced into
 // C in global memory (the default, 56 KB of shared memory per block, four
 // blocks per SM) or summed in shared memory 6144 ranks at a time (104 KB in
@@ -230,17 +250,17 @@ static cudaError_t tiny_dispatch(const int* hist, int lo, int hi, F8 f8, F16 f16
   return cudaSuccess;
 }
 
-// First bin of the block window.  Rows of more than 65,536 products always take
-// it; a bin below does when it has fewer than 40 rows per SM: the warp window
-// runs one warp per row, 27 at a time on an SM, and with fewer rows the longest
-// of them run alone at the end (40,000 columns, 316 K nonzeros, rows above 4096
-// products in FP64: 2.4 ms with warps up to 65,536 products, 0.57 with blocks;
-// R-MAT scale 18, 7 K to 16 K rows a bin: 13.1 ms with warps, 15.6 with blocks).
+// With the banded accumulator as the default, the block window takes over (on
+// narrow FP32 products, see numeric_block_bin) when fewer than 40 rows per SM
+// are in its bins: the longest row then sets the time, and two dense windows
+// with adds that need no compare-and-swap finish it sooner than bands do
+// (12,345 columns: 0.22 ms against 0.26; 20,000 columns and 2 M nonzeros:
+// 3.5 against 3.3).
 static int block_lo(const Tuning& tu, const int* hist, int nsm) {
-  if (!tu.block_auto || !hist) return tu.num_lo_block;
-  int b = bin_of(65536) + 1;
-  while (b > tu.num_lo_block && hist[b - 1] < 40 * nsm) --b;
-  return b;
+  if (tu.num_lo_band >= NBINS || tu.num_lo_block >= NBINS) return tu.num_lo_block;
+  long long rows = 0;
+  for (int b = tu.num_lo_block; hist && b < NBINS; ++b) rows += hist[b];
+  return hist && rows < 40ll * nsm ? tu.num_lo_block : NBINS;
 }
 
 template <typename T, int SR>
@@ -295,9 +315,10 @@ static cudaError_t numeric_t(const LaunchCtx& c, const Csr& A, const Csr& B, con
     timer_mark(c, T_NUM_HASH, 1);
     if (e) return e;
   }
-  // every other row: the warp-owned dense window up to block_lo,
-  // the block-wide window from there on (rows of the symbolic warp and block
-  // paths both land here)
+  // every other row (rows of the symbolic warp and block paths both land
+  // here): the block-wide window from block_lo on, the banded accumulator from
+  // num_lo_band on, below them the register path and, where an option asks
+  // for it, the warp-owned dense window
   int lo = NBINS, hi = 0;
   for (int p : {PATH_WARP, PATH_BLOCK})
     if (pb.hi[p] >= pb.lo[p]) {
@@ -325,6 +346,19 @@ static cudaError_t numeric_t(const LaunchCtx& c, const Csr& A, const Csr& B, con
     if (e) return e;
   }
   if (hi >= blo) hi = blo - 1;
+  // with many rows of 2,049 to 4,096 products the register path keeps them
+  // (64 products of 1,024 to 50,000 rows: 0.55 ms, 0.83 in bands)
+  int band = tu.num_lo_band > lo ? tu.num_lo_band : lo;
+  if (hist && band == bin_of(2048) + 1 && hist[band] >= 40 * c.nsm) ++band;
+  if (blo >= NBINS && hi >= band) {
+    if (!empty_bins(hist, band, hi)) {
+      timer_mark(c, T_NUM_BLOCK, 0);
+      e = band_num<T, SR>(c, A, B, av, bv, ri, band, hi, cur, nxt, c_rp, c_ci, c_v);
+      timer_mark(c, T_NUM_BLOCK, 1);
+      if (e) return e;
+    }
+    hi = band - 1;
+  }
   // rows of the rank bins (below the block window) take the rank-compacted
   // accumulator, unless heavy rows are split (the warp kernel owns those)
   const bool split = sp.heavy_bin < NBINS && sp.hcap > 0;
