@@ -41,18 +41,6 @@ static cudaError_t tiny_num(const LaunchCtx& c, const Csr& A, const Csr& B, cons
   return cudaGetLastError();
 }
 
-template <typename T, int E, int SR>
-static cudaError_t hash_num(const LaunchCtx& c, const Csr& A, const Csr& B, const T* av, const T* bv,
-                            const RowInfo& ri, int lo, int hi, const int32_t* c_rp, int32_t* c_ci, T* c_v,
-                            long long rows) {
-  auto k = k_hash_num<E, T, SR>;
-  const int occ = kernel_blocks_per_sm(k, HASH_WARPS * 32, 0);
-  const int grid = persistent_grid(rows, HASH_WARPS, c.nsm, occ);
-  k<<<grid, HASH_WARPS * 32, 0, c.stream>>>(A, B, av, bv, ri, c.st, lo, hi, c_rp, c_ci, c_v, c.err);
-  count_launch(c);
-  return cudaGetLastError();
-}
-
 // Whether bins lo..hi hold no row (hist: rows per bin on the host, as the
 // symbolic pass read them; null: unknown, never empty).
 static bool empty_bins(const int* hist, int lo, int hi) {
@@ -62,18 +50,58 @@ static bool empty_bins(const int* hist, int lo, int hi) {
   return true;
 }
 
-// Hash bins: 6 -> 1 product per lane (P <= 32), 7 -> 2 (P <= 64), 8 -> 4 (P <= 128).
-template <typename F1, typename F2, typename F4>
-static cudaError_t hash_dispatch(const int* hist, int lo, int hi, F1 f1, F2 f2, F4 f4) {
-  cudaError_t e = cudaSuccess;
-  auto clip = [&](int a, int b, auto f) -> cudaError_t {
-    const int l = lo > a ? lo : a, h = hi < b ? hi : b;
-    return (l <= h && !empty_bins(hist, l, h)) ? f(l, h) : cudaSuccess;
-  };
-  if ((e = clip(1, 6, f1))) return e;
-  if ((e = clip(7, 7, f2))) return e;
-  if ((e = clip(8, 8, f4))) return e;
-  return cudaSuccess;
+// Small rows in one launch, each warp taking its share of every kind: a warp
+// and its table for 17 to 128 products, register sorts below.  (Five launches
+// of kernels that each fill a few SMs, one after the other, cost a product of
+// 12,345 vertices 31 us of 570.)
+constexpr int SMALL_WARPS = 4;
+
+struct SmallBins {  // inclusive; lo > hi: none
+  int tiny_lo, tiny_hi;  // at most bin 5
+  int hash_lo, hash_hi;  // bins 6..8
+};
+
+template <typename T, int SR>
+__global__ void __launch_bounds__(SMALL_WARPS * 32)
+k_num_small(Csr A, Csr B, const T* __restrict__ av, const T* __restrict__ bv, RowInfo ri, const DevStats* st,
+            SmallBins b, const int32_t* __restrict__ c_rp, int32_t* __restrict__ c_ci, T* __restrict__ c_v,
+            uint32_t* err) {
+  __shared__ __align__(16) HashWarp<T> s_hash[SMALL_WARPS];
+  __shared__ int s_r[5][2];
+  const int warp = threadIdx.x >> 5, lane = lane_id();
+  auto range = [&](int i, int lo, int hi) { block_bin_range(st, lo, hi, &s_r[i][0], &s_r[i][1]); };
+  range(0, max(b.hash_lo, 8), min(b.hash_hi, 8));
+  range(1, max(b.hash_lo, 7), min(b.hash_hi, 7));
+  range(2, max(b.hash_lo, 6), min(b.hash_hi, 6));
+  range(3, max(b.tiny_lo, 5), min(b.tiny_hi, 5));
+  range(4, b.tiny_lo, min(b.tiny_hi, 4));
+  HashWarp<T>& sm = s_hash[warp];
+  if (b.hash_hi >= b.hash_lo)
+    for (int t = lane; t < 256; t += 32) sm.key[t] = HASH_EMPTY;
+  if (block_skip(st)) return;
+  const long long w = (long long)blockIdx.x * SMALL_WARPS + warp, nw = (long long)gridDim.x * SMALL_WARPS;
+  hash_num_rows<4, T, SR>(A, B, av, bv, ri, s_r[0][0], s_r[0][1], w, nw, sm, c_rp, c_ci, c_v, err);
+  hash_num_rows<2, T, SR>(A, B, av, bv, ri, s_r[1][0], s_r[1][1], w, nw, sm, c_rp, c_ci, c_v, err);
+  hash_num_rows<1, T, SR>(A, B, av, bv, ri, s_r[2][0], s_r[2][1], w, nw, sm, c_rp, c_ci, c_v, err);
+  tiny_rows<16, 1, true, T, SR>(A, B, av, bv, ri, s_r[3][0], s_r[3][1], w, nw, nullptr, c_rp, c_ci, c_v, err);
+  tiny_rows<8, 1, true, T, SR>(A, B, av, bv, ri, s_r[4][0], s_r[4][1], w, nw, nullptr, c_rp, c_ci, c_v, err);
+}
+
+template <typename T, int SR>
+static cudaError_t small_num(const LaunchCtx& c, const Csr& A, const Csr& B, const T* av, const T* bv,
+                             const RowInfo& ri, const SmallBins& b, const int32_t* c_rp, int32_t* c_ci, T* c_v,
+                             const int* hist) {
+  long long warps = 0;  // hash rows take a warp each, the others a part of one
+  for (int k = b.hash_lo; hist && k <= b.hash_hi; ++k) warps += hist[k];
+  for (int k = b.tiny_lo; hist && k <= b.tiny_hi; ++k) warps += (hist[k] + 1) / 2;
+  if (hist && warps == 0) return cudaSuccess;
+  auto k = k_num_small<T, SR>;
+  const int occ = kernel_blocks_per_sm(k, SMALL_WARPS * 32, 0);
+  if (occ <= 0) return cudaErrorInvalidConfiguration;
+  k<<<persistent_grid(hist ? warps : -1, SMALL_WARPS, c.nsm, occ), SMALL_WARPS * 32, 0, c.stream>>>(
+      A, B, av, bv, ri, c.st, b, c_rp, c_ci, c_v, c.err);
+  count_launch(c);
+  return cudaGetLastError();
 }
 
 template <typename T, int NT, int SR>
@@ -269,14 +297,33 @@ static cudaError_t numeric_t(const LaunchCtx& c, const Csr& A, const Csr& B, con
                              const T* bv, int32_t* cur, int32_t* nxt, const int32_t* c_rp, int32_t* c_ci,
                              T* c_v, const int* path_rows, long long rows_wide, long long rows_wide8, const int* hist) {
   cudaError_t e = cudaSuccess;
-  // When no row has more than LANE_MERGE_K nonzeros (stencil products, and
-  // stencils times an aggregation), rows of at most 64 products are merged by
-  // one lane each, the smallest ones too: the register sort exchanges every
-  // product of a row with its neighbours log2(P)^2 / 2 times (96^3 Galerkin,
-  // A*P with 7 products a row: 107 us).
-  const bool merge = rows_wide8 == 0 && path_rows && pb.hi[PATH_HASH] >= pb.lo[PATH_HASH] &&
-                     pb.hi[PATH_TINY] + 1 == pb.lo[PATH_HASH];
-  if (pb.hi[PATH_TINY] >= pb.lo[PATH_TINY] && !merge) {
+  if (pb.hi[PATH_HASH] >= pb.lo[PATH_HASH]) {  // with it, register sorts stop at 16 products
+    timer_mark(c, T_NUM_HASH, 0);
+    SmallBins b{pb.lo[PATH_TINY], pb.hi[PATH_TINY], pb.lo[PATH_HASH], pb.hi[PATH_HASH]};
+    // Rows of up to 64 products by one lane each when they are most of the
+    // product's rows and enough to give every SM several warps (stencil and
+    // Galerkin products): throughput over many similar rows.  When no row has
+    // more than LANE_MERGE_K nonzeros (they are merged), the smallest ones
+    // too: the register sort exchanges every product of a row with its
+    // neighbours log2(P)^2 / 2 times (96^3 Galerkin, A*P with 7 products a
+    // row: 107 us).  Fewer rows keep a warp each, whose latency per row is
+    // lower.
+    long long all_rows = 0, lane_rows_n = 0;
+    const bool merge = rows_wide8 == 0 && b.tiny_hi + 1 == b.hash_lo;
+    if (path_rows && hist) {
+      for (int q = 0; q < NPATHS; ++q) all_rows += path_rows[q];
+      for (int k = merge ? b.tiny_lo : b.hash_lo; k <= b.hash_hi && k <= 7; ++k) lane_rows_n += hist[k];
+    }
+    if (lane_rows_n >= lane_rows_from(rows_wide8, c.nsm) && (merge || 2 * (long long)path_rows[PATH_HASH] >= all_rows)) {
+      const int llo = merge ? b.tiny_lo : b.hash_lo, lhi = b.hash_hi < 7 ? b.hash_hi : 7;
+      e = lane_rows<T, SR>(c, A, B, av, bv, ri, llo, lhi, c_rp, c_ci, c_v, lane_rows_n, rows_wide8);
+      b.hash_lo = lhi + 1;
+      if (merge) b.tiny_hi = b.tiny_lo - 1;
+    }
+    if (!e) e = small_num<T, SR>(c, A, B, av, bv, ri, b, c_rp, c_ci, c_v, hist);
+    timer_mark(c, T_NUM_HASH, 1);
+    if (e) return e;
+  } else if (pb.hi[PATH_TINY] >= pb.lo[PATH_TINY]) {
     const long long rows = rows_in(path_rows, PATH_TINY);
     timer_mark(c, T_NUM_TINY, 0);
     e = tiny_dispatch(hist, pb.lo[PATH_TINY], pb.hi[PATH_TINY],
@@ -288,31 +335,6 @@ static cudaError_t numeric_t(const LaunchCtx& c, const Csr& A, const Csr& B, con
         [&](int l, int h) { return tiny_num_wide<T, 32, 8, SR>(c, A, B, av, bv, ri, l, h, c_rp, c_ci, c_v, rows); },
         [&](int l, int h) { return tiny_num_wide<T, 32, 16, SR>(c, A, B, av, bv, ri, l, h, c_rp, c_ci, c_v, rows); });
     timer_mark(c, T_NUM_TINY, 1);
-    if (e) return e;
-  }
-  if (pb.hi[PATH_HASH] >= pb.lo[PATH_HASH]) {
-    const long long rows = rows_in(path_rows, PATH_HASH);
-    timer_mark(c, T_NUM_HASH, 0);
-    // When the hash rows are most of the product's rows (stencil and
-    // Galerkin products, where every row lands here), rows of at most 64
-    // products take one lane per row: throughput over many similar rows.
-    // A few such rows among larger ones (a power-law product) keep the warp
-    // per row, whose latency per row is lower.
-    long long all_rows = 0;
-    if (path_rows)
-      for (int q = 0; q < NPATHS; ++q) all_rows += path_rows[q];
-    const bool lanes = merge || (path_rows && 2 * (long long)path_rows[PATH_HASH] >= all_rows);
-    const int llo = merge ? pb.lo[PATH_TINY] : pb.lo[PATH_HASH], lhi = lanes ? (pb.hi[PATH_HASH] < 7 ? pb.hi[PATH_HASH] : 7) : 0;
-    if (llo <= lhi && !empty_bins(hist, llo, lhi))
-      e = lane_rows<T, SR>(c, A, B, av, bv, ri, llo, lhi, c_rp, c_ci, c_v,
-                           merge ? rows + path_rows[PATH_TINY] : rows, rows_wide8);
-    const int wlo = lhi >= llo ? lhi + 1 : llo;
-    if (!e && pb.hi[PATH_HASH] >= wlo)
-      e = hash_dispatch(hist, wlo, pb.hi[PATH_HASH],
-          [&](int l, int h) { return hash_num<T, 1, SR>(c, A, B, av, bv, ri, l, h, c_rp, c_ci, c_v, rows); },
-          [&](int l, int h) { return hash_num<T, 2, SR>(c, A, B, av, bv, ri, l, h, c_rp, c_ci, c_v, rows); },
-          [&](int l, int h) { return hash_num<T, 4, SR>(c, A, B, av, bv, ri, l, h, c_rp, c_ci, c_v, rows); });
-    timer_mark(c, T_NUM_HASH, 1);
     if (e) return e;
   }
   // every other row (rows of the symbolic warp and block paths both land

@@ -28,7 +28,6 @@
 namespace sg {
 
 constexpr int HASH_EMPTY = -1;   // free slot (columns are >= 0)
-constexpr int HASH_WARPS = 8;    // warps (rows in flight) per block
 
 // Slot of column c in a table of 2^lg slots: Fibonacci hashing of the column.
 template <int LG>
@@ -225,35 +224,36 @@ __device__ __forceinline__ void hash_sym_rows(const Csr& A, const Csr& B, const 
   });
 }
 
+// Shared memory of one warp of the numeric pass.
+template <typename T>
+struct HashWarp {
+  T val[256];
+  T dv[128];
+  int key[256];     // all HASH_EMPTY between rows
+  int dk[128 + 4];  // +4: INT_MAX padding of the ranking reads
+};
+
 // Numeric pass: C's columns (ascending) and values for each row, at the
 // positions [c_rp[r], c_rp[r+1]) the symbolic pass and the scan fixed.
 // The product that claims a column's slot stores its value there; the
 // others add theirs with a shared-memory reduction after a warp barrier.
+// Rows at list positions [lb, le), warp w of nw takes its share.
 template <int E, typename T, int SR = SPGEMM_PLUS_TIMES>
-__global__ void __launch_bounds__(HASH_WARPS * 32)
-k_hash_num(Csr A, Csr B, const T* __restrict__ av, const T* __restrict__ bv, RowInfo ri, const DevStats* st,
-           int bin_lo, int bin_hi, const int32_t* __restrict__ c_rp, int32_t* __restrict__ c_ci,
-           T* __restrict__ c_v, uint32_t* err) {
+__device__ __forceinline__ void hash_num_rows(const Csr& A, const Csr& B, const T* __restrict__ av,
+                                              const T* __restrict__ bv, const RowInfo& ri, long long lb,
+                                              long long le, long long w, long long nw, HashWarp<T>& sm,
+                                              const int32_t* __restrict__ c_rp, int32_t* __restrict__ c_ci,
+                                              T* __restrict__ c_v, uint32_t* err) {
   constexpr int LG = 6 + (E >= 4 ? 2 : (E >= 2 ? 1 : 0));
   constexpr int H = 1 << LG;
   constexpr int D = 32 * E;  // distinct columns of a row: at most its products
   static_assert(H == 64 * E, "table of twice the slots");
-  __shared__ int s_lb, s_le;
-  __shared__ __align__(16) int s_key[HASH_WARPS][H];
-  __shared__ __align__(16) T s_val[HASH_WARPS][H];
-  __shared__ __align__(16) int s_dk[HASH_WARPS][D + 4];  // +4: INT_MAX padding of the ranking reads
-  __shared__ __align__(16) T s_dv[HASH_WARPS][D];
-  const int warp = threadIdx.x >> 5, lane = lane_id();
-  int* key = s_key[warp];
-  T* val = s_val[warp];
-  int* dk = s_dk[warp];
-  T* dv = s_dv[warp];
-  for (int t = lane; t < H; t += 32) key[t] = HASH_EMPTY;
-  block_bin_range(st, bin_lo, bin_hi, &s_lb, &s_le);
-  if (block_skip(st)) return;
-  const long long nw = (long long)gridDim.x * HASH_WARPS;
-  hash_row_loop<true, T>(A, B, av, ri, s_lb, s_le, (long long)blockIdx.x * HASH_WARPS + warp, nw,
-                         [&](int r, int a0, int a1, const Chunk0<T>& c0, auto& between) {
+  const int lane = lane_id();
+  int* const key = sm.key;
+  T* const val = sm.val;
+  int* const dk = sm.dk;
+  T* const dv = sm.dv;
+  hash_row_loop<true, T>(A, B, av, ri, lb, le, w, nw, [&](int r, int a0, int a1, const Chunk0<T>& c0, auto& between) {
     const int ob = c_rp[r], oe = c_rp[r + 1];
     int col[E];
     T pv[E];

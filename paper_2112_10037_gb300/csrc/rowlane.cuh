@@ -35,6 +35,17 @@ namespace sg {
 constexpr int LANE_SLOTS = 64;     // table slots per lane (rows of at most 64 products)
 constexpr int LANE_WARPS = 4;      // warps per block
 constexpr int LANE_EMPTY = -1;
+// Fewest rows per SM that take a lane each; with rows of more than
+// LANE_MERGE_K nonzeros among them (wide8) many more, since their tables walk
+// one entry at a time.  A warp and its table per row otherwise: 24,013 rows of
+// 49 products on random columns 69 us by lanes, 31 by warps; 85,184 rows of a
+// 44^3 stencil 25 and 74; 50,000 rows of 2 to 12 nonzeros 246 and 71.
+constexpr int LANE_ROWS_PER_SM = 160;
+constexpr int LANE_ROWS_PER_SM_WIDE = 1024;
+
+__host__ __device__ inline long long lane_rows_from(long long wide8, int nsm) {
+  return (long long)nsm * (wide8 ? LANE_ROWS_PER_SM_WIDE : LANE_ROWS_PER_SM);
+}
 
 template <int SLOTS>
 __device__ __forceinline__ unsigned lane_hash(int c) {

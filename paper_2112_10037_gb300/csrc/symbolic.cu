@@ -49,7 +49,7 @@ static cudaError_t tiny_dispatch(int lo, int hi, F8 f8, F16 f16, F32 f32, F64 f6
 // Rows of at most 128 products in one launch: one lane and its table per row
 // of 17 to 64 products, and of fewer when no row has more than LANE_MERGE_K
 // nonzeros (a lane walks its nonzeros one by one; otherwise register sorts), a
-// warp and its table above.  The host does not know yet which bins have rows,
+// warp and its table above and where the rows are too few for lanes.  The host does not know yet which bins have rows,
 // so separate kernels would cost a small product four launches that find
 // nothing to do.  (Counting by the numeric pass's merge instead of the lane's
 // table: 98 us against 73 on the 96^3 stencil's square.)
@@ -62,7 +62,8 @@ struct SymBins {
 };
 
 __global__ void __launch_bounds__(SYM_SMALL_WARPS * 32)
-k_sym_small(Csr A, Csr B, RowInfo ri, const DevStats* st, SymBins b, int32_t* __restrict__ c_cnt, uint32_t* err) {
+k_sym_small(Csr A, Csr B, RowInfo ri, const DevStats* st, SymBins b, int nsm, int32_t* __restrict__ c_cnt,
+            uint32_t* err) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int s_t8[2], s_t16[2], s_lane[2], s_hash[2], s_wide8;
   const int warp = threadIdx.x >> 5, lane = lane_id();
@@ -74,7 +75,9 @@ k_sym_small(Csr A, Csr B, RowInfo ri, const DevStats* st, SymBins b, int32_t* __
   if (block_skip(st)) return;
   const long long gw = (long long)blockIdx.x * SYM_SMALL_WARPS + warp;
   const long long nw = (long long)gridDim.x * SYM_SMALL_WARPS;
-  const bool lanes = s_wide8 == 0;
+  const long long from = lane_rows_from(s_wide8, nsm);
+  const bool many = s_lane[1] - s_lane[0] >= from;
+  const bool lanes = s_wide8 == 0 && s_t8[1] - s_t16[0] >= from;
   int* const keys = reinterpret_cast<int*>(smem_raw) + (size_t)warp * LANE_SLOTS * 32;
   if (s_hash[1] > s_hash[0] || s_lane[1] > s_lane[0] || lanes) {
     for (int h = 0; h < LANE_SLOTS; ++h) keys[h * 32 + lane] = LANE_EMPTY;
@@ -82,8 +85,12 @@ k_sym_small(Csr A, Csr B, RowInfo ri, const DevStats* st, SymBins b, int32_t* __
   }
   // the warp tables first: their rows are the longest
   hash_sym_rows<4>(A, B, ri, s_hash[0], s_hash[1], gw, nw, keys, c_cnt, err);
-  lane_hash_rows<false, float>(A, B, nullptr, nullptr, ri, s_lane[0], s_lane[1], gw, nw, keys, nullptr, c_cnt,
-                               nullptr, nullptr, nullptr, err, -1);
+  if (!many) {  // too few rows to give every SM several warps of lanes
+    hash_sym_rows<2>(A, B, ri, s_lane[0], s_lane[1], gw, nw, keys, c_cnt, err);
+  } else {
+    lane_hash_rows<false, float>(A, B, nullptr, nullptr, ri, s_lane[0], s_lane[1], gw, nw, keys, nullptr, c_cnt,
+                                 nullptr, nullptr, nullptr, err, -1);
+  }
   if (lanes) {
     lane_hash_rows<false, float, SPGEMM_PLUS_TIMES, 32>(A, B, nullptr, nullptr, ri, s_t16[0], s_t8[1], gw, nw, keys,
                                                         nullptr, c_cnt, nullptr, nullptr, nullptr, err, -1);
@@ -106,7 +113,7 @@ static cudaError_t small_sym(const LaunchCtx& c, const Csr& A, const Csr& B, con
   const int occ = kernel_blocks_per_sm(k_sym_small, SYM_SMALL_WARPS * 32, smem);
   if (occ <= 0) return cudaErrorInvalidConfiguration;
   k_sym_small<<<persistent_grid(ri.mloc, SYM_SMALL_WARPS, c.nsm, occ), SYM_SMALL_WARPS * 32, smem, c.stream>>>(
-      A, B, ri, c.st, b, c_cnt, c.err);
+      A, B, ri, c.st, b, c.nsm, c_cnt, c.err);
   count_launch(c);
   return cudaGetLastError();
 }

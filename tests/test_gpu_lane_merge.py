@@ -1,8 +1,9 @@
 """GPU parity of the lane-per-row merge (rows of at most 8 nonzeros of A and
 64 products): one to eight B rows of uneven and zero length, 1 to 64 outputs
 (the collected groups of 8 full, ragged and empty), columns that all meet or
-all stay apart, a last warp of few rows; and the same rows beside one row of 9
-nonzeros, which routes the small rows to the other accumulators."""
+all stay apart, a last warp of few rows; the same rows beside one row of 9
+nonzeros; and both in numbers below and above those that take a lane per row
+(fewer take a warp each)."""
 import numpy as np
 import pytest
 
@@ -23,12 +24,12 @@ def api():
     return a
 
 
-def _operands(ncols, nine, seed=3):
+def _operands(ncols, nine, nrows=1003, seed=3):
     rng = np.random.default_rng(seed)
     blen = np.minimum(np.repeat([0, 1, 2, 7, 8, 9, 16, 31, 64], 40), ncols)
     B = gen.random_rows(len(blen), ncols, blen, rng)
     rows = []
-    for i in range(1003):
+    for i in range(nrows):
         n = 1 + i % 8
         ks = np.sort(rng.choice(len(blen), n, replace=False))
         while blen[ks].sum() > 64:
@@ -44,8 +45,9 @@ def _operands(ncols, nine, seed=3):
 @pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
 @pytest.mark.parametrize("ncols", [64, 100_000])
 @pytest.mark.parametrize("nine", [False, True])
-def test_rows(api, oracle_mod, ncols, nine, dtype):
-    A, B = _operands(ncols, nine)
+@pytest.mark.parametrize("nrows", [1003, 50_003, 320_003])
+def test_rows(api, oracle_mod, nrows, ncols, nine, dtype):
+    A, B = _operands(ncols, nine, nrows)
     got = api.spgemm(api.DeviceCSR.from_host(A, dtype=dtype), api.DeviceCSR.from_host(B, dtype=dtype)).to_host()
     if dtype == torch.float32:
         A, B = (M.astype(np.float32).astype(np.float64) for M in (A, B))
@@ -55,8 +57,9 @@ def test_rows(api, oracle_mod, ncols, nine, dtype):
 
 
 @pytest.mark.parametrize("semiring", ["min_plus", "max_plus", "or_and"])
-def test_semirings(api, oracle_mod, semiring):
-    A, B = _operands(64, False)
+@pytest.mark.parametrize("nrows,nine", [(1003, False), (50_003, False), (320_003, True)])
+def test_semirings(api, oracle_mod, nrows, nine, semiring):
+    A, B = _operands(64, nine, nrows)
     got = api.spgemm_semiring(api.DeviceCSR.from_host(A), api.DeviceCSR.from_host(B), semiring).to_host()
     R = oracle_mod.spgemm(A, B)
     assert_structure_equal(got, R)
