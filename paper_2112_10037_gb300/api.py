@@ -89,8 +89,9 @@ class DeviceCSR:
 
 
 def _stream_handle(stream=None) -> int:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return int(s.cuda_stream)
+    if stream is None:  # the handle itself, without building a Stream object
+        return int(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+    return int(stream.cuda_stream)
 
 
 def make_opts(dtype=torch.float64, validate=False, row_range=None, force_path=-1, warp_max=0,

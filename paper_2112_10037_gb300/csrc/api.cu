@@ -359,10 +359,55 @@ sg::RowInfo rowinfo_of(const spgemm_plan* p) {
   return ri;
 }
 
-spgemm_status read_stats(spgemm_plan* p, cudaStream_t s) {
-  if (cudaMemcpyAsync(&p->host_st, p->st, sizeof(sg::DevStats), cudaMemcpyDeviceToHost, s) != cudaSuccess)
+// Host memory that kernels write, for statistics that a blocking call waits
+// for: the scan's last block leaves them there and no copy follows the pass
+// (a copy to pageable memory and the wait for it took 5 us of a small
+// product's 87).  A block serves one call at a time and goes back to the pool;
+// at most POOL are kept (a call that finds none free and cannot get another
+// copies instead).
+class StatsPool {
+ public:
+  sg::DevStats* take() {
+    std::lock_guard<std::mutex> g(mu_);
+    if (!free_.empty()) {
+      sg::DevStats* p = free_.back();
+      free_.pop_back();
+      return p;
+    }
+    if (made_ >= POOL) return nullptr;
+    void* p = nullptr;
+    if (cudaHostAlloc(&p, sizeof(sg::DevStats), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    ++made_;
+    return (sg::DevStats*)p;
+  }
+  void give(sg::DevStats* p) {
+    if (!p) return;
+    std::lock_guard<std::mutex> g(mu_);
+    free_.push_back(p);
+  }
+
+ private:
+  static constexpr int POOL = 64;
+  std::mutex mu_;
+  std::vector<sg::DevStats*> free_;
+  int made_ = 0;
+};
+
+StatsPool& stats_pool() {
+  static StatsPool* pool = new StatsPool;  // never destroyed: calls may outlive static objects
+  return *pool;
+}
+
+// mirror: where the stream's work leaves the statistics (null: copied here).
+spgemm_status read_stats(spgemm_plan* p, cudaStream_t s, const sg::DevStats* mirror = nullptr) {
+  if (!mirror &&
+      cudaMemcpyAsync(&p->host_st, p->st, sizeof(sg::DevStats), cudaMemcpyDeviceToHost, s) != cudaSuccess)
     return SPGEMM_ERR_CUDA;
   if (cudaStreamSynchronize(s) != cudaSuccess) return SPGEMM_ERR_CUDA;
+  if (mirror) std::memcpy(&p->host_st, mirror, sizeof(sg::DevStats));
   for (int q = 0; q < sg::NPATHS; ++q) {
     int n = 0;
     for (int b = p->pb.lo[q]; b <= p->pb.hi[q]; ++b) n += p->host_st.hist[b];
@@ -617,10 +662,14 @@ spgemm_status spgemm_symbolic(spgemm_plan* p, int32_t* c_row_ptr, int64_t* c_nnz
   cudaError_t e = cudaSuccess;
   if (p->mloc > 0) e = sg::launch_symbolic(c, p->A, p->B, ri, p->pb, p->sp, p->cursor, c_row_ptr);
   // rows without products were not visited: the scan takes them as empty
-  if (e == cudaSuccess) e = sg::launch_scan(c, c_row_ptr, p->mloc, p->scan_part, nullptr, p->prod, &p->st->work[4]);
-  if (e != cudaSuccess) return SPGEMM_ERR_CUDA;
-  spgemm_status s = read_stats(p, st);
-  if (s != SPGEMM_OK) return s;
+  sg::DevStats* const mirror = stats_pool().take();
+  sg::DevStats* dev_mirror = nullptr;  // its address on the device
+  if (mirror && cudaHostGetDevicePointer((void**)&dev_mirror, mirror, 0) != cudaSuccess) dev_mirror = nullptr;
+  if (e == cudaSuccess)
+    e = sg::launch_scan(c, c_row_ptr, p->mloc, p->scan_part, nullptr, p->prod, &p->st->work[4], dev_mirror);
+  spgemm_status s = e == cudaSuccess ? read_stats(p, st, dev_mirror ? mirror : nullptr) : SPGEMM_ERR_CUDA;
+  if (s != SPGEMM_OK) return s;  // (the stream was not waited for: it may still write the mirror)
+  stats_pool().give(mirror);
   s = from_err_word(p->host_st.err);
   if (s != SPGEMM_OK) return s;
   p->nnz_c = p->host_st.nnz_c;

@@ -301,9 +301,11 @@ cudaError_t launch_runs(const LaunchCtx& c, const Csr& B, const SplitInfo& sp, l
 cudaError_t launch_symbolic(const LaunchCtx& c, const Csr& A, const Csr& B, const RowInfo& ri,
                             const PathBins& pb, const SplitInfo& sp, int32_t* cursor, int32_t* c_rp);
 // prod: rows of no product count as size 0 whatever c_rp holds (null: no
-// such rows); reset: two words set to zero (null: none).
+// such rows); reset: two words set to zero (null: none); mirror: host memory
+// that the device can write, receives the statistics (null: none).
 cudaError_t launch_scan(const LaunchCtx& c, int32_t* c_rp, long long mloc, long long* partials,
-                        long long* total_out = nullptr, const long long* prod = nullptr, unsigned* reset = nullptr);
+                        long long* total_out = nullptr, const long long* prod = nullptr, unsigned* reset = nullptr,
+                        DevStats* mirror = nullptr);
 // The run pointers of B's window-run lists (rrb may be null), both sums in the
 // same launches; win_lo as for launch_runs.
 cudaError_t launch_scan_runs(const LaunchCtx& c, int32_t* rr, int32_t* rrb, long long m, long long* partials,

@@ -61,17 +61,26 @@ __device__ __forceinline__ int scan_size(const int32_t* __restrict__ rp, const l
   return r < m && (!prod || prod[r] > 0) ? rp[r] : 0;
 }
 
+// Every thread of the last block must call it.
 __device__ __forceinline__ void scan_finish(const ScanArgs& a, long long m, long long total, DevStats* st,
-                                            unsigned* reset) {
-  *a.total = total;
-  if (total >= (1ll << 31)) atomicOr(&st->err, EB_OVERFLOW);
-  a.rp[m] = (int32_t)(total < (1ll << 31) ? total : 0);
-  if (reset) reset[0] = reset[1] = 0u;
+                                            unsigned* reset, DevStats* mirror) {
+  if (threadIdx.x == 0) {
+    *a.total = total;
+    if (total >= (1ll << 31)) atomicOr(&st->err, EB_OVERFLOW);
+    a.rp[m] = (int32_t)(total < (1ll << 31) ? total : 0);
+    if (reset) reset[0] = reset[1] = 0u;
+  }
+  if (!mirror) return;
+  __threadfence();
+  __syncthreads();
+  static_assert(sizeof(DevStats) % 4 == 0, "copied by words");
+  for (unsigned w = threadIdx.x; w < sizeof(DevStats) / 4; w += blockDim.x)
+    reinterpret_cast<volatile unsigned*>(mirror)[w] = reinterpret_cast<const volatile unsigned*>(st)[w];
 }
 
 __global__ void __launch_bounds__(SCAN_SMALL_THREADS) k_scan_small(ScanArgs a0, ScanArgs a1, long long m,
                                                                   const long long* __restrict__ prod, DevStats* st,
-                                                                  unsigned* reset) {
+                                                                  unsigned* reset, DevStats* mirror) {
   const ScanArgs a = blockIdx.y ? a1 : a0;
   if (no_window_rows(st, a.win_lo)) return;
   long long carry = 0, total;
@@ -92,7 +101,7 @@ __global__ void __launch_bounds__(SCAN_SMALL_THREADS) k_scan_small(ScanArgs a0, 
     }
     carry += total;
   }
-  if (threadIdx.x == 0) scan_finish(a, m, carry, st, blockIdx.y ? nullptr : reset);
+  scan_finish(a, m, carry, st, blockIdx.y ? nullptr : reset, blockIdx.y ? nullptr : mirror);
 }
 
 __global__ void __launch_bounds__(SCAN_THREADS) k_scan_reduce(ScanArgs a0, ScanArgs a1, long long m,
@@ -129,7 +138,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_partials(ScanArgs a0, Sca
 template <bool SCANNED>
 __global__ void __launch_bounds__(SCAN_THREADS) k_scan_down(ScanArgs a0, ScanArgs a1, long long m,
                                                            const long long* __restrict__ prod, DevStats* st,
-                                                           unsigned* reset) {
+                                                           unsigned* reset, DevStats* mirror) {
   __shared__ int s_tile[SCAN_TILE + SCAN_TILE / 16];  // one word of padding per thread's 16
   const ScanArgs a = blockIdx.y ? a1 : a0;
   if (no_window_rows(st, a.win_lo)) return;
@@ -168,25 +177,26 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_down(ScanArgs a0, ScanArg
     const int q = j * SCAN_THREADS + tid;
     if (base + q < m) a.rp[base + q] = s_tile[q + (q >> 4)];
   }
-  if (blockIdx.x == gridDim.x - 1 && tid == 0) scan_finish(a, m, before + total, st, blockIdx.y ? nullptr : reset);
+  if (blockIdx.x == gridDim.x - 1)
+    scan_finish(a, m, before + total, st, blockIdx.y ? nullptr : reset, blockIdx.y ? nullptr : mirror);
 }
 
 static cudaError_t scan_launch(const LaunchCtx& c, int sums, const ScanArgs& a0, const ScanArgs& a1, long long m,
-                               const long long* prod, unsigned* reset) {
+                               const long long* prod, unsigned* reset, DevStats* mirror) {
   const long long ntiles = (m + SCAN_TILE - 1) / SCAN_TILE;
   timer_mark(c, T_SCAN, 0);
   if (m <= SCAN_SMALL) {
-    k_scan_small<<<dim3(1, sums), SCAN_SMALL_THREADS, 0, c.stream>>>(a0, a1, m, prod, c.st, reset);
+    k_scan_small<<<dim3(1, sums), SCAN_SMALL_THREADS, 0, c.stream>>>(a0, a1, m, prod, c.st, reset, mirror);
     count_launch(c);
   } else {
     k_scan_reduce<<<dim3((unsigned)ntiles, sums), SCAN_THREADS, 0, c.stream>>>(a0, a1, m, prod, c.st);
     count_launch(c);
     if (ntiles <= SCAN_TWO) {
-      k_scan_down<false><<<dim3((unsigned)ntiles, sums), SCAN_THREADS, 0, c.stream>>>(a0, a1, m, prod, c.st, reset);
+      k_scan_down<false><<<dim3((unsigned)ntiles, sums), SCAN_THREADS, 0, c.stream>>>(a0, a1, m, prod, c.st, reset, mirror);
     } else {
       k_scan_partials<<<dim3(1, sums), SCAN_THREADS, 0, c.stream>>>(a0, a1, ntiles, c.st);
       count_launch(c);
-      k_scan_down<true><<<dim3((unsigned)ntiles, sums), SCAN_THREADS, 0, c.stream>>>(a0, a1, m, prod, c.st, reset);
+      k_scan_down<true><<<dim3((unsigned)ntiles, sums), SCAN_THREADS, 0, c.stream>>>(a0, a1, m, prod, c.st, reset, mirror);
     }
     count_launch(c);
   }
@@ -195,16 +205,16 @@ static cudaError_t scan_launch(const LaunchCtx& c, int sums, const ScanArgs& a0,
 }
 
 cudaError_t launch_scan(const LaunchCtx& c, int32_t* c_rp, long long m, long long* part, long long* total_out,
-                        const long long* prod, unsigned* reset) {
+                        const long long* prod, unsigned* reset, DevStats* mirror) {
   const ScanArgs a{c_rp, part, total_out ? total_out : &c.st->nnz_c, 0};
-  return scan_launch(c, 1, a, a, m, prod, reset);
+  return scan_launch(c, 1, a, a, m, prod, reset, mirror);
 }
 
 cudaError_t launch_scan_runs(const LaunchCtx& c, int32_t* rr, int32_t* rrb, long long m, long long* partials,
                              int win_lo) {
   const ScanArgs a{rr, partials, &c.st->nruns, win_lo};
   const ScanArgs b{rrb, partials + scan_partials_count(m), &c.st->nruns_b, win_lo};
-  return scan_launch(c, rrb ? 2 : 1, a, b, m, nullptr, nullptr);
+  return scan_launch(c, rrb ? 2 : 1, a, b, m, nullptr, nullptr, nullptr);
 }
 
 }  // namespace sg
