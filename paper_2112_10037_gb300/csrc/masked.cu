@@ -6,10 +6,11 @@
 // order of Sec. 2.2 (A's entries of the row, each with its row of B) and
 // keeps only the products whose column lies in M's row.
 //
-// Work is cut into units of 32 consecutive nonzeros of A (so rows of any
-// length spread over many warps and the dense core of a power-law graph
-// does not hold one warp for long).  A warp finds the row of its unit's first
-// nonzero by a 32-way search over A's row pointer, the others follow from it.
+// Rows of A with at least 64 nonzeros, and a mask row of at most 4 columns for
+// each, go to blocks (k_masked_rows, below), the other rows to warps
+// (k_masked): their work is cut into units of 32 consecutive nonzeros of A.  A
+// warp finds the row of its unit's first nonzero by a 32-way search over A's
+// row pointer, the others follow from it.
 // A product whose column lies in its row of M adds its rounded value
 // A(i,k)*B(k,j) to that entry.
 //
@@ -36,20 +37,22 @@
 // no more columns than products).
 //
 // A block is one warp and takes one unit, so that the hardware's block
-// scheduler balances units of very different work.
+// scheduler balances units of very different work.  (Long rows on warps left
+// 40 % of the SM cycles idle: the warps of the longest row of a power-law graph
+// alone took two thirds of the kernel's time.)
 //
-// Strictly lower triangles of R-MAT graphs, a search of the mask row per
-// product and this: scale 16 (147 M products) 1.61 and 1.14 ms, scale 18
-// (1.1 G products) 10.0 and 5.4 ms; 70 % of the products are never formed.
-// What bounds it now is the latency of the searches' loads (1.3 of 4
-// instructions issued per clock with 20 warps on an SM).  The full pattern of
-// the 96^3 stencil's square as the mask stays at 0.82 ms (min-plus).
+// Strictly lower triangles of R-MAT graphs, with a search of the mask row per
+// product, with warps alone, and now: scale 16 (147 M products) 1.61, 1.15 and
+// 0.47 ms (blocks 0.31, warps 0.15), scale 18 (1.1 G products) 10.1, 5.6 and
+// 2.2 ms; 3000 rows, edge factor 8: 56, 50 and 49 us.  The full pattern of the
+// 96^3 stencil's square as the mask stays at 0.66 ms.
 //
 // The output is zeroed before and, with M's values, scaled by them after
 // (the sum is finished before the factor, as in the definition).
 #include <type_traits>
 
 #include "launch_util.cuh"
+#include "segstream.cuh"
 
 namespace sg {
 
@@ -59,6 +62,14 @@ constexpr int MASK_FILTER_MAX = 2048;     // longest mask row worth the bitmap (
 constexpr int MASK_MIN_PRODUCTS = 128;    // fewest products worth staging a row,
 constexpr int MASK_RATIO = 4;             // and per mask column,
 constexpr int MASK_UNIT_PRODUCTS = 512;   // in a unit of this many in all (a stencil's units have 224)
+constexpr int MASK_ROW_MIN = 64;          // nonzeros of a row that blocks take,
+constexpr int MASK_ROW_RATIO = 4;         // with at most this many mask columns each
+constexpr int MASK_BLOCK = 256;           // threads of such a block, most nonzeros of its unit
+constexpr int MASK_UNITS_PER_SM = 10;     // units below which they are made smaller
+constexpr int MASK_BLOCK_CAP = 1536;      // mask columns staged with accumulators per block
+constexpr int MASK_BLOCK_BITS = 65536;    // bits of its hashed bitmap
+constexpr int MASK_BLOCK_QUEUE = 160;     // products of a warp that passed it (fewer than 32 wait)
+constexpr int MASK_ROUND = 1 << 22;       // entries of one row of B in a block's list at a time
 constexpr int MASK_QUEUE = 64;            // products that passed the bitmap (fewer than 32 wait)
 
 // Largest r with rp[r] <= e (the row holding position e) over rows [0, m),
@@ -162,6 +173,11 @@ __device__ __forceinline__ void sr_reduce_global(T* p, T v) {
   else *p = T(1);
 }
 
+// Rows that k_masked_rows takes whole; k_masked leaves them out.
+__device__ __forceinline__ bool mask_row_blocked(int la, int n) {
+  return la >= MASK_ROW_MIN && n > 0 && (n + MASK_ROW_RATIO - 1) / MASK_ROW_RATIO <= la;
+}
+
 // Shared memory of one warp.
 template <typename T>
 struct MaskWarp {
@@ -201,7 +217,7 @@ k_masked(Csr A, Csr B, Csr M, const T* __restrict__ av, const T* __restrict__ bv
     T a = T(0);
     if (ve) {
       i = row_from(A.rp, (int)A.nrows, i, e);
-      const int k = A.ci[e];
+      const int k = mask_row_blocked(A.rp[i + 1] - A.rp[i], M.rp[i + 1] - M.rp[i]) ? -1 : A.ci[e];
       if (k >= 0 && (long long)k < B.nrows) {  // a column of A out of range names no row of B
         sb = B.rp[k];
         len = B.rp[k + 1] - sb;
@@ -356,6 +372,203 @@ k_masked(Csr A, Csr B, Csr M, const T* __restrict__ av, const T* __restrict__ bv
   }
 }
 
+// Shared memory of a block of k_masked_rows.
+template <typename T>
+struct MaskBlock {
+  // up to MASK_BLOCK_CAP accumulators and columns, or COLS columns alone
+  static constexpr int COLS = MASK_BLOCK_CAP * (int)(sizeof(T) + sizeof(int)) / (int)sizeof(int);
+  union {
+    struct {
+      T acc[MASK_BLOCK_CAP];
+      int col[MASK_BLOCK_CAP];
+    };
+    int only_col[COLS];
+  };
+  T seg_a[MASK_BLOCK];                                // the list: multiplier,
+  unsigned long long pack;                            // (segments << 32) | products,
+  int seg_off[MASK_BLOCK], seg_s[MASK_BLOCK];         // stream offset, start in B
+  int2 queue[MASK_BLOCK / 32][MASK_BLOCK_QUEUE];            // per warp: (entry of B, segment)
+  int row[MASK_BLOCK];                                // row of each nonzero
+  int part[MASK_BLOCK / MASK_ROW_MIN + 4], parts;     // first nonzeros of the rows to take
+  uint32_t bits[MASK_BLOCK_BITS / 32];
+};
+
+// Long rows: a block takes a unit of up to 256 consecutive nonzeros of A and
+// one after the other the rows in it that mask_row_blocked names (the other
+// parts of such a row are other blocks'; their sums meet in the output).  The
+// mask row's columns set bits of a hashed bitmap (the low 16 bits) and are
+// listed in shared memory with an accumulator each (up to 1536 columns; up to
+// 4608, 3072 in FP32, without accumulators; in global memory beyond).  The
+// products of the part are one stream, cut into equal shares for the warps
+// (segstream.cuh): rows of B of hundreds of entries and of one weigh the same.
+// A product costs its column, one test of the bitmap and a ballot; those that
+// pass wait in the warp's queue and are looked up 32 at a time, because an FP64
+// product and its addition cost a warp the same with one lane as with all.
+//
+// What bounds it: the latency of a batch's loads in a warp (four batches in
+// flight) in units of hundreds of thousands of products, and about 30
+// instructions a batch elsewhere.  R-MAT scale 16: 0.31 ms; 0.35 with a queue
+// check after each batch or with 2048 columns (four blocks on an SM instead of
+// five), 0.39 without the list for rows beyond the accumulators, 0.35 and 0.41
+// with 512 and 128 threads, and no less with the next four loads issued before
+// the tests.  Rows from 32 and from 128 nonzeros on: 2 % slower and 5 %.
+template <typename T, int SR>
+__global__ void __launch_bounds__(MASK_BLOCK, 5)
+k_masked_rows(Csr A, Csr B, Csr M, const T* __restrict__ av, const T* __restrict__ bv, T* __restrict__ out,
+              int unit) {
+  constexpr int NT = MASK_BLOCK;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  MaskBlock<T>& sm = *reinterpret_cast<MaskBlock<T>*>(smem_raw);
+  const int tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
+  const unsigned lt = lanemask_lt();
+  const int u0 = (int)(unit * (long long)blockIdx.x), u1 = (int)min(A.nnz - u0, (long long)unit);  // u0 + [0, u1)
+  // ---- rows of the unit's nonzeros, and the parts to take
+  int row = -1, sb = 0, len = 0;
+  bool take = false;
+  if (warp * 32 < u1) {
+    row = warp_row_of(A.rp, (int)A.nrows, u0 + warp * 32);
+    if (tid < u1) {
+      row = row_from(A.rp, (int)A.nrows, row, u0 + tid);
+      take = mask_row_blocked(A.rp[row + 1] - A.rp[row], M.rp[row + 1] - M.rp[row]);
+    }
+  }
+  sm.row[tid] = row;
+  if (tid == 0) {
+    sm.parts = 0;
+    sm.pack = 0ull;
+  }
+  if (!__syncthreads_or(take)) return;
+  if (take && (tid == 0 || sm.row[tid - 1] != row)) {  // (rows of at least MASK_ROW_MIN nonzeros: a few parts)
+    const int x = atomicAdd(&sm.parts, 1);
+    if (x < MASK_BLOCK / MASK_ROW_MIN + 4) sm.part[x] = tid;
+  }
+  T a = T(0);
+  if (take) {
+    const int k = A.ci[u0 + tid];
+    if (k >= 0 && (long long)k < B.nrows) {  // a column of A out of range names no row of B
+      sb = B.rp[k];
+      len = max(B.rp[k + 1] - sb, 0);
+      a = av[u0 + tid];
+    }
+  }
+  for (int t = tid; t < MASK_BLOCK_BITS / 32; t += NT) sm.bits[t] = 0u;
+  __syncthreads();
+  const int parts = min(sm.parts, MASK_BLOCK / MASK_ROW_MIN + 4);
+  int2* const queue = sm.queue[warp];
+  for (int x = 0; x < parts; ++x) {
+    const int i = sm.row[sm.part[x]];
+    const int m0 = M.rp[i], n = M.rp[i + 1] - m0;
+    const bool staged = n <= MASK_BLOCK_CAP;  // accumulators; products go to the output otherwise
+    const bool listed = n <= MaskBlock<T>::COLS;
+    int* const cols = staged ? sm.col : sm.only_col;
+    for (int t = tid; t < n; t += NT) {
+      const int c = M.ci[m0 + t];
+      atomicOr(&sm.bits[(c >> 5) & (MASK_BLOCK_BITS / 32 - 1)], 1u << (c & 31));
+      if (listed) cols[t] = c;
+      if (staged) sm.acc[t] = sr_zero<SR, T>();
+    }
+    int rest = take && row == i ? len : 0;
+    do {  // one round, but for rows of B of millions of entries
+      const int now = min(rest, MASK_ROUND);
+      seg_append<T>(&sm.pack, sb, now, a, sm.seg_off, sm.seg_s, sm.seg_a);
+      rest -= now;
+      sb += now;
+      __syncthreads();  // the list and the mask are complete
+      const int nseg = (int)(sm.pack >> 32), tot = (int)(unsigned)(sm.pack & 0xffffffffull);
+      const int share = ((tot + NT - 1) / NT) * 32;
+      const int lo = warp * share, hi = min(tot, lo + share);
+      int qn = 0;  // waiting products
+      auto look_up = [&](int cnt) {  // the last cnt (at most 32) of the queue
+        if (lane < cnt) {
+          const int2 w = queue[qn - cnt + lane];
+          const int j = B.ci[w.x];
+          const T b = bv[w.x];
+          const int p = listed ? find_in(cols, 0, n, j) : find_in(M.ci + m0, 0, n, j);
+          if (p >= 0) {
+            const T x = sr_product<SR>(sm.seg_a[w.y], b);
+            if (staged) sr_reduce_shared<SR>(&sm.acc[p], x);
+            else sr_reduce_global<SR>(&out[m0 + p], x);
+          }
+        }
+        qn -= cnt;
+        __syncwarp();  // the entries are read before later ones overwrite them
+      };
+      auto offer = [&](int j, int bi, int k, bool act) {
+        const bool pass = act && (sm.bits[(j >> 5) & (MASK_BLOCK_BITS / 32 - 1)] >> (j & 31) & 1u);
+        const unsigned b = __ballot_sync(FULL, pass);
+        if (!b) return;
+        if (pass) queue[qn + __popc(b & lt)] = make_int2(bi, k);
+        qn += __popc(b);
+        __syncwarp();
+        if (qn >= 32) look_up(32);
+      };
+      if (lo < hi) {
+        int f = seg_find(sm.seg_off, nseg, lo);
+        int p = lo;
+        while (p < hi) {
+          const int so = sm.seg_off[f];
+          const int se = f + 1 < nseg ? sm.seg_off[f + 1] : tot;
+          const int run = min(se, hi) - p;
+          if (run >= 32) {  // whole batches inside segment f, four loads in flight
+            const int nw = run & ~31;
+            const int q = sm.seg_s[f] + (p - so) + lane;
+            const int* __restrict__ ci = B.ci + q;
+            int t = 0;
+            for (; t + 96 < nw; t += 128) {
+              const int j[4] = {ci[t], ci[t + 32], ci[t + 64], ci[t + 96]};
+              bool pass[4];
+              unsigned b[4];
+#pragma unroll
+              for (int v = 0; v < 4; ++v) {
+                pass[v] = sm.bits[(j[v] >> 5) & (MASK_BLOCK_BITS / 32 - 1)] >> (j[v] & 31) & 1u;
+                b[v] = __ballot_sync(FULL, pass[v]);
+              }
+              if (!(b[0] | b[1] | b[2] | b[3])) continue;
+#pragma unroll
+              for (int v = 0; v < 4; ++v) {
+                if (pass[v]) queue[qn + __popc(b[v] & lt)] = make_int2(q + t + 32 * v, f);
+                qn += __popc(b[v]);
+              }
+              __syncwarp();
+              while (qn >= 32) look_up(32);
+            }
+            for (; t < nw; t += 32) offer(ci[t], q + t, f, true);
+            p += nw;
+            if (p == se) ++f;
+            continue;
+          }
+          // one batch across segments: lane j holds the end of segment f + j
+          const int nx = f + lane + 1;
+          const int end = nx < nseg ? sm.seg_off[nx] : (nx == nseg ? tot : INT_MAX);
+          const int d = end == INT_MAX ? INT_MAX : end - p;
+          const unsigned m = __reduce_or_sync(FULL, d <= 31 ? (1u << d) : 0u);
+          const int k = f + __popc(m & (lane == 31 ? FULL : ((2u << lane) - 1u)));
+          const int q = p + lane;
+          const bool act = q < hi;
+          const int bi = act ? sm.seg_s[k] + (q - sm.seg_off[k]) : 0;
+          offer(act ? B.ci[bi] : 0, bi, k, act);
+          const int pn = p + 32;
+          if (pn < hi) {  // segment of the next product
+            const int c = __popc(__ballot_sync(FULL, end <= pn));
+            f = c < 32 ? f + c : seg_find(sm.seg_off, nseg, pn);
+          }
+          p = pn;
+        }
+        if (qn > 0) look_up(qn);
+      }
+      __syncthreads();  // all products in; the list may be refilled
+      if (tid == 0) sm.pack = 0ull;
+    } while (__syncthreads_or(rest > 0));
+    // (the barrier above: every accumulator is final)
+    for (int t = tid; t < n; t += NT) {
+      const int c = listed ? cols[t] : M.ci[m0 + t];
+      sm.bits[(c >> 5) & (MASK_BLOCK_BITS / 32 - 1)] = 0u;
+      if (staged) sr_reduce_global<SR>(&out[m0 + t], sm.acc[t]);
+    }
+    __syncthreads();  // the next row's columns and bits come after
+  }
+}
+
 // out[p] *= mv[p] for the nnz(M) entries.
 template <typename T>
 __global__ void __launch_bounds__(256) k_scale(T* __restrict__ out, const T* __restrict__ mv, long long n) {
@@ -385,6 +598,15 @@ static cudaError_t masked_t(const LaunchCtx& c, const Csr& A, const Csr& B, cons
   }
   if (e != cudaSuccess || A.nnz <= 0) return e;
   auto k = k_masked<T, SR>;
+  auto kr = k_masked_rows<T, SR>;
+  if (kernel_blocks_per_sm(kr, MASK_BLOCK, sizeof(MaskBlock<T>)) <= 0) return cudaErrorInvalidConfiguration;
+  // smaller units where few would be left for the SMs: 3000 rows 68 -> 49 us
+  int unit = MASK_BLOCK;
+  while (unit > 32 && A.nnz < (long long)MASK_UNITS_PER_SM * c.nsm * unit) unit >>= 1;
+  kr<<<(unsigned)((A.nnz + unit - 1) / unit), MASK_BLOCK, sizeof(MaskBlock<T>), c.stream>>>(A, B, M, av, bv, out,
+                                                                                        unit);
+  count_launch(c);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   k<<<(unsigned)((A.nnz + 31) / 32), 32, 0, c.stream>>>(A, B, M, av, bv, out);
   count_launch(c);
   if ((e = cudaGetLastError()) != cudaSuccess || SR != 0 || !mv) return e;
