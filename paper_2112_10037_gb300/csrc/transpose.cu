@@ -13,7 +13,7 @@
 //     count of every digit value, stored digit-major (table[d*T + t]); the
 //     first pass also checks the column range,
 //  2. exclusive prefix sum of the table,
-//  3. scatter pass per digit: a block takes a tile; each warp ranks its 512
+//  3. scatter pass per digit: a block takes a tile; each warp ranks its 256
 //     consecutive entries among the equal digits of its earlier entries
 //     (lanes of equal digit found by one ballot per digit bit -- the warp
 //     match instruction takes 64 cycles of an SM, a ballot and its mask 1 --
@@ -33,7 +33,11 @@
 //     every column by atomics and a scan follows.)
 // R-MAT scale 20 (15.7 M entries, three passes, FP64 values): 1.05 ms with warp
 // matches, a row search per entry, column atomics and positions that nobody
-// reads; 0.68 ms now (a later pass moves 0.5 GB at 3.5 TB/s).
+// reads, 0.68 ms with ballots, row marks and tiles of 4096 entries, 0.63 ms now
+// (a later pass moves 0.5 GB at 3.8 TB/s).  A tile is a chain of phases with
+// barriers between them, so what bounds a pass is how many blocks an SM holds:
+// 4096 entries leave two (16 entries a lane, 122 registers), 2048 four; 3072
+// with three take 0.63 ms too but lose on small matrices, five blocks spill.
 // The source positions let a caller move new values of the same structure
 // (t_v[q] = v[t_src[q]]) without transposing again.
 #include "launch_util.cuh"
@@ -41,8 +45,8 @@
 namespace sg {
 
 constexpr int TR_WARPS = 8;                         // warps of a scatter block
-constexpr int TR_ITEMS = 16;                        // entries per lane and tile
-constexpr int TR_TILE = TR_WARPS * 32 * TR_ITEMS;   // 4096 entries per tile
+constexpr int TR_ITEMS = 8;                         // entries per lane and tile
+constexpr int TR_TILE = TR_WARPS * 32 * TR_ITEMS;   // 2048 entries per tile
 constexpr int TR_DIGIT = 9;                         // at most 512 digit values per pass
 constexpr int TR_HIST_THREADS = 256;
 static_assert(TR_WARPS * 32 >= (1 << TR_DIGIT) / 2, "two digits per thread at most");
@@ -190,7 +194,7 @@ __global__ void __launch_bounds__(256) k_tr_row_ptr(const int32_t* __restrict__ 
 // memory, so the global stores go out as runs of consecutive positions (one
 // run per digit value).
 template <bool FIRST, bool LAST, int VB, bool POS>
-__global__ void __launch_bounds__(TR_WARPS * 32) k_tr_scatter(const int32_t* __restrict__ rp, int m,
+__global__ void __launch_bounds__(TR_WARPS * 32, 4) k_tr_scatter(const int32_t* __restrict__ rp, int m,
                                                               const int32_t* __restrict__ kin,
                                                               const int32_t* __restrict__ rin,
                                                               const int32_t* __restrict__ pin,
