@@ -231,8 +231,13 @@ Layout layout_for(const spgemm_opts& o, long long mloc, long long nnz_a, long lo
   L.hcnt = off; off = align_up(off + sizeof(int32_t) * nh);
   L.rrb = L.runsb = 0;
   if (own_b && numeric_block_bin(o, ncols_b) < sg::NBINS) {  // run list at the block window's width
-    L.rrb = off; off = align_up(off + sizeof(int32_t) * (size_t)(nrows_b + 1));
-    L.runsb = off; off = align_up(off + sizeof(int2) * (size_t)(nnz_b + nrows_b + sg::RUNS_PAD));
+    if (default_long_rows(o)) {  // no row takes the warp window: one list, the block window's
+      L.rrb = L.rr;
+      L.runsb = L.runs;
+    } else {
+      L.rrb = off; off = align_up(off + sizeof(int32_t) * (size_t)(nrows_b + 1));
+      L.runsb = off; off = align_up(off + sizeof(int2) * (size_t)(nnz_b + nrows_b + sg::RUNS_PAD));
+    }
   }
   if (o.backward) {
     L.at_rp = off; off = align_up(off + sizeof(int32_t) * (size_t)(nrows_b + 1));
@@ -527,7 +532,13 @@ static spgemm_status analyse_impl(const spgemm_csr* A, const spgemm_csr* B, cons
     if (block_lo < win_lo || p->tu.num_lo_band < sg::NBINS) win_lo = block_lo;  // (bands need no lists)
     const bool never = win_lo >= sg::NBINS && p->tu.num_lo_band < sg::NBINS;
     if (rb != 0 || re != A->nrows) win_lo = 0;
-    if (!never) e = sg::launch_runs(c, p->B, p->sp, p->runs_part, win_lo);
+    sg::SplitInfo lists = p->sp;
+    if (default_long_rows(o)) {  // (see layout_for)
+      lists.wf_shift = lists.wb_shift;
+      lists.rrb = nullptr;
+      lists.runsb = nullptr;
+    }
+    if (!never) e = sg::launch_runs(c, p->B, lists, p->runs_part, win_lo);
   }
   if (e == cudaSuccess && o.backward) {
     p->at_rp = (int32_t*)(p->ws + L.at_rp);
