@@ -76,7 +76,7 @@ struct Layout {
 // `off`; returns the end offset.
 size_t transpose_layout(size_t off, long long n, long long nnz, int vbytes, size_t* tmp, size_t* table,
                         size_t* part) {
-  const sg::TransposeScratch s = sg::transpose_scratch(n, nnz, vbytes);
+  const sg::TransposeScratch s = sg::transpose_scratch(n, nnz, vbytes, sg::transpose_items(n));
   *tmp = off; off = align_up(off + sizeof(int32_t) * s.tmp_ints);
   *table = off; off = align_up(off + sizeof(int32_t) * s.table_ints);
   *part = off; off = align_up(off + sizeof(long long) * s.part_count);
@@ -546,7 +546,8 @@ static spgemm_status analyse_impl(const spgemm_csr* A, const spgemm_csr* B, cons
     p->at_src = (int32_t*)(p->ws + L.at_src);
     e = sg::launch_transpose(c, A->nrows, A->ncols, A->nnz, A->row_ptr, A->col_idx, p->at_rp, p->at_ci, p->at_src,
                              0, nullptr, nullptr, (int32_t*)(p->ws + L.at_tmp), (int32_t*)(p->ws + L.at_table),
-                             (long long*)(p->ws + L.at_part), (int32_t*)(p->ws + L.a_row) /* filled below */);
+                             (long long*)(p->ws + L.at_part), (int32_t*)(p->ws + L.a_row) /* filled below */,
+                             sg::transpose_items(A->ncols));
     p->a_row = (int32_t*)(p->ws + L.a_row);
     p->b_row = (int32_t*)(p->ws + L.b_row);
     if (e == cudaSuccess) e = sg::launch_row_index(c, A->row_ptr, A->nrows, p->a_row);
@@ -854,7 +855,7 @@ spgemm_status spgemm_transpose(const spgemm_csr* M, int32_t dtype, int32_t* t_ro
   if (e == cudaSuccess)
     e = sg::launch_transpose(c, M->nrows, M->ncols, M->nnz, M->row_ptr, M->col_idx, t_row_ptr, t_col_idx, t_src,
                              vbytes, M->vals, t_vals, (int32_t*)(ws + tmp), (int32_t*)(ws + table),
-                             (long long*)(ws + part), sorted);
+                             (long long*)(ws + part), sorted, sg::transpose_items(M->ncols));
   return e == cudaSuccess ? SPGEMM_OK : SPGEMM_ERR_CUDA;
 }
 

@@ -337,14 +337,16 @@ SG_NUMERIC_SR_DECL(launch_numeric_or_and);
 struct TransposeScratch {
   size_t tmp_ints, table_ints, part_count;
 };
-TransposeScratch transpose_scratch(long long n, long long nnz, int vbytes);
+TransposeScratch transpose_scratch(long long n, long long nnz, int vbytes, int items);
+// Entries per lane and tile for a matrix with n columns: 8 or 16.
+int transpose_items(long long n);
 // M^T: t_rp (n+1), t_ci and, unless null, t_src (nnz), and with vbytes 4 or 8
 // and both value pointers, t_vals[q] = vals[t_src[q]].  sorted: scratch of nnz
 // integers for the sorted columns, or null (slower).
 cudaError_t launch_transpose(const LaunchCtx& c, long long m, long long n, long long nnz, const int32_t* rp,
                              const int32_t* ci, int32_t* t_rp, int32_t* t_ci, int32_t* t_src, int vbytes,
                              const void* vals, void* t_vals, int32_t* tmp, int32_t* table, long long* partials,
-                             int32_t* sorted);
+                             int32_t* sorted, int items);
 // Masked product on M's pattern over a semiring (spgemm_semiring; 0 is
 // C<M> = (A*B) .* M, mv null for the pattern only; mv is unused otherwise).
 cudaError_t launch_masked(const LaunchCtx& c, int dtype, int semiring, const Csr& A, const Csr& B, const Csr& M,

@@ -37,9 +37,12 @@ struct NaLayout {
 
 // The sorted columns get scratch only when the caller passes no t_src (what
 // fits the fixed array does not depend on how the row pointer is found);
-// values (vbytes each, 0 without t_vals) travel through the scratch.
+// values (vbytes each, 0 without t_vals) travel through the scratch.  Tiles are
+// the large ones at every size: the digit table of the small ones is twice as
+// large and would turn away inputs that fit.
+constexpr int NA_ITEMS = 16;
 NaLayout na_layout(long long ncols, long long nnz, bool need_src, int vbytes) {
-  const TransposeScratch s = transpose_scratch(ncols, nnz, vbytes);
+  const TransposeScratch s = transpose_scratch(ncols, nnz, vbytes, NA_ITEMS);
   NaLayout L{};
   size_t off = 0;
   L.st = off; off = na_align(off + sizeof(DevStats));
@@ -110,6 +113,6 @@ extern "C" spgemm_status spgemm_transpose_noalloc(const spgemm_csr* M, int32_t d
   if (e == cudaSuccess)
     e = launch_transpose(c, M->nrows, M->ncols, M->nnz, M->row_ptr, M->col_idx, t_row_ptr, t_col_idx, t_src,
                          vbytes, M->vals, t_vals, (int32_t*)(ws + L.tmp), (int32_t*)(ws + L.table),
-                         (long long*)(ws + L.part), sorted);
+                         (long long*)(ws + L.part), sorted, NA_ITEMS);
   return e == cudaSuccess ? SPGEMM_OK : SPGEMM_ERR_CUDA;
 }

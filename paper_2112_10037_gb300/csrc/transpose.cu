@@ -9,18 +9,17 @@
 // every pass a stable counting scatter.  No output row is sorted afterwards
 // and no source position is searched for, whatever the column lengths.
 //
-//  1. histogram pass per digit: per tile of TR_TILE consecutive entries the
+//  1. histogram pass per digit: per tile of 2048 or 4096 consecutive entries the
 //     count of every digit value, stored digit-major (table[d*T + t]); the
 //     first pass also checks the column range,
 //  2. exclusive prefix sum of the table,
-//  3. scatter pass per digit: a block takes a tile; each warp ranks its 256
+//  3. scatter pass per digit: a block takes a tile; each warp ranks its
 //     consecutive entries among the equal digits of its earlier entries
 //     (lanes of equal digit found by one ballot per digit bit -- the warp
 //     match instruction takes 64 cycles of an SM, a ballot and its mask 1 --
 //     and one running count per digit and warp in shared memory), the block
-//     turns the
-//     per-warp counts into offsets, reorders the tile by digit in shared
-//     memory and writes every digit's entries as one run from its table
+//     turns the per-warp counts into offsets, reorders the tile by digit in
+//     shared memory and writes every digit's entries as one run from its table
 //     offset.  The first pass reads M itself (source row by a search over
 //     the row pointer, source position = entry index); the last writes the
 //     source row (M^T's column index), the source position and the sorted
@@ -45,8 +44,6 @@
 namespace sg {
 
 constexpr int TR_WARPS = 8;                         // warps of a scatter block
-constexpr int TR_ITEMS = 8;                         // entries per lane and tile
-constexpr int TR_TILE = TR_WARPS * 32 * TR_ITEMS;   // 2048 entries per tile
 constexpr int TR_DIGIT = 9;                         // at most 512 digit values per pass
 constexpr int TR_HIST_THREADS = 256;
 static_assert(TR_WARPS * 32 >= (1 << TR_DIGIT) / 2, "two digits per thread at most");
@@ -75,8 +72,18 @@ static TrPasses tr_passes(long long n) {
   return p;
 }
 
-TransposeScratch transpose_scratch(long long n, long long nnz, int vbytes) {
+// Entries of a tile with `items` entries per lane: 2048 or 4096.
+static constexpr int tr_tile(int items) { return TR_WARPS * 32 * items; }
+
+// With digits of at most 7 bits a tile of 2048 entries still leaves as runs of
+// 16 and more, and four blocks share an SM; with 8 and 9 bits the runs fall
+// below a 32-byte sector of columns (164 M entries with positions, 65,536
+// columns: 6.6 ms, 5.0 with 4096).
+int transpose_items(long long n) { return tr_passes(n).bits[0] <= 7 ? 8 : 16; }
+
+TransposeScratch transpose_scratch(long long n, long long nnz, int vbytes, int items) {
   TransposeScratch s{};
+  const int TR_TILE = tr_tile(items);
   const TrPasses p = tr_passes(n);
   const long long tiles = (nnz + TR_TILE - 1) / TR_TILE;
   // pass outputs: X = (values, key, source row, source position) feeds the
@@ -94,19 +101,20 @@ __device__ __forceinline__ int tr_digit(int32_t key, int shift, int bits) {
   return (int)(((uint32_t)key >> shift) & ((1u << bits) - 1u));
 }
 
-// Digit counts of every tile; check: the columns' range; with cnt, also the
+// Digit counts of every `tile` entries; check: the columns' range; with cnt, also the
 // entries of every column.
 __global__ void __launch_bounds__(TR_HIST_THREADS) k_tr_hist(const int32_t* __restrict__ key, long long nnz,
                                                              int shift, int bits, long long tiles,
                                                              int32_t* __restrict__ table, bool check,
-                                                             int32_t* __restrict__ cnt, long long n, uint32_t* err) {
+                                                             int32_t* __restrict__ cnt, long long n, int tile,
+                                                             uint32_t* err) {
   __shared__ int h[1 << TR_DIGIT];
   const int nb = 1 << bits;
   for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
     for (int d = threadIdx.x; d < nb; d += TR_HIST_THREADS) h[d] = 0;
     __syncthreads();
-    const long long e0 = t * TR_TILE;
-    const long long e1 = e0 + TR_TILE < nnz ? e0 + TR_TILE : nnz;
+    const long long e0 = t * tile;
+    const long long e1 = e0 + tile < nnz ? e0 + tile : nnz;
     for (long long e = e0 + threadIdx.x; e < e1; e += TR_HIST_THREADS) {
       const int32_t c = key[e];
       if (check) {
@@ -141,9 +149,9 @@ __device__ __forceinline__ int tr_warp_row(const int32_t* __restrict__ rp, int m
 template <int VB> struct TrVal { using type = unsigned int; };
 template <> struct TrVal<8> { using type = unsigned long long; };
 
-static size_t tr_scatter_smem(int bits, int vbytes, bool pos) {
+static size_t tr_scatter_smem(int bits, int vbytes, bool pos, int items) {
   return sizeof(int) * ((size_t)(TR_WARPS + 2) << bits) +
-         (sizeof(int) * (pos ? 3 : 2) + (size_t)vbytes) * (size_t)TR_TILE;
+         (sizeof(int) * (pos ? 3 : 2) + (size_t)vbytes) * (size_t)tr_tile(items);
 }
 
 // t_rp[k] = first position whose column is at least k, from the sorted columns
@@ -193,8 +201,8 @@ __global__ void __launch_bounds__(256) k_tr_row_ptr(const int32_t* __restrict__ 
 // The tile is first reordered by digit in shared
 // memory, so the global stores go out as runs of consecutive positions (one
 // run per digit value).
-template <bool FIRST, bool LAST, int VB, bool POS>
-__global__ void __launch_bounds__(TR_WARPS * 32, 4) k_tr_scatter(const int32_t* __restrict__ rp, int m,
+template <int TR_ITEMS, bool FIRST, bool LAST, int VB, bool POS>
+__global__ void __launch_bounds__(TR_WARPS * 32, TR_ITEMS == 8 ? 4 : 2) k_tr_scatter(const int32_t* __restrict__ rp, int m,
                                                               const int32_t* __restrict__ kin,
                                                               const int32_t* __restrict__ rin,
                                                               const int32_t* __restrict__ pin,
@@ -204,7 +212,7 @@ __global__ void __launch_bounds__(TR_WARPS * 32, 4) k_tr_scatter(const int32_t* 
                                                               int32_t* __restrict__ kout, int32_t* __restrict__ rout,
                                                               int32_t* __restrict__ pout, void* __restrict__ vout_) {
   using V = typename TrVal<VB>::type;
-  constexpr int NT = TR_WARPS * 32;
+  constexpr int NT = TR_WARPS * 32, TR_TILE = tr_tile(TR_ITEMS);
   const V* __restrict__ vin = (const V*)vin_;
   V* __restrict__ vout = (V*)vout_;
   extern __shared__ __align__(16) int tr_smem[];
@@ -382,14 +390,14 @@ static int grid_cap(long long units, int per_block, int nsm, int per_sm = 8) {
   return (int)(g < 1 ? 1 : g);
 }
 
-template <int VB, bool POS>
+template <int ITEMS, int VB, bool POS>
 static cudaError_t tr_scatter_launch(const LaunchCtx& c, bool first, bool last, const int32_t* rp, int m,
                                      const int32_t* kin, const int32_t* rin, const int32_t* pin, const void* vin,
                                      long long nnz, int shift, int bits, long long tiles, const int32_t* table,
                                      int32_t* ko, int32_t* ro, int32_t* po, void* vo) {
-  const size_t smem = tr_scatter_smem(bits, VB, POS);
-  auto k = first ? (last ? k_tr_scatter<true, true, VB, POS> : k_tr_scatter<true, false, VB, POS>)
-                 : (last ? k_tr_scatter<false, true, VB, POS> : k_tr_scatter<false, false, VB, POS>);
+  const size_t smem = tr_scatter_smem(bits, VB, POS, ITEMS);
+  auto k = first ? (last ? k_tr_scatter<ITEMS, true, true, VB, POS> : k_tr_scatter<ITEMS, true, false, VB, POS>)
+                 : (last ? k_tr_scatter<ITEMS, false, true, VB, POS> : k_tr_scatter<ITEMS, false, false, VB, POS>);
   const int per_sm = kernel_blocks_per_sm(k, TR_WARPS * 32, smem);
   if (per_sm <= 0) return cudaErrorInvalidConfiguration;
   k<<<grid_cap(tiles, 1, c.nsm, per_sm), TR_WARPS * 32, smem, c.stream>>>(rp, m, kin, rin, pin, vin, nnz, shift,
@@ -399,20 +407,19 @@ static cudaError_t tr_scatter_launch(const LaunchCtx& c, bool first, bool last, 
 }
 
 template <int VB>
-static cudaError_t tr_scatter_any(bool pos, const LaunchCtx& c, bool first, bool last, const int32_t* rp, int m,
-                                  const int32_t* kin, const int32_t* rin, const int32_t* pin, const void* vin,
+static cudaError_t tr_scatter_any(int items, bool pos, const LaunchCtx& c, bool first, bool last, const int32_t* rp,
+                                  int m, const int32_t* kin, const int32_t* rin, const int32_t* pin, const void* vin,
                                   long long nnz, int shift, int bits, long long tiles, const int32_t* table,
                                   int32_t* ko, int32_t* ro, int32_t* po, void* vo) {
-  return pos ? tr_scatter_launch<VB, true>(c, first, last, rp, m, kin, rin, pin, vin, nnz, shift, bits, tiles, table,
-                                           ko, ro, po, vo)
-             : tr_scatter_launch<VB, false>(c, first, last, rp, m, kin, rin, pin, vin, nnz, shift, bits, tiles, table,
-                                            ko, ro, po, vo);
+  auto* run = items == 8 ? (pos ? tr_scatter_launch<8, VB, true> : tr_scatter_launch<8, VB, false>)
+                         : (pos ? tr_scatter_launch<16, VB, true> : tr_scatter_launch<16, VB, false>);
+  return run(c, first, last, rp, m, kin, rin, pin, vin, nnz, shift, bits, tiles, table, ko, ro, po, vo);
 }
 
 cudaError_t launch_transpose(const LaunchCtx& c, long long m, long long n, long long nnz, const int32_t* rp,
                              const int32_t* ci, int32_t* t_rp, int32_t* t_ci, int32_t* t_src, int vbytes,
                              const void* vals, void* t_vals, int32_t* tmp, int32_t* table, long long* partials,
-                             int32_t* sorted) {
+                             int32_t* sorted, int items) {
   cudaError_t e = cudaSuccess;
   // row pointer from the sorted columns, unless empty columns prevail
   if (n > 4 * nnz || m <= 0 || n <= 0) sorted = nullptr;
@@ -422,10 +429,11 @@ cudaError_t launch_transpose(const LaunchCtx& c, long long m, long long n, long 
   if (vbytes != 0 && vbytes != 4 && vbytes != 8) return cudaErrorInvalidValue;
   if (!t_vals || !vals) vbytes = 0;
   const TrPasses ps = tr_passes(n);
-  const long long tiles = (nnz + TR_TILE - 1) / TR_TILE;
+  const int tile = tr_tile(items);
+  const long long tiles = (nnz + tile - 1) / tile;
   if (n <= 0) {  // no column exists: every entry is out of range (reported), M^T is empty
     k_tr_hist<<<grid_cap(tiles, 1, c.nsm, 8), TR_HIST_THREADS, 0, c.stream>>>(ci, nnz, 0, 1, tiles, table, true, t_rp,
-                                                                             n, c.err);
+                                                                             n, tile, c.err);
     count_launch(c);
     return launch_scan(c, t_rp, n, partials, &c.st->scratch_total);
   }
@@ -439,7 +447,7 @@ cudaError_t launch_transpose(const LaunchCtx& c, long long m, long long n, long 
   for (int i = 0; i < ps.passes; ++i) {
     const bool first = i == 0, last = i == ps.passes - 1;
     k_tr_hist<<<grid_cap(tiles, 1, c.nsm, 8), TR_HIST_THREADS, 0, c.stream>>>(
-        kin, nnz, ps.shift[i], ps.bits[i], tiles, table, first, first && !sorted ? t_rp : nullptr, n, c.err);
+        kin, nnz, ps.shift[i], ps.bits[i], tiles, table, first, first && !sorted ? t_rp : nullptr, n, tile, c.err);
     count_launch(c);
     if (first && !sorted && (e = launch_scan(c, t_rp, n, partials, &c.st->scratch_total)) != cudaSuccess) return e;
     if ((e = launch_scan(c, table, tiles << ps.bits[i], partials, &c.st->scratch_total)) != cudaSuccess) return e;
@@ -454,13 +462,13 @@ cudaError_t launch_transpose(const LaunchCtx& c, long long m, long long n, long 
     }
     const int mm = (int)m;
     if (vbytes == 8)
-      e = tr_scatter_any<8>(t_src != nullptr, c, first, last, rp, mm, kin, rin, pin, vin, nnz, ps.shift[i], ps.bits[i], tiles,
+      e = tr_scatter_any<8>(items, t_src != nullptr, c, first, last, rp, mm, kin, rin, pin, vin, nnz, ps.shift[i], ps.bits[i], tiles,
                                table, ko, ro, po, vo);
     else if (vbytes == 4)
-      e = tr_scatter_any<4>(t_src != nullptr, c, first, last, rp, mm, kin, rin, pin, vin, nnz, ps.shift[i], ps.bits[i], tiles,
+      e = tr_scatter_any<4>(items, t_src != nullptr, c, first, last, rp, mm, kin, rin, pin, vin, nnz, ps.shift[i], ps.bits[i], tiles,
                                table, ko, ro, po, vo);
     else
-      e = tr_scatter_any<0>(t_src != nullptr, c, first, last, rp, mm, kin, rin, pin, nullptr, nnz, ps.shift[i], ps.bits[i], tiles,
+      e = tr_scatter_any<0>(items, t_src != nullptr, c, first, last, rp, mm, kin, rin, pin, nullptr, nnz, ps.shift[i], ps.bits[i], tiles,
                                table, ko, ro, po, nullptr);
     if (e != cudaSuccess) return e;
     kin = ko; rin = ro; pin = po; vin = vo;

@@ -1,0 +1,43 @@
+"""GPU transpose where its tiles end: matrices whose digits take tiles of 2048
+and of 4096 entries, with entry counts just below, at and above one and several
+tiles, with and without source positions."""
+import numpy as np
+import pytest
+
+from paper_2112_10037_gb300 import gen
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def api():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2112_10037_gb300 import build
+    build.build()
+    from paper_2112_10037_gb300 import api as a
+    return a
+
+
+# columns: 7 bits in one pass, 2 x 5, 2 x 7 (small tiles); 9, 2 x 8, 2 x 9 (large)
+@pytest.mark.parametrize("ncols", [128, 600, 16384, 512, 65536, 262144])
+@pytest.mark.parametrize("nnz", [2047, 2048, 2049, 4095, 4096, 4097, 20481])
+def test_tile_edges(api, ncols, nnz):
+    rng = np.random.default_rng(nnz)
+    nrows = 400
+    lens = np.full(nrows, nnz // nrows)
+    lens[: nnz - lens.sum()] += 1
+    M = gen.random_rows(nrows, ncols, lens, rng, values="int")
+    dM = api.DeviceCSR.from_host(M)
+    order = np.argsort(M.col_idx, kind="stable")
+    rows = np.repeat(np.arange(nrows), np.diff(M.row_ptr))[order]
+    rp = np.concatenate([[0], np.cumsum(np.bincount(M.col_idx, minlength=ncols))])
+    for want_src in (False, True):
+        got = api.transpose(dM, want_src=want_src)
+        T, src = got if want_src else (got, None)
+        assert np.array_equal(T.row_ptr.cpu().numpy(), rp)
+        assert np.array_equal(T.col_idx.cpu().numpy(), rows)
+        assert np.array_equal(T.vals.cpu().numpy(), M.vals[order])
+        if want_src:
+            assert np.array_equal(src.cpu().numpy(), order)
