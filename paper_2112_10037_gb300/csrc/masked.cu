@@ -44,8 +44,10 @@
 // Strictly lower triangles of R-MAT graphs, with a search of the mask row per
 // product, with warps alone, and now: scale 16 (147 M products) 1.61, 1.15 and
 // 0.47 ms (blocks 0.31, warps 0.15), scale 18 (1.1 G products) 10.1, 5.6 and
-// 2.2 ms; 3000 rows, edge factor 8: 56, 50 and 49 us.  The full pattern of the
-// 96^3 stencil's square as the mask stays at 0.66 ms.
+// 2.2 ms; 3000 rows, edge factor 8: 56, 50 and 49 us.  The full pattern of a
+// square as the mask, where nearly every product hits: 96^3 stencil 0.54 ms with
+// a search per product and 0.57 now (min-plus 0.98 and 0.94), R-MAT scale 15
+// 5.8 and 5.3 ms (min-plus 8.0 and 8.1).
 //
 // The output is zeroed before and, with M's values, scaled by them after
 // (the sum is finished before the factor, as in the definition).
@@ -205,7 +207,7 @@ __device__ __forceinline__ bool mask_search_pays(int n, int len) {
 
 template <typename T, int SR>
 __global__ void __launch_bounds__(32, 32)
-k_masked(Csr A, Csr B, Csr M, const T* __restrict__ av, const T* __restrict__ bv, T* __restrict__ out) {
+k_masked(Csr A, Csr B, Csr M, const T* __restrict__ av, const T* __restrict__ bv, T* __restrict__ out, bool blocks) {
   __shared__ MaskWarp<T> sm;
   const int lane = lane_id();
   const unsigned lt = lanemask_lt();
@@ -217,7 +219,7 @@ k_masked(Csr A, Csr B, Csr M, const T* __restrict__ av, const T* __restrict__ bv
     T a = T(0);
     if (ve) {
       i = row_from(A.rp, (int)A.nrows, i, e);
-      const int k = mask_row_blocked(A.rp[i + 1] - A.rp[i], M.rp[i + 1] - M.rp[i]) ? -1 : A.ci[e];
+      const int k = blocks && mask_row_blocked(A.rp[i + 1] - A.rp[i], M.rp[i + 1] - M.rp[i]) ? -1 : A.ci[e];
       if (k >= 0 && (long long)k < B.nrows) {  // a column of A out of range names no row of B
         sb = B.rp[k];
         len = B.rp[k + 1] - sb;
@@ -598,16 +600,22 @@ static cudaError_t masked_t(const LaunchCtx& c, const Csr& A, const Csr& B, cons
   }
   if (e != cudaSuccess || A.nnz <= 0) return e;
   auto k = k_masked<T, SR>;
-  auto kr = k_masked_rows<T, SR>;
-  if (kernel_blocks_per_sm(kr, MASK_BLOCK, sizeof(MaskBlock<T>)) <= 0) return cudaErrorInvalidConfiguration;
-  // smaller units where few would be left for the SMs: 3000 rows 68 -> 49 us
-  int unit = MASK_BLOCK;
-  while (unit > 32 && A.nnz < (long long)MASK_UNITS_PER_SM * c.nsm * unit) unit >>= 1;
-  kr<<<(unsigned)((A.nnz + unit - 1) / unit), MASK_BLOCK, sizeof(MaskBlock<T>), c.stream>>>(A, B, M, av, bv, out,
-                                                                                        unit);
-  count_launch(c);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  k<<<(unsigned)((A.nnz + 31) / 32), 32, 0, c.stream>>>(A, B, M, av, bv, out);
+  // A mask with more than twice A's entries has few rows that blocks take: its
+  // long rows stay with the warps, and looking for such rows is saved (the 96^3
+  // stencil with its square's pattern, min-plus: 1.04 -> 0.94 ms).
+  const bool long_rows = M.nnz <= 2 * A.nnz;
+  if (long_rows) {
+    auto kr = k_masked_rows<T, SR>;
+    if (kernel_blocks_per_sm(kr, MASK_BLOCK, sizeof(MaskBlock<T>)) <= 0) return cudaErrorInvalidConfiguration;
+    // smaller units where few would be left for the SMs: 3000 rows 68 -> 49 us
+    int unit = MASK_BLOCK;
+    while (unit > 32 && A.nnz < (long long)MASK_UNITS_PER_SM * c.nsm * unit) unit >>= 1;
+    kr<<<(unsigned)((A.nnz + unit - 1) / unit), MASK_BLOCK, sizeof(MaskBlock<T>), c.stream>>>(A, B, M, av, bv, out,
+                                                                                          unit);
+    count_launch(c);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  k<<<(unsigned)((A.nnz + 31) / 32), 32, 0, c.stream>>>(A, B, M, av, bv, out, long_rows);
   count_launch(c);
   if ((e = cudaGetLastError()) != cudaSuccess || SR != 0 || !mv) return e;
   k_scale<T><<<eg, 256, 0, c.stream>>>(out, mv, M.nnz);

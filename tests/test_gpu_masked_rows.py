@@ -56,11 +56,12 @@ def test_rows_for_blocks(api, oracle_mod, semiring, dtype):
     n = 12000
     B = gen.random_rows(len(blen), n, blen, rng, values="int")
     alen = np.array([63, 64, 64, 65, 3, 255, 256, 257, 0, 520, 700, 600, 64, 1, 100, 512, 513, 66, 1100, 1100,
-                     1600, 1600])
+                     1600, 1600] + [1600] * 5)
     mlen = np.array([252, 256, 257, 1, 40, 0, 1024, 1028, 5, 1535, 1536, 1537, 64, 9, 401, 2400, 2052, 264, 3072, 3073,
-                     4608, 4609])
+                     4608, 4609] + [3] * 5)
     A = gen.random_rows(len(alen), B.nrows, alen, rng, values="int")
     M = gen.random_rows(len(mlen), n, mlen, rng, values="int")
+    assert M.nnz <= 2 * A.nnz  # denser masks leave every row to the warps
     dA, dB, dM = (api.DeviceCSR.from_host(X, dtype=dtype) for X in (A, B, M))
     got = api.masked_semiring(dA, dB, dM, semiring).double().cpu().numpy()
     ref = (oracle_mod.masked(A, B, M, use_mask_values=False) if semiring == "plus_times"
