@@ -39,12 +39,11 @@ sys.path.insert(0, HERE)
 from paper_2112_10037_gb300 import gen  # noqa: E402
 
 L2_BYTES = 129 * 1024 * 1024
-# default row classes of the library (register sort <= 16 products, hash
-# accumulator 17..128; numeric warp window up to 65536 products, bins rounded
-# to powers of two; block window above)
-TINY_MAX = 16
+# default row classes of the library (one launch for rows of up to 128
+# products; numeric: registers of a block up to 4096, bands of ranks above, on
+# products of more than 65536 columns)
 HASH_MAX = 128
-NUM_BLOCK_MIN = 65536
+NUM_BLOCK_MIN = 4096
 PEAKS_FILE = os.path.join(HERE, "MEASURED_PEAKS.json")
 FALLBACK_HBM_GBS = 6800.0
 
@@ -359,15 +358,14 @@ def kernel_bytes(A, B, prod_rows, c_rp, kernel, row_begin):
     kernel's rows."""
     P = np.asarray(prod_rows, np.int64)
     path = kernel.split("_", 1)[1]
-    # register sort up to 16 products, hash accumulator up to 128; every
-    # larger row runs in the warp window kernel (numeric) / the bitmap
-    # kernels (symbolic warp <= 8192 < block)
-    small = {"tiny": (1, TINY_MAX), "hash": (TINY_MAX + 1, HASH_MAX)}
+    # the timers' row classes: "hash" holds every row of up to 128 products;
+    # numeric "warp" the rows in a block's registers, "block" the bands;
+    # symbolic "block" every larger row
     if kernel.startswith("num"):
-        lo, hi = dict(small, warp=(HASH_MAX + 1, NUM_BLOCK_MIN), block=(NUM_BLOCK_MIN + 1, 1 << 62)).get(
-            path, (0, -1))
+        lo, hi = {"hash": (1, HASH_MAX), "warp": (HASH_MAX + 1, NUM_BLOCK_MIN),
+                  "block": (NUM_BLOCK_MIN + 1, 1 << 62)}.get(path, (0, -1))
     else:
-        lo, hi = dict(small, warp=(HASH_MAX + 1, 8192), block=(8193, 1 << 62)).get(path, (0, -1))
+        lo, hi = {"hash": (1, HASH_MAX), "block": (HASH_MAX + 1, 1 << 62)}.get(path, (0, -1))
     rows = np.flatnonzero((P >= lo) & (P <= hi))
     if len(rows) == 0:
         return 0.0
@@ -390,10 +388,8 @@ def kernel_bytes(A, B, prod_rows, c_rp, kernel, row_begin):
 def kernel_products(prod_rows, kernel):
     """Products handled by the numeric kernel of this path (host bookkeeping)."""
     P = np.asarray(prod_rows, np.int64)
-    if kernel == "num_tiny":
-        return int(P[(P >= 1) & (P <= TINY_MAX)].sum())
     if kernel == "num_hash":
-        return int(P[(P > TINY_MAX) & (P <= HASH_MAX)].sum())
+        return int(P[(P >= 1) & (P <= HASH_MAX)].sum())
     if kernel == "num_warp":
         return int(P[(P > HASH_MAX) & (P <= NUM_BLOCK_MIN)].sum())
     return int(P[P > NUM_BLOCK_MIN].sum())
@@ -415,7 +411,8 @@ def fp64_peak_gflops(torch, dev):
 # Sources of the numeric pass's kernels: numeric.cu and everything it
 # includes.  A DRAM-traffic record stays valid while these are unchanged.
 NUMERIC_SOURCES = ["numeric.cu", "numdispatch.cuh", "semiring.cuh", "launch_util.cuh", "internal.cuh", "numblock.cuh",
-                   "numrank.cuh", "numwarp.cuh", "rowhash.cuh", "rowlane.cuh", "rowpass.cuh", "segstream.cuh"]
+                   "numband.cuh", "numonce.cuh", "numrank.cuh", "numwarp.cuh", "rowhash.cuh", "rowlane.cuh", "rowpass.cuh",
+                   "segstream.cuh", "symblock.cuh"]
 
 
 def numeric_digest() -> str:

@@ -5,13 +5,14 @@ It replaces the paper's analytical choice of architecture parameters
 with measurement on this GPU.  The options it picks, per product:
 
 * the accumulator of the short rows, by bin: the warp hash table for rows of
-  17 .. hash_max products (32, 64 or 128), with dense column windows above,
+  17 .. hash_max products (32, 64 or 128), with the register path above,
   or no hash table at all and the register sort up to sort_max products
   (128 or 256) -- the dense-versus-hash choice per bin;
 * the product count above which rows take the rank-compacted accumulator
   (a presence bitmap ranks the output columns, values sit in an array of the
-  row's outputs) instead of the warp's dense column windows;
-* the numeric window width of a warp (columns per dense accumulator);
+  row's outputs) instead of the default routes;
+* the numeric window width of a warp (columns per dense accumulator; another
+  width than 1024 sends rows to it that the register path takes otherwise);
 * the product count above which rows take the block-wide window, that
   window's width and the number of warps sharing it;
 * the product count at which the symbolic pass switches from one warp to a
@@ -49,8 +50,8 @@ DEFAULT_CACHE = os.path.join(os.path.expanduser("~"), ".cache", "paper_2112_1003
 # named by the key, or a dict of several options set together.
 SMALL_ROW_ACCUMULATORS = [
     {"hash_max": 128, "sort_max": 128},   # hash table for 17..128 products (default)
-    {"hash_max": 64, "sort_max": 128},    # hash for 17..64, dense windows above
-    {"hash_max": 32, "sort_max": 128},    # hash for 17..32, dense windows above
+    {"hash_max": 64, "sort_max": 128},    # hash for 17..64, registers above
+    {"hash_max": 32, "sort_max": 128},    # hash for 17..32, registers above
     {"hash_max": -1, "sort_max": 128},    # no hash: register sort up to 128
     {"hash_max": -1, "sort_max": 256},    # no hash: register sort up to 256
 ]

@@ -1,4 +1,5 @@
-// Numeric pass, dense-window accumulator owned by one warp.
+// Numeric pass, dense-window accumulator owned by one warp: the rows an option
+// sends here (by default numonce.cuh and numband.cuh take them).
 //
 // Row i of C is the sum over A(i,k) of A(i,k) * B(k,:) (Sec. 2.2).  A warp
 // owns a window of W consecutive columns in shared memory: a dense value
