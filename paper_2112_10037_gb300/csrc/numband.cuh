@@ -26,7 +26,7 @@
 // and, below 65,536 products, the latency of a row's phases with two rows on
 // an SM.  R-MAT scale 18, FP64: rows of 8,193 to 65,536 products 10.3 ms with
 // a warp's 1024-column windows and 7.4 in bands; with the longer rows, which a
-// block's 8192-column windows took 14.6 ms for, 21.8 ms together.  262,144
+// block's 8192-column windows took 14.6 ms for, 22.9 ms together.  262,144
 // columns, edge factor 8, FP32: 8.5 and 4.4 ms; 150,000 columns, edge factor 4,
 // FP64: 1.4 and 1.2 ms.
 #pragma once
