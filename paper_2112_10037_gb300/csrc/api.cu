@@ -37,7 +37,6 @@ struct spgemm_plan {
   long long grad_buf_entries = 0;
   std::mutex grad_mu;                // calls that use the buffer follow one another
   cudaEvent_t grad_done = nullptr;   // end of the last one outside a capture
-  cudaStream_t grad_stream = nullptr;
   // host state
   sg::PathBins pb{};
   sg::Tuning tu{};
@@ -796,8 +795,11 @@ spgemm_status spgemm_backward(spgemm_plan* p, const void* a_vals, const void* b_
   g.buf_entries = p->grad_buf_entries;
   if (e == cudaSuccess && p->mloc > 0) {
     // the product buffer serves one call at a time: the launches of a call are
-    // not mixed with another thread's, and a call on another stream waits for
-    // the last one (not inside a capture, which takes no outside event)
+    // not mixed with another thread's, and every call waits for the last one
+    // (not inside a capture, which takes no outside event).  Equal handles do
+    // not make the wait unnecessary: the per-thread stream has one handle for
+    // a different stream in every thread, and a destroyed stream's handle may
+    // come back for a new one
     std::lock_guard<std::mutex> lock(p->grad_mu);
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     const bool order = p->grad_buf_entries > 0 && db_vals;
@@ -805,12 +807,12 @@ spgemm_status spgemm_backward(spgemm_plan* p, const void* a_vals, const void* b_
     const bool eager = order && cs == cudaStreamCaptureStatusNone;
     if (e == cudaSuccess && eager && !p->grad_done)
       e = cudaEventCreateWithFlags(&p->grad_done, cudaEventDisableTiming);
-    else if (e == cudaSuccess && eager && p->grad_stream != c.stream)
+    else if (e == cudaSuccess && eager)
       e = cudaStreamWaitEvent(c.stream, p->grad_done, 0);
     if (e == cudaSuccess) e = sg::launch_backward(c, p->opts.dtype, g, a_vals, b_vals, dc_vals, da_vals, db_vals);
-    if (e == cudaSuccess && eager) {
-      e = cudaEventRecord(p->grad_done, c.stream);
-      p->grad_stream = c.stream;
+    if (eager && p->grad_done) {  // after a failure too: some of its launches may run
+      const cudaError_t r = cudaEventRecord(p->grad_done, c.stream);
+      if (e == cudaSuccess) e = r;
     }
   }
   return e == cudaSuccess ? SPGEMM_OK : SPGEMM_ERR_CUDA;

@@ -2,7 +2,10 @@
 C at the edges of what a block stages in shared memory (128 and 4096 entries,
 one bitmap of columns), rows of B of average length below and above the lane
 groups' sizes, columns of A with more terms than a lane's chain takes, one
-gradient at a time, and calls on two streams."""
+gradient at a time, and calls on two streams, named by two handles or by one
+(the per-thread stream's)."""
+import threading
+
 import numpy as np
 import pytest
 
@@ -104,4 +107,45 @@ def test_two_streams(api):
     plan.stream = home
     for i, (da, db) in enumerate(got):
         assert torch.equal(da, alone[i % 2][0]) and torch.equal(db, alone[i % 2][1])
+    plan.close()
+
+
+def test_per_thread_streams(api):
+    """Two host threads that both name the per-thread stream: one handle, a
+    different stream in each thread, one product buffer."""
+    from paper_2112_10037_gb300 import _native as nat
+    A = gen.random_rows(3000, 3000, np.full(3000, 40), np.random.default_rng(3))
+    dA = api.DeviceCSR.from_host(A)
+    plan = api.Plan(dA, dA, backward=True)
+    _, nnz = plan.symbolic()
+    plan.numeric(dA.vals, dA.vals)
+    gen_ = torch.Generator(device="cuda").manual_seed(1)
+    ws = [torch.randn(nnz, generator=gen_, device="cuda", dtype=torch.float64) for _ in range(2)]
+    alone = [plan.backward(dA.vals, dA.vals, w) for w in ws]
+    reps = 8
+    out = [[(torch.zeros_like(dA.vals), torch.zeros_like(dA.vals)) for _ in range(reps)] for _ in ws]
+    torch.cuda.synchronize()
+    start, failed = threading.Barrier(2), []
+
+    def work(i):
+        try:
+            torch.cuda.set_device(0)
+            start.wait()
+            for da, db in out[i]:
+                nat.spgemm_backward(plan.handle, dA.vals.data_ptr(), dA.vals.data_ptr(), plan.row_ptr.data_ptr(),
+                                    plan.col_idx.data_ptr(), ws[i].data_ptr(), da.data_ptr(), db.data_ptr(),
+                                    2)  # cudaStreamPerThread
+        except Exception as e:  # reported by the main thread
+            failed.append(e)
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not failed
+    for i, pairs in enumerate(out):
+        for da, db in pairs:
+            assert torch.equal(da, alone[i][0]) and torch.equal(db, alone[i][1])
     plan.close()
