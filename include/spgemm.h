@@ -250,8 +250,10 @@ spgemm_status spgemm_plan_check(spgemm_plan* plan, spgemm_stream_t stream);
  * of A's nonzeros; entries of rows outside the plan's row range are left
  * untouched) and db_vals (aligned with B's col_idx; sums over the plan's
  * rows only) are overwritten; either may be NULL to skip it.  Each output is
- * summed in a fixed order (chains of fused multiply-adds and fixed trees of
- * additions), so the result is deterministic (the same bits on every call).
+ * summed in a fixed order, so the result is deterministic (the same bits on
+ * every call): db_vals by one chain of fused multiply-adds for at most 128
+ * terms (nonzeros of A's column), otherwise by 32 chains of every 32nd term and
+ * a fixed tree; da_vals by chains of at most 128 terms and a fixed tree.
  * db_vals uses a buffer of at most 128 MB in the plan's workspace: calls on
  * one plan follow one another on the GPU whatever streams they are given; a
  * graph captured from this call must not run beside another of the plan's.

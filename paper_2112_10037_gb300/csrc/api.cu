@@ -557,8 +557,8 @@ static spgemm_status analyse_impl(const spgemm_csr* A, const spgemm_csr* B, cons
       p->t_off = (long long*)(p->ws + L.t_off);
       p->grad_buf = p->ws + L.gbuf;
       p->grad_buf_entries = L.gbuf_entries;
-      e = sg::launch_grad_offsets(c, p->A, p->B, p->row_begin, p->mloc, p->prod, p->at_ci, p->at_src, p->row_off,
-                                  (long long*)(p->ws + L.off_part), p->p_off, p->t_off);
+      e = sg::launch_grad_offsets(c, p->A, p->B, p->row_begin, p->mloc, p->prod, p->at_rp, p->at_ci, p->at_src,
+                                  p->row_off, (long long*)(p->ws + L.off_part), p->p_off, p->t_off);
     }
   }
   if (e != cudaSuccess) { delete p; return SPGEMM_ERR_CUDA; }
@@ -790,6 +790,7 @@ spgemm_status spgemm_backward(spgemm_plan* p, const void* a_vals, const void* b_
   g.c_rp = c_row_ptr; g.c_ci = c_col_idx;
   g.row_off = p->row_off; g.p_off = p->p_off; g.t_off = p->t_off;
   g.total = (long long)p->host_st.total_products;
+  g.max_col = p->host_st.max_col;
   g.hist = p->host_st.hist;
   g.buf = p->grad_buf;
   g.buf_entries = p->grad_buf_entries;

@@ -278,12 +278,20 @@ __global__ void __launch_bounds__(256) k_product_offsets(Csr A, Csr B, long long
 }
 
 // The same offsets in the order of A^T; rows before and after the plan's
-// range lie below and above every product.
+// range lie below and above every product.  Also the length of A's longest
+// column, into the plan's statistics.
 __global__ void __launch_bounds__(256) k_transposed_offsets(long long nnz, const int32_t* __restrict__ t_ci,
                                                             const int32_t* __restrict__ t_src, long long row_begin,
                                                             long long row_end, const long long* __restrict__ p_off,
-                                                            long long* __restrict__ t_off, const DevStats* st) {
+                                                            long long* __restrict__ t_off,
+                                                            const int32_t* __restrict__ t_rp, long long ncols,
+                                                            DevStats* st) {
   if (block_skip(st)) return;
+  int most = 0;
+  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < ncols; k += (long long)gridDim.x * blockDim.x)
+    most = max(most, t_rp[k + 1] - t_rp[k]);
+  most = warp_max(most);
+  if (lane_id() == 0 && most > 0) atomicMax(&st->max_col, most);
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < nnz; t += (long long)gridDim.x * blockDim.x) {
     const long long i = t_ci[t];
     t_off[t] = i < row_begin ? -1ll : (i >= row_end ? LLONG_MAX : p_off[t_src[t]]);
@@ -600,13 +608,16 @@ k_grad_slabs(Csr A, Csr B, const T* __restrict__ bv, RowInfo ri, const int32_t* 
   }
 }
 
-// dB from one chunk of the buffer: slabs of 32 outputs of B per warp, each
-// output its lane's chain over the chunk's nonzeros of A^T(k,:) (lanes of one
-// row of B read consecutive buffer entries).  A slab with an output of more
-// than GRAD_COL_MAX terms is summed by the whole block, each warp an eighth of
-// every output's terms, the eighths added in order.
-constexpr int GRAD_COL_MAX = 512;
-
+// dB from one chunk of the buffer, in the order that k_grad_b sums in: slabs of
+// 32 outputs of B per warp, an output of at most GRAD_LANE_MAX terms (of the
+// whole column of A, not of the chunk) its lane's chain over the chunk's
+// nonzeros of A^T(k,:), which the next chunk takes up from dB (lanes of one row
+// of B read consecutive buffer entries).  Longer sums are 32 chains and a fixed
+// tree; their chains cannot be taken up from one number, so they are summed here
+// only when one chunk holds every product (LONG; a kernel of its own, because
+// its registers leave fewer warps), by the whole block: warp w runs the chains
+// w, w + 8, w + 16 and w + 24 of the slab's 32 outputs, each lane an output.  (FP32, positive terms, root mean square error over the sum:
+// 512 terms 3.0e-7 in one chain, 4.5e-8 in 32.)
 template <typename T>
 __device__ __forceinline__ T grad_col_sum(const T* __restrict__ av, const int32_t* __restrict__ t_src,
                                           const long long* __restrict__ t_off, const T* __restrict__ buf,
@@ -626,14 +637,37 @@ __device__ __forceinline__ T grad_col_sum(const T* __restrict__ av, const int32_
   return acc;
 }
 
+// Chains w, w + 8, w + 16, w + 24 of the 32 over the terms [t0, t1), added as
+// warp_sum_fixed adds their lanes (16 apart, then 8 apart).  Rows outside the
+// plan's range (offsets -1 and LLONG_MAX) keep their place and add nothing.
 template <typename T>
+__device__ __forceinline__ T grad_wide_part(const T* __restrict__ av, const int32_t* __restrict__ t_src,
+                                            const long long* __restrict__ t_off, const T* __restrict__ buf, int l,
+                                            int t0, int t1, int w) {
+  T p[4] = {T(0), T(0), T(0), T(0)};
+  for (int t = t0 + w; t < t1; t += 32) {
+    T a[4], d[4];
+    bool in[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int x = t + 8 * u;
+      const long long o = x < t1 ? t_off[x] : -1ll;
+      in[u] = o >= 0 && o < LLONG_MAX;
+      a[u] = in[u] ? av[t_src[x]] : T(0);
+      d[u] = in[u] ? buf[o + l] : T(0);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (in[u]) p[u] = fma(a[u], d[u], p[u]);
+  }
+  return (p[0] + p[2]) + (p[1] + p[3]);
+}
+
+template <typename T, bool LONG>
 __global__ void __launch_bounds__(256)
 k_grad_cols(Csr B, const T* __restrict__ av, const int32_t* __restrict__ b_row, const int32_t* __restrict__ t_rp,
             const int32_t* __restrict__ t_src, const long long* __restrict__ t_off, const T* __restrict__ buf,
             T* __restrict__ db, long long c0, long long c1, int first, int whole) {
-  __shared__ int s_big[8];
-  __shared__ int s_l[32], s_t0[32], s_t1[32];
-  __shared__ T s_part[8][32];
   const int warp = threadIdx.x >> 5, lane = lane_id();
   const long long nslab = (B.nnz + 31) >> 5;
   for (long long s0 = blockIdx.x * 8ll; s0 < nslab; s0 += gridDim.x * 8ll) {
@@ -645,36 +679,40 @@ k_grad_cols(Csr B, const T* __restrict__ av, const int32_t* __restrict__ b_row, 
       l = (int)(q - B.rp[k]);
       t0 = t_rp[k];
       t1 = t_rp[k + 1];
+    }
+    const bool wide = LONG && t1 - t0 > GRAD_LANE_MAX;
+    if (have && !wide) {
+      int u0 = t0, u1 = t1;
       if (!whole) {  // one chunk of every row of A needs no search
-        t0 = first_at_least(t_off, t0, t1, c0);
-        t1 = first_at_least(t_off, t0, t1, c1);
+        u0 = first_at_least(t_off, t0, t1, c0);
+        u1 = first_at_least(t_off, u0, t1, c1);
       }
+      if (first || u1 > u0) db[q] = grad_col_sum(av, t_src, t_off, buf, c0, l, u0, u1, first ? T(0) : db[q]);
     }
-    const bool big = __any_sync(FULL, t1 - t0 > GRAD_COL_MAX);
-    if (!big && have && (first || t1 > t0))
-      db[q] = grad_col_sum(av, t_src, t_off, buf, c0, l, t0, t1, first ? T(0) : db[q]);
-    if (lane == 0) s_big[warp] = big;
-    if (!__syncthreads_or(big)) continue;
-    for (int w = 0; w < 8; ++w) {
-      if (!s_big[w]) continue;  // block-uniform
-      if (warp == w) {
-        s_l[lane] = l;
-        s_t0[lane] = t0;
-        s_t1[lane] = t1;
-      }
-      __syncthreads();
-      const int u0 = s_t0[lane], n = s_t1[lane] - u0;
-      s_part[warp][lane] = grad_col_sum(av, t_src, t_off, buf, c0, s_l[lane], u0 + (int)((long long)n * warp / 8),
-                                        u0 + (int)((long long)n * (warp + 1) / 8), T(0));
-      __syncthreads();
-      if (warp == w && have) {
-        T acc = first ? T(0) : db[q];
-        for (int v = 0; v < 8; ++v) acc += s_part[v][lane];
-        db[q] = acc;
+    if constexpr (LONG) {
+      __shared__ int s_any[8];
+      __shared__ int s_l[32], s_t0[32], s_t1[32];
+      __shared__ T s_part[8][32];
+      const bool any = __any_sync(FULL, wide);
+      if (lane == 0) s_any[warp] = any;
+      if (!__syncthreads_or(any)) continue;
+      for (int w = 0; w < 8; ++w) {
+        if (!s_any[w]) continue;  // block-uniform
+        if (warp == w) {
+          s_l[lane] = l;
+          s_t0[lane] = wide ? t0 : 0;
+          s_t1[lane] = wide ? t1 : 0;
+        }
+        __syncthreads();
+        s_part[warp][lane] = grad_wide_part(av, t_src, t_off, buf, s_l[lane], s_t0[lane], s_t1[lane], warp);
+        __syncthreads();
+        if (warp == w && wide)  // 4, 2 and 1 apart
+          db[q] = ((s_part[0][lane] + s_part[4][lane]) + (s_part[2][lane] + s_part[6][lane])) +
+                  ((s_part[1][lane] + s_part[5][lane]) + (s_part[3][lane] + s_part[7][lane]));
+        __syncthreads();
       }
       __syncthreads();
     }
-    __syncthreads();
   }
 }
 
@@ -702,8 +740,8 @@ long long grad_buffer_entries(long long nnz_a, long long nnz_b, long long ncols_
 }
 
 cudaError_t launch_grad_offsets(const LaunchCtx& c, const Csr& A, const Csr& B, long long row_begin, long long mloc,
-                                const long long* prod, const int32_t* t_ci, const int32_t* t_src, long long* row_off,
-                                long long* part, long long* p_off, long long* t_off) {
+                                const long long* prod, const int32_t* t_rp, const int32_t* t_ci, const int32_t* t_src,
+                                long long* row_off, long long* part, long long* p_off, long long* t_off) {
   if (mloc <= 0) return cudaSuccess;
   const long long tiles = (mloc + OFF_TILE - 1) / OFF_TILE;
   k_off_tiles<<<(unsigned)tiles, OFF_THREADS, 0, c.stream>>>(prod, mloc, part);
@@ -711,7 +749,7 @@ cudaError_t launch_grad_offsets(const LaunchCtx& c, const Csr& A, const Csr& B, 
   k_off_down<<<(unsigned)tiles, OFF_THREADS, 0, c.stream>>>(prod, mloc, part, row_off);
   k_product_offsets<<<grid_for(mloc, c.nsm), 256, 0, c.stream>>>(A, B, row_begin, mloc, row_off, p_off, c.st);
   k_transposed_offsets<<<grid_for((A.nnz + 31) / 32, c.nsm), 256, 0, c.stream>>>(
-      A.nnz, t_ci, t_src, row_begin, row_begin + mloc, p_off, t_off, c.st);
+      A.nnz, t_ci, t_src, row_begin, row_begin + mloc, p_off, t_off, t_rp, A.ncols, c.st);
   for (int i = 0; i < 5; ++i) count_launch(c);
   return cudaGetLastError();
 }
@@ -729,11 +767,27 @@ static cudaError_t grad_rows(const LaunchCtx& c, const GradArgs& g, const T* bv,
   return cudaGetLastError();
 }
 
-// Both gradients through the product buffer (g.buf_entries > 0).
+// dB with a search in C's rows per term.
+template <typename T>
+static cudaError_t search_db(const LaunchCtx& c, const GradArgs& g, const T* av, const T* dc, T* db) {
+  k_grad_b<T><<<grid_for((g.B.nnz + 31) / 32, c.nsm), 256, 0, c.stream>>>(
+      g.B, av, g.b_row, g.t_rp, g.t_ci, g.t_src, g.ri.row_begin, g.ri.row_begin + g.ri.mloc, g.c_rp, g.c_ci, dc, db,
+      c.err);
+  count_launch(c);
+  return cudaGetLastError();
+}
+
+// Both gradients, dB through the product buffer (g.buf_entries > 0) unless
+// sums that need 32 chains would have to go on from chunk to chunk.
 template <typename T>
 static cudaError_t backward_buffered(const LaunchCtx& c, const GradArgs& g, const T* av, const T* bv, const T* dc,
                                      T* da, T* db) {
   const long long longest = g.B.ncols < g.B.nnz ? g.B.ncols : g.B.nnz;
+  if (db && g.total > g.buf_entries - longest && g.max_col > GRAD_LANE_MAX) {
+    const cudaError_t e = search_db(c, g, av, dc, db);
+    if (e != cudaSuccess || !da) return e;
+    db = nullptr;
+  }
   const long long chunk = db ? g.buf_entries - longest : LLONG_MAX;
   T* const buf = db ? (T*)g.buf : nullptr;
   // rows of C staged in shared memory: a row has at most its products'
@@ -768,7 +822,9 @@ static cudaError_t backward_buffered(const LaunchCtx& c, const GradArgs& g, cons
         g.A, g.B, bv, g.ri, g.a_row, g.p_off, g.c_rp, g.c_ci, dc, da, buf, c0, c1, hi > 0 ? cap : 0, wlog, c.err);
     count_launch(c);
     if (db) {
-      k_grad_cols<T><<<grid_for((g.B.nnz + 31) / 32, c.nsm), 256, 0, c.stream>>>(
+      // (long sums in several chunks were left to search_db)
+      auto k = g.max_col > GRAD_LANE_MAX ? k_grad_cols<T, true> : k_grad_cols<T, false>;
+      k<<<grid_for((g.B.nnz + 31) / 32, c.nsm), 256, 0, c.stream>>>(
           g.B, av, g.b_row, g.t_rp, g.t_src, g.t_off, buf, db, c0, c1, c0 == 0 ? 1 : 0,
           c0 == 0 && last && g.ri.row_begin == 0 && g.ri.mloc == g.A.nrows ? 1 : 0);
       count_launch(c);
@@ -778,11 +834,22 @@ static cudaError_t backward_buffered(const LaunchCtx& c, const GradArgs& g, cons
   return cudaSuccess;
 }
 
+template <typename T>
+static cudaError_t backward_searched(const LaunchCtx& c, const GradArgs& g, const T* av, const T* bv, const T* dc,
+                                     T* da, T* db) {
+  if (da && g.ri.mloc > 0) {
+    k_grad_a<T><<<grid_for(g.A.nnz / 32 + 1, c.nsm), 256, 0, c.stream>>>(  // (the kernel reads the range's own extent)
+        g.A, g.B, bv, g.ri.row_begin, g.ri.mloc, g.a_row, g.c_rp, g.c_ci, dc, da, c.err);
+    count_launch(c);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return db && g.B.nnz > 0 ? search_db(c, g, av, dc, db) : cudaSuccess;
+}
+
 cudaError_t launch_backward(const LaunchCtx& c, int dtype, const GradArgs& g, const void* av, const void* bv,
                             const void* dc, void* da, void* db) {
-  const Csr &A = g.A, &B = g.B;
-  const long long row_begin = g.ri.row_begin, mloc = g.ri.mloc;
-  if (g.buf_entries > 0 && mloc > 0 && B.nnz > 0) {
+  if (g.buf_entries > 0 && g.ri.mloc > 0 && g.B.nnz > 0) {
     if (dtype == SPGEMM_F32)
       return backward_buffered<float>(c, g, (const float*)av, (const float*)bv, (const float*)dc, (float*)da,
                                       (float*)db);
@@ -790,35 +857,10 @@ cudaError_t launch_backward(const LaunchCtx& c, int dtype, const GradArgs& g, co
                                      (double*)db);
   }
   // rows of B longer than the buffer: a search per product and gradient
-  if (db && B.nnz > 0) {
-    const cudaError_t e = cudaMemsetAsync(db, 0, (size_t)B.nnz * (dtype == SPGEMM_F32 ? 4 : 8), c.stream);
-    if (e != cudaSuccess) return e;
-  }
-  if (da && mloc > 0) {
-    const long long slabs = A.nnz / 32 + 1;  // an upper bound; the kernel reads the range's own extent
-    if (dtype == SPGEMM_F32)
-      k_grad_a<float><<<grid_for(slabs, c.nsm), 256, 0, c.stream>>>(A, B, (const float*)bv, row_begin, mloc, g.a_row,
-                                                                    g.c_rp, g.c_ci, (const float*)dc, (float*)da, c.err);
-    else
-      k_grad_a<double><<<grid_for(slabs, c.nsm), 256, 0, c.stream>>>(A, B, (const double*)bv, row_begin, mloc, g.a_row,
-                                                                     g.c_rp, g.c_ci, (const double*)dc, (double*)da, c.err);
-    count_launch(c);
-  }
-  if (db && B.nnz > 0) {
-    const long long slabs = (B.nnz + 31) / 32;
-    if (dtype == SPGEMM_F32)
-      k_grad_b<float><<<grid_for(slabs, c.nsm), 256, 0, c.stream>>>(B, (const float*)av, g.b_row, g.t_rp, g.t_ci,
-                                                                     g.t_src, row_begin, row_begin + mloc, g.c_rp,
-                                                                     g.c_ci, (const float*)dc,
-                                                                     (float*)db, c.err);
-    else
-      k_grad_b<double><<<grid_for(slabs, c.nsm), 256, 0, c.stream>>>(B, (const double*)av, g.b_row, g.t_rp, g.t_ci,
-                                                                      g.t_src,
-                                                                      row_begin, row_begin + mloc, g.c_rp, g.c_ci,
-                                                                      (const double*)dc, (double*)db, c.err);
-    count_launch(c);
-  }
-  return cudaGetLastError();
+  if (dtype == SPGEMM_F32)
+    return backward_searched<float>(c, g, (const float*)av, (const float*)bv, (const float*)dc, (float*)da, (float*)db);
+  return backward_searched<double>(c, g, (const double*)av, (const double*)bv, (const double*)dc, (double*)da,
+                                   (double*)db);
 }
 
 }  // namespace sg

@@ -48,6 +48,7 @@ struct DevStats {
   uint32_t err;
   uint32_t rows_wide;  // rows of the plan with more than 32 nonzeros of A
   uint32_t rows_wide8;  // rows with more than 8 (LANE_MERGE_K)
+  int max_col;       // nonzeros of A's longest column (plans for the adjoint)
   int hist[NBINS];   // rows per bin
   int fill[NBINS];   // scatter cursors
   unsigned int work[8];  // dynamic work counters (0, 1, 3: reset before each use; 4, 5: the symbolic
@@ -364,14 +365,15 @@ struct GradArgs {
   const int32_t *a_row, *b_row, *t_rp, *t_ci, *t_src, *c_rp, *c_ci;
   const long long *row_off, *p_off, *t_off;
   long long total;   // products of the plan's rows
+  int max_col;       // nonzeros of A's longest column
   const int* hist;   // host: rows per bin
   void* buf;
   long long buf_entries;
 };
 long long grad_buffer_entries(long long nnz_a, long long nnz_b, long long ncols_b, int vbytes);
 cudaError_t launch_grad_offsets(const LaunchCtx& c, const Csr& A, const Csr& B, long long row_begin, long long mloc,
-                                const long long* prod, const int32_t* t_ci, const int32_t* t_src, long long* row_off,
-                                long long* part, long long* p_off, long long* t_off);
+                                const long long* prod, const int32_t* t_rp, const int32_t* t_ci, const int32_t* t_src,
+                                long long* row_off, long long* part, long long* p_off, long long* t_off);
 cudaError_t launch_backward(const LaunchCtx& c, int dtype, const GradArgs& g, const void* av, const void* bv,
                             const void* dc, void* da, void* db);
 

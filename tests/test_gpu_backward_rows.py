@@ -110,6 +110,37 @@ def test_two_streams(api):
     plan.close()
 
 
+# (4500, 4000): 18 M products, more than one chunk of the buffer
+@pytest.mark.parametrize("terms,width", [(129, 64), (256, 64), (512, 64), (4096, 300), (4500, 4000)])
+def test_long_sums_keep_their_chains(api, terms, width):
+    """dB's sums of more than 128 terms are 32 chains of every 32nd term and a
+    tree of five levels.  A = one column, B = one row, positive FP32 operands:
+    a rounding is u/sqrt(3) of its partial sum in the root mean square (u =
+    2^-24); the m = terms/32 of a chain, whose partial sums grow evenly, come to
+    sqrt(m/3) of the chain's sum, over 32 chains sqrt(m/96) of the whole, the
+    tree's levels to 1, 1/2, ... of it, squared: less than 2.  1.3 for the
+    sample.  (One chain of 256
+    terms comes to sqrt(256/3), six times the bound.)"""
+    rng = np.random.default_rng(terms)
+    arp = np.arange(terms + 1, dtype=np.int32)
+    A = gen.CSR(terms, 1, arp, np.zeros(terms, np.int32), rng.uniform(0.5, 1.5, terms).astype(np.float32))
+    B = gen.CSR(1, width, np.array([0, width], np.int32), np.arange(width, dtype=np.int32),
+                rng.uniform(0.5, 1.5, width).astype(np.float32))
+    dA, dB = (api.DeviceCSR.from_host(M, dtype=torch.float32) for M in (A, B))
+    plan = api.Plan(dA, dB, dtype=torch.float32, backward=True)
+    _, nnz = plan.symbolic()
+    plan.numeric(dA.vals, dB.vals)
+    W = rng.uniform(0.5, 1.5, nnz).astype(np.float32)
+    _, db = plan.backward(dA.vals, dB.vals, torch.from_numpy(W).cuda())
+    torch.cuda.synchronize()
+    plan.check()
+    plan.close()
+    ref = A.vals.astype(np.float64) @ W.reshape(terms, width).astype(np.float64)
+    err = np.sqrt(np.mean(((db.double().cpu().numpy() - ref) / ref) ** 2))
+    bound = 1.3 * 2.0 ** -24 / np.sqrt(3.0) * np.sqrt(-(-terms // 32) / 96.0 + 2.0)
+    assert err <= bound
+
+
 def test_per_thread_streams(api):
     """Two host threads that both name the per-thread stream: one handle, a
     different stream in each thread, one product buffer."""
