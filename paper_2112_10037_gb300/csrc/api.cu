@@ -790,7 +790,9 @@ spgemm_status spgemm_backward(spgemm_plan* p, const void* a_vals, const void* b_
   g.c_rp = c_row_ptr; g.c_ci = c_col_idx;
   g.row_off = p->row_off; g.p_off = p->p_off; g.t_off = p->t_off;
   g.total = (long long)p->host_st.total_products;
+  g.nnz_c = p->nnz_c;
   g.max_col = p->host_st.max_col;
+  g.max_row_b = p->host_st.max_row_b;
   g.hist = p->host_st.hist;
   g.buf = p->grad_buf;
   g.buf_entries = p->grad_buf_entries;

@@ -28,6 +28,8 @@
 // Here k_grad_rows takes 0.62 ms for four chunks (bound by the latency of a
 // row's loads, 8 of 16 warps per scheduler resident at 64 registers),
 // k_grad_cols 0.20 ms (2.6 TB/s of DRAM and L1 59 % busy).
+#include <cmath>
+
 #include "launch_util.cuh"
 
 namespace sg {
@@ -278,20 +280,26 @@ __global__ void __launch_bounds__(256) k_product_offsets(Csr A, Csr B, long long
 }
 
 // The same offsets in the order of A^T; rows before and after the plan's
-// range lie below and above every product.  Also the length of A's longest
-// column, into the plan's statistics.
+// range lie below and above every product.  Also the lengths of A's longest
+// column and B's longest row, into the plan's statistics.
 __global__ void __launch_bounds__(256) k_transposed_offsets(long long nnz, const int32_t* __restrict__ t_ci,
                                                             const int32_t* __restrict__ t_src, long long row_begin,
                                                             long long row_end, const long long* __restrict__ p_off,
                                                             long long* __restrict__ t_off,
-                                                            const int32_t* __restrict__ t_rp, long long ncols,
+                                                            const int32_t* __restrict__ t_rp,
+                                                            const int32_t* __restrict__ b_rp, long long nrows_b,
                                                             DevStats* st) {
   if (block_skip(st)) return;
-  int most = 0;
-  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < ncols; k += (long long)gridDim.x * blockDim.x)
-    most = max(most, t_rp[k + 1] - t_rp[k]);
-  most = warp_max(most);
-  if (lane_id() == 0 && most > 0) atomicMax(&st->max_col, most);
+  int col = 0, row = 0;
+  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < nrows_b;
+       k += (long long)gridDim.x * blockDim.x) {
+    col = max(col, t_rp[k + 1] - t_rp[k]);
+    row = max(row, b_rp[k + 1] - b_rp[k]);
+  }
+  col = warp_max(col);
+  row = warp_max(row);
+  if (lane_id() == 0 && col > 0) atomicMax(&st->max_col, col);
+  if (lane_id() == 0 && row > 0) atomicMax(&st->max_row_b, row);
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < nnz; t += (long long)gridDim.x * blockDim.x) {
     const long long i = t_ci[t];
     t_off[t] = i < row_begin ? -1ll : (i >= row_end ? LLONG_MAX : p_off[t_src[t]]);
@@ -749,7 +757,7 @@ cudaError_t launch_grad_offsets(const LaunchCtx& c, const Csr& A, const Csr& B, 
   k_off_down<<<(unsigned)tiles, OFF_THREADS, 0, c.stream>>>(prod, mloc, part, row_off);
   k_product_offsets<<<grid_for(mloc, c.nsm), 256, 0, c.stream>>>(A, B, row_begin, mloc, row_off, p_off, c.st);
   k_transposed_offsets<<<grid_for((A.nnz + 31) / 32, c.nsm), 256, 0, c.stream>>>(
-      A.nnz, t_ci, t_src, row_begin, row_begin + mloc, p_off, t_off, t_rp, A.ncols, c.st);
+      A.nnz, t_ci, t_src, row_begin, row_begin + mloc, p_off, t_off, t_rp, B.rp, B.nrows, c.st);
   for (int i = 0; i < 5; ++i) count_launch(c);
   return cudaGetLastError();
 }
@@ -777,52 +785,116 @@ static cudaError_t search_db(const LaunchCtx& c, const GradArgs& g, const T* av,
   return cudaGetLastError();
 }
 
-// Both gradients, dB through the product buffer (g.buf_entries > 0) unless
-// sums that need 32 chains would have to go on from chunk to chunk.
+// dA with a search in C's rows per term.
 template <typename T>
-static cudaError_t backward_buffered(const LaunchCtx& c, const GradArgs& g, const T* av, const T* bv, const T* dc,
-                                     T* da, T* db) {
-  const long long longest = g.B.ncols < g.B.nnz ? g.B.ncols : g.B.nnz;
-  if (db && g.total > g.buf_entries - longest && g.max_col > GRAD_LANE_MAX) {
-    const cudaError_t e = search_db(c, g, av, dc, db);
-    if (e != cudaSuccess || !da) return e;
-    db = nullptr;
-  }
-  const long long chunk = db ? g.buf_entries - longest : LLONG_MAX;
-  T* const buf = db ? (T*)g.buf : nullptr;
-  // rows of C staged in shared memory: a row has at most its products'
-  // entries, so the rows' bins bound them
+static cudaError_t search_da(const LaunchCtx& c, const GradArgs& g, const T* bv, const T* dc, T* da) {
+  k_grad_a<T><<<grid_for(g.A.nnz / 32 + 1, c.nsm), 256, 0, c.stream>>>(  // (the kernel reads the range's own extent)
+      g.A, g.B, bv, g.ri.row_begin, g.ri.mloc, g.a_row, g.c_rp, g.c_ci, dc, da, c.err);
+  count_launch(c);
+  return cudaGetLastError();
+}
+
+// How a plan's gradients are formed.
+struct GradRoute {
+  bool staged;    // rows of C of more than 128 entries in shared memory (k_grad_rows)
+  bool buffered;  // dB through the product buffer
+  int cap, wlog;  // entries and column bits that k_grad_rows stages
+  int lanes;      // per nonzero of A
+  long long rows, chunk;
+};
+
+// Staged rows pay where rows of C fit (more than half of the rows can have
+// more than 128 entries, and a bitmap holds every column), where a row has
+// enough products to carry its barriers (10,007 columns, k a row, dA alone, FP64:
+// k = 20, 400 products, 75 us staged and 66 with searches; k = 24, 84 and 89;
+// FP32: k = 18 58 and 50, k = 20 59 and 61) and where rows of B are alike: a
+// group of lanes walks the longest of eight rows of B, so that on power-law
+// graphs, whose products come from rows of B many times the average (weighted
+// by their use 22 times on an R-MAT of 32,768 columns), most lanes wait: dA there
+// 4.49 ms staged, 1.57 with searches.  At most 4 times the average.  A row of B
+// of more than 128 entries is summed by 32 lanes, or not here.  The choice
+// depends on the plan alone: dA has the same bits with dB and without.
+//
+// Through the buffer dB shares dA's searches, or staged rows' look-ups.  Alone
+// and without either a search per term is no more work (40^3 stencil, FP64: 37 us
+// against 51; with dA 61 against 56), unless columns of A are long, whose terms
+// one warp would search (R-MAT, 3,000 columns: 1.18 ms against 0.33).  More than
+// one chunk: every chunk passes over all of dB, so what counts is the terms of an
+// output in a chunk and the steps that the search of each would take.  With dA,
+// buffered against searched, terms x steps: 5 (96^3 stencil FP64) 1.06 ms and
+// 0.44, 11 (FP32) 0.48 and 0.41, 13 (200,000 columns, 16 to 48 a row, FP64) 13.0
+// and 11.1, 16 (300,000 columns, 2 to 10, FP64) 0.28 and 0.35, 25 (200,000 columns
+// in FP32) 6.7 and 9.9, 40 (65,536 columns, 32, FP64) 1.2 and 3.0.  Long sums do
+// not go on from chunk to chunk (k_grad_cols).
+template <typename T>
+static GradRoute grad_route(const GradArgs& g, bool da, bool db, bool has_buffer) {
+  GradRoute r{};
   int hi = 0;
-  long long rows = 0;
-  for (int b = bin_of(GRAD_ROW_MIN + 1); b < NBINS; ++b)
-    if (g.hist[b]) {
+  long long all = 0;
+  for (int b = 1; b < NBINS; ++b) {
+    all += g.hist[b];
+    if (b >= bin_of(GRAD_ROW_MIN + 1) && g.hist[b]) {
       hi = b;
-      rows += g.hist[b];
+      r.rows += g.hist[b];
     }
-  int cap = 256;
-  while (cap < GRAD_ROW_CAP && cap < (hi > 0 ? (hi < 14 ? 1 << (hi - 1) : GRAD_ROW_CAP) : 0)) cap *= 2;
-  int wlog = 10;
-  while (wlog < (cap > 2048 ? 18 : 17) && (1ll << wlog) < g.B.ncols) ++wlog;
+  }
+  // a row has at most its products' entries, so the rows' bins bound them
+  r.cap = 256;
+  while (r.cap < GRAD_ROW_CAP && r.cap < (hi > 0 ? (hi < 14 ? 1 << (hi - 1) : GRAD_ROW_CAP) : 0)) r.cap *= 2;
+  r.wlog = 10;
+  const int widest = r.cap > 2048 ? 18 : 17;
+  while (r.wlog < widest && (1ll << r.wlog) < g.B.ncols) ++r.wlog;
   const double avg = g.B.nrows > 0 ? (double)g.B.nnz / (double)g.B.nrows : 0.0;
+  r.lanes = avg >= 20 ? 32 : (avg >= 10 ? 16 : 8);
+  const double share = g.A.nrows > 0 ? (double)g.ri.mloc / (double)g.A.nrows : 0.0;  // of A's nonzeros, about
+  r.staged = has_buffer && g.total >= (sizeof(T) == 8 ? 512 : 384) * all && 2 * r.rows > all && (1ll << r.wlog) >= g.B.ncols &&
+             (double)g.total <= 4.0 * avg * share * (double)g.A.nnz &&
+             (r.lanes == 32 || g.max_row_b <= GRAD_LANE_MAX);
+  const long long longest = g.B.ncols < g.B.nnz ? g.B.ncols : g.B.nnz;
+  r.chunk = g.buf_entries - longest;
+  r.buffered = db && has_buffer && (da || r.staged || g.max_col > GRAD_LANE_MAX);
+  if (r.buffered && g.total > r.chunk) {
+    const double chunks = (double)((g.total + r.chunk - 1) / r.chunk);
+    const double terms = (double)g.total / (chunks * (double)g.B.nnz);
+    const double steps = log2(1.0 + (double)g.nnz_c / (double)(all > 0 ? all : 1));
+    r.buffered = g.max_col <= GRAD_LANE_MAX && terms * steps >= 15.0;
+  }
+  return r;
+}
+
+template <typename T>
+static cudaError_t backward_t(const LaunchCtx& c, const GradArgs& g, const T* av, const T* bv, const T* dc, T* da,
+                              T* db) {
+  // no buffer: rows of B longer than one, which have no product offsets either
+  const GradRoute r = grad_route<T>(g, da != nullptr, db != nullptr, g.buf_entries > 0 && g.B.nnz > 0);
+  if (db && g.B.nnz > 0 && !r.buffered) {
+    const cudaError_t e = search_db(c, g, av, dc, db);
+    if (e != cudaSuccess) return e;
+  }
+  if (!r.buffered) db = nullptr;
+  if (!da && !db) return cudaSuccess;
+  if (!db && !r.staged) return search_da(c, g, bv, dc, da);
+  const long long chunk = db ? r.chunk : LLONG_MAX;
+  T* const buf = db ? (T*)g.buf : nullptr;
+  const int cap = r.staged ? r.cap : 0;
   for (long long c0 = 0; c0 < g.total || c0 == 0; c0 += chunk) {
     const bool last = c0 + chunk >= g.total || chunk == LLONG_MAX;
     const long long c1 = last ? LLONG_MAX - 1 : c0 + chunk;
     cudaError_t e = cudaSuccess;
-    if (hi > 0) {
-#define SG_GRAD_ROWS(GG)                                                                               \
-  e = cap > 2048 ? grad_rows<256, GG, T>(c, g, bv, dc, da, buf, c0, c1, cap, wlog, rows)                \
-                 : grad_rows<128, GG, T>(c, g, bv, dc, da, buf, c0, c1, cap, wlog, rows)
-      if (avg >= 20) SG_GRAD_ROWS(32);
-      else if (avg >= 10) SG_GRAD_ROWS(16);
+    if (r.staged) {
+#define SG_GRAD_ROWS(GG)                                                                                    \
+  e = cap > 2048 ? grad_rows<256, GG, T>(c, g, bv, dc, da, buf, c0, c1, cap, r.wlog, r.rows)                 \
+                 : grad_rows<128, GG, T>(c, g, bv, dc, da, buf, c0, c1, cap, r.wlog, r.rows)
+      if (r.lanes == 32) SG_GRAD_ROWS(32);
+      else if (r.lanes == 16) SG_GRAD_ROWS(16);
       else SG_GRAD_ROWS(8);
 #undef SG_GRAD_ROWS
       if (e != cudaSuccess) return e;
     }
     k_grad_slabs<T><<<grid_for(g.A.nnz / 32 + 1, c.nsm), 256, 0, c.stream>>>(
-        g.A, g.B, bv, g.ri, g.a_row, g.p_off, g.c_rp, g.c_ci, dc, da, buf, c0, c1, hi > 0 ? cap : 0, wlog, c.err);
+        g.A, g.B, bv, g.ri, g.a_row, g.p_off, g.c_rp, g.c_ci, dc, da, buf, c0, c1, cap, r.wlog, c.err);
     count_launch(c);
     if (db) {
-      // (long sums in several chunks were left to search_db)
       auto k = g.max_col > GRAD_LANE_MAX ? k_grad_cols<T, true> : k_grad_cols<T, false>;
       k<<<grid_for((g.B.nnz + 31) / 32, c.nsm), 256, 0, c.stream>>>(
           g.B, av, g.b_row, g.t_rp, g.t_src, g.t_off, buf, db, c0, c1, c0 == 0 ? 1 : 0,
@@ -834,33 +906,11 @@ static cudaError_t backward_buffered(const LaunchCtx& c, const GradArgs& g, cons
   return cudaSuccess;
 }
 
-template <typename T>
-static cudaError_t backward_searched(const LaunchCtx& c, const GradArgs& g, const T* av, const T* bv, const T* dc,
-                                     T* da, T* db) {
-  if (da && g.ri.mloc > 0) {
-    k_grad_a<T><<<grid_for(g.A.nnz / 32 + 1, c.nsm), 256, 0, c.stream>>>(  // (the kernel reads the range's own extent)
-        g.A, g.B, bv, g.ri.row_begin, g.ri.mloc, g.a_row, g.c_rp, g.c_ci, dc, da, c.err);
-    count_launch(c);
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
-  return db && g.B.nnz > 0 ? search_db(c, g, av, dc, db) : cudaSuccess;
-}
-
 cudaError_t launch_backward(const LaunchCtx& c, int dtype, const GradArgs& g, const void* av, const void* bv,
                             const void* dc, void* da, void* db) {
-  if (g.buf_entries > 0 && g.ri.mloc > 0 && g.B.nnz > 0) {
-    if (dtype == SPGEMM_F32)
-      return backward_buffered<float>(c, g, (const float*)av, (const float*)bv, (const float*)dc, (float*)da,
-                                      (float*)db);
-    return backward_buffered<double>(c, g, (const double*)av, (const double*)bv, (const double*)dc, (double*)da,
-                                     (double*)db);
-  }
-  // rows of B longer than the buffer: a search per product and gradient
   if (dtype == SPGEMM_F32)
-    return backward_searched<float>(c, g, (const float*)av, (const float*)bv, (const float*)dc, (float*)da, (float*)db);
-  return backward_searched<double>(c, g, (const double*)av, (const double*)bv, (const double*)dc, (double*)da,
-                                   (double*)db);
+    return backward_t<float>(c, g, (const float*)av, (const float*)bv, (const float*)dc, (float*)da, (float*)db);
+  return backward_t<double>(c, g, (const double*)av, (const double*)bv, (const double*)dc, (double*)da, (double*)db);
 }
 
 }  // namespace sg

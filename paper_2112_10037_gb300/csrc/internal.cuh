@@ -48,7 +48,7 @@ struct DevStats {
   uint32_t err;
   uint32_t rows_wide;  // rows of the plan with more than 32 nonzeros of A
   uint32_t rows_wide8;  // rows with more than 8 (LANE_MERGE_K)
-  int max_col;       // nonzeros of A's longest column (plans for the adjoint)
+  int max_col, max_row_b;  // nonzeros of A's longest column and B's longest row (plans for the adjoint)
   int hist[NBINS];   // rows per bin
   int fill[NBINS];   // scatter cursors
   unsigned int work[8];  // dynamic work counters (0, 1, 3: reset before each use; 4, 5: the symbolic
@@ -365,7 +365,8 @@ struct GradArgs {
   const int32_t *a_row, *b_row, *t_rp, *t_ci, *t_src, *c_rp, *c_ci;
   const long long *row_off, *p_off, *t_off;
   long long total;   // products of the plan's rows
-  int max_col;       // nonzeros of A's longest column
+  long long nnz_c;   // entries of C
+  int max_col, max_row_b;      // nonzeros of A's longest column and of B's longest row
   const int* hist;   // host: rows per bin
   void* buf;
   long long buf_entries;

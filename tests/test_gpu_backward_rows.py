@@ -110,6 +110,84 @@ def test_two_streams(api):
     plan.close()
 
 
+def _staged_operands(ncols, blen, seed):
+    """Every row of A reaches 127..130, 1000 or 4094..4098 distinct columns or
+    none, from rows of B of `blen` columns; products enough for staged rows."""
+    rng = np.random.default_rng(seed)
+    runs = 4200 // blen
+    place = np.sort(rng.choice(ncols, runs * blen + 64, replace=False))
+    order = rng.permutation(runs * blen)
+    lens = np.concatenate([np.full(runs, blen), np.ones(64, np.int64), [0]])
+    rp = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    ci = np.concatenate([np.sort(place[order[k * blen:(k + 1) * blen]]) for k in range(runs)] + [place[runs * blen:]])
+    # `blen` columns in a row of B, 64 rows of one more: an average near blen
+    B = gen.CSR(len(lens), ncols, rp, ci.astype(np.int32), rng.standard_normal(len(ci))).check()
+    rows = []
+    for want in [127, 128, 129, 130, 1000, 0] + [4094, 4095, 4096, 4097, 4098, 2000, 2500] * 6:
+        n = min(want // blen, runs)
+        ks = np.concatenate([rng.choice(runs, n, replace=False), runs + np.arange(min(want - n * blen, 64))])
+        rows.append(np.sort(ks).astype(np.int64))
+    arp = np.concatenate([[0], np.cumsum([len(r) for r in rows])]).astype(np.int32)
+    aci = np.concatenate(rows).astype(np.int32)
+    return gen.CSR(len(rows), B.nrows, arp, aci, rng.standard_normal(len(aci))).check(), B
+
+
+def _run(api, A, B, dtype, **want):
+    """(dA, dB, launches of the call, dC) of one plan."""
+    from paper_2112_10037_gb300 import _native as nat
+    dA, dB = api.DeviceCSR.from_host(A, dtype=dtype), api.DeviceCSR.from_host(B, dtype=dtype)
+    plan = api.Plan(dA, dB, dtype=dtype, backward=True)
+    _, nnz = plan.symbolic()
+    plan.numeric(dA.vals, dB.vals)
+    W = np.random.default_rng(1).standard_normal(nnz).astype(np.float32).astype(np.float64)
+    before = nat.spgemm_plan_launches(plan.handle)
+    da, db = plan.backward(dA.vals, dB.vals, torch.from_numpy(W).to(device="cuda", dtype=dtype), **want)
+    n = nat.spgemm_plan_launches(plan.handle) - before
+    torch.cuda.synchronize()
+    plan.check()
+    plan.close()
+    return da, db, n, W
+
+
+@pytest.mark.parametrize("dtype,tol", [(torch.float64, 1e-12), (torch.float32, 2e-4)])
+@pytest.mark.parametrize("ncols", [5000, 100_000])
+@pytest.mark.parametrize("blen", [9, 16, 60])
+def test_staged_rows(api, oracle_mod, blen, ncols, dtype, tol):
+    A, B = _staged_operands(ncols, blen, blen)
+    da, db, n, W = _run(api, A, B, dtype)
+    assert n == 3  # staged rows, the other rows, the columns
+    only_a, _, _, _ = _run(api, A, B, dtype, need_b=False)
+    _, only_b, _, _ = _run(api, A, B, dtype, need_a=False)
+    assert torch.equal(da, only_a) and torch.equal(db, only_b)
+    if dtype == torch.float32:
+        A, B = (M.astype(np.float32).astype(np.float64) for M in (A, B))
+    ra, rb, sa, sb = _reference(oracle_mod, A, B, W)
+    assert max_rel_err(da.double().cpu().numpy(), ra, sa) <= tol
+    assert max_rel_err(db.double().cpu().numpy(), rb, sb) <= tol
+
+
+@pytest.mark.parametrize("kind", ["stencil", "power", "short"])
+def test_searched_rows(api, oracle_mod, kind):
+    """Products that staged rows or a buffer in chunks would slow down: a stencil
+    of three chunks (a search per term of each gradient), a power-law graph and
+    uniform rows of few products (one search for both, then the columns).  dA
+    alone is one launch, and the same bits."""
+    rng = np.random.default_rng(2)
+    if kind == "stencil":
+        A = gen.laplacian_3d(80)
+    elif kind == "power":
+        A = gen.rmat(11, 16, seed=3)
+    else:
+        A = gen.random_rows(20000, 20000, rng.integers(6, 13, 20000), rng)
+    da, db, n, W = _run(api, A, A, torch.float64)
+    assert n == 2
+    only_a, _, n, _ = _run(api, A, A, torch.float64, need_b=False)
+    assert n == 1 and torch.equal(da, only_a)
+    ra, rb, sa, sb = _reference(oracle_mod, A, A, W)
+    assert max_rel_err(da.cpu().numpy(), ra, sa) <= 1e-12
+    assert max_rel_err(db.cpu().numpy(), rb, sb) <= 1e-12
+
+
 # (4500, 4000): 18 M products, more than one chunk of the buffer
 @pytest.mark.parametrize("terms,width", [(129, 64), (256, 64), (512, 64), (4096, 300), (4500, 4000)])
 def test_long_sums_keep_their_chains(api, terms, width):
