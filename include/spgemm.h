@@ -254,10 +254,11 @@ spgemm_status spgemm_plan_check(spgemm_plan* plan, spgemm_stream_t stream);
  * every call): db_vals by one chain of fused multiply-adds for at most 128
  * terms (nonzeros of A's column), otherwise by 32 chains of every 32nd term and
  * a fixed tree; da_vals by chains of at most 128 terms and a fixed tree.
- * db_vals uses a buffer of at most 128 MB in the plan's workspace: calls on
- * one plan follow one another on the GPU whatever streams they are given; a
- * graph captured from this call must not run beside another of the plan's.
- * Does not block, allocates nothing. */
+ * db_vals may pass through a buffer in the plan's workspace (at most 64 MB and
+ * the longest row of B): such calls on one plan follow one another on the GPU,
+ * whatever streams they are given.  A captured call does not use the buffer, so
+ * its graph may run beside any other call of the plan.  Does not block,
+ * allocates nothing. */
 spgemm_status spgemm_backward(spgemm_plan* plan, const void* a_vals, const void* b_vals,
                               const int32_t* c_row_ptr, const int32_t* c_col_idx,
                               const void* dc_vals, void* da_vals, void* db_vals,

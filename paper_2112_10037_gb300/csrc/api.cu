@@ -36,7 +36,7 @@ struct spgemm_plan {
   void* grad_buf = nullptr;
   long long grad_buf_entries = 0;
   std::mutex grad_mu;                // calls that use the buffer follow one another
-  cudaEvent_t grad_done = nullptr;   // end of the last one outside a capture
+  cudaEvent_t grad_done = nullptr;   // end of the last one
   // host state
   sg::PathBins pb{};
   sg::Tuning tu{};
@@ -781,7 +781,7 @@ spgemm_status spgemm_backward(spgemm_plan* p, const void* a_vals, const void* b_
   cudaError_t e = cudaSuccess;
   if (db_vals && p->B.nnz > 0 && p->mloc <= 0)
     e = cudaMemsetAsync(db_vals, 0, (size_t)p->B.nnz * (p->opts.dtype == SPGEMM_F32 ? 4 : 8), c.stream);
-  sg::GradArgs g;
+  sg::GradArgs g{};
   g.A = p->A;
   g.B = p->B;
   g.ri = rowinfo_of(p);
@@ -797,23 +797,26 @@ spgemm_status spgemm_backward(spgemm_plan* p, const void* a_vals, const void* b_
   g.buf = p->grad_buf;
   g.buf_entries = p->grad_buf_entries;
   if (e == cudaSuccess && p->mloc > 0) {
-    // the product buffer serves one call at a time: the launches of a call are
-    // not mixed with another thread's, and every call waits for the last one
-    // (not inside a capture, which takes no outside event).  Equal handles do
-    // not make the wait unnecessary: the per-thread stream has one handle for
-    // a different stream in every thread, and a destroyed stream's handle may
-    // come back for a new one
-    std::lock_guard<std::mutex> lock(p->grad_mu);
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    const bool order = p->grad_buf_entries > 0 && db_vals;
-    if (order) e = cudaStreamIsCapturing(c.stream, &cs);
-    const bool eager = order && cs == cudaStreamCaptureStatusNone;
-    if (e == cudaSuccess && eager && !p->grad_done)
+    if (db_vals && g.buf_entries > 0) e = cudaStreamIsCapturing(c.stream, &cs);
+    g.captured = cs != cudaStreamCaptureStatusNone;
+    if (e != cudaSuccess) return SPGEMM_ERR_CUDA;
+    if (!sg::grad_uses_buffer(p->opts.dtype, g, da_vals != nullptr, db_vals != nullptr)) {
+      e = sg::launch_backward(c, p->opts.dtype, g, a_vals, b_vals, dc_vals, da_vals, db_vals);
+      return e == cudaSuccess ? SPGEMM_OK : SPGEMM_ERR_CUDA;
+    }
+    // the product buffer serves one call at a time: the launches of a call are
+    // not mixed with another thread's, and every call waits for the last one.
+    // Equal handles do not make the wait unnecessary: the per-thread stream has
+    // one handle for a different stream in every thread, and a destroyed
+    // stream's handle may come back for a new one
+    std::lock_guard<std::mutex> lock(p->grad_mu);
+    if (!p->grad_done)
       e = cudaEventCreateWithFlags(&p->grad_done, cudaEventDisableTiming);
-    else if (e == cudaSuccess && eager)
+    else
       e = cudaStreamWaitEvent(c.stream, p->grad_done, 0);
     if (e == cudaSuccess) e = sg::launch_backward(c, p->opts.dtype, g, a_vals, b_vals, dc_vals, da_vals, db_vals);
-    if (eager && p->grad_done) {  // after a failure too: some of its launches may run
+    if (p->grad_done) {  // after a failure too: some of its launches may run
       const cudaError_t r = cudaEventRecord(p->grad_done, c.stream);
       if (e == cudaSuccess) e = r;
     }

@@ -825,10 +825,14 @@ struct GradRoute {
 // 0.44, 11 (FP32) 0.48 and 0.41, 13 (200,000 columns, 16 to 48 a row, FP64) 13.0
 // and 11.1, 16 (300,000 columns, 2 to 10, FP64) 0.28 and 0.35, 25 (200,000 columns
 // in FP32) 6.7 and 9.9, 40 (65,536 columns, 32, FP64) 1.2 and 3.0.  Long sums do
-// not go on from chunk to chunk (k_grad_cols).
+// not go on from chunk to chunk (k_grad_cols).  A captured call stays off the
+// buffer: nothing orders its replays against the plan's other calls.  Whichever
+// way, dB's sums have the same order and bits.
 template <typename T>
-static GradRoute grad_route(const GradArgs& g, bool da, bool db, bool has_buffer) {
+static GradRoute grad_route(const GradArgs& g, bool da, bool db) {
   GradRoute r{};
+  // none: rows of B longer than one, and then no product offsets either
+  const bool has_buffer = g.buf_entries > 0 && g.B.nnz > 0;
   int hi = 0;
   long long all = 0;
   for (int b = 1; b < NBINS; ++b) {
@@ -852,7 +856,7 @@ static GradRoute grad_route(const GradArgs& g, bool da, bool db, bool has_buffer
              (r.lanes == 32 || g.max_row_b <= GRAD_LANE_MAX);
   const long long longest = g.B.ncols < g.B.nnz ? g.B.ncols : g.B.nnz;
   r.chunk = g.buf_entries - longest;
-  r.buffered = db && has_buffer && (da || r.staged || g.max_col > GRAD_LANE_MAX);
+  r.buffered = db && has_buffer && !g.captured && (da || r.staged || g.max_col > GRAD_LANE_MAX);
   if (r.buffered && g.total > r.chunk) {
     const double chunks = (double)((g.total + r.chunk - 1) / r.chunk);
     const double terms = (double)g.total / (chunks * (double)g.B.nnz);
@@ -865,8 +869,7 @@ static GradRoute grad_route(const GradArgs& g, bool da, bool db, bool has_buffer
 template <typename T>
 static cudaError_t backward_t(const LaunchCtx& c, const GradArgs& g, const T* av, const T* bv, const T* dc, T* da,
                               T* db) {
-  // no buffer: rows of B longer than one, which have no product offsets either
-  const GradRoute r = grad_route<T>(g, da != nullptr, db != nullptr, g.buf_entries > 0 && g.B.nnz > 0);
+  const GradRoute r = grad_route<T>(g, da != nullptr, db != nullptr);
   if (db && g.B.nnz > 0 && !r.buffered) {
     const cudaError_t e = search_db(c, g, av, dc, db);
     if (e != cudaSuccess) return e;
@@ -904,6 +907,10 @@ static cudaError_t backward_t(const LaunchCtx& c, const GradArgs& g, const T* av
     if ((e = cudaGetLastError()) != cudaSuccess || last) return e;
   }
   return cudaSuccess;
+}
+
+bool grad_uses_buffer(int dtype, const GradArgs& g, bool da, bool db) {
+  return (dtype == SPGEMM_F32 ? grad_route<float>(g, da, db) : grad_route<double>(g, da, db)).buffered;
 }
 
 cudaError_t launch_backward(const LaunchCtx& c, int dtype, const GradArgs& g, const void* av, const void* bv,

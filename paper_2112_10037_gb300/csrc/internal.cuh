@@ -370,7 +370,11 @@ struct GradArgs {
   const int* hist;   // host: rows per bin
   void* buf;
   long long buf_entries;
+  bool captured;     // recorded into a graph: no use of buf
 };
+// Whether this call writes the product buffer (then it must not run beside
+// another that does).
+bool grad_uses_buffer(int dtype, const GradArgs& g, bool da, bool db);
 long long grad_buffer_entries(long long nnz_a, long long nnz_b, long long ncols_b, int vbytes);
 cudaError_t launch_grad_offsets(const LaunchCtx& c, const Csr& A, const Csr& B, long long row_begin, long long mloc,
                                 const long long* prod, const int32_t* t_rp, const int32_t* t_ci, const int32_t* t_src,

@@ -258,3 +258,51 @@ def test_per_thread_streams(api):
         for da, db in pairs:
             assert torch.equal(da, alone[i][0]) and torch.equal(db, alone[i][1])
     plan.close()
+
+
+@pytest.mark.parametrize("kind,dtype", [("staged", torch.float64), ("chunks", torch.float32), ("long", torch.float64)])
+def test_captured_calls_run_beside_others(api, kind, dtype):
+    """Two graphs captured from one plan's adjoint and eager calls, all at once
+    on three streams: the bits of an eager call alone.  Rows staged in shared
+    memory, two chunks of the buffer, sums of more than 128 terms."""
+    from paper_2112_10037_gb300 import _native as nat
+    rng = np.random.default_rng(5)
+    if kind == "staged":
+        A = gen.random_rows(3000, 3000, np.full(3000, 40), rng)
+    elif kind == "chunks":
+        A = gen.random_rows(20000, 20000, np.full(20000, 32), rng)
+    else:
+        A = gen.random_rows(2000, 90, rng.integers(2, 20, 2000), rng)
+    B = gen.random_rows(90, 4000, np.full(90, 60), rng) if kind == "long" else A
+    dA, dB = api.DeviceCSR.from_host(A, dtype=dtype), api.DeviceCSR.from_host(B, dtype=dtype)
+    plan = api.Plan(dA, dB, dtype=dtype, backward=True)
+    _, nnz = plan.symbolic()
+    plan.numeric(dA.vals, dB.vals)
+    gen_ = torch.Generator(device="cuda").manual_seed(1)
+    ws = [torch.randn(nnz, generator=gen_, device="cuda", dtype=dtype) for _ in range(3)]
+    alone = [plan.backward(dA.vals, dB.vals, w) for w in ws]
+    outs = [(torch.zeros_like(dA.vals), torch.zeros_like(dB.vals)) for _ in ws]
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in ws]
+
+    def call(i):
+        nat.spgemm_backward(plan.handle, dA.vals.data_ptr(), dB.vals.data_ptr(), plan.row_ptr.data_ptr(),
+                            plan.col_idx.data_ptr(), ws[i].data_ptr(), outs[i][0].data_ptr(), outs[i][1].data_ptr(),
+                            int(streams[i].cuda_stream))
+
+    graphs = []
+    for i in range(2):
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=streams[i]):
+            call(i)
+        graphs.append(g)
+    for _ in range(10):
+        for i in range(2):
+            with torch.cuda.stream(streams[i]):
+                graphs[i].replay()
+        call(2)
+    torch.cuda.synchronize()
+    plan.check()
+    for (da, db), (ra, rb) in zip(outs, alone):
+        assert torch.equal(da, ra) and torch.equal(db, rb)
+    plan.close()
