@@ -41,3 +41,22 @@ def test_tile_edges(api, ncols, nnz):
         assert np.array_equal(T.vals.cpu().numpy(), M.vals[order])
         if want_src:
             assert np.array_equal(src.cpu().numpy(), order)
+
+
+# rows walked from entry to entry (below 16 rows per entry and tile), searched
+# per entry (above), and both in one matrix
+@pytest.mark.parametrize("nrows,nnz", [(32_000, 2048), (40_000, 2048), (3_000_000, 1), (3_000_000, 2), (3_000_000, 5001),
+                                       (70_000, 4097)])
+@pytest.mark.parametrize("ncols", [600, 65536])
+def test_far_more_rows_than_entries(api, nrows, nnz, ncols):
+    rng = np.random.default_rng(nnz)
+    lens = np.zeros(nrows, np.int64)
+    at = np.concatenate([[0, nrows - 1], rng.integers(0, nrows, max(0, nnz - 2))])[:nnz]  # both ends
+    np.add.at(lens, at[: nnz // 2], 1)
+    np.add.at(lens, at[nnz // 2:] // 50, 1)  # half of them among the first rows
+    M = gen.random_rows(nrows, ncols, np.minimum(lens, ncols), rng, values="int")
+    T = api.transpose(api.DeviceCSR.from_host(M))
+    order = np.argsort(M.col_idx, kind="stable")
+    assert np.array_equal(T.row_ptr.cpu().numpy(), np.concatenate([[0], np.cumsum(np.bincount(M.col_idx, minlength=ncols))]))
+    assert np.array_equal(T.col_idx.cpu().numpy(), np.repeat(np.arange(nrows), np.diff(M.row_ptr))[order])
+    assert np.array_equal(T.vals.cpu().numpy(), M.vals[order])
