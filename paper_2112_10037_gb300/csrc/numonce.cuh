@@ -214,20 +214,25 @@ k_num_once(Csr A, Csr B, const T* __restrict__ av, const T* __restrict__ bv, Row
     for (int t = tid; t < HW; t += NT) marks[t] = 0u;
 
     while (true) {  // windows of W columns from base on
-      // ---- presence bits; owners are the products that set them
+      // ---- presence bits; owners are the products that set them.  Columns
+      // outside [base, cmx], only in unsorted rows of B, would use words of the
+      // bitmap that have no rank and are not cleared: reported and left out
+      const int nwords = (min(W, cmx - base + 1) + 31) >> 5;
       unsigned own = 0, here = 0;
       int next = INT_MAX;
 #pragma unroll
       for (int u = 0; u < E; ++u) {
+        if (col[u] < 0) continue;  // no product, or emitted with an earlier window
         const int j = col[u] - base;
-        if (j >= 0) {  // col -1: no product, or emitted with an earlier window
-          if (j < W) {
-            const unsigned m = 1u << (j & 31);
-            here |= 1u << u;
-            if (!(atomicOr(&bits[j >> 5], m) & m)) own |= 1u << u;
-          } else {
-            next = min(next, col[u]);
-          }
+        if ((j >> 5) >= 0 && (j >> 5) < nwords) {
+          const unsigned m = 1u << (j & 31);
+          here |= 1u << u;
+          if (!(atomicOr(&bits[j >> 5], m) & m)) own |= 1u << u;
+        } else if (j >= W && col[u] <= cmx) {
+          next = min(next, col[u]);
+        } else {
+          atomicOr(err, EB_UNSORTED);
+          col[u] = -1;
         }
       }
       next = warp_min(next);
@@ -235,7 +240,6 @@ k_num_once(Csr A, Csr B, const T* __restrict__ av, const T* __restrict__ bv, Row
       __syncthreads();
 
       // ---- prefix of the words' popcounts; a lane takes 8 consecutive words
-      const int nwords = (min(W, cmx - base + 1) + 31) >> 5;
       const int tiles = (nwords + 255) >> 8, per = (tiles + NW - 1) / NW;
       const int t0 = min(tiles, warp * per), t1 = min(tiles, t0 + per);
       int sum = 0;

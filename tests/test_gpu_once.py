@@ -110,3 +110,23 @@ def test_block_window_before_the_registers(api, oracle_mod, ncols, num_block_min
     R, S = oracle_with_scale(oracle_mod, A, B)
     assert_structure_equal(got, R)
     assert_values_close(got.vals, R.vals, S)
+
+
+@pytest.mark.parametrize("ncols", [5000, 70001])
+def test_unsorted_rows_of_b_are_reported(api, oracle_mod, ncols):
+    """Rows of B whose last column is their second smallest (the span that the
+    analysis takes from their ends is too narrow), not validated: an error, and
+    nothing outside the blocks' bitmaps."""
+    from paper_2112_10037_gb300 import _native as nat
+    A, B = _operands(ncols, "spread", 9)
+    A = oracle_mod.select_rows(A, np.flatnonzero(np.array(EDGES) <= 2048))
+    for k in range(128):
+        s, e = B.row_ptr[k], B.row_ptr[k + 1]
+        B.col_idx[s + 1:e] = B.col_idx[s + 1:e][::-1].copy()
+    dA, dB = api.DeviceCSR.from_host(A), api.DeviceCSR.from_host(B)
+    with pytest.raises(nat.SpgemmError) as e:
+        plan = api.Plan(dA, dB)
+        plan.symbolic()
+        plan.numeric(dA.vals, dB.vals)
+        plan.check()
+    assert nat.STATUS_NAMES[e.value.status] == "SPGEMM_ERR_UNSORTED_INPUT"
