@@ -155,11 +155,17 @@ static size_t tr_scatter_smem(int bits, int vbytes, bool pos, int items) {
          (sizeof(int) * (pos ? 3 : 2) + (size_t)vbytes) * (size_t)tr_tile(items);
 }
 
-// t_rp[k] = first position whose column is at least k, from the sorted columns
-// (out-of-range ones, reported by the first pass, write nothing).  Long gaps
-// of empty columns are filled by the whole warp.
+// t_rp[k] = first position whose column is at least k, from the sorted columns.
+// Long gaps of empty columns are filled by the whole warp.  Columns out of range
+// (reported by the first pass) are not in order, and every step down would be
+// such a gap: M^T has empty rows then.
 __global__ void __launch_bounds__(256) k_tr_row_ptr(const int32_t* __restrict__ key, long long nnz, long long n,
-                                                    int32_t* __restrict__ t_rp) {
+                                                    int32_t* __restrict__ t_rp, const DevStats* st) {
+  if (block_skip(st)) {
+    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k <= n; k += (long long)gridDim.x * blockDim.x)
+      t_rp[k] = 0;
+    return;
+  }
   const int lane = lane_id();
   constexpr int U = 8;  // positions per lane and step, their loads in flight together
   const long long step = (long long)gridDim.x * (blockDim.x >> 5) * 32 * U;
@@ -490,7 +496,7 @@ cudaError_t launch_transpose(const LaunchCtx& c, long long m, long long n, long 
     kin = ko; rin = ro; pin = po; vin = vo;
   }
   if (sorted) {
-    k_tr_row_ptr<<<grid_cap(nnz + 1, 2048, c.nsm), 256, 0, c.stream>>>(sorted, nnz, n, t_rp);
+    k_tr_row_ptr<<<grid_cap(nnz + 1, 2048, c.nsm), 256, 0, c.stream>>>(sorted, nnz, n, t_rp, c.st);
     count_launch(c);
   }
   return cudaGetLastError();

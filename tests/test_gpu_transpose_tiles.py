@@ -43,6 +43,27 @@ def test_tile_edges(api, ncols, nnz):
             assert np.array_equal(src.cpu().numpy(), order)
 
 
+def test_columns_out_of_range_leave_empty_rows(api):
+    """Every other entry's column is out of range: an error, and a row pointer
+    of an empty matrix (every step down of the columns would fill rows)."""
+    from paper_2112_10037_gb300 import _native as nat
+    n, nnz = 10_000, 3000
+    rp = torch.tensor([0, nnz], dtype=torch.int32, device="cuda")
+    ci = torch.arange(nnz, dtype=torch.int32, device="cuda")
+    ci[1::2] += 3 << 16
+    t_rp = torch.full((n + 1,), -1, dtype=torch.int32, device="cuda")
+    t_ci = torch.zeros(nnz, dtype=torch.int32, device="cuda")
+    M = api.DeviceCSR(1, n, rp, ci, torch.ones(nnz, dtype=torch.float64, device="cuda")).c_struct()
+    size = nat.spgemm_transpose_workspace_size(1, n, nnz)
+    ws = torch.empty(size, dtype=torch.uint8, device="cuda")
+    s = int(torch.cuda.current_stream().cuda_stream)
+    nat.spgemm_transpose(M, 0, t_rp.data_ptr(), t_ci.data_ptr(), 0, 0, ws.data_ptr(), size, s)
+    with pytest.raises(nat.SpgemmError) as e:
+        nat.spgemm_transpose_check(ws.data_ptr(), s)
+    assert nat.STATUS_NAMES[e.value.status] == "SPGEMM_ERR_UNSORTED_INPUT"
+    assert not t_rp.any()
+
+
 # rows walked from entry to entry (below 16 rows per entry and tile), searched
 # per entry (above), and both in one matrix
 @pytest.mark.parametrize("nrows,nnz", [(32_000, 2048), (40_000, 2048), (3_000_000, 1), (3_000_000, 2), (3_000_000, 5001),
