@@ -130,7 +130,8 @@ typedef struct spgemm_opts {
                           each row of C then the semiring sum over A(i,k) of the products
                           A(i,k) (x) B(k,:) on the same pattern (Sec. 2.2 with + and *
                           replaced; min, max and or do not depend on the order of the sums,
-                          so those values are exact).  With another semiring sort_max,
+                          so those values are exact; a product that is not a number
+                          counts for nothing in min and max).  With another semiring sort_max,
                           rank_min, split_min, window_warp, window_block and block_warps
                           are ignored (defaults; no rank-compacted accumulator, no split
                           rows), and backward must be 0 */

@@ -291,7 +291,7 @@ k_num_once(Csr A, Csr B, const T* __restrict__ av, const T* __restrict__ bv, Row
           const int j = col[u] - base;
           rk[u] = pre[j >> 5] + __popc(bits[j >> 5] & ((1u << (j & 31)) - 1u));
           if (own >> u & 1u) {
-            acc[rk[u]] = val[u];
+            acc[rk[u]] = Ops::first(val[u]);
             ccol[rk[u]] = col[u];
           }
         }

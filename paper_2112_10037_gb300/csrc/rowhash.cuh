@@ -269,7 +269,7 @@ __device__ __forceinline__ void hash_num_rows(const Csr& A, const Csr& B, const 
     between();
 #pragma unroll
     for (int s = 0; s < E; ++s)
-      if (fresh[s]) val[slot[s]] = pv[s];
+      if (fresh[s]) val[slot[s]] = SrOps<T, SR>::first(pv[s]);
     __syncwarp();
 #pragma unroll
     for (int s = 0; s < E; ++s)

@@ -125,7 +125,7 @@ __device__ __forceinline__ void lane_hash_rows(const Csr& A, const Csr& B, const
             if (fresh) ++nd;
             if (NUM) {
               T* vp = &vals[h * 32 + lane];
-              *vp = fresh ? SrOps<T, SR>::mul(a, bb[u]) : SrOps<T, SR>::madd(a, bb[u], *vp);
+              *vp = fresh ? SrOps<T, SR>::first(SrOps<T, SR>::mul(a, bb[u])) : SrOps<T, SR>::madd(a, bb[u], *vp);
             }
           }
         }

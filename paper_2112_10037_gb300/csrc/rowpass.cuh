@@ -96,7 +96,7 @@ __device__ __forceinline__ void tiny_rows(const Csr& A, const Csr& B, const T* _
         if (q >= 0 && q < tot) {
           const int bi = os + q - oex;
           col[s] = B.ci[bi];
-          if (NUM) val[s] = SrOps<T, SR>::mul(oa, bv[bi]);
+          if (NUM) val[s] = SrOps<T, SR>::first(SrOps<T, SR>::mul(oa, bv[bi]));
         }
       }
       done += tot;

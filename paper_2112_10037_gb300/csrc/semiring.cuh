@@ -6,7 +6,10 @@
 // operands, so those products are exact.
 //
 // Each policy gives the sum's identity (the cleared state of an
-// accumulator word), the product, the sum, their fusion acc (+) a (*) b, and
+// accumulator word), the product, the sum, their fusion acc (+) a (*) b, what
+// an accumulator holds after its first product (first: the product itself, but
+// in min-plus and max-plus the identity where the product is not a number, so
+// that a NaN counts for nothing whichever product comes first), and
 // shared-memory updates that other lanes may race with: red_value (*p (+)=
 // x), red_shared (*p (+)= a (*) b) and madd_shared (the same, returning
 // whether the word still held the identity when read, i.e. whether this may
@@ -54,6 +57,7 @@ template <typename T> struct SrOps<T, SPGEMM_PLUS_TIMES> {
   __device__ static T zero() { return T(0); }
   __device__ static bool cleared(T v) { return is_cleared(v); }
   __device__ static T mul(T a, T b) { return a * b; }
+  __device__ static T first(T x) { return x; }
   __device__ static T add(T x, T y) { return x + y; }
   __device__ static T madd(T a, T b, T acc) { return fma(a, b, acc); }
   __device__ static void red_value(T* p, T x, uint32_t*) { red_add_shared(p, x); }
@@ -66,6 +70,7 @@ template <typename T> struct SrOps<T, SPGEMM_MIN_PLUS> {
   __device__ static bool cleared(T v) { return sr_bits(v) == sr_bits(zero()); }
   __device__ static T mul(T a, T b) { return a + b; }
   __device__ static T add(T x, T y) { return y < x ? y : x; }
+  __device__ static T first(T x) { return add(zero(), x); }
   __device__ static T madd(T a, T b, T acc) { return add(acc, a + b); }
   __device__ static void red_value(T* p, T x, uint32_t* err) { minmax_shared<true>(p, x, zero(), err); }
   __device__ static void red_shared(T* p, T a, T b, uint32_t* err) { minmax_shared<true>(p, a + b, zero(), err); }
@@ -79,6 +84,7 @@ template <typename T> struct SrOps<T, SPGEMM_MAX_PLUS> {
   __device__ static bool cleared(T v) { return sr_bits(v) == sr_bits(zero()); }
   __device__ static T mul(T a, T b) { return a + b; }
   __device__ static T add(T x, T y) { return y > x ? y : x; }
+  __device__ static T first(T x) { return add(zero(), x); }
   __device__ static T madd(T a, T b, T acc) { return add(acc, a + b); }
   __device__ static void red_value(T* p, T x, uint32_t* err) { minmax_shared<false>(p, x, zero(), err); }
   __device__ static void red_shared(T* p, T a, T b, uint32_t* err) { minmax_shared<false>(p, a + b, zero(), err); }
@@ -91,6 +97,7 @@ template <typename T> struct SrOps<T, SPGEMM_OR_AND> {
   __device__ static T zero() { return T(0); }
   __device__ static bool cleared(T v) { return is_cleared(v); }
   __device__ static T mul(T a, T b) { return (a != T(0) && b != T(0)) ? T(1) : T(0); }
+  __device__ static T first(T x) { return x; }
   __device__ static T add(T x, T y) { return (x != T(0) || y != T(0)) ? T(1) : T(0); }
   __device__ static T madd(T a, T b, T acc) { return add(acc, mul(a, b)); }
   // every writer stores the same 1, so racing stores need no atomics

@@ -184,3 +184,33 @@ def test_semiring_degenerate_and_errors(api, oracle_mod):
     with pytest.raises(nat.SpgemmError) as ei:
         nat.spgemm_semiring(A.c_struct(), B.c_struct(), M.c_struct(), 0, 7, 0, 0)
     assert ei.value.status == 1
+
+
+# (rows, nonzeros of a row of A, of B, columns): register sort, warp tables,
+# merged lanes, lane tables, long warp tables, block registers, bands
+@pytest.mark.parametrize("shape", [(400, 3, 4, 9), (400, 5, 8, 20), (40_000, 5, 8, 20), (160_000, 9, 5, 20),
+                                   (400, 12, 9, 50), (300, 30, 40, 500), (40, 100, 100, 900)])
+@pytest.mark.parametrize("semiring", SEMIRINGS)
+def test_nan_counts_for_nothing(api, oracle_mod, semiring, shape):
+    """Products that are not a number (NaN factors, infinities of both signs)
+    leave an entry to its other products, whichever kernel forms it and whichever
+    product comes first; an entry of such products alone holds the identity."""
+    m, na, nb, n = shape
+    rng = np.random.default_rng(m)
+    A = gen.random_rows(m, 300, np.full(m, na), rng)
+    B = gen.random_rows(300, n, np.full(300, nb), rng)
+    A.vals[rng.random(A.nnz) < 0.4] = np.nan
+    A.vals[rng.random(A.nnz) < 0.1] = np.inf
+    B.vals[rng.random(B.nnz) < 0.3] = np.nan
+    B.vals[rng.random(B.nnz) < 0.1] = -np.inf
+    C = oracle_mod.spgemm(A, B)
+    ref = oracle_mod.masked_semiring(A, B, C, semiring)
+    for dtype in (torch.float64, torch.float32):
+        for _ in range(3):
+            got = api.spgemm_semiring(api.DeviceCSR.from_host(A, dtype=dtype), api.DeviceCSR.from_host(B, dtype=dtype),
+                                      semiring, dtype=dtype).to_host()
+            assert np.array_equal(got.col_idx, C.col_idx)
+            want = ref if dtype == torch.float64 else oracle_mod.masked_semiring(
+                A.astype(np.float32).astype(np.float64), B.astype(np.float32).astype(np.float64), C,
+                semiring).astype(np.float32)
+            assert np.array_equal(got.vals, want)
