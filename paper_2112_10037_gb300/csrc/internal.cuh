@@ -204,6 +204,22 @@ __device__ __forceinline__ bool fma_shared(float* p, float a, float b, uint32_t*
   return true;
 }
 
+// The same in FP32 with one rounding, by compare-and-swap: for rows whose
+// products meet seldom, where a product's own rounding is much of the error.
+__device__ __forceinline__ void fma_shared_cas(float* p, float a, float b, uint32_t* err) {
+  const unsigned s = (unsigned)__cvta_generic_to_shared(p);
+  unsigned old;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(old) : "r"(s) : "memory");
+  for (int it = 0; it < CAS_RETRY_LIMIT; ++it) {
+    const unsigned nv = __float_as_uint(fmaf(a, b, __uint_as_float(old)));
+    unsigned prev;
+    asm volatile("atom.shared.cas.b32 %0, [%1], %2, %3;" : "=r"(prev) : "r"(s), "r"(old), "r"(nv) : "memory");
+    if (prev == old) return;
+    old = prev;
+  }
+  atomicOr(err, EB_INTERNAL);  // never expected: each failed swap is another update's success
+}
+
 // Index of the first lane whose inclusive prefix `incl` exceeds p (incl is
 // non-decreasing over the 32 lanes).  Every lane must call it.
 __device__ __forceinline__ int warp_owner(int incl, int p) {

@@ -15,7 +15,7 @@
 //     column's owner (the others found the bit set),
 //  3. a prefix sum of the words' popcounts turns (word, bit) into the rank,
 //  4. owners store their product and column at their rank, the others add
-//     theirs there with a shared-memory reduction after a barrier,
+//     theirs there (HeldProduct in semiring.cuh) after a barrier,
 //  5. the row leaves in one coalesced copy.
 //
 // A bitmap spans up to 262,144 columns; a wider row takes the next
@@ -84,7 +84,6 @@ __global__ void __launch_bounds__(NT, once_blocks_per_sm<NT>())
 k_num_once(Csr A, Csr B, const T* __restrict__ av, const T* __restrict__ bv, RowInfo ri, const DevStats* st,
            int bin_lo, int bin_hi, int wlog, const int32_t* __restrict__ c_rp, int32_t* __restrict__ c_ci,
            T* __restrict__ c_v, uint32_t* err) {
-  using Ops = SrOps<T, SR>;
   constexpr int E = ONCE_E, CAP = NT * E, NW = NT / 32, HW = CAP / 32;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int s_lb, s_le;
@@ -173,7 +172,7 @@ k_num_once(Csr A, Csr B, const T* __restrict__ av, const T* __restrict__ bv, Row
 
     // ---- products: batches of 32, 8 consecutive batches per warp
     int col[E];
-    T val[E];
+    HeldProduct<T, SR> pv[E];
     {
       int k0 = 0;  // segments that start before this warp's products
       for (int t = lane; t < warp * E; t += 32) k0 += __popc(marks[t]);
@@ -195,7 +194,8 @@ k_num_once(Csr A, Csr B, const T* __restrict__ av, const T* __restrict__ bv, Row
         }
       }
 #pragma unroll
-      for (int u = 0; u < E; ++u) val[u] = col[u] >= 0 ? Ops::mul(acc[ks[u]], bb[u]) : T(0);
+      for (int u = 0; u < E; ++u)
+        if (col[u] >= 0) pv[u].set(acc[ks[u]], bb[u]);
     }
     // the next row's first nonzeros and the row after that, in flight from here on
     m0 = T(0);
@@ -282,26 +282,29 @@ k_num_once(Csr A, Csr B, const T* __restrict__ av, const T* __restrict__ bv, Row
       }
       __syncthreads();
 
-      // ---- ranks: owners store, the others add after the barrier
-      int rk[E];
+      // ---- ranks: owners store, the others (col -2 - rank from here) add
+      // after the barrier
 #pragma unroll
       for (int u = 0; u < E; ++u) {
-        rk[u] = 0;
         if (here >> u & 1u) {
           const int j = col[u] - base;
-          rk[u] = pre[j >> 5] + __popc(bits[j >> 5] & ((1u << (j & 31)) - 1u));
+          const int rk = pre[j >> 5] + __popc(bits[j >> 5] & ((1u << (j & 31)) - 1u));
           if (own >> u & 1u) {
-            acc[rk[u]] = Ops::first(val[u]);
-            ccol[rk[u]] = col[u];
+            acc[rk] = pv[u].first();
+            ccol[rk] = col[u];
+            col[u] = -1;
+          } else {
+            col[u] = -2 - rk;
           }
         }
       }
       __syncthreads();
 #pragma unroll
-      for (int u = 0; u < E; ++u) {
-        if ((here & ~own) >> u & 1u) Ops::red_value(&acc[rk[u]], val[u], err);
-        if (here >> u & 1u) col[u] = -1;
-      }
+      for (int u = 0; u < E; ++u)
+        if (col[u] < -1) {
+          pv[u].add_to(&acc[-2 - col[u]], err);
+          col[u] = -1;
+        }
       // the bitmap is clear again for the next window or row
       for (int t = tid * 4; t < nwords; t += NT * 4) *reinterpret_cast<uint4*>(bits + t) = make_uint4(0, 0, 0, 0);
       __syncthreads();

@@ -83,18 +83,15 @@ __device__ __forceinline__ void b_bounds(const Csr& B, int k, int* sb, int* len)
 // gives every entry's first product, and each lane finds the entry owning
 // its product by a search over those sums.  The first chunk's operands come
 // preloaded in c0; later chunks (rows of more than 32 nonzeros) load their
-// own.  NUM: pv = A(i,k) * B(k,j), one rounded multiply per product.  Empty
-// slots hold column INT_MAX.  Returns the row's product count.
+// own.  NUM: pv holds A(i,k) * B(k,j).  Empty slots hold column INT_MAX.
+// Returns the row's product count.
 template <int E, bool NUM, typename T, int SR = SPGEMM_PLUS_TIMES>
 __device__ __forceinline__ int hash_gather(const Csr& A, const Csr& B, const T* __restrict__ av,
                                            const T* __restrict__ bv, int a0, int a1, const Chunk0<T>& c0,
-                                           int (&col)[E], T (&pv)[E]) {
+                                           int (&col)[E], HeldProduct<T, SR> (&pv)[E]) {
   const int lane = lane_id();
 #pragma unroll
-  for (int s = 0; s < E; ++s) {
-    col[s] = INT_MAX;
-    pv[s] = T(0);
-  }
+  for (int s = 0; s < E; ++s) col[s] = INT_MAX;
   int done = 0;
   for (int e0 = a0; e0 < a1; e0 += 32) {
     int sb = c0.sb, len = c0.len;
@@ -124,7 +121,7 @@ __device__ __forceinline__ int hash_gather(const Csr& A, const Csr& B, const T* 
       if (q >= 0 && q < tot) {
         const int bi = os + q - oex;
         col[s] = B.ci[bi];
-        if (NUM) pv[s] = SrOps<T, SR>::mul(oa, bv[bi]);
+        if (NUM) pv[s].set(oa, bv[bi]);
       }
     }
     done += tot;
@@ -202,7 +199,7 @@ __device__ __forceinline__ void hash_sym_rows(const Csr& A, const Csr& B, const 
   hash_row_loop<false, float>(A, B, nullptr, ri, lb, le, w, nw,
                               [&](int r, int a0, int a1, const Chunk0<float>& c0, auto& between) {
     int col[E];
-    float pv[E];
+    HeldProduct<float, SPGEMM_PLUS_TIMES> pv[E];
     const int P = hash_gather<E, false, float>(A, B, nullptr, nullptr, a0, a1, c0, col, pv);
     if (P > 32 * E && lane == 0) atomicOr(err, EB_INTERNAL);  // the row's bin rules this out
     int slot[E];
@@ -236,7 +233,7 @@ struct HashWarp {
 // Numeric pass: C's columns (ascending) and values for each row, at the
 // positions [c_rp[r], c_rp[r+1]) the symbolic pass and the scan fixed.
 // The product that claims a column's slot stores its value there; the
-// others add theirs with a shared-memory reduction after a warp barrier.
+// others are added there (HeldProduct) after a warp barrier.
 // Rows at list positions [lb, le), warp w of nw takes its share.
 template <int E, typename T, int SR = SPGEMM_PLUS_TIMES>
 __device__ __forceinline__ void hash_num_rows(const Csr& A, const Csr& B, const T* __restrict__ av,
@@ -256,7 +253,7 @@ __device__ __forceinline__ void hash_num_rows(const Csr& A, const Csr& B, const 
   hash_row_loop<true, T>(A, B, av, ri, lb, le, w, nw, [&](int r, int a0, int a1, const Chunk0<T>& c0, auto& between) {
     const int ob = c_rp[r], oe = c_rp[r + 1];
     int col[E];
-    T pv[E];
+    HeldProduct<T, SR> pv[E];
     const int P = hash_gather<E, true, T, SR>(A, B, av, bv, a0, a1, c0, col, pv);
     if (P > 32 * E && lane == 0) atomicOr(err, EB_INTERNAL);  // the row's bin rules this out
     int slot[E];
@@ -269,11 +266,11 @@ __device__ __forceinline__ void hash_num_rows(const Csr& A, const Csr& B, const 
     between();
 #pragma unroll
     for (int s = 0; s < E; ++s)
-      if (fresh[s]) val[slot[s]] = SrOps<T, SR>::first(pv[s]);
+      if (fresh[s]) val[slot[s]] = pv[s].first();
     __syncwarp();
 #pragma unroll
     for (int s = 0; s < E; ++s)
-      if (!fresh[s] && slot[s] >= 0) SrOps<T, SR>::red_value(&val[slot[s]], pv[s], err);
+      if (!fresh[s] && slot[s] >= 0) pv[s].add_to(&val[slot[s]], err);
     __syncwarp();
     // Compaction: the occupied slots, in slot order, into the list dk/dv;
     // each slot's key is cleared by the lane that read it.

@@ -130,3 +130,24 @@ def test_unsorted_rows_of_b_are_reported(api, oracle_mod, ncols):
         plan.numeric(dA.vals, dB.vals)
         plan.check()
     assert nat.STATUS_NAMES[e.value.status] == "SPGEMM_ERR_UNSORTED_INPUT"
+
+
+@pytest.mark.parametrize("width", [9, 30, 60, 100, 250, 500, 1000, 2000])
+@pytest.mark.parametrize("nrows", [40, 30_000])
+def test_fp32_products_that_meet_are_fused(api, nrows, width):
+    """Every column is x*y and -x*y: the first is rounded, the second fused, so
+    what is left is exactly the first one's rounding error, with either sign (a
+    rounded second product would leave 0).  Warp tables, lanes (many rows),
+    block registers."""
+    if nrows * width > 1_000_000:
+        nrows = 500
+    rng = np.random.default_rng(width)
+    x, y = (rng.uniform(1, 2, n).astype(np.float32) for n in (nrows, width))
+    cols = np.sort(rng.choice(70_001, width, replace=False)).astype(np.int32)
+    B = gen.CSR(2, 70_001, np.array([0, width, 2 * width], np.int32), np.tile(cols, 2), np.tile(y, 2).astype(np.float64))
+    A = gen.CSR(nrows, 2, (2 * np.arange(nrows + 1)).astype(np.int32), np.tile(np.array([0, 1], np.int32), nrows),
+                np.stack([x, -x], 1).ravel().astype(np.float64))
+    got = api.spgemm(*(api.DeviceCSR.from_host(M, dtype=torch.float32) for M in (A, B))).to_host()
+    err = (x[:, None] * y).astype(np.float64) - x[:, None].astype(np.float64) * y
+    assert np.count_nonzero(err) > 0.9 * err.size
+    assert np.array_equal(np.abs(got.vals.reshape(nrows, width).astype(np.float64)), np.abs(err))
