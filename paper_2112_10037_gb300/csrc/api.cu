@@ -1052,6 +1052,10 @@ spgemm_status spgemm_batched(int32_t n, const spgemm_csr* As, const spgemm_csr* 
   B.row_ptr = b->b_rp; B.col_idx = b->b_nnz ? b->b_ci : nullptr; B.vals = b->b_v;
   s = spgemm_analyse(&A, &B, &o, ws + L.plan, workspace_bytes - L.plan, stream, &b->plan);
   if (s != SPGEMM_OK) { delete b; return s; }
+  if (o.validate && sg::launch_batch_validate(ctx_of(b->plan, stream), n, b->d_desc, b->a_nnz, b->b_nnz) != cudaSuccess) {
+    delete b;
+    return SPGEMM_ERR_CUDA;
+  }
   *batch = b;
   return SPGEMM_OK;
 }

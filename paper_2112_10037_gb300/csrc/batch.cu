@@ -91,6 +91,38 @@ k_stack_structure(const BatchDesc* __restrict__ d, int n, int32_t* __restrict__ 
                 [](const BatchDesc&) { return 0; });
 }
 
+// Columns of every instance inside its own matrices: the stacked arrays alone
+// allow B_i the columns of the widest instance, and A_i the rows of the next
+// instance's B.  Chunks of A's entries, then of B's (only with opts.validate).
+__global__ void __launch_bounds__(STACK_THREADS)
+k_batch_validate(const BatchDesc* __restrict__ d, int n, long long total_a_nnz, long long total_b_nnz, long long c0,
+                 uint32_t* err) {
+  const bool b = blockIdx.x >= c0;
+  const long long p0 = (b ? blockIdx.x - c0 : (long long)blockIdx.x) * STACK_CHUNK + threadIdx.x;
+  const long long total = b ? total_b_nnz : total_a_nnz;
+  long long BatchDesc::*const off = b ? &BatchDesc::boff : &BatchDesc::aoff;
+  if (p0 >= total) return;
+  int i = instance_at(d, n, off, p0);
+  bool bad = false;
+  for (int u = 0; u < STACK_ITEMS; ++u) {
+    const long long p = p0 + u * STACK_THREADS;
+    if (p >= total) break;
+    while (i + 1 < n && d[i + 1].*off <= p) ++i;
+    const int c = (b ? d[i].b_ci : d[i].a_ci)[p - d[i].*off];
+    bad |= c < 0 || (long long)c >= (b ? d[i].n : d[i].k);
+  }
+  if (bad) atomicOr(err, EB_UNSORTED);
+}
+
+cudaError_t launch_batch_validate(const LaunchCtx& c, int n, const BatchDesc* d, long long total_a_nnz,
+                                  long long total_b_nnz) {
+  const long long c0 = stack_chunks(total_a_nnz), blocks = c0 + stack_chunks(total_b_nnz);
+  if (n <= 0 || blocks <= 0) return cudaSuccess;
+  k_batch_validate<<<(unsigned)blocks, STACK_THREADS, 0, c.stream>>>(d, n, total_a_nnz, total_b_nnz, c0, c.err);
+  count_launch(c);
+  return cudaGetLastError();
+}
+
 // V: an unsigned type of the values' width (the values are only moved).
 template <typename V>
 __global__ void __launch_bounds__(STACK_THREADS)

@@ -413,6 +413,8 @@ struct BatchDesc {
 cudaError_t launch_stack_structure(const LaunchCtx& c, int n, const BatchDesc* d, long long total_rows,
                                    long long total_k, int32_t* a_rp, int32_t* a_ci, int32_t* b_rp, int32_t* b_ci,
                                    long long total_a_nnz, long long total_b_nnz);
+cudaError_t launch_batch_validate(const LaunchCtx& c, int n, const BatchDesc* d, long long total_a_nnz,
+                                  long long total_b_nnz);
 cudaError_t launch_stack_values(const LaunchCtx& c, int n, int dtype, const BatchDesc* d, void* a_v, void* b_v,
                                 long long total_a_nnz, long long total_b_nnz);
 cudaError_t launch_batch_bounds(const LaunchCtx& c, int n, const BatchDesc* d, const int32_t* c_rp, long long total_rows,

@@ -138,3 +138,31 @@ def test_galerkin_96_matches_two_plain_calls(api, oracle_mod):
     ref = oracle_mod.spgemm(oracle_mod.transpose(P), oracle_mod.spgemm(A, P))
     assert_structure_equal(Ac, ref)
     assert_values_exact(Ac.vals, ref.vals)
+
+
+@pytest.mark.parametrize("bad", [None, "last B", "first B", "A"])
+def test_batch_validates_every_instance_by_its_own_width(api, oracle_mod, bad):
+    """A column that only a wider instance has (or, in A, only the next
+    instance's B has rows for) is refused with validate."""
+    from paper_2112_10037_gb300 import _native as nat
+    rng = np.random.default_rng(6)
+    pairs = []
+    for m, k, n in ((60, 50, 40), (70, 30, 90), (80, 45, 20)):
+        pairs.append((gen.random_rows(m, k, np.full(m, 4), rng), gen.random_rows(k, n, np.full(k, 5), rng)))
+    if bad == "last B":
+        pairs[2][1].col_idx[pairs[2][1].row_ptr[9] - 1] = 20  # n = 20; the batch's widest has 90
+    elif bad == "first B":
+        pairs[0][1].col_idx[pairs[0][1].row_ptr[9] - 1] = 41
+    elif bad == "A":
+        pairs[0][0].col_idx[pairs[0][0].row_ptr[9] - 1] = 50
+    batch = api.Batch([tuple(api.DeviceCSR.from_host(M) for M in p) for p in pairs], validate=True)
+    if bad:
+        with pytest.raises(nat.SpgemmError) as e:
+            batch.symbolic()
+        assert nat.STATUS_NAMES[e.value.status] == "SPGEMM_ERR_UNSORTED_INPUT"
+    else:
+        batch.symbolic()
+        batch.numeric()
+        for (A, B), C in zip(pairs, batch.results()):
+            assert_structure_equal(_host(C), oracle_mod.spgemm(A, B))
+    batch.close()
