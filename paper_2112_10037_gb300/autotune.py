@@ -25,15 +25,17 @@ search is coordinate descent: starting from the library defaults, each
 option group in turn tries its candidates with the others held at the best
 values found so far, for ``sweeps`` sweeps (the exhaustive product of all
 candidates is available as ``strategy="grid"``).  Winners are cached in a
-JSON file keyed by the GPU (name, SM count), the value type and a size class
-of the product (log2 buckets of rows, nnz(A) and total and largest row
-product counts), so products of the same shape reuse the choice.
+JSON file keyed by the GPU (name, SM count), the library's sources, the value
+type and a size class of the product (log2 buckets of rows, nnz(A) and total and
+largest row product counts), so products of the same shape reuse the choice; a
+choice timed with other kernels is not found.
 
 The cache holds only option values and timings, never results of the
 product.
 """
 from __future__ import annotations
 
+import functools
 import itertools
 import json
 import math
@@ -42,6 +44,7 @@ import threading
 
 import torch
 
+from . import build
 from .api import DeviceCSR, Plan
 
 DEFAULT_CACHE = os.path.join(os.path.expanduser("~"), ".cache", "paper_2112_10037_gb300", "autotune.json")
@@ -89,12 +92,18 @@ def expand(choice: dict) -> dict:
     return out
 
 
+@functools.lru_cache(maxsize=None)
+def kernels_key() -> str:
+    """Digest of the library's sources."""
+    return "k" + build.source_digest()[:12]
+
+
 def signature(A: DeviceCSR, B: DeviceCSR, dtype, stats) -> str:
-    """Cache key: device, dtype and log2 size classes of the product."""
+    """Cache key: device, kernels, dtype and log2 size classes of the product."""
     dev = A.row_ptr.device
     props = torch.cuda.get_device_properties(dev)
     total, mx, _ = stats
-    parts = [props.name.replace(" ", "_"), str(props.multi_processor_count), str(dtype).split(".")[-1],
+    parts = [props.name.replace(" ", "_"), str(props.multi_processor_count), kernels_key(), str(dtype).split(".")[-1],
              "r%d" % _bucket(A.nrows), "c%d" % _bucket(B.ncols), "a%d" % _bucket(A.nnz),
              "p%d" % _bucket(total), "m%d" % _bucket(mx)]
     return "|".join(parts)
@@ -231,8 +240,8 @@ def batch_signature(pairs, dtype) -> str:
     rows = sum(a.nrows for a, _ in pairs)
     dev = pairs[0][0].row_ptr.device
     props = torch.cuda.get_device_properties(dev)
-    return "|".join([props.name.replace(" ", "_"), str(props.multi_processor_count), str(dtype).split(".")[-1],
-                     "batch", "n%d" % _bucket(len(pairs)), "r%d" % _bucket(rows), "a%d" % _bucket(a_nnz)])
+    return "|".join([props.name.replace(" ", "_"), str(props.multi_processor_count), kernels_key(),
+                     str(dtype).split(".")[-1], "batch", "n%d" % _bucket(len(pairs)), "r%d" % _bucket(rows), "a%d" % _bucket(a_nnz)])
 
 
 def autotune_batch(pairs, dtype=torch.float64, candidates=None, cache_path=DEFAULT_CACHE, reps: int = 1,

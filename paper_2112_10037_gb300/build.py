@@ -35,7 +35,8 @@ def _sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
-def _deps_digest() -> str:
+def source_digest() -> str:
+    """Digest of every source and of the flags."""
     h = hashlib.sha1()
     files = sorted(glob.glob(os.path.join(CSRC, "*"))) + [os.path.join(INCLUDE, "spgemm.h")]
     for f in files:
@@ -51,7 +52,7 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
     source, the header or the flags changed (content digest)."""
     os.makedirs(BUILD, exist_ok=True)
     stamp = os.path.join(BUILD, "digest")
-    digest = _deps_digest() + "|" + " ".join(extra_flags)
+    digest = source_digest() + "|" + " ".join(extra_flags)
     if not force and os.path.exists(LIB) and os.path.exists(stamp):
         with open(stamp) as fh:
             if fh.read() == digest:

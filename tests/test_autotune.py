@@ -39,6 +39,30 @@ def test_candidates_cover_the_accumulator_choice():
     assert opts["hash_max"] == 128 and opts["window_block"] == 8192 and opts["block_warps"] == 8
 
 
+def test_choices_of_other_kernels_are_not_found(tmp_path, monkeypatch):
+    """A winner stored under other library sources (say a window that beat a
+    kernel since replaced) is timed again, for products and for batches."""
+    at = _at()
+    from types import SimpleNamespace as NS
+    monkeypatch.setattr(at.torch.cuda, "get_device_properties",
+                        lambda dev: NS(name="Some GPU", multi_processor_count=152))
+    M = NS(nrows=1000, ncols=1000, nnz=5000, row_ptr=NS(device="cuda:0"))
+    cache = str(tmp_path / "tune.json")
+    cand = {"window_warp": [1024, 2048]}
+    for sign in (lambda: at.signature(M, M, "torch.float64", (40_000, 90, None)),
+                 lambda: at.batch_signature([(M, M)], "torch.float64")):
+        old = sign()
+        assert at._tune(old, cand, lambda o: float(o["window_warp"] == 1024), cache, False, "grid", 1) == {"window_warp": 2048}
+        assert sign() == old
+        monkeypatch.setattr(at, "kernels_key", lambda: "kother")
+        assert sign() != old
+        assert at._tune(sign(), cand, lambda o: float(o["window_warp"]), cache, False, "grid", 1) == {"window_warp": 1024}
+        monkeypatch.undo()
+        monkeypatch.setattr(at.torch.cuda, "get_device_properties",
+                            lambda dev: NS(name="Some GPU", multi_processor_count=152))
+    assert at.kernels_key() == at.kernels_key() != "k"
+
+
 def _separable_cost(opts):
     """A cost whose minimum is known: each option contributes on its own."""
     cost = {1024: 3.0, 2048: 1.0}[opts["window_warp"]]
