@@ -36,18 +36,21 @@
 // does not pay, and masks that most products hit (the full pattern of A*B has
 // no more columns than products).
 //
-// A block is one warp and takes one unit, so that the hardware's block
-// scheduler balances units of very different work.  (Long rows on warps left
-// 40 % of the SM cycles idle: the warps of the longest row of a power-law graph
-// alone took two thirds of the kernel's time.)
+// A block is two warps and takes two units, so that the hardware's block
+// scheduler balances units of very different work.  (One warp a block spends
+// more on starting blocks: 96^3 stencil with its square's pattern 0.58 ms, 0.54
+// with two and with four; R-MAT of 65,536 columns with its square's 4.84, 4.44
+// and 4.78.  Long rows on warps left 40 % of the SM cycles idle: the warps of the
+// longest row of a power-law graph alone took two thirds of the kernel's time.)
 //
 // Strictly lower triangles of R-MAT graphs, with a search of the mask row per
 // product, with warps alone, and now: scale 16 (147 M products) 1.61, 1.15 and
 // 0.47 ms (blocks 0.31, warps 0.15), scale 18 (1.1 G products) 10.1, 5.6 and
-// 2.2 ms; 3000 rows, edge factor 8: 56, 50 and 49 us.  The full pattern of a
-// square as the mask, where nearly every product hits: 96^3 stencil 0.54 ms with
-// a search per product and 0.57 now (min-plus 0.98 and 0.94), R-MAT scale 15
-// 5.8 and 5.3 ms (min-plus 8.0 and 8.1).
+// 2.2 ms.  Masks that nearly every product hits, with a search per product and
+// now: the pattern of a square, 96^3 stencil 0.55 and 0.54 ms (min-plus 0.96 and
+// 0.93), R-MAT of 65,536 columns 6.3 and 4.4 ms.  The stencil with its own
+// pattern as the mask pays for the pass that looks for long rows: 0.43 and
+// 0.49 ms.
 //
 // The output is zeroed before and, with M's values, scaled by them after
 // (the sum is finished before the factor, as in the definition).
@@ -58,6 +61,7 @@
 
 namespace sg {
 
+constexpr int MASK_WARPS = 2;             // warps per block, each with a unit of its own
 constexpr int MASK_CAP = 384;             // mask columns staged per warp (32 warps share an SM)
 constexpr int MASK_BITS = 4096;           // bits of the hashed bitmap
 constexpr int MASK_FILTER_MAX = 2048;     // longest mask row worth the bitmap (two bits per column)
@@ -206,13 +210,15 @@ __device__ __forceinline__ bool mask_search_pays(int n, int len) {
 }
 
 template <typename T, int SR>
-__global__ void __launch_bounds__(32, 32)
+__global__ void __launch_bounds__(MASK_WARPS * 32, 32 / MASK_WARPS)
 k_masked(Csr A, Csr B, Csr M, const T* __restrict__ av, const T* __restrict__ bv, T* __restrict__ out, bool blocks) {
-  __shared__ MaskWarp<T> sm;
+  __shared__ MaskWarp<T> s_warp[MASK_WARPS];
+  MaskWarp<T>& sm = s_warp[threadIdx.x >> 5];
   const int lane = lane_id();
   const unsigned lt = lanemask_lt();
   {
-    const long long u = blockIdx.x;
+    const long long u = (long long)blockIdx.x * MASK_WARPS + (threadIdx.x >> 5);
+    if (32 * u >= A.nnz) return;
     const int e = (int)(32 * u) + lane;
     const bool ve = e < A.nnz;
     int i = warp_row_of(A.rp, (int)A.nrows, (int)(32 * u)), sb = 0, len = 0;
@@ -615,7 +621,8 @@ static cudaError_t masked_t(const LaunchCtx& c, const Csr& A, const Csr& B, cons
     count_launch(c);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  k<<<(unsigned)((A.nnz + 31) / 32), 32, 0, c.stream>>>(A, B, M, av, bv, out, long_rows);
+  const long long per_block = 32 * MASK_WARPS;
+  k<<<(unsigned)((A.nnz + per_block - 1) / per_block), MASK_WARPS * 32, 0, c.stream>>>(A, B, M, av, bv, out, long_rows);
   count_launch(c);
   if ((e = cudaGetLastError()) != cudaSuccess || SR != 0 || !mv) return e;
   k_scale<T><<<eg, 256, 0, c.stream>>>(out, mv, M.nnz);
