@@ -97,23 +97,37 @@ __device__ __forceinline__ void analyse_walk(const Csr& A, const Csr& B, int a0,
   }
 }
 
+// Whether a row forms so many products on few columns that a warp with dense
+// 1024-column windows sums it sooner than the paths that rank the columns (when
+// such rows are many, see window_rows in api.cu): windows need neither marks
+// nor ranks nor, for one row of B at a time, atomics, but a row walks every
+// window of its span.  Up to 4096 products (block registers instead) four
+// products per column of the span, or one window while the registers are half
+// empty; above (bands instead) 256 per window.
+__device__ __forceinline__ bool row_is_dense(long long p, int mn, int mx, bool count) {
+  if (!count || p <= 128) return false;
+  const int windows = (mx >> 10) - (mn >> 10) + 1;
+  if (p > 4096) return p >= 256ll * windows;
+  return p >= 4ll * (mx - mn + 1) || (p <= 256 && windows == 1);
+}
+
 // One warp per row of A: P_i, the smallest and largest column any product of
 // the row reaches (first and last column of each touched B row, since B's rows
 // are sorted), histogram of bins, total and maximum P.
 __global__ void __launch_bounds__(256) k_analyse(Csr A, Csr B, long long row_begin, long long mloc,
                                                  long long* __restrict__ prod, int* __restrict__ cmin,
-                                                 int* __restrict__ cmax, DevStats* st) {
+                                                 int* __restrict__ cmax, DevStats* st, bool count_dense) {
   __shared__ int s_hist[NBINS];
   __shared__ unsigned long long s_total, s_max;
-  __shared__ unsigned s_wide, s_wide8;
+  __shared__ unsigned s_wide, s_wide8, s_dense;
   if (threadIdx.x < NBINS) s_hist[threadIdx.x] = 0;
-  if (threadIdx.x == 0) { s_total = 0; s_max = 0; s_wide = 0; s_wide8 = 0; }
+  if (threadIdx.x == 0) { s_total = 0; s_max = 0; s_wide = 0; s_wide8 = 0; s_dense = 0; }
   if (block_skip(st)) return;  // validated input was rejected
   const int lane = lane_id(), gl = lane;
   const long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const long long nw = (gridDim.x * (long long)blockDim.x) >> 5;
   unsigned long long my_total = 0, my_max = 0;
-  unsigned my_wide = 0, my_wide8 = 0;
+  unsigned my_wide = 0, my_wide8 = 0, my_dense = 0;
   bool bad = false;
   for (long long r = w; r < mloc; r += nw) {
     const int a0 = A.rp[row_begin + r], a1 = A.rp[row_begin + r + 1];
@@ -126,6 +140,7 @@ __global__ void __launch_bounds__(256) k_analyse(Csr A, Csr B, long long row_beg
     if (lane == 0) {
       my_wide += a1 - a0 > 32 ? 1u : 0u;
       my_wide8 += a1 - a0 > 8 ? 1u : 0u;
+      my_dense += row_is_dense(p, mn, mx, count_dense) ? 1u : 0u;
       prod[r] = p;
       cmin[r] = mn;
       cmax[r] = mx;
@@ -140,6 +155,7 @@ __global__ void __launch_bounds__(256) k_analyse(Csr A, Csr B, long long row_beg
   }
   if (gl == 0 && my_wide) atomicAdd(&s_wide, my_wide);
   if (gl == 0 && my_wide8) atomicAdd(&s_wide8, my_wide8);
+  if (gl == 0 && my_dense) atomicAdd(&s_dense, my_dense);
   if (__any_sync(FULL, bad) && lane == 0) atomicOr(&st->err, EB_UNSORTED);
   __syncthreads();
   if (threadIdx.x < NBINS && s_hist[threadIdx.x]) atomicAdd(&st->hist[threadIdx.x], s_hist[threadIdx.x]);
@@ -149,6 +165,7 @@ __global__ void __launch_bounds__(256) k_analyse(Csr A, Csr B, long long row_beg
   }
   if (threadIdx.x == 0 && s_wide) atomicAdd(&st->rows_wide, s_wide);
   if (threadIdx.x == 0 && s_wide8) atomicAdd(&st->rows_wide8, s_wide8);
+  if (threadIdx.x == 0 && s_dense) atomicAdd(&st->rows_dense, s_dense);
 }
 
 // The same for matrices of short rows (stencils, aggregation operators): 8
@@ -159,20 +176,21 @@ __global__ void __launch_bounds__(256) k_analyse(Csr A, Csr B, long long row_beg
 // squared: 76 us with one row per group and every row's span, 40 us here.
 __global__ void __launch_bounds__(256) k_analyse_short(Csr A, Csr B, long long row_begin, long long mloc,
                                                        long long* __restrict__ prod, int* __restrict__ cmin,
-                                                       int* __restrict__ cmax, DevStats* st, long long span_min) {
+                                                       int* __restrict__ cmax, DevStats* st, long long span_min,
+                                                       bool count_dense) {
   constexpr int G = 8, RPW = 32 / G, U = 4;
   __shared__ int s_hist[NBINS];
   __shared__ unsigned long long s_total, s_max;
-  __shared__ unsigned s_wide, s_wide8;
+  __shared__ unsigned s_wide, s_wide8, s_dense;
   if (threadIdx.x < NBINS) s_hist[threadIdx.x] = 0;
-  if (threadIdx.x == 0) { s_total = 0; s_max = 0; s_wide = 0; s_wide8 = 0; }
+  if (threadIdx.x == 0) { s_total = 0; s_max = 0; s_wide = 0; s_wide8 = 0; s_dense = 0; }
   if (block_skip(st)) return;  // validated input was rejected
   const int lane = lane_id();
   const int gl = lane & (G - 1), g = lane / G;
   const long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const long long nw = (gridDim.x * (long long)blockDim.x) >> 5;
   unsigned long long my_total = 0, my_max = 0;
-  unsigned my_wide = 0, my_wide8 = 0;
+  unsigned my_wide = 0, my_wide8 = 0, my_dense = 0;
   bool bad = false;
   for (long long r0 = w * RPW * U; r0 < mloc; r0 += nw * RPW * U) {
     int a0[U], a1[U], k[U];
@@ -219,6 +237,7 @@ __global__ void __launch_bounds__(256) k_analyse_short(Csr A, Csr B, long long r
         mx = warp_max(mx);
         if (g == L / G) p[u] = wp;
         if (lane == L) {
+          my_dense += row_is_dense(wp, mn, mx, count_dense) ? 1u : 0u;
           cmin[r] = mn;
           cmax[r] = mx;
         }
@@ -239,6 +258,7 @@ __global__ void __launch_bounds__(256) k_analyse_short(Csr A, Csr B, long long r
         mn = group_min<G>(mn);
         mx = group_max<G>(mx);
         if (gl == 0 && r < mloc && p[u] > span_min && !wide) {
+          my_dense += row_is_dense(p[u], mn, mx, count_dense) ? 1u : 0u;
           cmin[r] = mn;
           cmax[r] = mx;
         }
@@ -259,6 +279,7 @@ __global__ void __launch_bounds__(256) k_analyse_short(Csr A, Csr B, long long r
   }
   if (gl == 0 && my_wide) atomicAdd(&s_wide, my_wide);
   if (gl == 0 && my_wide8) atomicAdd(&s_wide8, my_wide8);
+  if (gl == 0 && my_dense) atomicAdd(&s_dense, my_dense);
   if (__any_sync(FULL, bad) && lane == 0) atomicOr(&st->err, EB_UNSORTED);
   __syncthreads();
   if (threadIdx.x < NBINS && s_hist[threadIdx.x]) atomicAdd(&st->hist[threadIdx.x], s_hist[threadIdx.x]);
@@ -268,6 +289,7 @@ __global__ void __launch_bounds__(256) k_analyse_short(Csr A, Csr B, long long r
   }
   if (threadIdx.x == 0 && s_wide) atomicAdd(&st->rows_wide, s_wide);
   if (threadIdx.x == 0 && s_wide8) atomicAdd(&st->rows_wide8, s_wide8);
+  if (threadIdx.x == 0 && s_dense) atomicAdd(&st->rows_dense, s_dense);
 }
 
 // Counting sort of the non-empty rows by bin, largest bin first.  Each block
@@ -448,15 +470,16 @@ cudaError_t launch_validate(const LaunchCtx& c, const Csr& M) {
 
 cudaError_t launch_analyse(const LaunchCtx& c, const Csr& A, const Csr& B, long long row_begin,
                            long long mloc, long long* prod, int* cmin, int* cmax, int* rows,
-                           long long span_min) {
+                           long long span_min, bool count_dense) {
   if (mloc <= 0) return cudaSuccess;
   timer_mark(c, T_ANALYSE, 0);
   // short rows on average (stencils, aggregation operators): 8 lanes per row
   if (A.nrows > 0 && A.nnz <= 12 * A.nrows)
     k_analyse_short<<<grid_for_warps((mloc + 15) / 16, 8, c.nsm), 256, 0, c.stream>>>(A, B, row_begin, mloc, prod,
-                                                                                     cmin, cmax, c.st, span_min);
+                                                                                     cmin, cmax, c.st, span_min, count_dense);
   else
-    k_analyse<<<grid_for_warps(mloc, 8, c.nsm), 256, 0, c.stream>>>(A, B, row_begin, mloc, prod, cmin, cmax, c.st);
+    k_analyse<<<grid_for_warps(mloc, 8, c.nsm), 256, 0, c.stream>>>(A, B, row_begin, mloc, prod, cmin, cmax, c.st,
+                                                                    count_dense);
   count_launch(c);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;

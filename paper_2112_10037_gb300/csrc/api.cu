@@ -1,5 +1,6 @@
 // C ABI of the library (declared in include/spgemm.h): argument checks,
 // workspace carving, plan state and the order of the passes.
+#include <atomic>
 #include <cstring>
 #include <mutex>
 #include <new>
@@ -41,6 +42,8 @@ struct spgemm_plan {
   sg::PathBins pb{};
   sg::Tuning tu{};
   sg::SplitInfo sp{};
+  const spgemm_plan* base = nullptr;       // plan whose run lists this one reads (null: its own)
+  std::atomic<bool> window_lists{false};   // the 1024-column lists are built (default routes, see window_rows)
   bool symbolic_done = false;
   long long nnz_c = -1;
   int path_rows[sg::NPATHS] = {0, 0, 0, 0};
@@ -229,14 +232,13 @@ Layout layout_for(const spgemm_opts& o, long long mloc, long long nnz_a, long lo
   }
   L.hcnt = off; off = align_up(off + sizeof(int32_t) * nh);
   L.rrb = L.runsb = 0;
-  if (own_b && numeric_block_bin(o, ncols_b) < sg::NBINS) {  // run list at the block window's width
-    if (default_long_rows(o)) {  // no row takes the warp window: one list, the block window's
-      L.rrb = L.rr;
-      L.runsb = L.runs;
-    } else {
-      L.rrb = off; off = align_up(off + sizeof(int32_t) * (size_t)(nrows_b + 1));
-      L.runsb = off; off = align_up(off + sizeof(int2) * (size_t)(nnz_b + nrows_b + sg::RUNS_PAD));
-    }
+  // run list at the block window's width (by default only narrow FP32 products
+  // have it; FP64 keeps the room too: a plan never takes more in FP32)
+  spgemm_opts of = o;
+  of.dtype = SPGEMM_F32;
+  if (own_b && numeric_block_bin(of, ncols_b) < sg::NBINS) {
+    L.rrb = off; off = align_up(off + sizeof(int32_t) * (size_t)(nrows_b + 1));
+    L.runsb = off; off = align_up(off + sizeof(int2) * (size_t)(nnz_b + nrows_b + sg::RUNS_PAD));
   }
   if (o.backward) {
     L.at_rp = off; off = align_up(off + sizeof(int32_t) * (size_t)(nrows_b + 1));
@@ -420,6 +422,39 @@ spgemm_status read_stats(spgemm_plan* p, cudaStream_t s, const sg::DevStats* mir
   return SPGEMM_OK;
 }
 
+// Whether the default routes give a plan's rows above the small ones (up to
+// 65,536 products) to warps with dense windows of 1024 columns: most of them
+// dense (row_is_dense: bands, blocks, finite elements of several unknowns), in
+// numbers that give every SM its warps, and products enough for the lists of B's
+// runs and one more wait.  FP64, ranked and in windows: band of 61 entries a row,
+// 50,000 rows 3.60 and 1.46 ms; blocks of 64, 64,000 rows 5.23 and 1.86, of 16,
+// 160,000 rows 0.83 and 0.65; 27-point stencil of 3 unknowns on 30^3 points 6.25
+// and 4.26.  Left to the ranks: 7,000 rows of a band of 41 entries (12 M products)
+// 0.31 and 0.29, in FP32 0.24 and 0.29; 100,000 rows of 484 products on 2000 random
+// columns 0.54 and 0.65; 8,000 random rows of 60 entries 0.41 and 0.52.
+constexpr long long WINDOW_PRODUCTS = 16000000;
+
+bool window_rows(const spgemm_plan* p) {
+  if (!default_long_rows(p->opts)) return false;
+  long long rows = 0;
+  for (int b = small_hi_bin(p->opts) + 1; b < sg::NBINS; ++b) rows += p->host_st.hist[b];
+  const long long dense = (long long)p->host_st.rows_dense;
+  return dense >= 40ll * p->nsm && 2 * dense > rows && (long long)p->host_st.total_products >= WINDOW_PRODUCTS;
+}
+
+// After the statistics are on the host: the run lists of B for such rows, once
+// per plan, complete on return (derived plans read them on any stream).
+spgemm_status build_window_lists(spgemm_plan* p, const sg::LaunchCtx& c) {
+  if (p->base || p->window_lists.load() || !p->runs_part || !window_rows(p)) return SPGEMM_OK;
+  sg::SplitInfo lists = p->sp;
+  lists.rrb = nullptr;
+  lists.runsb = nullptr;
+  if (sg::launch_runs(c, p->B, lists, p->runs_part, 0) != cudaSuccess) return SPGEMM_ERR_CUDA;
+  if (cudaStreamSynchronize(c.stream) != cudaSuccess) return SPGEMM_ERR_CUDA;
+  p->window_lists.store(true);
+  return SPGEMM_OK;
+}
+
 }  // namespace
 
 // Other semirings than plus-times skip the rank-compacted accumulator,
@@ -488,6 +523,7 @@ static spgemm_status analyse_impl(const spgemm_csr* A, const spgemm_csr* B, cons
     p->sp.hcnt = nh ? (int32_t*)(p->ws + L.hcnt) : nullptr;
     p->sp.wb_shift = 0;
     while ((1 << p->sp.wb_shift) < p->tu.window_block) ++p->sp.wb_shift;
+    p->base = base;
     if (base) {
       p->sp.rr = base->sp.rr;
       p->sp.runs = base->sp.runs;
@@ -518,7 +554,7 @@ static spgemm_status analyse_impl(const spgemm_csr* A, const spgemm_csr* B, cons
     if (e == cudaSuccess) e = sg::launch_validate(c, p->B);
   }
   if (e == cudaSuccess) e = sg::launch_analyse(c, p->A, p->B, p->row_begin, p->mloc, p->prod, p->cmin, p->cmax, p->rows,
-                                               span_min);
+                                               span_min, default_long_rows(o));
   if (e == cudaSuccess && !base) {
     // Only the numeric window paths read the run lists.  A plan of every row
     // of A may leave them unbuilt when none of its rows can take such a path:
@@ -532,8 +568,10 @@ static spgemm_status analyse_impl(const spgemm_csr* A, const spgemm_csr* B, cons
     const bool never = win_lo >= sg::NBINS && p->tu.num_lo_band < sg::NBINS;
     if (rb != 0 || re != A->nrows) win_lo = 0;
     sg::SplitInfo lists = p->sp;
-    if (default_long_rows(o)) {  // (see layout_for)
+    if (default_long_rows(o)) {  // the block window's alone; the others when the rows are known (window_rows)
       lists.wf_shift = lists.wb_shift;
+      lists.rr = lists.rrb;
+      lists.runs = lists.runsb;
       lists.rrb = nullptr;
       lists.runsb = nullptr;
     }
@@ -683,6 +721,8 @@ spgemm_status spgemm_symbolic(spgemm_plan* p, int32_t* c_row_ptr, int64_t* c_nnz
   stats_pool().give(mirror);
   s = from_err_word(p->host_st.err);
   if (s != SPGEMM_OK) return s;
+  s = build_window_lists(p, c);
+  if (s != SPGEMM_OK) return s;
   p->nnz_c = p->host_st.nnz_c;
   *c_nnz = p->nnz_c;
   p->symbolic_done = true;
@@ -699,6 +739,8 @@ spgemm_status spgemm_plan_adopt_row_ptr(spgemm_plan* p, int64_t nnz, spgemm_stre
   if (s != SPGEMM_OK) return s;
   s = from_err_word(p->host_st.err);
   if (s != SPGEMM_OK) return s;
+  s = build_window_lists(p, ctx_of(p, stream));
+  if (s != SPGEMM_OK) return s;
   p->nnz_c = nnz;
   p->symbolic_done = true;
   return SPGEMM_OK;
@@ -713,7 +755,9 @@ spgemm_status spgemm_numeric(spgemm_plan* p, const void* a_vals, const void* b_v
   if (!a_vals || !b_vals || !c_col_idx || !c_vals) return SPGEMM_ERR_INVALID_ARG;
   sg::LaunchCtx c = ctx_of(p, stream);
   const sg::RowInfo ri = rowinfo_of(p);
-  cudaError_t e = sg::launch_numeric(c, p->A, p->B, ri, p->pb, p->tu, p->sp, p->opts.dtype, a_vals, b_vals,
+  sg::Tuning tu = p->tu;
+  tu.windows = (p->base ? p->base : p)->window_lists.load() && window_rows(p);
+  cudaError_t e = sg::launch_numeric(c, p->A, p->B, ri, p->pb, tu, p->sp, p->opts.dtype, a_vals, b_vals,
                                      p->cursor, p->nxt, c_row_ptr, c_col_idx, c_vals, p->path_rows,
                                      (long long)p->host_st.rows_wide,
                                      (long long)p->host_st.rows_wide8, p->host_st.hist, p->opts.semiring);

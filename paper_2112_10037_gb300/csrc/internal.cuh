@@ -48,6 +48,7 @@ struct DevStats {
   uint32_t err;
   uint32_t rows_wide;  // rows of the plan with more than 32 nonzeros of A
   uint32_t rows_wide8;  // rows with more than 8 (LANE_MERGE_K)
+  uint32_t rows_dense;  // rows of many products per window of columns (row_is_dense)
   int max_col, max_row_b;  // nonzeros of A's longest column and B's longest row (plans for the adjoint)
   int hist[NBINS];   // rows per bin
   int fill[NBINS];   // scatter cursors
@@ -89,6 +90,7 @@ struct Tuning {
   int hash_max;        // largest P of the hash path (0: path disabled)
   int warp_max;        // largest P of the symbolic warp path
   int num_hi_once;     // numeric bins <= this (above the small-row bins) keep a row in registers (0: none)
+  bool windows;        // rows above the small ones and of at most 65,536 products take the warp window
   int num_lo_block;    // numeric bins >= this use the block kernel (NBINS: never)
   int num_lo_band;     // numeric bins >= this use the banded accumulator (NBINS: never); then the block
                        // kernel serves few rows only
@@ -310,7 +312,8 @@ inline void count_launch(const LaunchCtx& c) {
 cudaError_t launch_validate(const LaunchCtx& c, const Csr& M);
 cudaError_t launch_analyse(const LaunchCtx& c, const Csr& A, const Csr& B, long long row_begin,
                            long long mloc, long long* prod, int* cmin, int* cmax, int* rows,
-                           long long span_min /* rows of at most this many products need no column span */);
+                           long long span_min /* rows of at most this many products need no column span */,
+                           bool count_dense /* rows_dense is wanted */);
 // win_lo > 0: skip building the lists when the analysis put no row in bins
 // win_lo and above (only valid when no other plan reads this plan's lists
 // for rows outside it).

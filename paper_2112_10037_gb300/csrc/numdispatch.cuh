@@ -338,7 +338,8 @@ static cudaError_t numeric_t(const LaunchCtx& c, const Csr& A, const Csr& B, con
     if (e) return e;
   }
   // every other row (rows of the symbolic warp and block paths both land
-  // here): the block-wide window from block_lo on, the banded accumulator from
+  // here): the warp-owned dense window for all but the longest when most are
+  // dense (tu.windows); the block-wide window from block_lo on, the banded accumulator from
   // num_lo_band on, below them the register path and, where an option asks
   // for it, the warp-owned dense window
   int lo = NBINS, hi = 0;
@@ -347,6 +348,16 @@ static cudaError_t numeric_t(const LaunchCtx& c, const Csr& A, const Csr& B, con
       lo = pb.lo[p] < lo ? pb.lo[p] : lo;
       hi = pb.hi[p] > hi ? pb.hi[p] : hi;
     }
+  if (tu.windows && hi >= lo) {
+    const int whi = hi < bin_of(65536) ? hi : bin_of(65536);
+    if (whi >= lo && !empty_bins(hist, lo, whi)) {
+      timer_mark(c, T_NUM_WARP, 0);
+      e = warp_num<T, 1024, SR>(c, A, B, av, bv, ri, lo, whi, sp, cur, nxt, c_rp, c_ci, c_v, rows_wide);
+      timer_mark(c, T_NUM_WARP, 1);
+      if (e) return e;
+    }
+    if (whi >= lo) lo = whi + 1;
+  }
   const int nlo = block_lo(tu, hist, c.nsm);
   const int blo = nlo > lo ? nlo : lo;
   if (hi >= blo && !empty_bins(hist, blo, hi)) {

@@ -94,3 +94,73 @@ def test_semirings(api, oracle_mod, semiring):
     R = oracle_mod.spgemm(A, B)
     assert_structure_equal(got, R)
     assert np.array_equal(got.vals, oracle_mod.masked_semiring(A, B, R, semiring))
+
+
+def _block_rows(n, kind, rng):
+    """At least 16 M products in rows that the windows take: a band that
+    straddles windows, dense blocks, 3000 columns that all rows share (one row of
+    more than 65,536 products among them), every 50th row short."""
+    if kind == "band":
+        cols = np.arange(n)[:, None] + np.arange(-20, 21)[None, :]
+        rows = [c[(c >= 0) & (c < n)] for c in cols]
+    elif kind == "blocks":
+        rows = [i // 40 * 40 + np.arange(min(40, n - i // 40 * 40)) for i in range(n)]
+    else:
+        rows = [np.sort(rng.choice(3000, 70, replace=False)) for _ in range(n)]
+        rows[7] = np.sort(rng.choice(n, 1500, replace=False))
+    for i in range(0, n, 50):
+        rows[i] = rows[i][:3]
+    rp = np.concatenate([[0], np.cumsum([len(r) for r in rows])]).astype(np.int32)
+    ci = np.concatenate(rows).astype(np.int32)
+    return gen.CSR(n, n, rp, ci, rng.standard_normal(len(ci))).check()
+
+
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+@pytest.mark.parametrize("kind,n", [("band", 12_000), ("blocks", 12_001), ("shared", 9_000), ("band", 40_000)])
+def test_dense_rows_take_windows(api, oracle_mod, kind, n, dtype):
+    """Many rows of many products on few columns: the windows' lists are built
+    with the symbolic pass; a plan of a range of the rows reads them, and ranks its
+    columns while they do not exist."""
+    from paper_2112_10037_gb300 import _native as nat
+    A = _block_rows(n, kind, np.random.default_rng(n))
+    assert oracle_mod.row_products(A, A).sum() >= 16_000_000
+    dA = api.DeviceCSR.from_host(A, dtype=dtype)
+    plan = api.Plan(dA, dA, dtype=dtype)
+    early = plan.rows(0, n - 300)
+    early_rp, _ = early.symbolic()
+    first = early.numeric(dA.vals, dA.vals)  # before the lists exist
+    before = nat.spgemm_plan_launches(plan.handle)
+    rp, _ = plan.symbolic()
+    assert nat.spgemm_plan_launches(plan.handle) - before >= 6  # two symbolic, a scan, the lists' three
+    ci, v = plan.numeric(dA.vals, dA.vals)
+    late = plan.rows(100, n)
+    late_rp, _ = late.symbolic()
+    got = [(first, early_rp, 0, n - 300), (early.numeric(dA.vals, dA.vals), early_rp, 0, n - 300),
+           (late.numeric(dA.vals, dA.vals), late_rp, 100, n)]
+    torch.cuda.synchronize()
+    plan.check()
+    for p in (early, late):
+        p.check()
+    if dtype == torch.float32:
+        A = A.astype(np.float32).astype(np.float64)
+    R, S = oracle_with_scale(oracle_mod, A, A)
+    C = gen.CSR(n, n, rp.cpu().numpy(), ci.cpu().numpy(), v.double().cpu().numpy())
+    assert_structure_equal(C, R)
+    assert_values_close(C.vals, R.vals, S, *([RTOL_F32] if dtype == torch.float32 else []))
+    for (pci, pv), r, a, b in got:
+        s, e = R.row_ptr[a], R.row_ptr[b]
+        assert np.array_equal(r.cpu().numpy(), R.row_ptr[a:b + 1] - s)
+        assert np.array_equal(pci.cpu().numpy(), R.col_idx[s:e])
+        assert np.all(np.abs(pv.double().cpu().numpy() - R.vals[s:e]) <=
+                      (RTOL_F32 if dtype == torch.float32 else 1e-12) * S[s:e])
+    for p in (early, late, plan):
+        p.close()
+
+
+@pytest.mark.parametrize("semiring", ["min_plus", "or_and"])
+def test_dense_rows_semirings(api, oracle_mod, semiring):
+    A = _block_rows(12_000, "blocks", np.random.default_rng(1))
+    got = api.spgemm_semiring(api.DeviceCSR.from_host(A), api.DeviceCSR.from_host(A), semiring).to_host()
+    R = oracle_mod.spgemm(A, A)
+    assert_structure_equal(got, R)
+    assert np.array_equal(got.vals, oracle_mod.masked_semiring(A, A, R, semiring))
