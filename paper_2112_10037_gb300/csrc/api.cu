@@ -285,14 +285,16 @@ spgemm_status check_csr(const spgemm_csr* M) {
 
 // Window columns and warps of the numeric block kernel: one of the compiled
 // pairs, the default where the options name none or an unsupported one: 8192
-// columns and 8 warps (three blocks on an SM), or 16,384 and 16 where B has at
-// most two such windows: there the longest rows set the time, and a row is
-// done in half of it (12,345 columns FP32: 0.36 ms for the rows above 4096
-// products with 8192 and 8, 0.22 so).
+// columns and 8 warps (three blocks on an SM), or on the default routes 16,384
+// and 16 where B has at most two such windows: there few rows are left to the
+// block window, the longest sets the time, and a row is done in half of it
+// (12,345 columns FP32: 0.36 ms for the rows above 4096 products with 8192 and
+// 8, 0.22 so; every row of a graph of 30,000 vertices, FP64: 1.06 and 1.34).
 static void block_geometry(const spgemm_opts& o, long long ncols_b, int* w, int* nw) {
   static const int pairs[][2] = {{2048, 4}, {2048, 8}, {4096, 4}, {4096, 8}, {4096, 16}, {8192, 8}, {8192, 16},
                                  {16384, 16}};
-  const int dw = ncols_b <= 32768 ? 16384 : 8192, dn = ncols_b <= 32768 ? 16 : 8;
+  const bool two = default_long_rows(o) && ncols_b <= 32768;
+  const int dw = two ? 16384 : 8192, dn = two ? 16 : 8;
   const int ww = o.window_block > 0 ? o.window_block : dw, nn = o.block_warps > 0 ? o.block_warps : dn;
   *w = dw;
   *nw = dn;
