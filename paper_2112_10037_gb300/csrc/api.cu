@@ -446,7 +446,8 @@ bool window_rows(const spgemm_plan* p) {
 
 // After the statistics are on the host: the run lists of B for such rows, once
 // per plan, complete on return (derived plans read them on any stream).
-spgemm_status build_window_lists(spgemm_plan* p, const sg::LaunchCtx& c) {
+spgemm_status build_window_lists(spgemm_plan* p, sg::LaunchCtx c) {
+  c.timers = nullptr;  // (the scan's timer is the symbolic pass's)
   if (p->base || p->window_lists.load() || !p->runs_part || !window_rows(p)) return SPGEMM_OK;
   sg::SplitInfo lists = p->sp;
   lists.rrb = nullptr;
