@@ -285,12 +285,10 @@ __device__ __forceinline__ int lane_merge_rows(const Csr& A, const Csr& B, const
     }
     if (act) {
       T acc = Ops::zero();
-      bool any = false;
 #pragma unroll
       for (int k = 0; k < K; ++k) {
         if (hc[k] == m) {
-          acc = Ops::madd(a[k], v[k], any ? acc : Ops::zero());  // one FP64 instruction per head test
-          any = true;
+          acc = Ops::madd(a[k], v[k], acc);  // one FP64 instruction per head test
           ++hs[k];
           hc[k] = hn[k];
           hn[k] = hs[k] + 1 < he[k] ? B.ci[hs[k] + 1] : INT_MAX;
