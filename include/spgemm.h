@@ -91,11 +91,13 @@ typedef struct spgemm_opts {
   int32_t window_warp; /* columns of the numeric dense window (one per warp):
                           1024, 2048 or 4096 (0: default 1024).  With 1024, rows of up
                           to 8192 products that no other option routes elsewhere keep
-                          their products in a block's registers instead */
+                          their products in a block's registers instead, unless most
+                          of the long rows form many products on few columns */
   int32_t window_block;/* columns of the numeric block window, with block_warps one of
                           the pairs (2048, 4), (2048, 8), (4096, 4), (4096, 8),
                           (4096, 16), (8192, 8), (8192, 16), (16384, 16); 0 or any
-                          other pair: (8192, 8) */
+                          other pair: (8192, 8), but (16384, 16) on the default routes
+                          (see num_block_min) of a B of at most 32,768 columns */
   int32_t split_min;   /* rows with more products than this are split into column
                           tiles of window_warp columns, processed independently
                           (0: default 131072; -1: never split); used only for rows
@@ -106,9 +108,12 @@ typedef struct spgemm_opts {
                           with a block-wide window (-1: never, then heavy rows are split
                           as split_min says).  0 or 65536 with the other options that
                           choose a kernel for such rows (rank_min, split_min, window_warp,
-                          window_block, block_warps) at 0 or their defaults: rows of more
-                          than 4096 products (2048 on at most 65,536 columns) accumulate
-                          in bands of ranks, see csrc/numband.cuh */
+                          window_block, block_warps) at 0 or their defaults means the
+                          default routes: rows of more than 4096 products (2048 on at
+                          most 65,536 columns) accumulate in bands of ranks, see
+                          csrc/numband.cuh, but where most long rows form many products
+                          on few columns those of up to 65,536 products take the warps'
+                          windows */
   int32_t block_warps; /* warps sharing a numeric block window (see window_block) */
   int32_t sort_max;    /* rows of at most this many products are merged by a sort in
                           registers: 128, 256 or 512 (0: 128); rows of 17 or more

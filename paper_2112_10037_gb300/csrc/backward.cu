@@ -18,16 +18,17 @@
 // Rows of C that are too short to be worth a block or too long or too wide
 // for its shared memory are searched in global memory by k_grad_slabs.
 //
-// Orders are fixed (a lane's own chain, fixed shuffle trees, chunks in
-// order), nothing is accumulated atomically: the same bits on every run.
+// Orders are fixed (a lane's own chain, fixed trees, chunks in order), nothing
+// is accumulated atomically: the same bits on every run, and for dB whether it
+// passes through the buffer or not (grad_route says when it does).
 //
 // 65,536 rows of 32 x 32 products, FP32: a binary search in C's row per
-// product and gradient (the kernels that still serve products whose rows of
-// B exceed the buffer) took 0.82 ms for dA and 1.88 ms for dB, bound by the
-// memory latency and the 32-byte sectors of scattered searches in C (533 MB).
-// Here k_grad_rows takes 0.62 ms for four chunks (bound by the latency of a
-// row's loads, 8 of 16 warps per scheduler resident at 64 registers),
-// k_grad_cols 0.20 ms (2.6 TB/s of DRAM and L1 59 % busy).
+// product and gradient (k_grad_a, k_grad_b) took 0.82 ms for dA and 1.88 ms for
+// dB, bound by the memory latency and the 32-byte sectors of scattered searches
+// in C (533 MB).  Here k_grad_rows takes 0.44 ms for four chunks (bound by the
+// latency of a row's loads, 7.3 of 13 stalled warps per issue, 8 of 16 warps per
+// scheduler resident at 64 registers), k_grad_cols 0.18 ms (load latency; L1 50 %
+// and DRAM 31 % busy).
 #include <cmath>
 
 #include "launch_util.cuh"

@@ -19,7 +19,8 @@
 // five times as long, so that a warp's 32 products mostly come from one row of
 // B -- distinct columns, no retries of the shared-memory compare-and-swap --
 // without mapping products to segments one by one.  The price is the first
-// walk over the columns and a bitmap look-up per product.
+// walk over the columns and a bitmap look-up per product; rows on few columns,
+// which need one or two windows, stay with the warps' windows (numwarp.cuh).
 //
 // What bounds it is the shared-memory pipe (the swap of 64-bit words at 17
 // cycles a warp, look-ups and stores of a batch of 32 products about 30 more)

@@ -26,16 +26,17 @@
 // COLUMN, so a row of 1,000 products over 65,536 columns walks 64 windows of
 // 16 products each and pays a segment search, an emission and a clear for
 // every one.  Here a row costs one pass whatever its width.  What bounds it is
-// instruction issue (2.4 of 4 per clock, 152 warp instructions per 32 products
-// at 16,384 rows of 32 x 32) and the shared-memory traffic of random bits and
-// ranks (L1 74 % busy).  65,536 rows of 32 x 32 products over 65,536 columns
+// instruction issue (2.5 of 4 per clock, 155 warp instructions per 32 products
+// at 16,384 rows of 32 x 32, FP64, 0.11 ms) and the shared-memory traffic of
+// random bits and ranks (L1 72 % busy).  65,536 rows of 32 x 32 products over 65,536 columns
 // in FP32: 1.58 ms with the warp window, 0.40 ms here; 64 products of 1,024 to
 // 50,000 rows (rows of up to 4,096 products, FP64): 10.9 ms and 4.1 ms; R-MAT
 // scale 18, rows of 129 to 8,192 products: 6.0 ms and 2.6 ms.
 //
-// The threads follow the row's products, 8 per thread.  Rows above 8192
-// products stay with the windows: their products no longer fit 64 registers
-// at the 1024 threads of a block.
+// The threads follow the row's products, 8 per thread: rows of up to 8192 fit
+// the 64 registers of a block's 1024 threads.  Rows that form many products on
+// few columns stay with the warps' windows, which add them without marks and
+// ranks (row_is_dense in analyse.cu).
 #pragma once
 
 #include "internal.cuh"

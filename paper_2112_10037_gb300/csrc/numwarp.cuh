@@ -1,5 +1,6 @@
-// Numeric pass, dense-window accumulator owned by one warp: the rows an option
-// sends here (by default numonce.cuh and numband.cuh take them).
+// Numeric pass, dense-window accumulator owned by one warp: rows that form many
+// products on few columns, when they are many (window_rows in api.cu), and rows
+// that an option sends here.  numonce.cuh and numband.cuh take the others.
 //
 // Row i of C is the sum over A(i,k) of A(i,k) * B(k,:) (Sec. 2.2).  A warp
 // owns a window of W consecutive columns in shared memory: a dense value
