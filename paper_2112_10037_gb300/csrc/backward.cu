@@ -26,7 +26,7 @@
 // product and gradient (k_grad_a, k_grad_b) took 0.82 ms for dA and 1.88 ms for
 // dB, bound by the memory latency and the 32-byte sectors of scattered searches
 // in C (533 MB).  Here k_grad_rows takes 0.44 ms for four chunks (bound by the
-// latency of a row's loads, 7.3 of 13 stalled warps per issue, 8 of 16 warps per
+// latency of a row's loads, 7.3 of 14 stalled warps per issue, 8 of 16 warps per
 // scheduler resident at 64 registers), k_grad_cols 0.18 ms (load latency; L1 50 %
 // and DRAM 31 % busy).
 #include <cmath>
