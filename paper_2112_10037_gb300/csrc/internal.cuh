@@ -206,20 +206,41 @@ __device__ __forceinline__ bool fma_shared(float* p, float a, float b, uint32_t*
   return true;
 }
 
-// The same in FP32 with one rounding, by compare-and-swap: for rows whose
-// products meet seldom, where a product's own rounding is much of the error.
-__device__ __forceinline__ void fma_shared_cas(float* p, float a, float b, uint32_t* err) {
-  const unsigned s = (unsigned)__cvta_generic_to_shared(p);
-  unsigned old;
-  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(old) : "r"(s) : "memory");
-  for (int it = 0; it < CAS_RETRY_LIMIT; ++it) {
-    const unsigned nv = __float_as_uint(fmaf(a, b, __uint_as_float(old)));
+// The same in FP32 with one rounding, by compare-and-swap: acc[at[u]] += a[u] *
+// b[u] for the at[u] >= 0, the loads of the words and the first swaps of all of
+// them in flight together.
+template <int N>
+__device__ __forceinline__ void fma_shared_cas(float* acc, const float (&a)[N], const float (&b)[N], const int (&at)[N],
+                                               uint32_t* err) {
+  const unsigned s0 = (unsigned)__cvta_generic_to_shared(acc);
+  auto swap = [&](int u, unsigned old) {
     unsigned prev;
-    asm volatile("atom.shared.cas.b32 %0, [%1], %2, %3;" : "=r"(prev) : "r"(s), "r"(old), "r"(nv) : "memory");
-    if (prev == old) return;
-    old = prev;
+    asm volatile("atom.shared.cas.b32 %0, [%1], %2, %3;"
+                 : "=r"(prev)
+                 : "r"(s0 + 4u * (unsigned)at[u]), "r"(old), "r"(__float_as_uint(fmaf(a[u], b[u], __uint_as_float(old))))
+                 : "memory");
+    return prev;
+  };
+  unsigned old[N], prev[N];
+#pragma unroll
+  for (int u = 0; u < N; ++u) {
+    old[u] = 0u;
+    if (at[u] >= 0) asm volatile("ld.shared.u32 %0, [%1];" : "=r"(old[u]) : "r"(s0 + 4u * (unsigned)at[u]) : "memory");
   }
-  atomicOr(err, EB_INTERNAL);  // never expected: each failed swap is another update's success
+#pragma unroll
+  for (int u = 0; u < N; ++u) prev[u] = at[u] >= 0 ? swap(u, old[u]) : old[u];
+#pragma unroll
+  for (int u = 0; u < N; ++u) {
+    int it = 0;
+    while (prev[u] != old[u]) {  // another product came first
+      if (++it > CAS_RETRY_LIMIT) {  // never expected: each failed swap is another update's success
+        atomicOr(err, EB_INTERNAL);
+        break;
+      }
+      old[u] = prev[u];
+      prev[u] = swap(u, old[u]);
+    }
+  }
 }
 
 // Index of the first lane whose inclusive prefix `incl` exceeds p (incl is

@@ -300,12 +300,16 @@ k_num_once(Csr A, Csr B, const T* __restrict__ av, const T* __restrict__ bv, Row
         }
       }
       __syncthreads();
+      int at[E];
 #pragma unroll
-      for (int u = 0; u < E; ++u)
+      for (int u = 0; u < E; ++u) {
+        at[u] = -1;
         if (col[u] < -1) {
-          pv[u].add_to(&acc[-2 - col[u]], err);
+          at[u] = -2 - col[u];
           col[u] = -1;
         }
+      }
+      add_held<1>(pv, acc, at, err);
       // the bitmap is clear again for the next window or row
       for (int t = tid * 4; t < nwords; t += NT * 4) *reinterpret_cast<uint4*>(bits + t) = make_uint4(0, 0, 0, 0);
       __syncthreads();

@@ -268,9 +268,10 @@ __device__ __forceinline__ void hash_num_rows(const Csr& A, const Csr& B, const 
     for (int s = 0; s < E; ++s)
       if (fresh[s]) val[slot[s]] = pv[s].first();
     __syncwarp();
+    int at[E];
 #pragma unroll
-    for (int s = 0; s < E; ++s)
-      if (!fresh[s] && slot[s] >= 0) pv[s].add_to(&val[slot[s]], err);
+    for (int s = 0; s < E; ++s) at[s] = fresh[s] ? -1 : slot[s];
+    add_held<E>(pv, val, at, err);
     __syncwarp();
     // Compaction: the occupied slots, in slot order, into the list dk/dv;
     // each slot's key is cleared by the lane that read it.
