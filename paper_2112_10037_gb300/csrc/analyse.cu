@@ -111,6 +111,13 @@ __device__ __forceinline__ bool row_is_dense(long long p, int mn, int mx, bool c
   return p >= 4ll * (mx - mn + 1) || (p <= 256 && windows == 1);
 }
 
+// Rows that stay inside half of B's columns (bands, stencils, finite elements):
+// neighbouring rows of C then share cache lines and searches in them are cheap
+// (see grad_route in backward.cu).
+__device__ __forceinline__ bool row_is_local(long long p, int mn, int mx, long long ncols) {
+  return p > 128 && 2 * ((long long)mx - mn + 1) <= ncols;
+}
+
 // One warp per row of A: P_i, the smallest and largest column any product of
 // the row reaches (first and last column of each touched B row, since B's rows
 // are sorted), histogram of bins, total and maximum P.
@@ -119,15 +126,15 @@ __global__ void __launch_bounds__(256) k_analyse(Csr A, Csr B, long long row_beg
                                                  int* __restrict__ cmax, DevStats* st, bool count_dense) {
   __shared__ int s_hist[NBINS];
   __shared__ unsigned long long s_total, s_max;
-  __shared__ unsigned s_wide, s_wide8, s_dense;
+  __shared__ unsigned s_wide, s_wide8, s_dense, s_local;
   if (threadIdx.x < NBINS) s_hist[threadIdx.x] = 0;
-  if (threadIdx.x == 0) { s_total = 0; s_max = 0; s_wide = 0; s_wide8 = 0; s_dense = 0; }
+  if (threadIdx.x == 0) { s_total = 0; s_max = 0; s_wide = 0; s_wide8 = 0; s_dense = 0; s_local = 0; }
   if (block_skip(st)) return;  // validated input was rejected
   const int lane = lane_id(), gl = lane;
   const long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const long long nw = (gridDim.x * (long long)blockDim.x) >> 5;
   unsigned long long my_total = 0, my_max = 0;
-  unsigned my_wide = 0, my_wide8 = 0, my_dense = 0;
+  unsigned my_wide = 0, my_wide8 = 0, my_dense = 0, my_local = 0;
   bool bad = false;
   for (long long r = w; r < mloc; r += nw) {
     const int a0 = A.rp[row_begin + r], a1 = A.rp[row_begin + r + 1];
@@ -141,6 +148,7 @@ __global__ void __launch_bounds__(256) k_analyse(Csr A, Csr B, long long row_beg
       my_wide += a1 - a0 > 32 ? 1u : 0u;
       my_wide8 += a1 - a0 > 8 ? 1u : 0u;
       my_dense += row_is_dense(p, mn, mx, count_dense) ? 1u : 0u;
+      my_local += row_is_local(p, mn, mx, B.ncols) ? 1u : 0u;
       prod[r] = p;
       cmin[r] = mn;
       cmax[r] = mx;
@@ -156,6 +164,7 @@ __global__ void __launch_bounds__(256) k_analyse(Csr A, Csr B, long long row_beg
   if (gl == 0 && my_wide) atomicAdd(&s_wide, my_wide);
   if (gl == 0 && my_wide8) atomicAdd(&s_wide8, my_wide8);
   if (gl == 0 && my_dense) atomicAdd(&s_dense, my_dense);
+  if (gl == 0 && my_local) atomicAdd(&s_local, my_local);
   if (__any_sync(FULL, bad) && lane == 0) atomicOr(&st->err, EB_UNSORTED);
   __syncthreads();
   if (threadIdx.x < NBINS && s_hist[threadIdx.x]) atomicAdd(&st->hist[threadIdx.x], s_hist[threadIdx.x]);
@@ -166,6 +175,7 @@ __global__ void __launch_bounds__(256) k_analyse(Csr A, Csr B, long long row_beg
   if (threadIdx.x == 0 && s_wide) atomicAdd(&st->rows_wide, s_wide);
   if (threadIdx.x == 0 && s_wide8) atomicAdd(&st->rows_wide8, s_wide8);
   if (threadIdx.x == 0 && s_dense) atomicAdd(&st->rows_dense, s_dense);
+  if (threadIdx.x == 0 && s_local) atomicAdd(&st->rows_local, s_local);
 }
 
 // The same for matrices of short rows (stencils, aggregation operators): 8
@@ -181,16 +191,16 @@ __global__ void __launch_bounds__(256) k_analyse_short(Csr A, Csr B, long long r
   constexpr int G = 8, RPW = 32 / G, U = 4;
   __shared__ int s_hist[NBINS];
   __shared__ unsigned long long s_total, s_max;
-  __shared__ unsigned s_wide, s_wide8, s_dense;
+  __shared__ unsigned s_wide, s_wide8, s_dense, s_local;
   if (threadIdx.x < NBINS) s_hist[threadIdx.x] = 0;
-  if (threadIdx.x == 0) { s_total = 0; s_max = 0; s_wide = 0; s_wide8 = 0; s_dense = 0; }
+  if (threadIdx.x == 0) { s_total = 0; s_max = 0; s_wide = 0; s_wide8 = 0; s_dense = 0; s_local = 0; }
   if (block_skip(st)) return;  // validated input was rejected
   const int lane = lane_id();
   const int gl = lane & (G - 1), g = lane / G;
   const long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const long long nw = (gridDim.x * (long long)blockDim.x) >> 5;
   unsigned long long my_total = 0, my_max = 0;
-  unsigned my_wide = 0, my_wide8 = 0, my_dense = 0;
+  unsigned my_wide = 0, my_wide8 = 0, my_dense = 0, my_local = 0;
   bool bad = false;
   for (long long r0 = w * RPW * U; r0 < mloc; r0 += nw * RPW * U) {
     int a0[U], a1[U], k[U];
@@ -238,6 +248,7 @@ __global__ void __launch_bounds__(256) k_analyse_short(Csr A, Csr B, long long r
         if (g == L / G) p[u] = wp;
         if (lane == L) {
           my_dense += row_is_dense(wp, mn, mx, count_dense) ? 1u : 0u;
+          my_local += row_is_local(wp, mn, mx, B.ncols) ? 1u : 0u;
           cmin[r] = mn;
           cmax[r] = mx;
         }
@@ -259,6 +270,7 @@ __global__ void __launch_bounds__(256) k_analyse_short(Csr A, Csr B, long long r
         mx = group_max<G>(mx);
         if (gl == 0 && r < mloc && p[u] > span_min && !wide) {
           my_dense += row_is_dense(p[u], mn, mx, count_dense) ? 1u : 0u;
+          my_local += row_is_local(p[u], mn, mx, B.ncols) ? 1u : 0u;
           cmin[r] = mn;
           cmax[r] = mx;
         }
@@ -280,6 +292,7 @@ __global__ void __launch_bounds__(256) k_analyse_short(Csr A, Csr B, long long r
   if (gl == 0 && my_wide) atomicAdd(&s_wide, my_wide);
   if (gl == 0 && my_wide8) atomicAdd(&s_wide8, my_wide8);
   if (gl == 0 && my_dense) atomicAdd(&s_dense, my_dense);
+  if (gl == 0 && my_local) atomicAdd(&s_local, my_local);
   if (__any_sync(FULL, bad) && lane == 0) atomicOr(&st->err, EB_UNSORTED);
   __syncthreads();
   if (threadIdx.x < NBINS && s_hist[threadIdx.x]) atomicAdd(&st->hist[threadIdx.x], s_hist[threadIdx.x]);
@@ -290,6 +303,7 @@ __global__ void __launch_bounds__(256) k_analyse_short(Csr A, Csr B, long long r
   if (threadIdx.x == 0 && s_wide) atomicAdd(&st->rows_wide, s_wide);
   if (threadIdx.x == 0 && s_wide8) atomicAdd(&st->rows_wide8, s_wide8);
   if (threadIdx.x == 0 && s_dense) atomicAdd(&st->rows_dense, s_dense);
+  if (threadIdx.x == 0 && s_local) atomicAdd(&st->rows_local, s_local);
 }
 
 // Counting sort of the non-empty rows by bin, largest bin first.  Each block

@@ -840,6 +840,7 @@ spgemm_status spgemm_backward(spgemm_plan* p, const void* a_vals, const void* b_
   g.nnz_c = p->nnz_c;
   g.max_col = p->host_st.max_col;
   g.max_row_b = p->host_st.max_row_b;
+  g.rows_local = (long long)p->host_st.rows_local;
   g.hist = p->host_st.hist;
   g.buf = p->grad_buf;
   g.buf_entries = p->grad_buf_entries;

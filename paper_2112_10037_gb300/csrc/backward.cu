@@ -812,9 +812,15 @@ struct GradRoute {
 // group of lanes walks the longest of eight rows of B, so that on power-law
 // graphs, whose products come from rows of B many times the average (weighted
 // by their use 22 times on an R-MAT of 32,768 columns), most lanes wait: dA there
-// 4.49 ms staged, 1.57 with searches.  At most 4 times the average.  A row of B
-// of more than 128 entries is summed by 32 lanes, or not here.  The choice
-// depends on the plan alone: dA has the same bits with dB and without.
+// 4.49 ms staged, 1.57 with searches.  At most 4 times the average, 8 with 32
+// lanes (R-MAT of 2,000 vertices, edge factor 32: 0.25 and 0.40; of 9,000: 1.89
+// and 1.16).  A row of B of more than 128 entries is summed by 32 lanes, or not
+// here.  The choice depends on the plan alone: dA has the same bits with dB and
+// without.  Where most rows stay inside half of B's columns, searches meet each
+// other's cache lines and cost a fifth (6 ps a term instead of 30), and neither
+// staging nor more than one chunk pays: 27-point stencil on 40^3 points, FP64,
+// both gradients 0.96 ms and 0.52 with searches, blocks of 64 (20,032 rows) 2.20
+// and 1.06, a band of 41 entries (20,000 rows) 0.63 and 0.35.
 //
 // Through the buffer dB shares dA's searches, or staged rows' look-ups.  Alone
 // and without either a search per term is no more work (40^3 stencil, FP64: 37 us
@@ -851,9 +857,10 @@ static GradRoute grad_route(const GradArgs& g, bool da, bool db) {
   while (r.wlog < widest && (1ll << r.wlog) < g.B.ncols) ++r.wlog;
   const double avg = g.B.nrows > 0 ? (double)g.B.nnz / (double)g.B.nrows : 0.0;
   r.lanes = avg >= 20 ? 32 : (avg >= 10 ? 16 : 8);
+  const bool local = 2 * g.rows_local > r.rows;
   const double share = g.A.nrows > 0 ? (double)g.ri.mloc / (double)g.A.nrows : 0.0;  // of A's nonzeros, about
   r.staged = has_buffer && g.total >= (sizeof(T) == 8 ? 512 : 384) * all && 2 * r.rows > all && (1ll << r.wlog) >= g.B.ncols &&
-             (double)g.total <= 4.0 * avg * share * (double)g.A.nnz &&
+             (double)g.total <= (r.lanes == 32 ? 8.0 : 4.0) * avg * share * (double)g.A.nnz && !local &&
              (r.lanes == 32 || g.max_row_b <= GRAD_LANE_MAX);
   const long long longest = g.B.ncols < g.B.nnz ? g.B.ncols : g.B.nnz;
   r.chunk = g.buf_entries - longest;
@@ -862,7 +869,7 @@ static GradRoute grad_route(const GradArgs& g, bool da, bool db) {
     const double chunks = (double)((g.total + r.chunk - 1) / r.chunk);
     const double terms = (double)g.total / (chunks * (double)g.B.nnz);
     const double steps = log2(1.0 + (double)g.nnz_c / (double)(all > 0 ? all : 1));
-    r.buffered = g.max_col <= GRAD_LANE_MAX && terms * steps >= 15.0;
+    r.buffered = g.max_col <= GRAD_LANE_MAX && !local && terms * steps >= 15.0;
   }
   return r;
 }

@@ -49,6 +49,7 @@ struct DevStats {
   uint32_t rows_wide;  // rows of the plan with more than 32 nonzeros of A
   uint32_t rows_wide8;  // rows with more than 8 (LANE_MERGE_K)
   uint32_t rows_dense;  // rows of many products per window of columns (row_is_dense)
+  uint32_t rows_local;  // rows of more than 128 products inside half of B's columns
   int max_col, max_row_b;  // nonzeros of A's longest column and B's longest row (plans for the adjoint)
   int hist[NBINS];   // rows per bin
   int fill[NBINS];   // scatter cursors
@@ -407,6 +408,7 @@ struct GradArgs {
   long long total;   // products of the plan's rows
   long long nnz_c;   // entries of C
   int max_col, max_row_b;      // nonzeros of A's longest column and of B's longest row
+  long long rows_local;        // rows of more than 128 products inside half of B's columns
   const int* hist;   // host: rows per bin
   void* buf;
   long long buf_entries;

@@ -166,17 +166,22 @@ def test_staged_rows(api, oracle_mod, blen, ncols, dtype, tol):
     assert max_rel_err(db.double().cpu().numpy(), rb, sb) <= tol
 
 
-@pytest.mark.parametrize("kind", ["stencil", "power", "short"])
+@pytest.mark.parametrize("kind", ["stencil", "power", "short", "band"])
 def test_searched_rows(api, oracle_mod, kind):
     """Products that staged rows or a buffer in chunks would slow down: a stencil
-    of three chunks (a search per term of each gradient), a power-law graph and
-    uniform rows of few products (one search for both, then the columns).  dA
-    alone is one launch, and the same bits."""
+    of three chunks and a band of two (a search per term of each gradient), a
+    power-law graph and uniform rows of few products (one search for both, then
+    the columns).  dA alone is one launch, and the same bits."""
     rng = np.random.default_rng(2)
     if kind == "stencil":
         A = gen.laplacian_3d(80)
     elif kind == "power":
         A = gen.rmat(11, 16, seed=3)
+    elif kind == "band":
+        cols = np.arange(9000)[:, None] + np.arange(-16, 17)[None, :]
+        ok = (cols >= 0) & (cols < 9000)
+        A = gen.CSR(9000, 9000, np.concatenate([[0], np.cumsum(ok.sum(1))]).astype(np.int32),
+                    cols[ok].astype(np.int32), rng.standard_normal(int(ok.sum()))).check()
     else:
         A = gen.random_rows(20000, 20000, rng.integers(6, 13, 20000), rng)
     da, db, n, W = _run(api, A, A, torch.float64)
