@@ -625,8 +625,9 @@ k_grad_slabs(Csr A, Csr B, const T* __restrict__ bv, RowInfo ri, const int32_t* 
 // tree; their chains cannot be taken up from one number, so they are summed here
 // only when one chunk holds every product (LONG; a kernel of its own, because
 // its registers leave fewer warps), by the whole block: warp w runs the chains
-// w, w + 8, w + 16 and w + 24 of the slab's 32 outputs, each lane an output.  (FP32, positive terms, root mean square error over the sum:
-// 512 terms 3.0e-7 in one chain, 4.5e-8 in 32.)
+// w, w + 8, w + 16 and w + 24 of the slab's 32 outputs, each lane an output.
+// (FP32, positive terms, root mean square error over the sum: 512 terms 3.0e-7
+// in one chain, 4.5e-8 in 32.)
 template <typename T>
 __device__ __forceinline__ T grad_col_sum(const T* __restrict__ av, const int32_t* __restrict__ t_src,
                                           const long long* __restrict__ t_off, const T* __restrict__ buf,
@@ -859,8 +860,9 @@ static GradRoute grad_route(const GradArgs& g, bool da, bool db) {
   r.lanes = avg >= 20 ? 32 : (avg >= 10 ? 16 : 8);
   const bool local = 2 * g.rows_local > r.rows;
   const double share = g.A.nrows > 0 ? (double)g.ri.mloc / (double)g.A.nrows : 0.0;  // of A's nonzeros, about
-  r.staged = has_buffer && g.total >= (sizeof(T) == 8 ? 512 : 384) * all && 2 * r.rows > all && (1ll << r.wlog) >= g.B.ncols &&
-             (double)g.total <= (r.lanes == 32 ? 8.0 : 4.0) * avg * share * (double)g.A.nnz && !local &&
+  const double alike = (r.lanes == 32 ? 8.0 : 4.0) * avg * share * (double)g.A.nnz;
+  r.staged = has_buffer && !local && 2 * r.rows > all && g.total >= (sizeof(T) == 8 ? 512 : 384) * all &&
+             (1ll << r.wlog) >= g.B.ncols && (double)g.total <= alike &&
              (r.lanes == 32 || g.max_row_b <= GRAD_LANE_MAX);
   const long long longest = g.B.ncols < g.B.nnz ? g.B.ncols : g.B.nnz;
   r.chunk = g.buf_entries - longest;
