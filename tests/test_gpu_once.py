@@ -151,3 +151,15 @@ def test_fp32_products_that_meet_are_fused(api, nrows, width):
     err = (x[:, None] * y).astype(np.float64) - x[:, None].astype(np.float64) * y
     assert np.count_nonzero(err) > 0.9 * err.size
     assert np.array_equal(np.abs(got.vals.reshape(nrows, width).astype(np.float64)), np.abs(err))
+
+
+def test_fp32_infinities_and_nan(api, oracle_mod):
+    """The same for FP32, whose products are fused by compare-and-swap."""
+    A, B = _operands(5000, "meet", 7)
+    A.vals[::37], A.vals[5::91], B.vals[3::113] = np.inf, np.nan, -np.inf
+    got = api.spgemm(*(api.DeviceCSR.from_host(M, dtype=torch.float32) for M in (A, B))).to_host()
+    R = oracle_mod.spgemm(A, B)
+    assert_structure_equal(got, R)
+    assert np.array_equal(np.isnan(got.vals), np.isnan(R.vals))
+    inf = np.isinf(R.vals)
+    assert np.array_equal(got.vals[inf], R.vals[inf]) and np.array_equal(np.isinf(got.vals), inf)
