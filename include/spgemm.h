@@ -259,7 +259,8 @@ spgemm_status spgemm_plan_check(spgemm_plan* plan, spgemm_stream_t stream);
  * summed in a fixed order, so the result is deterministic (the same bits on
  * every call): db_vals by one chain of fused multiply-adds for at most 128
  * terms (nonzeros of A's column), otherwise by 32 chains of every 32nd term and
- * a fixed tree; da_vals by chains of at most 128 terms and a fixed tree.
+ * a fixed tree; da_vals the same (terms: entries of B's row) or, where the plan's
+ * rows suit it, by 8, 16 or 32 such chains and a tree whatever the terms.
  * db_vals may pass through a buffer in the plan's workspace (at most 64 MB and
  * the longest row of B): such calls on one plan follow one another on the GPU,
  * whatever streams they are given.  A captured call does not use the buffer, so
